@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(kBT) k_weight_grad(int64_t n, int d, int k,
                                                      const double* __restrict__ f,
                                                      const float* __restrict__ ls,
                                                      float* __restrict__ dX) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const int D = d + 1;
@@ -101,6 +102,7 @@ __global__ void k_filter_in(int64_t n, int d, int k, int col0, int kc,
                             const float* __restrict__ X, const float* __restrict__ ls,
                             const float* __restrict__ V, const float* __restrict__ G,
                             float* __restrict__ out) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n * kc) return;
   const int64_t i = e / kc;
@@ -126,6 +128,7 @@ __global__ void k_filter_acc(int64_t n, int d, int k, int col0, int kc,
                              const float* __restrict__ X, const float* __restrict__ ls,
                              const float* __restrict__ V, const float* __restrict__ G,
                              const float* __restrict__ F, float* __restrict__ dZ) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int kd = k * d;
@@ -150,6 +153,7 @@ __global__ void k_filter_acc(int64_t n, int d, int k, int col0, int kc,
 
 __global__ void k_filter_finish(int64_t n, int d, float scale, const float* __restrict__ ls,
                                 float* __restrict__ dX) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n * d) return;
   dX[e] = scale * dX[e] / ls[e % d];
@@ -161,6 +165,7 @@ __global__ void k_filter_finish(int64_t n, int d, float scale, const float* __re
 __global__ void __launch_bounds__(256) k_dls_partial(int64_t n, int d, const float* __restrict__ X,
                                                      const float* __restrict__ dX,
                                                      double* __restrict__ partial) {
+  pdl_enter();
   __shared__ double sh[256];
   const int P = 256 / d;
   const int t = threadIdx.x;
@@ -182,6 +187,7 @@ __global__ void __launch_bounds__(256) k_dls_partial(int64_t n, int d, const flo
 
 __global__ void k_dls_final(int nblk, int d, const double* __restrict__ partial,
                             const float* __restrict__ ls, float* __restrict__ dls) {
+  pdl_enter();
   const int j = threadIdx.x;
   if (j >= d) return;
   double s = 0.0;
@@ -216,7 +222,7 @@ void launch_weight_grad(const Lattice* L, int k, const void* BU, const void* BS,
   const unsigned grid = (unsigned)ceil_div(L->n, kBT);
   const int D = L->D;
 #define SGP_WG(MAXD)                                                                        \
-  k_weight_grad<MAXD, VEC, S><<<grid, kBT, 0, st>>>(L->n, L->d, k, L->perm, L->idx, L->rank, \
+  launch_pdl(k_weight_grad<MAXD, VEC, S>, grid, kBT, st, L->n, L->d, k, L->perm, L->idx, L->rank, \
                                                     (const S*)BU, (const S*)BS, Vp, Gp,      \
                                                     alpha, f, ls, dX)
   if (D <= 8) SGP_WG(8);
@@ -298,23 +304,23 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
       BW_CHECK(cudaMemsetAsync(dXw, 0, (size_t)n * d * sizeof(float), st), "clear dX");
       for (int col0 = 0; col0 < kk; col0 += chunk) {
         const int kc = std::min(chunk, kk - col0);
-        k_filter_in<<<(unsigned)ceil_div(n * kc, 256), 256, 0, st>>>(n, d, k, col0, kc, X, ls, V,
+        launch_pdl(k_filter_in, (unsigned)ceil_div(n * kc, 256), 256, st, n, d, k, col0, kc, X, ls, V,
                                                                       G, in);
         enqueue_mvm(L, in, kc, blur, 1.f, 0.f, F, st);
-        k_filter_acc<<<(unsigned)ceil_div(n, kBT), kBT, 0, st>>>(n, d, k, col0, kc, X, ls, V, G,
+        launch_pdl(k_filter_acc, (unsigned)ceil_div(n, kBT), kBT, st, n, d, k, col0, kc, X, ls, V, G,
                                                                  F, dXw);
         note_launches(2);
       }
       // dz = 2 alpha (k'/k) dZ with k' = -k/2 for the RBF; dX = dz / l
-      k_filter_finish<<<(unsigned)ceil_div(n * d, 256), 256, 0, st>>>(n, d, -alpha, ls, dXw);
+      launch_pdl(k_filter_finish, (unsigned)ceil_div(n * d, 256), 256, st, n, d, -alpha, ls, dXw);
       note_launches(1);
     }
   }
   if (dls) {
     double* part = nullptr;
     BW_CHECK(w.get(&part, (size_t)kDlsBlocks * d * sizeof(double)), "alloc partials");
-    k_dls_partial<<<kDlsBlocks, 256, 0, st>>>(n, d, X, dXw, part);
-    k_dls_final<<<1, 128, 0, st>>>(kDlsBlocks, d, part, ls, dls);
+    launch_pdl(k_dls_partial, kDlsBlocks, 256, st, n, d, X, dXw, part);
+    launch_pdl(k_dls_final, 1, 128, st, kDlsBlocks, d, part, ls, dls);
     note_launches(2);
   }
   BW_CHECK(cudaGetLastError(), "launching the MVM backward");

@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(128) k_elevate(const float* __restrict__ X,
                                                  float* __restrict__ w_out,
                                                  int* __restrict__ qmin, int* __restrict__ qmax,
                                                  unsigned* __restrict__ err, int inject_nan) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int D = d + 1;
@@ -218,6 +219,7 @@ struct CellPack {
 
 __global__ void k_point_key(const int16_t* __restrict__ rem0, int64_t n, int D, CellPack pk,
                             uint32_t* __restrict__ key, uint32_t* __restrict__ val) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   uint32_t k = 0;
@@ -237,6 +239,7 @@ __global__ void __launch_bounds__(256) k_insert(const int32_t* __restrict__ perm
                                                 int d, unsigned long long* __restrict__ table,
                                                 uint64_t mask, int32_t* __restrict__ entry_slot,
                                                 unsigned* __restrict__ err) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nD) return;
   const int D = d + 1;
@@ -272,6 +275,7 @@ __global__ void __launch_bounds__(256) k_insert(const int32_t* __restrict__ perm
 __global__ void k_owner_flags(const int32_t* __restrict__ entry_slot,
                               const unsigned long long* __restrict__ table, int64_t nD,
                               uint32_t* __restrict__ flags) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nD) return;
   const int32_t s = entry_slot[e];
@@ -286,6 +290,7 @@ __global__ void k_assign_ids(const uint32_t* __restrict__ scanned,
                              int32_t* __restrict__ slot_id, int16_t* __restrict__ keys,
                              uint64_t* __restrict__ vhash, int2* __restrict__ vrange,
                              uint32_t* __restrict__ bloom, uint64_t bloom_mask) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nD) return;
   const int32_t s = entry_slot[e];
@@ -336,6 +341,7 @@ __global__ void k_entry_ids(const int32_t* __restrict__ entry_slot,
                             const uint8_t* __restrict__ rank_user, int64_t nD, int D,
                             int32_t* __restrict__ idx, float* __restrict__ w,
                             uint8_t* __restrict__ rank) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nD) return;
   const int32_t s = entry_slot[e];
@@ -382,6 +388,7 @@ __global__ void __launch_bounds__(256) k_neighbours(
     const int16_t* __restrict__ rem0, const uint8_t* __restrict__ rank,
     const uint32_t* __restrict__ bloom, uint64_t bloom_mask, int32_t* __restrict__ nbr,
     unsigned long long* __restrict__ counts, uint32_t* __restrict__ hasnb) {
+  pdl_enter();
   __shared__ unsigned block_count[kMaxD];  // this block's vertices with a neighbour along j
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int D = d + 1;
@@ -482,6 +489,7 @@ constexpr int kFillThreads = 512;
 __global__ void __launch_bounds__(kFillThreads) k_active_fill(
     const uint32_t* __restrict__ hasnb, int64_t m, int D, const int64_t* __restrict__ off,
     unsigned long long* __restrict__ fill, int32_t* __restrict__ act) {
+  pdl_enter();
   constexpr int kWarps = kFillThreads / 32;
   __shared__ unsigned wpos[kWarps][kMaxD];  // counts, then each warp's offset in the list
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -532,6 +540,7 @@ __global__ void __launch_bounds__(kFillThreads) k_active_fill(
 __global__ void k_splat_items(const uint32_t* __restrict__ sorted_entries,
                               const float* __restrict__ w,
                               int64_t nD, int D, int2* __restrict__ items) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= nD) return;
   const uint32_t e = sorted_entries[p];
@@ -542,6 +551,7 @@ __global__ void k_splat_items(const uint32_t* __restrict__ sorted_entries,
 __global__ void k_seg_count(const int32_t* __restrict__ row_ptr, int64_t m,
                             uint32_t* __restrict__ nseg, uint32_t* __restrict__ nslot,
                             uint32_t* __restrict__ med, uint32_t* __restrict__ huge) {
+  pdl_enter();
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= m) return;
   const int len = row_ptr[v + 1] - row_ptr[v];
@@ -559,6 +569,7 @@ __global__ void k_seg_fill(const int32_t* __restrict__ row_ptr, int64_t m,
                            const uint32_t* __restrict__ med_off,
                            const uint32_t* __restrict__ huge_off, int4* __restrict__ seg,
                            int4* __restrict__ med_rows, int4* __restrict__ huge_rows) {
+  pdl_enter();
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= m) return;
   const int b = row_ptr[v], e = row_ptr[v + 1];
@@ -582,6 +593,7 @@ constexpr int kSegWindow = 128;
 __global__ void __launch_bounds__(kSegWindow) k_seg_window_sort(const int4* __restrict__ in,
                                                                 int64_t nseg,
                                                                 int4* __restrict__ out) {
+  pdl_enter();
   __shared__ int len[kSegWindow];
   const int64_t s = (int64_t)blockIdx.x * kSegWindow + threadIdx.x;
   const int4 sg = s < nseg ? in[s] : make_int4(0, 0, 0, 0);
@@ -598,12 +610,14 @@ __global__ void __launch_bounds__(kSegWindow) k_seg_window_sort(const int4* __re
 }
 
 __global__ void k_iota(uint32_t* __restrict__ out, int64_t count) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p < count) out[p] = (uint32_t)p;
 }
 
 __global__ void k_row_ptr(const uint32_t* __restrict__ sorted_ids, int64_t nD, int64_t m,
                           int32_t* __restrict__ row_ptr) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p > nD) return;
   if (p == nD) {
@@ -645,11 +659,11 @@ int bits_for(uint64_t v) {  // bits needed to hold values 0..v
 
 #define SGP_DISPATCH_D(D, KERNEL, GRID, BLOCK, ST, ...)                            \
   do {                                                                              \
-    if ((D) <= 8) KERNEL<8><<<(GRID), (BLOCK), 0, (ST)>>>(__VA_ARGS__);             \
-    else if ((D) <= 16) KERNEL<16><<<(GRID), (BLOCK), 0, (ST)>>>(__VA_ARGS__);      \
-    else if ((D) <= 32) KERNEL<32><<<(GRID), (BLOCK), 0, (ST)>>>(__VA_ARGS__);      \
-    else if ((D) <= 64) KERNEL<64><<<(GRID), (BLOCK), 0, (ST)>>>(__VA_ARGS__);      \
-    else KERNEL<128><<<(GRID), (BLOCK), 0, (ST)>>>(__VA_ARGS__);                    \
+    if ((D) <= 8) launch_pdl(KERNEL<8>, (GRID), (BLOCK), (ST), __VA_ARGS__);             \
+    else if ((D) <= 16) launch_pdl(KERNEL<16>, (GRID), (BLOCK), (ST), __VA_ARGS__);      \
+    else if ((D) <= 32) launch_pdl(KERNEL<32>, (GRID), (BLOCK), (ST), __VA_ARGS__);      \
+    else if ((D) <= 64) launch_pdl(KERNEL<64>, (GRID), (BLOCK), (ST), __VA_ARGS__);      \
+    else launch_pdl(KERNEL<128>, (GRID), (BLOCK), (ST), __VA_ARGS__);                    \
     note_launches(1);                                                               \
   } while (0)
 
@@ -762,7 +776,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     SGP_CHECK(tmp.get(&kb, n), "alloc sort");
     SGP_CHECK(tmp.get(&vb, n), "alloc sort");
     SGP_CHECK(tmp.get(&rt, radix_temp_elems(n)), "alloc sort");
-    k_point_key<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(rem0, n, D, pk, ka, va);
+    launch_pdl(k_point_key, (unsigned)ceil_div(n, 256), 256, st, rem0, n, D, pk, ka, va);
     note_launches(1);
     // the packed cell occupies the top `used` bits; bits below are zero
     const bool in_alt = used > 0 ? radix_sort_pairs(ka, va, kb, vb, n, 32, rt, st) : false;
@@ -792,7 +806,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   SGP_CHECK(tmp.get(&flags, nD), "alloc flags");
   SGP_CHECK(tmp.get(&scan_tmp, scan_temp_elems(nD)), "alloc scan");
   SGP_CHECK(tmp.get(&total, 1), "alloc total");
-  k_owner_flags<<<(unsigned)ceil_div(nD, 256), 256, 0, st>>>(entry_slot, table, nD, flags);
+  launch_pdl(k_owner_flags, (unsigned)ceil_div(nD, 256), 256, st, entry_slot, table, nD, flags);
   note_launches(1);
   exclusive_scan_u32(flags, nD, total, scan_tmp, st);
   uint32_t hm = 0;
@@ -820,7 +834,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   uint32_t* bloom = nullptr;
   SGP_CHECK(tmp.get(&bloom, bloom_bits / 32), "alloc vertex filter");
   SGP_CHECK(cudaMemsetAsync(bloom, 0, bloom_bits / 8, st), "clear vertex filter");
-  k_assign_ids<<<(unsigned)ceil_div(nD, 256), 256, 0, st>>>(flags, entry_slot, table, L->perm,
+  launch_pdl(k_assign_ids, (unsigned)ceil_div(nD, 256), 256, st, flags, entry_slot, table, L->perm,
                                                            rem0, rank, nD, d, slot_id, L->keys,
                                                            vhash, vrange, bloom, bloom_bits - 1);
   note_launches(1);
@@ -828,7 +842,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   SGP_CHECK(dalloc(&L->w, nD, st), "alloc w");
   SGP_CHECK(dalloc(&L->rank, nD, st), "alloc rank");
   L->bytes += nD * (sizeof(int32_t) + sizeof(float) + sizeof(uint8_t));
-  k_entry_ids<<<(unsigned)ceil_div(nD, 256), 256, 0, st>>>(entry_slot, slot_id, L->perm, w_user,
+  launch_pdl(k_entry_ids, (unsigned)ceil_div(nD, 256), 256, st, entry_slot, slot_id, L->perm, w_user,
                                                           rank, nD, D, L->idx, L->w, L->rank);
   note_launches(1);
   SGP_CHECK(cudaGetLastError(), "numbering");
@@ -845,7 +859,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     // sum_c A_c over the D coordinates, as the kernels compute A_c
     uint64_t sum_A = 0;
     for (int c = 0; c < D; ++c) sum_A += host_coord_mult(c);
-    k_neighbours<<<(unsigned)ceil_div(m, 256), 256, 0, st>>>(
+    launch_pdl(k_neighbours, (unsigned)ceil_div(m, 256), 256, st, 
         L->keys, vhash, vrange, m, d, r, sum_A, table, mask, slot_id, L->perm, rem0, rank,
         bloom, bloom_bits - 1, L->nbr, counts, hasnb);
     note_launches(1);
@@ -862,7 +876,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     SGP_CHECK(tmp.get(&rt, radix_temp_elems(nD)), "alloc csr");
     SGP_CHECK(cudaMemcpyAsync(ka, L->idx, nD * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st),
               "copy ids");
-    k_iota<<<(unsigned)ceil_div(nD, 256), 256, 0, st>>>(va, nD);
+    launch_pdl(k_iota, (unsigned)ceil_div(nD, 256), 256, st, va, nD);
     note_launches(1);
     const int bits = std::max(1, bits_for((uint64_t)(m > 0 ? m - 1 : 0)));
     const bool in_alt = radix_sort_pairs(ka, va, kb, vb, nD, bits, rt, st);
@@ -871,10 +885,10 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     SGP_CHECK(dalloc(&L->items, nD, st), "alloc items");
     SGP_CHECK(dalloc(&L->row_ptr, m + 1, st), "alloc row_ptr");
     L->bytes += nD * sizeof(int2) + (m + 1) * sizeof(int32_t);
-    k_splat_items<<<(unsigned)ceil_div(nD, 256), 256, 0, st>>>(sorted_entries, L->w, nD, D,
+    launch_pdl(k_splat_items, (unsigned)ceil_div(nD, 256), 256, st, sorted_entries, L->w, nD, D,
                                                               L->items);
     note_launches(1);
-    k_row_ptr<<<(unsigned)ceil_div(nD + 1, 256), 256, 0, st>>>(sorted_ids, nD, m, L->row_ptr);
+    launch_pdl(k_row_ptr, (unsigned)ceil_div(nD + 1, 256), 256, st, sorted_ids, nD, m, L->row_ptr);
     note_launches(1);
     SGP_CHECK(cudaGetLastError(), "splat lists");
   }
@@ -888,7 +902,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     SGP_CHECK(tmp.get(&huge, m), "alloc seg");
     SGP_CHECK(tmp.get(&tot, 4), "alloc seg");
     SGP_CHECK(tmp.get(&stmp, scan_temp_elems(m)), "alloc seg");
-    k_seg_count<<<(unsigned)ceil_div(m, 256), 256, 0, st>>>(L->row_ptr, m, cnt, slots, med, huge);
+    launch_pdl(k_seg_count, (unsigned)ceil_div(m, 256), 256, st, L->row_ptr, m, cnt, slots, med, huge);
     note_launches(1);
     exclusive_scan_u32(cnt, m, tot + 0, stmp, st);
     exclusive_scan_u32(slots, m, tot + 1, stmp, st);
@@ -907,11 +921,11 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     L->bytes += (L->nseg + L->nmed + L->nhuge) * sizeof(int4);
     int4* seg_unsorted = nullptr;
     SGP_CHECK(tmp.get(&seg_unsorted, std::max<int64_t>(L->nseg, 1)), "alloc seg");
-    k_seg_fill<<<(unsigned)ceil_div(m, 256), 256, 0, st>>>(L->row_ptr, m, cnt, slots, med, huge,
+    launch_pdl(k_seg_fill, (unsigned)ceil_div(m, 256), 256, st, L->row_ptr, m, cnt, slots, med, huge,
                                                           seg_unsorted, L->med_rows,
                                                           L->huge_rows);
     if (L->nseg > 0)
-      k_seg_window_sort<<<(unsigned)ceil_div(L->nseg, kSegWindow), kSegWindow, 0, st>>>(
+      launch_pdl(k_seg_window_sort, (unsigned)ceil_div(L->nseg, kSegWindow), kSegWindow, st, 
           seg_unsorted, L->nseg, L->seg);
     note_launches(2);
     SGP_CHECK(cudaGetLastError(), "splat segments");
@@ -940,7 +954,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
       SGP_CHECK(cudaMemcpyAsync(L->act_off_dev, L->act_off.data(), (D + 1) * sizeof(int64_t),
                                 cudaMemcpyHostToDevice, st),
                 "copy list offsets");
-      k_active_fill<<<(unsigned)ceil_div(m, kFillThreads), kFillThreads, 0, st>>>(
+      launch_pdl(k_active_fill, (unsigned)ceil_div(m, kFillThreads), kFillThreads, st, 
           hasnb, m, D, L->act_off_dev, counts + D, L->act);
       note_launches(1);
       // powers of the symmetric blur's centre tap g_0 (stored rows are rescaled lazily)

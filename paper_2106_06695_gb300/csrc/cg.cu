@@ -77,6 +77,7 @@ __global__ void k_cg_init(const float* __restrict__ B, int kb, const int32_t* __
                           float* __restrict__ xh, float* __restrict__ xl,
                           float* __restrict__ rh, float* __restrict__ rl, float* __restrict__ p,
                           int64_t n, int k, double* __restrict__ partial) {
+  pdl_enter();
   dfloat acc[VEC];
 #pragma unroll
   for (int j = 0; j < VEC; ++j) acc[j] = {0.f, 0.f};
@@ -120,6 +121,7 @@ __device__ __forceinline__ double column_total(const double* __restrict__ partia
 
 __global__ void k_cg_init_scalars(const double* __restrict__ partial, int nblk, int k,
                                   float tol, int max_iter, CgState S) {
+  pdl_enter();
   const double rr = column_total(partial, nblk, k);
   if (threadIdx.x != 0) return;
   const int c = blockIdx.x;
@@ -139,6 +141,7 @@ __global__ void k_cg_init_scalars(const double* __restrict__ partial, int nblk, 
 
 // <p, A p> from the slice's block partials, then alpha = rho / <p, A p>.
 __global__ void k_cg_alpha(int nblk, int k, CgState S) {
+  pdl_enter();
   const double pap = column_total(S.partial, nblk, k);
   if (threadIdx.x != 0) return;
   const int c = blockIdx.x;
@@ -163,6 +166,7 @@ __global__ void k_cg_update_xr(float* __restrict__ xh, float* __restrict__ xl,
                                float* __restrict__ rh, float* __restrict__ rl,
                                const float* __restrict__ p, const float* __restrict__ Ap,
                                int64_t n, int k, CgState S) {
+  pdl_enter();
   dfloat acc[VEC], a[VEC], na[VEC];
   bool on[VEC];
   {
@@ -223,6 +227,7 @@ __global__ void k_cg_update_xr(float* __restrict__ xh, float* __restrict__ xl,
 }
 
 __global__ void k_cg_beta(int nblk, int k, float tol, int max_iter, CgState S) {
+  pdl_enter();
   const double rr = column_total(S.partial, nblk, k);
   if (threadIdx.x != 0) return;
   const int c = blockIdx.x;
@@ -243,6 +248,7 @@ __global__ void k_cg_beta(int nblk, int k, float tol, int max_iter, CgState S) {
 
 // Preconditioned CG: convergence check on <r, r> (no beta yet).
 __global__ void k_cg_check(int nblk, int k, float tol, int max_iter, CgState S) {
+  pdl_enter();
   const double rr = column_total(S.partial, nblk, k);
   if (threadIdx.x != 0) return;
   const int c = blockIdx.x;
@@ -257,6 +263,7 @@ __global__ void k_cg_check(int nblk, int k, float tol, int max_iter, CgState S) 
 
 // Preconditioned CG: rho = <r, z> at the start.
 __global__ void k_cg_rho_init(int nblk, int k, CgState S) {
+  pdl_enter();
   const double rz = column_total(S.partial, nblk, k);
   if (threadIdx.x != 0) return;
   const int c = blockIdx.x;
@@ -266,6 +273,7 @@ __global__ void k_cg_rho_init(int nblk, int k, CgState S) {
 
 // Preconditioned CG: beta = <r, z>_new / <r, z>_old on active columns.
 __global__ void k_cg_beta_pcg(int nblk, int k, CgState S) {
+  pdl_enter();
   const double rz = column_total(S.partial, nblk, k);
   if (threadIdx.x != 0) return;
   const int c = blockIdx.x;
@@ -282,6 +290,7 @@ __global__ void k_cg_beta_pcg(int nblk, int k, CgState S) {
 template <int VEC, bool FIRST>
 __global__ void k_cg_update_p_z(float* __restrict__ p, const float* __restrict__ z, int64_t n,
                                 int k, CgState S) {
+  pdl_enter();
   dfloat b[VEC];
   bool on[VEC];
   {
@@ -314,6 +323,7 @@ __global__ void k_cg_update_p_z(float* __restrict__ p, const float* __restrict__
 template <int VEC>
 __global__ void k_cg_update_p(float* __restrict__ p, const float* __restrict__ rh,
                               const float* __restrict__ rl, int64_t n, int k, CgState S) {
+  pdl_enter();
   dfloat b[VEC];
   bool on[VEC];
   {
@@ -345,6 +355,7 @@ template <int VEC>
 __global__ void k_cg_store_x(const float* __restrict__ xh, const float* __restrict__ xl,
                              const int32_t* __restrict__ perm, float* __restrict__ X, int kb,
                              int64_t n, int k) {
+  pdl_enter();
   SGP_ROWS_LOOP(row) {
     float hv[VEC], lv[VEC];
     ldf<VEC>(xh + row * k + c0, hv);
@@ -469,16 +480,16 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
   }
 
   if (vec == 4)
-    k_cg_init<4><<<vblocks, T, 0, st>>>(B, kb, L->perm, xh, xl, rh, rl, p, n, k, S.partial);
+    launch_pdl(k_cg_init<4>, vblocks, T, st, B, kb, L->perm, xh, xl, rh, rl, p, n, k, S.partial);
   else
-    k_cg_init<1><<<vblocks, T, 0, st>>>(B, kb, L->perm, xh, xl, rh, rl, p, n, k, S.partial);
-  k_cg_init_scalars<<<k, 256, 0, st>>>(S.partial, vblocks, k, tol, max_iter, S);
+    launch_pdl(k_cg_init<1>, vblocks, T, st, B, kb, L->perm, xh, xl, rh, rl, p, n, k, S.partial);
+  launch_pdl(k_cg_init_scalars, k, 256, st, S.partial, vblocks, k, tol, max_iter, S);
   note_launches(2);
   if (use_pre) {  // z = P^-1 r, rho = <r, z>, p = z
     cl.pre.apply(rh, rl, k, z, S.partial, st);
-    k_cg_rho_init<<<k, 256, 0, st>>>((int)cl.pre.dot_blocks(), k, S);
-    if (vec == 4) k_cg_update_p_z<4, true><<<vblocks, T, 0, st>>>(p, z, n, k, S);
-    else k_cg_update_p_z<1, true><<<vblocks, T, 0, st>>>(p, z, n, k, S);
+    launch_pdl(k_cg_rho_init, k, 256, st, (int)cl.pre.dot_blocks(), k, S);
+    if (vec == 4) launch_pdl(k_cg_update_p_z<4, true>, vblocks, T, st, p, z, n, k, S);
+    else launch_pdl(k_cg_update_p_z<1, true>, vblocks, T, st, p, z, n, k, S);
     note_launches(2);
   }
   CG_CHECK(cudaGetLastError(), "CG init");
@@ -489,20 +500,20 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
     // Ap = outputscale K~ p + noise p, with the slice also summing <p, Ap> per block
     passes = enqueue_mvm(L, p, k, blur, L->outputscale, noise, Ap, st, ev, /*internal=*/true,
                          S.partial);
-    k_cg_alpha<<<k, 256, 0, st>>>((int)sblocks, k, S);
-    if (vec == 4) k_cg_update_xr<4><<<vblocks, T, 0, st>>>(xh, xl, rh, rl, p, Ap, n, k, S);
-    else k_cg_update_xr<1><<<vblocks, T, 0, st>>>(xh, xl, rh, rl, p, Ap, n, k, S);
+    launch_pdl(k_cg_alpha, k, 256, st, (int)sblocks, k, S);
+    if (vec == 4) launch_pdl(k_cg_update_xr<4>, vblocks, T, st, xh, xl, rh, rl, p, Ap, n, k, S);
+    else launch_pdl(k_cg_update_xr<1>, vblocks, T, st, xh, xl, rh, rl, p, Ap, n, k, S);
     if (use_pre) {
-      k_cg_check<<<k, 256, 0, st>>>(vblocks, k, tol, max_iter, S);
+      launch_pdl(k_cg_check, k, 256, st, vblocks, k, tol, max_iter, S);
       cl.pre.apply(rh, rl, k, z, S.partial, st, ev ? ev + 4 : nullptr, S.r3 != nullptr);
-      k_cg_beta_pcg<<<k, 256, 0, st>>>((int)cl.pre.dot_blocks(), k, S);
-      if (vec == 4) k_cg_update_p_z<4, false><<<vblocks, T, 0, st>>>(p, z, n, k, S);
-      else k_cg_update_p_z<1, false><<<vblocks, T, 0, st>>>(p, z, n, k, S);
+      launch_pdl(k_cg_beta_pcg, k, 256, st, (int)cl.pre.dot_blocks(), k, S);
+      if (vec == 4) launch_pdl(k_cg_update_p_z<4, false>, vblocks, T, st, p, z, n, k, S);
+      else launch_pdl(k_cg_update_p_z<1, false>, vblocks, T, st, p, z, n, k, S);
       note_launches(5);
     } else {
-      k_cg_beta<<<k, 256, 0, st>>>(vblocks, k, tol, max_iter, S);
-      if (vec == 4) k_cg_update_p<4><<<vblocks, T, 0, st>>>(p, rh, rl, n, k, S);
-      else k_cg_update_p<1><<<vblocks, T, 0, st>>>(p, rh, rl, n, k, S);
+      launch_pdl(k_cg_beta, k, 256, st, vblocks, k, tol, max_iter, S);
+      if (vec == 4) launch_pdl(k_cg_update_p<4>, vblocks, T, st, p, rh, rl, n, k, S);
+      else launch_pdl(k_cg_update_p<1>, vblocks, T, st, p, rh, rl, n, k, S);
       note_launches(4);
     }
   };
@@ -543,8 +554,8 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
       }
     }
   }
-  if (vec == 4) k_cg_store_x<4><<<vblocks, T, 0, st>>>(xh, xl, L->perm, X, kb, n, k);
-  else k_cg_store_x<1><<<vblocks, T, 0, st>>>(xh, xl, L->perm, X, kb, n, k);
+  if (vec == 4) launch_pdl(k_cg_store_x<4>, vblocks, T, st, xh, xl, L->perm, X, kb, n, k);
+  else launch_pdl(k_cg_store_x<1>, vblocks, T, st, xh, xl, L->perm, X, kb, n, k);
   note_launches(1);
   CG_CHECK(cudaGetLastError(), "CG result");
   std::vector<double> hrel(k);

@@ -29,6 +29,7 @@ constexpr int kQlSweeps = 64;  // QL iterations allowed per eigenvalue
 __global__ void k_slq(const double* __restrict__ ha, const double* __restrict__ hb, int k, int cap,
                       const int* __restrict__ iters, const double* __restrict__ bnorm,
                       double* __restrict__ quad, int* __restrict__ bad) {
+  pdl_enter();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= k) return;
   const int m = min(iters[c], cap);
@@ -143,7 +144,7 @@ sgp_status run_logdet(Lattice* L, const float* Z, int s, float noise, int max_la
   sgp_status status = run_cg(L, Z, s, SGP_BLUR_SYMMETRIC, noise, tol, cap, X, nullptr, nullptr,
                              0, 0, &rec);
   if (status != SGP_OK) return status;
-  k_slq<<<(unsigned)ceil_div(s, 64), 64, 0, st>>>(rec.alpha, rec.beta, s, cap, rec.iters,
+  launch_pdl(k_slq, (unsigned)ceil_div(s, 64), 64, st, rec.alpha, rec.beta, s, cap, rec.iters,
                                                    rec.bnorm, dq, bad);
   note_launches(1);
   LZ_CHECK(cudaGetLastError(), "Lanczos quadrature");

@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(kThreads) k_splat(int64_t nseg, int G, int k,
                                                     const float* __restrict__ V,
                                                     S* __restrict__ lat,
                                                     float* __restrict__ partial) {
+  pdl_enter();
   using Vt = Vec<VEC>;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t s = gid / G;
@@ -72,6 +73,7 @@ __global__ void __launch_bounds__(kThreads) k_splat_med(int64_t nrows, int G, in
                                                         const int4* __restrict__ rows,
                                                         const float* __restrict__ partial,
                                                         S* __restrict__ lat) {
+  pdl_enter();
   using Vt = Vec<VEC>;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t q = gid / G;
@@ -89,6 +91,7 @@ template <int VEC, class S>
 __global__ void __launch_bounds__(kThreads) k_splat_huge(int G, int k, const int4* __restrict__ rows,
                                                          const float* __restrict__ partial,
                                                          S* __restrict__ lat) {
+  pdl_enter();
   using Vt = Vec<VEC>;
   __shared__ typename Vt::T red[kThreads];
   const int groups = blockDim.x / G;
@@ -114,6 +117,7 @@ template <class S>
 __global__ void __launch_bounds__(kThreads) k_blur(int64_t m, int k, int r, Taps tp,
                                                    const int32_t* __restrict__ nbr,
                                                    const S* __restrict__ in, S* __restrict__ out) {
+  pdl_enter();
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t v = gid / k;
   if (v >= m) return;
@@ -139,6 +143,7 @@ __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k,
                                                         const int32_t* __restrict__ nbr,
                                                         const S* __restrict__ in,
                                                         S* __restrict__ out) {
+  pdl_enter();
   static_assert(CH == 1 || CH == 2, "one or two groups of four columns per thread");
   const int rows_per_run = blockDim.x / G;
   const int col = (int)(threadIdx.x % G) * (4 * CH);
@@ -204,6 +209,7 @@ __global__ void __launch_bounds__(kThreads) k_blur_pipe(int64_t m, int G, int k,
                                                         const int32_t* __restrict__ nbr,
                                                         const S* __restrict__ in,
                                                         S* __restrict__ out) {
+  pdl_enter();
   const int rows_per_block = blockDim.x / G;
   const int col = (int)(threadIdx.x % G) * 8;
   const int64_t stride = (int64_t)gridDim.x * rows_per_block;
@@ -293,6 +299,7 @@ __global__ void __launch_bounds__(kThreads) k_sparse_blur(int64_t count, int G, 
                                                           const float* __restrict__ pw,
                                                           const S* __restrict__ stored,
                                                           S* __restrict__ tmp) {
+  pdl_enter();
   using Vt = Vec<VEC>;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t a = gid / G;
@@ -321,6 +328,7 @@ __global__ void __launch_bounds__(kThreads) k_sparse_store(int64_t count, int G,
                                                            const S* __restrict__ tmp,
                                                            S* __restrict__ stored,
                                                            int32_t* __restrict__ epoch) {
+  pdl_enter();
   using Vt = Vec<VEC>;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t a = gid / G;
@@ -336,6 +344,7 @@ __global__ void __launch_bounds__(kThreads) k_sparse_finish(int64_t m, int G, in
                                                             const int32_t* __restrict__ epoch,
                                                             const float* __restrict__ pw,
                                                             S* __restrict__ stored) {
+  pdl_enter();
   using Vt = Vec<VEC>;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t v = gid / G;
@@ -386,6 +395,7 @@ __global__ void __launch_bounds__(kThreads) k_slice(int64_t n, int G, int k, int
                                                     const S* __restrict__ lat,
                                                     const float* __restrict__ V, float alpha,
                                                     float beta, float* __restrict__ out) {
+  pdl_enter();
   using Vt = Vec<VEC>;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t p = gid / G;
@@ -409,6 +419,7 @@ __global__ void __launch_bounds__(kThreads) k_slice_dot(int64_t n, int G, int k,
                                                         const float* __restrict__ V, float alpha,
                                                         float beta, float* __restrict__ out,
                                                         double* __restrict__ dot_partial) {
+  pdl_enter();
   using Vt = Vec<VEC>;
   const int rows = blockDim.x / G;
   const int col = (int)(threadIdx.x % G) * VEC;
@@ -438,6 +449,7 @@ __global__ void __launch_bounds__(kThreads) k_permute_rows(int64_t n, int G, int
                                                            const int32_t* __restrict__ perm,
                                                            const float* __restrict__ V,
                                                            float* __restrict__ Vp) {
+  pdl_enter();
   using Vt = Vec<VEC>;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t p = gid / G;
@@ -457,18 +469,18 @@ void launch_splat_t(const Lattice* L, const float* V, int k, S* lat, float* part
   const bool v4 = vec4_ok(k, V, lat);
   const int G = v4 ? k / 4 : k;
   if (v4)
-    k_splat<4, S><<<(unsigned)ceil_div(L->nseg * G, kThreads), kThreads, 0, st>>>(
+    launch_pdl(k_splat<4, S>, (unsigned)ceil_div(L->nseg * G, kThreads), kThreads, st, 
         L->nseg, G, k, L->seg, L->items, V, lat, partial);
   else
-    k_splat<1, S><<<(unsigned)ceil_div(L->nseg * G, kThreads), kThreads, 0, st>>>(
+    launch_pdl(k_splat<1, S>, (unsigned)ceil_div(L->nseg * G, kThreads), kThreads, st, 
         L->nseg, G, k, L->seg, L->items, V, lat, partial);
   note_launches(1);
   if (L->nmed > 0) {
     if (v4)
-      k_splat_med<4, S><<<(unsigned)ceil_div(L->nmed * G, kThreads), kThreads, 0, st>>>(
+      launch_pdl(k_splat_med<4, S>, (unsigned)ceil_div(L->nmed * G, kThreads), kThreads, st, 
           L->nmed, G, k, L->med_rows, partial, lat);
     else
-      k_splat_med<1, S><<<(unsigned)ceil_div(L->nmed * G, kThreads), kThreads, 0, st>>>(
+      launch_pdl(k_splat_med<1, S>, (unsigned)ceil_div(L->nmed * G, kThreads), kThreads, st, 
           L->nmed, G, k, L->med_rows, partial, lat);
     note_launches(1);
   }
@@ -476,9 +488,9 @@ void launch_splat_t(const Lattice* L, const float* V, int k, S* lat, float* part
     int groups = 1;  // a power-of-two number of G-thread groups per block for the tree
     while (groups * 2 * G <= kThreads) groups *= 2;
     if (v4)
-      k_splat_huge<4, S><<<(unsigned)L->nhuge, groups * G, 0, st>>>(G, k, L->huge_rows, partial, lat);
+      launch_pdl(k_splat_huge<4, S>, (unsigned)L->nhuge, groups * G, st, G, k, L->huge_rows, partial, lat);
     else
-      k_splat_huge<1, S><<<(unsigned)L->nhuge, groups * G, 0, st>>>(G, k, L->huge_rows, partial, lat);
+      launch_pdl(k_splat_huge<1, S>, (unsigned)L->nhuge, groups * G, st, G, k, L->huge_rows, partial, lat);
     note_launches(1);
   }
 }
@@ -491,10 +503,10 @@ void launch_blur_rows(const Lattice* L, const int32_t* nbr, const Taps& taps, co
   const int64_t runs = ceil_div(L->m, threads / G);
   const unsigned grid = (unsigned)ceil_div(runs, U);
   switch (L->r) {
-    case 1: k_blur_rows<CH, U, 1, S><<<grid, threads, 0, st>>>(L->m, G, k, taps, nbr, in, out); break;
-    case 2: k_blur_rows<CH, U, 2, S><<<grid, threads, 0, st>>>(L->m, G, k, taps, nbr, in, out); break;
-    case 3: k_blur_rows<CH, U, 3, S><<<grid, threads, 0, st>>>(L->m, G, k, taps, nbr, in, out); break;
-    default: k_blur_rows<CH, U, 4, S><<<grid, threads, 0, st>>>(L->m, G, k, taps, nbr, in, out); break;
+    case 1: launch_pdl(k_blur_rows<CH, U, 1, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
+    case 2: launch_pdl(k_blur_rows<CH, U, 2, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
+    case 3: launch_pdl(k_blur_rows<CH, U, 3, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
+    default: launch_pdl(k_blur_rows<CH, U, 4, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
   }
 }
 
@@ -505,13 +517,13 @@ void launch_blur_t(const Lattice* L, int j, const Taps& taps, const S* in, S* ou
   if (k % 8 == 0 && k / 8 <= kThreads && L->r == 1) {  // eight columns, pipelined rows
     const int G = k / 8, threads = G * (kThreads / G);
     const int64_t blocks = std::min<int64_t>(blur_pipe_blocks<S>(), ceil_div(L->m, threads / G));
-    k_blur_pipe<S><<<(unsigned)blocks, threads, 0, st>>>(L->m, G, k, taps, nbr, in, out);
+    launch_pdl(k_blur_pipe<S>, (unsigned)blocks, threads, st, L->m, G, k, taps, nbr, in, out);
   } else if (k % 8 == 0 && k / 8 <= kThreads) {  // eight columns of two rows per thread
     launch_blur_rows<2, 2, S>(L, nbr, taps, in, out, k, st);
   } else if (k % 4 == 0 && k / 4 <= kThreads) {
     launch_blur_rows<1, 2, S>(L, nbr, taps, in, out, k, st);
   } else {
-    k_blur<S><<<(unsigned)ceil_div(L->m * k, kThreads), kThreads, 0, st>>>(L->m, k, L->r, taps, nbr,
+    launch_pdl(k_blur<S>, (unsigned)ceil_div(L->m * k, kThreads), kThreads, st, L->m, k, L->r, taps, nbr,
                                                                           in, out);
   }
   note_launches(1);
@@ -526,17 +538,17 @@ void launch_slice_t(const Lattice* L, const S* lat, const float* V, int k, float
   const bool use_beta = beta != 0.f && V != nullptr;
   if (v4) {
     if (use_beta)
-      k_slice<4, true, PERM, S><<<grid, kThreads, 0, st>>>(L->n, G, k, L->D, L->perm, L->idx, L->w,
+      launch_pdl(k_slice<4, true, PERM, S>, grid, kThreads, st, L->n, G, k, L->D, L->perm, L->idx, L->w,
                                                            lat, V, alpha, beta, out);
     else
-      k_slice<4, false, PERM, S><<<grid, kThreads, 0, st>>>(L->n, G, k, L->D, L->perm, L->idx,
+      launch_pdl(k_slice<4, false, PERM, S>, grid, kThreads, st, L->n, G, k, L->D, L->perm, L->idx,
                                                             L->w, lat, V, alpha, beta, out);
   } else {
     if (use_beta)
-      k_slice<1, true, PERM, S><<<grid, kThreads, 0, st>>>(L->n, G, k, L->D, L->perm, L->idx, L->w,
+      launch_pdl(k_slice<1, true, PERM, S>, grid, kThreads, st, L->n, G, k, L->D, L->perm, L->idx, L->w,
                                                            lat, V, alpha, beta, out);
     else
-      k_slice<1, false, PERM, S><<<grid, kThreads, 0, st>>>(L->n, G, k, L->D, L->perm, L->idx,
+      launch_pdl(k_slice<1, false, PERM, S>, grid, kThreads, st, L->n, G, k, L->D, L->perm, L->idx,
                                                             L->w, lat, V, alpha, beta, out);
   }
   note_launches(1);
@@ -549,10 +561,10 @@ void launch_slice_dot(const Lattice* L, const S* lat, const float* V, int k, flo
   const int T = column_block_threads(k, vec);
   const unsigned grid = (unsigned)slice_dot_blocks(L, k);
   if (vec == 4)
-    k_slice_dot<4, S><<<grid, T, 0, st>>>(L->n, k / 4, k, L->D, L->idx, L->w, lat, V, alpha, beta,
+    launch_pdl(k_slice_dot<4, S>, grid, T, st, L->n, k / 4, k, L->D, L->idx, L->w, lat, V, alpha, beta,
                                           out, dot_partial);
   else
-    k_slice_dot<1, S><<<grid, T, 0, st>>>(L->n, k, k, L->D, L->idx, L->w, lat, V, alpha, beta, out,
+    launch_pdl(k_slice_dot<1, S>, grid, T, st, L->n, k, k, L->D, L->idx, L->w, lat, V, alpha, beta, out,
                                           dot_partial);
   note_launches(1);
 }
@@ -560,10 +572,10 @@ void launch_slice_dot(const Lattice* L, const S* lat, const float* V, int k, flo
 void launch_permute(const Lattice* L, const float* V, int k, float* Vp, cudaStream_t st) {
   if (vec4_ok(k, V, Vp)) {
     const int G = k / 4;
-    k_permute_rows<4><<<(unsigned)ceil_div(L->n * G, kThreads), kThreads, 0, st>>>(
+    launch_pdl(k_permute_rows<4>, (unsigned)ceil_div(L->n * G, kThreads), kThreads, st, 
         L->n, G, k, L->perm, V, Vp);
   } else {
-    k_permute_rows<1><<<(unsigned)ceil_div(L->n * k, kThreads), kThreads, 0, st>>>(
+    launch_pdl(k_permute_rows<1>, (unsigned)ceil_div(L->n * k, kThreads), kThreads, st, 
         L->n, k, k, L->perm, V, Vp);
   }
   note_launches(1);
@@ -614,20 +626,20 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
     const int32_t* nbr_j = L->nbr + (size_t)j * L->r * 2 * L->m;
     const unsigned grid = (unsigned)ceil_div(count * G, kThreads);
     if (v4) {
-      k_sparse_blur<4, S><<<grid, kThreads, 0, st>>>(count, G, k, L->r, tp, t, act, nbr_j, L->m,
+      launch_pdl(k_sparse_blur<4, S>, grid, kThreads, st, count, G, k, L->r, tp, t, act, nbr_j, L->m,
                                                      L->epoch, pw, lat0, tmp);
-      k_sparse_store<4, S><<<grid, kThreads, 0, st>>>(count, G, k, t, act, tmp, lat0, L->epoch);
+      launch_pdl(k_sparse_store<4, S>, grid, kThreads, st, count, G, k, t, act, tmp, lat0, L->epoch);
     } else {
-      k_sparse_blur<1, S><<<grid, kThreads, 0, st>>>(count, G, k, L->r, tp, t, act, nbr_j, L->m,
+      launch_pdl(k_sparse_blur<1, S>, grid, kThreads, st, count, G, k, L->r, tp, t, act, nbr_j, L->m,
                                                      L->epoch, pw, lat0, tmp);
-      k_sparse_store<1, S><<<grid, kThreads, 0, st>>>(count, G, k, t, act, tmp, lat0, L->epoch);
+      launch_pdl(k_sparse_store<1, S>, grid, kThreads, st, count, G, k, t, act, tmp, lat0, L->epoch);
     }
     note_launches(2);
   }
   if (pw) {
     const unsigned grid = (unsigned)ceil_div(L->m * G, kThreads);
-    if (v4) k_sparse_finish<4, S><<<grid, kThreads, 0, st>>>(L->m, G, k, P, L->epoch, pw, lat0);
-    else k_sparse_finish<1, S><<<grid, kThreads, 0, st>>>(L->m, G, k, P, L->epoch, pw, lat0);
+    if (v4) launch_pdl(k_sparse_finish<4, S>, grid, kThreads, st, L->m, G, k, P, L->epoch, pw, lat0);
+    else launch_pdl(k_sparse_finish<1, S>, grid, kThreads, st, L->m, G, k, P, L->epoch, pw, lat0);
     note_launches(1);
   }
   return lat0;

@@ -48,6 +48,7 @@ __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
 
 __global__ void k_scan_reduce(const uint32_t* __restrict__ data, int64_t n,
                               uint32_t* __restrict__ block_sums) {
+  pdl_enter();
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
   uint32_t s = 0;
 #pragma unroll
@@ -60,6 +61,7 @@ __global__ void k_scan_reduce(const uint32_t* __restrict__ data, int64_t n,
 
 __global__ void k_scan_top(uint32_t* __restrict__ block_sums, int64_t nb,
                            uint32_t* __restrict__ total_out) {
+  pdl_enter();
   uint32_t carry = 0;
   for (int64_t base = 0; base < nb; base += kScanTile) {
     const int64_t my = base + (int64_t)threadIdx.x * kScanItems;
@@ -84,6 +86,7 @@ __global__ void k_scan_top(uint32_t* __restrict__ block_sums, int64_t nb,
 
 __global__ void k_scan_down(uint32_t* __restrict__ data, int64_t n,
                             const uint32_t* __restrict__ block_sums) {
+  pdl_enter();
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
   uint32_t v[kScanItems];
   uint32_t s = 0;
@@ -102,6 +105,7 @@ __global__ void k_scan_down(uint32_t* __restrict__ data, int64_t n,
 
 __global__ void k_radix_hist(const uint32_t* __restrict__ keys, int64_t n, int shift,
                              uint32_t* __restrict__ hist, int64_t nblk) {
+  pdl_enter();
   __shared__ uint32_t h[256];
   h[threadIdx.x] = 0;
   __syncthreads();
@@ -120,6 +124,7 @@ __global__ void k_radix_scatter(const uint32_t* __restrict__ kin,
                                 const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
                                 uint32_t* __restrict__ vout, int64_t n, int shift,
                                 const uint32_t* __restrict__ offs, int64_t nblk) {
+  pdl_enter();
   __shared__ uint32_t cnt[kSortWarps][256];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t base = (int64_t)blockIdx.x * kSortTile + (int64_t)warp * (kSortBatches * 32);
@@ -173,9 +178,9 @@ void exclusive_scan_u32(uint32_t* data, int64_t n, uint32_t* total, uint32_t* tm
     return;
   }
   const int64_t nb = ceil_div(n, kScanTile);
-  k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, st>>>(data, n, tmp);
-  k_scan_top<<<1, kScanThreads, 0, st>>>(tmp, nb, total);
-  k_scan_down<<<(unsigned)nb, kScanThreads, 0, st>>>(data, n, tmp);
+  launch_pdl(k_scan_reduce, (unsigned)nb, kScanThreads, st, data, n, tmp);
+  launch_pdl(k_scan_top, 1, kScanThreads, st, tmp, nb, total);
+  launch_pdl(k_scan_down, (unsigned)nb, kScanThreads, st, data, n, tmp);
   note_launches(3);
 }
 
@@ -196,9 +201,9 @@ bool radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32
     const uint32_t* vin = alt ? vals_alt : vals;
     uint32_t* kout = alt ? keys : keys_alt;
     uint32_t* vout = alt ? vals : vals_alt;
-    k_radix_hist<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, n, shift, hist, nblk);
+    launch_pdl(k_radix_hist, (unsigned)nblk, kSortThreads, st, kin, n, shift, hist, nblk);
     exclusive_scan_u32(hist, 256 * nblk, nullptr, scan_tmp, st);
-    k_radix_scatter<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, vin, kout, vout, n, shift,
+    launch_pdl(k_radix_scatter, (unsigned)nblk, kSortThreads, st, kin, vin, kout, vout, n, shift,
                                                             hist, nblk);
     note_launches(2);
     alt = !alt;
