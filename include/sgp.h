@@ -253,8 +253,8 @@ sgp_status sgp_cg_solve_history(sgp_lattice* h, const float* B, int k, int blur,
  * probe column z_s, plain CG on A x = z_s (at most max_lanczos iterations; App. A uses
  * 100; stopping early at ||r|| / ||z|| <= tol) gives the Lanczos tridiagonal T_s from its
  * coefficients (T[j][j] = 1/alpha_j + beta_{j-1}/alpha_{j-1}, T[j+1][j] =
- * sqrt(beta_j)/alpha_j); quad_s = ||z_s||^2 e1^T log(T_s) e1 (from T_s's eigenvalues and
- * the first components of its eigenvectors, implicit QL on the GPU), and
+ * sqrt(beta_j)/alpha_j); quad_s = ||z_s||^2 e1^T log(T_s) e1 (the integral of
+ * the resolvent e1^T (T_s + t I)^-1 e1 over t, on the GPU), and
  *   *logdet = (1/s) sum_s quad_s,
  * an unbiased estimate of tr log A when E[z z^T] = I (e.g. Rademacher probes).
  *   Z       device [n][s] fp32 probes (caller's order), 1 <= s <= 256.
