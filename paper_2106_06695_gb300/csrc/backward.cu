@@ -254,22 +254,25 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
   if (want_x && !dXw) BW_CHECK(w.get(&dXw, (size_t)n * d * sizeof(float)), "alloc dX");
 
   if (grad == SGP_GRAD_LATTICE) {
-    sgp_status s = ensure_lattice_values(L, k, st);
+    sgp_status s = ensure_product(L, k, st);
     if (s != SGP_OK) return s;
-    const size_t vb = lattice_value_bytes(L, k);
+    const int kp = value_cols(L, k);
+    const size_t vb = lattice_value_bytes(L, kp);
     void *b0 = nullptr, *b1 = nullptr;
     float *Vp = nullptr, *Gp = nullptr;
     BW_CHECK(w.get(&b0, vb), "alloc lattice values");
     BW_CHECK(w.get(&b1, vb), "alloc lattice values");
-    BW_CHECK(w.get(&Vp, (size_t)n * k * sizeof(float)), "alloc V");
-    BW_CHECK(w.get(&Gp, (size_t)n * k * sizeof(float)), "alloc G");
-    enqueue_permute(L, G, k, Gp, st);
+    BW_CHECK(w.get(&Vp, (size_t)n * kp * sizeof(float)), "alloc V");
+    BW_CHECK(w.get(&Gp, (size_t)n * kp * sizeof(float)), "alloc G");
+    enqueue_permute(L, G, k, kp, Gp, st);
     // B^T W^T G into (b0, b1), B W^T V into the handle's buffers
-    const void* BS = enqueue_splat_blur(L, Gp, k, transpose_blur(blur), b0, b1, L->partial, st);
-    if (dV) enqueue_slice_caller(L, BS, k, alpha, dV, st);
+    const void* BS = enqueue_splat_blur(L, Gp, kp, k, transpose_blur(blur), b0, b1, L->partial,
+                                        st);
+    if (dV) enqueue_slice_caller(L, BS, k, kp, alpha, dV, st);
     if (want_x) {
-      enqueue_permute(L, V, k, Vp, st);
-      const void* BU = enqueue_splat_blur(L, Vp, k, blur, L->lat[0], L->lat[1], L->partial, st);
+      enqueue_permute(L, V, k, kp, Vp, st);
+      const void* BU = enqueue_splat_blur(L, Vp, kp, k, blur, L->lat[0], L->lat[1],
+                                          L->partial, st);
       const double scale = std::sqrt((double)(d * (d + 1))) / L->s;
       std::vector<double> hf(d);
       for (int j = 0; j < d; ++j) hf[j] = scale / std::sqrt((double)((j + 1) * (j + 2)));
@@ -278,25 +281,25 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
       // pageable source: the call returns once hf has been staged
       BW_CHECK(cudaMemcpyAsync(f, hf.data(), d * sizeof(double), cudaMemcpyHostToDevice, st),
                "copy f");
-      const bool v4 = k % 4 == 0;
+      const bool v4 = kp % 4 == 0;
       if (L->value_dtype == SGP_VALUES_BF16) {
-        if (v4) launch_weight_grad<bf16, 4>(L, k, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
-        else launch_weight_grad<bf16, 1>(L, k, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
+        if (v4) launch_weight_grad<bf16, 4>(L, kp, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
+        else launch_weight_grad<bf16, 1>(L, kp, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
       } else {
-        if (v4) launch_weight_grad<float, 4>(L, k, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
-        else launch_weight_grad<float, 1>(L, k, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
+        if (v4) launch_weight_grad<float, 4>(L, kp, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
+        else launch_weight_grad<float, 1>(L, kp, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
       }
     }
   } else {  // SGP_GRAD_FILTER
     if (dV) {
-      sgp_status s = ensure_lattice_values(L, k, st);
+      sgp_status s = ensure_product(L, k, st);
       if (s != SGP_OK) return s;
       enqueue_mvm(L, G, k, transpose_blur(blur), alpha, 0.f, dV, st);
     }
     if (want_x) {
       const int kk = 2 * k * (d + 1);
       const int chunk = std::min(kk, kFilterChunk);
-      sgp_status s = ensure_lattice_values(L, chunk, st);
+      sgp_status s = ensure_product(L, chunk, st);
       if (s != SGP_OK) return s;
       float *in = nullptr, *F = nullptr;
       BW_CHECK(w.get(&in, (size_t)n * chunk * sizeof(float)), "alloc filter input");

@@ -375,10 +375,10 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
   const int64_t n = L->n;
   // The solver works on k rounded up to a multiple of 4 (zero right-hand sides in the
   // extra columns, inactive from the start), so that its vectors and the lattice values
-  // are rows of float4 and the MVM takes its vectorised kernels.  The Lanczos record of
-  // sgp_logdet is laid out for the caller's k: no padding then.
+  // are rows of float4 and the MVM takes its vectorised kernels.  One or two Lanczos probes
+  // (sgp_logdet) stay as they are; their huge vertices' sums keep the caller's k's shape.
   const int kb = k;
-  if (!rec) k = (k + 3) / 4 * 4;
+  k = rec ? padded_cols(k) : (k + 3) / 4 * 4;
   // CUDA graphs cannot be captured on the legacy default stream: use a private blocking
   // stream then (it is ordered with the legacy stream like any blocking stream).
   cudaStream_t st = L->stream;
@@ -499,7 +499,7 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
   auto iteration = [&]() {
     // Ap = outputscale K~ p + noise p, with the slice also summing <p, Ap> per block
     passes = enqueue_mvm(L, p, k, blur, L->outputscale, noise, Ap, st, ev, /*internal=*/true,
-                         S.partial);
+                         S.partial, rec ? kb : k);
     launch_pdl(k_cg_alpha, k, 256, st, (int)sblocks, k, S);
     if (vec == 4) launch_pdl(k_cg_update_xr<4>, vblocks, T, st, xh, xl, rh, rl, p, Ap, n, k, S);
     else launch_pdl(k_cg_update_xr<1>, vblocks, T, st, xh, xl, rh, rl, p, Ap, n, k, S);

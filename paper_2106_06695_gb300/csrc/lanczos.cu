@@ -125,13 +125,14 @@ sgp_status run_logdet(Lattice* L, const float* Z, int s, float noise, int max_la
   } while (0)
   LanczosRecord rec{};
   rec.cap = cap;
+  const int sp = padded_cols(s);  // columns of the record (run_cg pads its vectors alike)
   float* X = nullptr;
   double* dq = nullptr;
   int* bad = nullptr;
-  LZ_CHECK(get((void**)&rec.alpha, (size_t)cap * s * sizeof(double)), "alloc Lanczos record");
-  LZ_CHECK(get((void**)&rec.beta, (size_t)cap * s * sizeof(double)), "alloc Lanczos record");
-  LZ_CHECK(get((void**)&rec.bnorm, (size_t)s * sizeof(double)), "alloc Lanczos record");
-  LZ_CHECK(get((void**)&rec.iters, (size_t)s * sizeof(int)), "alloc Lanczos record");
+  LZ_CHECK(get((void**)&rec.alpha, (size_t)cap * sp * sizeof(double)), "alloc Lanczos record");
+  LZ_CHECK(get((void**)&rec.beta, (size_t)cap * sp * sizeof(double)), "alloc Lanczos record");
+  LZ_CHECK(get((void**)&rec.bnorm, (size_t)sp * sizeof(double)), "alloc Lanczos record");
+  LZ_CHECK(get((void**)&rec.iters, (size_t)sp * sizeof(int)), "alloc Lanczos record");
   LZ_CHECK(get((void**)&X, (size_t)L->n * s * sizeof(float)), "alloc CG solution");
   LZ_CHECK(get((void**)&dq, (size_t)s * kSlqWarps * sizeof(double)), "alloc quadratures");
   LZ_CHECK(get((void**)&bad, sizeof(int)), "alloc flag");
@@ -139,7 +140,7 @@ sgp_status run_logdet(Lattice* L, const float* Z, int s, float noise, int max_la
   sgp_status status = run_cg(L, Z, s, SGP_BLUR_SYMMETRIC, noise, tol, cap, X, nullptr, nullptr,
                              0, 0, &rec);
   if (status != SGP_OK) return status;
-  launch_pdl(k_slq, dim3(kSlqWarps + 1, (unsigned)s), 32, st, rec.alpha, rec.beta, s, cap,
+  launch_pdl(k_slq, dim3(kSlqWarps + 1, (unsigned)s), 32, st, rec.alpha, rec.beta, sp, cap,
              rec.iters, rec.bnorm, dq, bad);
   note_launches(1);
   LZ_CHECK(cudaGetLastError(), "Lanczos quadrature");

@@ -11,10 +11,15 @@
 //
 // All of them are bound by memory traffic.  The caller's vectors are fp32 [rows][k]
 // row-major.  Lattice values are stored as S = float or __nv_bfloat16 (SGP_VALUES_BF16:
-// half the bytes of the dominant blur traffic); every sum is accumulated in fp32.  A
-// thread owns 4 consecutive columns of a row when k is a multiple of 4 and the buffers are
-// aligned, else one column; the blur gives each thread 8 columns when k allows.
+// half the bytes of the dominant blur traffic); every sum is accumulated in fp32.
+//
+// Inside the operator a row has kp >= k columns (padded_cols): one or two columns as they
+// are, more rounded up to a multiple of 4 with zero columns, so that every row is float4
+// groups whatever k and however the caller's buffers are aligned; a thread owns 4 (2, 1)
+// consecutive columns of a row, the pipelined blur 8.  At n = 50k, d = 8, k = 9 a product
+// with 9 scalar columns took 100 us, with 12 padded ones 77.5 us (launches alike).
 #include <atomic>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 
@@ -34,7 +39,8 @@ constexpr int kThreads = 256;
 // sums keep the incidence order, so results do not change with the chunking.
 constexpr int kChunk = 8;
 
-// One thread-group of G threads per segment of at most kSplatSeg incidences.
+// One thread-group of G = k / VEC threads per segment of at most kSplatSeg incidences;
+// blockDim.x is a multiple of G.
 template <int VEC, class S>
 __global__ void __launch_bounds__(kThreads) k_splat(int64_t nseg, int G, int k,
                                                     const int4* __restrict__ seg,
@@ -44,10 +50,9 @@ __global__ void __launch_bounds__(kThreads) k_splat(int64_t nseg, int G, int k,
                                                     float* __restrict__ partial) {
   pdl_enter();
   using Vt = Vec<VEC>;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t s = gid / G;
+  const int64_t s = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
   if (s >= nseg) return;
-  const int col = (int)(gid - s * G) * VEC;
+  const int col = (int)(threadIdx.x % G) * VEC;
   const int4 sg = __ldg(seg + s);
   typename Vt::T acc = Vt::zero();
   for (int p0 = sg.y; p0 < sg.z; p0 += kChunk) {
@@ -75,44 +80,44 @@ __global__ void __launch_bounds__(kThreads) k_splat_med(int64_t nrows, int G, in
                                                         S* __restrict__ lat) {
   pdl_enter();
   using Vt = Vec<VEC>;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t q = gid / G;
+  const int64_t q = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
   if (q >= nrows) return;
-  const int col = (int)(gid - q * G) * VEC;
+  const int col = (int)(threadIdx.x % G) * VEC;
   const int4 rw = rows[q];
   typename Vt::T acc = Vt::zero();
   for (int j = 0; j < rw.z; ++j) acc = Vt::add(acc, Vt::ld(partial + (int64_t)(rw.y + j) * k + col));
   Vt::sts(lat + (int64_t)rw.x * k + col, acc);
 }
 
-// Fix-up for vertices with more segments: one block per vertex, groups of G threads take
-// strided partials, then a fixed-shape shared-memory tree combines the groups.
+// Fix-up for vertices with more segments: one block per vertex.  `groups` (a power of two,
+// groups G <= kThreads) strided partial sums, then a fixed-shape shared-memory tree over
+// them: the result depends on `groups` only, not on how the threads share the work.
 template <int VEC, class S>
-__global__ void __launch_bounds__(kThreads) k_splat_huge(int G, int k, const int4* __restrict__ rows,
+__global__ void __launch_bounds__(kThreads) k_splat_huge(int groups, int G, int k,
+                                                         const int4* __restrict__ rows,
                                                          const float* __restrict__ partial,
                                                          S* __restrict__ lat) {
   pdl_enter();
   using Vt = Vec<VEC>;
   __shared__ typename Vt::T red[kThreads];
-  const int groups = blockDim.x / G;
-  const int g = threadIdx.x / G;
-  const int col = (int)(threadIdx.x % G) * VEC;
   const int4 rw = rows[blockIdx.x];
-  typename Vt::T acc = Vt::zero();
-  if (g < groups)
-    for (int j = g; j < rw.z; j += groups)
-      acc = Vt::add(acc, Vt::ld(partial + (int64_t)(rw.y + j) * k + col));
-  red[threadIdx.x] = acc;
+  for (int q = threadIdx.x; q < groups * G; q += blockDim.x) {
+    typename Vt::T acc = Vt::zero();
+    for (int j = q / G; j < rw.z; j += groups)
+      acc = Vt::add(acc, Vt::ld(partial + (int64_t)(rw.y + j) * k + (q % G) * VEC));
+    red[q] = acc;
+  }
   __syncthreads();
   for (int half = groups / 2; half >= 1; half /= 2) {
-    if (g < half) red[threadIdx.x] = Vt::add(red[threadIdx.x], red[threadIdx.x + half * G]);
+    for (int q = threadIdx.x; q < half * G; q += blockDim.x)
+      red[q] = Vt::add(red[q], red[q + half * G]);
     __syncthreads();
   }
-  if (g == 0) Vt::sts(lat + (int64_t)rw.x * k + col, red[threadIdx.x]);
+  for (int q = threadIdx.x; q < G; q += blockDim.x) Vt::sts(lat + (int64_t)rw.x * k + q * VEC, red[q]);
 }
 
 // ---- blur ----------------------------------------------------------------------------
-// One value per thread (any k).
+// One value per thread (any k: the fixed work area's unpadded rows).
 template <class S>
 __global__ void __launch_bounds__(kThreads) k_blur(int64_t m, int k, int r, Taps tp,
                                                    const int32_t* __restrict__ nbr,
@@ -134,19 +139,21 @@ __global__ void __launch_bounds__(kThreads) k_blur(int64_t m, int k, int r, Taps
   Store<S>::st1(out + v * k + col, acc);
 }
 
-// Rows of k = 4 CH G values.  Each thread owns 4 CH consecutive columns of U rows (R =
+// Rows of k = VEC CH G values.  Each thread owns VEC CH consecutive columns of U rows (R =
 // stencil order): it issues all id loads, then all own and neighbour row loads, then the
 // arithmetic, so 3 U row loads per order are in flight at once.  A block covers U
 // consecutive runs of kThreads / G rows (coalesced per run, local per block).
-template <int CH, int U, int R, class S>
+template <int VEC, int CH, int U, int R, class S>
 __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k, Taps tp,
                                                         const int32_t* __restrict__ nbr,
                                                         const S* __restrict__ in,
                                                         S* __restrict__ out) {
+  static_assert(CH == 1 || (CH == 2 && VEC == 4), "one group of columns per thread, or 2 x 4");
   pdl_enter();
-  static_assert(CH == 1 || CH == 2, "one or two groups of four columns per thread");
+  using Vt = Vec<VEC>;
+  using T = typename Vt::T;
   const int rows_per_run = blockDim.x / G;
-  const int col = (int)(threadIdx.x % G) * (4 * CH);
+  const int col = (int)(threadIdx.x % G) * (VEC * CH);
   int64_t v[U];
   int ia[U][R], ic[U][R];
 #pragma unroll
@@ -158,21 +165,20 @@ __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k,
       ic[u][t] = v[u] < m ? __ldg(nbr + (int64_t)(2 * t + 1) * m + v[u]) : -1;
     }
   }
-  auto load = [&](int64_t row, float4* x) {
-    if (CH == 2) Store<S>::ldg8(in + row * k + col, x[0], x[CH - 1]);
-    else x[0] = Store<S>::ldg4(in + row * k + col);
+  auto load = [&](int64_t row, T* x) {
+    if constexpr (CH == 2) Store<S>::ldg8(in + row * k + col, x[0], x[1]);
+    else x[0] = Vt::ldgs(in + row * k + col);
   };
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  float4 own[U][CH], sa[U][R][CH], sc[U][R][CH];
+  T own[U][CH], sa[U][R][CH], sc[U][R][CH];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
 #pragma unroll
-    for (int c = 0; c < CH; ++c) own[u][c] = zero;
+    for (int c = 0; c < CH; ++c) own[u][c] = Vt::zero();
     if (v[u] < m) load(v[u], own[u]);
 #pragma unroll
     for (int t = 0; t < R; ++t) {
 #pragma unroll
-      for (int c = 0; c < CH; ++c) sa[u][t][c] = sc[u][t][c] = zero;
+      for (int c = 0; c < CH; ++c) sa[u][t][c] = sc[u][t][c] = Vt::zero();
       if (ia[u][t] >= 0) load(ia[u][t], sa[u][t]);
       if (ic[u][t] >= 0) load(ic[u][t], sc[u][t]);
     }
@@ -180,22 +186,16 @@ __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k,
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     if (v[u] >= m) continue;
-    float4 acc[CH];
+    T acc[CH];
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
-      acc[c] = make_float4(tp.t[0] * own[u][c].x, tp.t[0] * own[u][c].y, tp.t[0] * own[u][c].z,
-                           tp.t[0] * own[u][c].w);
+      acc[c] = Vt::scale(tp.t[0], own[u][c]);
 #pragma unroll
-      for (int t = 0; t < R; ++t) {
-        const float w = tp.t[t + 1];
-        acc[c].x = fmaf(w, sa[u][t][c].x + sc[u][t][c].x, acc[c].x);
-        acc[c].y = fmaf(w, sa[u][t][c].y + sc[u][t][c].y, acc[c].y);
-        acc[c].z = fmaf(w, sa[u][t][c].z + sc[u][t][c].z, acc[c].z);
-        acc[c].w = fmaf(w, sa[u][t][c].w + sc[u][t][c].w, acc[c].w);
-      }
+      for (int t = 0; t < R; ++t)
+        acc[c] = Vt::fma(tp.t[t + 1], Vt::add(sa[u][t][c], sc[u][t][c]), acc[c]);
     }
-    if (CH == 2) Store<S>::st8(out + v[u] * k + col, acc[0], acc[CH - 1]);
-    else Store<S>::st4(out + v[u] * k + col, acc[0]);
+    if constexpr (CH == 2) Store<S>::st8(out + v[u] * k + col, acc[0], acc[1]);
+    else Vt::sts(out + v[u] * k + col, acc[0]);
   }
 }
 
@@ -301,10 +301,9 @@ __global__ void __launch_bounds__(kThreads) k_sparse_blur(int64_t count, int G, 
                                                           S* __restrict__ tmp) {
   pdl_enter();
   using Vt = Vec<VEC>;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t a = gid / G;
+  const int64_t a = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
   if (a >= count) return;
-  const int col = (int)(gid - a * G) * VEC;
+  const int col = (int)(threadIdx.x % G) * VEC;
   const int64_t v = act[a];
   auto value = [&](int64_t x) {
     const float f = pw ? pw[t - epoch[x]] : 1.f;
@@ -330,10 +329,9 @@ __global__ void __launch_bounds__(kThreads) k_sparse_store(int64_t count, int G,
                                                            int32_t* __restrict__ epoch) {
   pdl_enter();
   using Vt = Vec<VEC>;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t a = gid / G;
+  const int64_t a = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
   if (a >= count) return;
-  const int col = (int)(gid - a * G) * VEC;
+  const int col = (int)(threadIdx.x % G) * VEC;
   const int64_t v = act[a];
   Vt::sts(stored + v * k + col, Vt::lds(tmp + a * k + col));
   if (col == 0) epoch[v] = t + 1;
@@ -346,12 +344,11 @@ __global__ void __launch_bounds__(kThreads) k_sparse_finish(int64_t m, int G, in
                                                             S* __restrict__ stored) {
   pdl_enter();
   using Vt = Vec<VEC>;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t v = gid / G;
+  const int64_t v = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
   if (v >= m) return;
   const int e = epoch[v];
   if (e == P) return;
-  const int col = (int)(gid - v * G) * VEC;
+  const int col = (int)(threadIdx.x % G) * VEC;
   Vt::sts(stored + v * k + col, Vt::scale(pw[P - e], Vt::lds(stored + v * k + col)));
 }
 
@@ -386,26 +383,34 @@ __device__ __forceinline__ typename Vec<VEC>::T slice_row(int64_t p, int D, int 
   return acc;
 }
 
-// PERM: V and out rows are in the caller's order (row perm[p]); else in locality order.
-template <int VEC, bool BETA, bool PERM, class S>
-__global__ void __launch_bounds__(kThreads) k_slice(int64_t n, int G, int k, int D,
+// out = alpha W lat (+ beta Vp, rows of k in locality order, when beta != 0).  PERM: out has
+// the caller's ko columns and row order (row perm[p]), written one value at a time unless
+// WIDE (ko = k, aligned rows); else out is [n][k] in locality order.
+template <int VEC, bool PERM, bool WIDE, class S>
+__global__ void __launch_bounds__(kThreads) k_slice(int64_t n, int G, int k, int ko, int D,
                                                     const int32_t* __restrict__ perm,
                                                     const int32_t* __restrict__ idx,
                                                     const float* __restrict__ w,
                                                     const S* __restrict__ lat,
-                                                    const float* __restrict__ V, float alpha,
+                                                    const float* __restrict__ Vp, float alpha,
                                                     float beta, float* __restrict__ out) {
   pdl_enter();
   using Vt = Vec<VEC>;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t p = gid / G;
+  const int64_t p = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
   if (p >= n) return;
-  const int col = (int)(gid - p * G) * VEC;
+  const int col = (int)(threadIdx.x % G) * VEC;
   const typename Vt::T acc = slice_row<VEC, S>(p, D, k, col, idx, w, lat);
   const int64_t i = PERM ? (int64_t)perm[p] : p;
   typename Vt::T res = Vt::scale(alpha, acc);
-  if (BETA) res = Vt::fma(beta, Vt::ld(V + i * k + col), res);
-  Vt::st(out + i * k + col, res);
+  if (beta != 0.f) res = Vt::fma(beta, Vt::ld(Vp + p * k + col), res);
+  if constexpr (!PERM || WIDE) {
+    Vt::st(out + i * k + col, res);
+  } else {
+    const float* rr = reinterpret_cast<const float*>(&res);
+#pragma unroll
+    for (int j = 0; j < VEC; ++j)
+      if (col + j < ko) out[i * ko + col + j] = rr[j];
+  }
 }
 
 // The CG's slice: V and out in locality order, out = alpha W lat + beta V, and the
@@ -443,70 +448,97 @@ __global__ void __launch_bounds__(kThreads) k_slice_dot(int64_t n, int G, int k,
   block_column_sums<VEC>(dd, k, dot_partial + (int64_t)blockIdx.x * k);
 }
 
-// Vp[p] = V[perm[p]]: the caller's rows in locality order.
-template <int VEC>
-__global__ void __launch_bounds__(kThreads) k_permute_rows(int64_t n, int G, int k,
+// Vp[p] = V[perm[p]]: the caller's rows (ki columns) in locality order, padded with zero
+// columns to k.  WIDE: ki = k and aligned rows.
+template <int VEC, bool WIDE>
+__global__ void __launch_bounds__(kThreads) k_permute_rows(int64_t n, int G, int k, int ki,
                                                            const int32_t* __restrict__ perm,
                                                            const float* __restrict__ V,
                                                            float* __restrict__ Vp) {
   pdl_enter();
   using Vt = Vec<VEC>;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t p = gid / G;
+  const int64_t p = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
   if (p >= n) return;
-  const int col = (int)(gid - p * G) * VEC;
-  Vt::st(Vp + p * k + col, Vt::ld(V + (int64_t)perm[p] * k + col));
+  const int col = (int)(threadIdx.x % G) * VEC;
+  const int64_t i = perm[p];
+  typename Vt::T x = Vt::zero();
+  if constexpr (WIDE) {
+    x = Vt::ld(V + i * k + col);
+  } else {
+    float* xx = reinterpret_cast<float*>(&x);
+#pragma unroll
+    for (int j = 0; j < VEC; ++j)
+      if (col + j < ki) xx[j] = V[i * ki + col + j];
+  }
+  Vt::st(Vp + p * k + col, x);
 }
 
-inline bool vec4_ok(int k, const void* a, const void* b) {
-  return (k % 4 == 0) && ((uintptr_t)a % 16 == 0) && ((uintptr_t)b % 16 == 0);
+// Columns per thread and launch shape for rows of kp columns in library buffers (16-byte
+// aligned): a whole number of G-thread rows per block.
+struct RowShape {
+  int vec, G, threads;
+  unsigned blocks;  // for `rows` rows
+};
+RowShape row_shape(int64_t rows, int kp) {
+  RowShape q;
+  q.vec = kp % 4 == 0 ? 4 : kp == 2 ? 2 : 1;
+  q.G = kp / q.vec;
+  q.threads = q.G * (kThreads / q.G);
+  q.blocks = (unsigned)ceil_div(rows, q.threads / q.G);
+  return q;
+}
+bool wide_ok(int k, int kp, const void* user) {
+  return k == kp && (uintptr_t)user % (kp % 4 == 0 ? 16 : kp == 2 ? 8 : 4) == 0;
+}
+// Calls f(std::integral_constant<int, vec>).
+template <class F>
+void by_vec(int vec, F f) {
+  if (vec == 4) f(std::integral_constant<int, 4>{});
+  else if (vec == 2) f(std::integral_constant<int, 2>{});
+  else f(std::integral_constant<int, 1>{});
 }
 
 // ---- launchers -----------------------------------------------------------------------
+// kt: the column count that fixes the shape of the huge vertices' summation tree (the
+// caller's k, so that padding does not change a result).
 template <class S>
-void launch_splat_t(const Lattice* L, const float* V, int k, S* lat, float* partial,
+void launch_splat_t(const Lattice* L, const float* V, int kp, int kt, S* lat, float* partial,
                     cudaStream_t st) {
-  const bool v4 = vec4_ok(k, V, lat);
-  const int G = v4 ? k / 4 : k;
-  if (v4)
-    launch_pdl(k_splat<4, S>, (unsigned)ceil_div(L->nseg * G, kThreads), kThreads, st, 
-        L->nseg, G, k, L->seg, L->items, V, lat, partial);
-  else
-    launch_pdl(k_splat<1, S>, (unsigned)ceil_div(L->nseg * G, kThreads), kThreads, st, 
-        L->nseg, G, k, L->seg, L->items, V, lat, partial);
-  note_launches(1);
-  if (L->nmed > 0) {
-    if (v4)
-      launch_pdl(k_splat_med<4, S>, (unsigned)ceil_div(L->nmed * G, kThreads), kThreads, st, 
-          L->nmed, G, k, L->med_rows, partial, lat);
-    else
-      launch_pdl(k_splat_med<1, S>, (unsigned)ceil_div(L->nmed * G, kThreads), kThreads, st, 
-          L->nmed, G, k, L->med_rows, partial, lat);
+  by_vec(row_shape(1, kp).vec, [&](auto vec) {
+    constexpr int VEC = decltype(vec)::value;
+    const RowShape q = row_shape(L->nseg, kp);
+    launch_pdl(k_splat<VEC, S>, q.blocks, q.threads, st, L->nseg, q.G, kp, L->seg, L->items, V, lat,
+               partial);
     note_launches(1);
-  }
-  if (L->nhuge > 0) {
-    int groups = 1;  // a power-of-two number of G-thread groups per block for the tree
-    while (groups * 2 * G <= kThreads) groups *= 2;
-    if (v4)
-      launch_pdl(k_splat_huge<4, S>, (unsigned)L->nhuge, groups * G, st, G, k, L->huge_rows, partial, lat);
-    else
-      launch_pdl(k_splat_huge<1, S>, (unsigned)L->nhuge, groups * G, st, G, k, L->huge_rows, partial, lat);
-    note_launches(1);
-  }
+    if (L->nmed > 0) {
+      const RowShape qm = row_shape(L->nmed, kp);
+      launch_pdl(k_splat_med<VEC, S>, qm.blocks, qm.threads, st, L->nmed, qm.G, kp, L->med_rows,
+                 partial, lat);
+      note_launches(1);
+    }
+    if (L->nhuge > 0) {
+      const int gt = kt % 4 == 0 ? kt / 4 : kt;
+      int groups = 1;
+      while (groups * 2 * gt <= kThreads) groups *= 2;
+      launch_pdl(k_splat_huge<VEC, S>, (unsigned)L->nhuge, kThreads, st, groups, q.G, kp,
+                 L->huge_rows, partial, lat);
+      note_launches(1);
+    }
+  });
 }
 
-template <int CH, int U, class S>
+template <int VEC, int CH, int U, class S>
 void launch_blur_rows(const Lattice* L, const int32_t* nbr, const Taps& taps, const S* in,
                       S* out, int k, cudaStream_t st) {
-  const int G = k / (4 * CH);
+  const int G = k / (VEC * CH);
   const int threads = G * (kThreads / G);  // a whole number of rows per run
   const int64_t runs = ceil_div(L->m, threads / G);
   const unsigned grid = (unsigned)ceil_div(runs, U);
   switch (L->r) {
-    case 1: launch_pdl(k_blur_rows<CH, U, 1, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
-    case 2: launch_pdl(k_blur_rows<CH, U, 2, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
-    case 3: launch_pdl(k_blur_rows<CH, U, 3, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
-    default: launch_pdl(k_blur_rows<CH, U, 4, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
+    case 1: launch_pdl(k_blur_rows<VEC, CH, U, 1, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
+    case 2: launch_pdl(k_blur_rows<VEC, CH, U, 2, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
+    case 3: launch_pdl(k_blur_rows<VEC, CH, U, 3, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
+    default: launch_pdl(k_blur_rows<VEC, CH, U, 4, S>, grid, threads, st, L->m, G, k, taps, nbr, in, out); break;
   }
 }
 
@@ -519,9 +551,13 @@ void launch_blur_t(const Lattice* L, int j, const Taps& taps, const S* in, S* ou
     const int64_t blocks = std::min<int64_t>(blur_pipe_blocks<S>(), ceil_div(L->m, threads / G));
     launch_pdl(k_blur_pipe<S>, (unsigned)blocks, threads, st, L->m, G, k, taps, nbr, in, out);
   } else if (k % 8 == 0 && k / 8 <= kThreads) {  // eight columns of two rows per thread
-    launch_blur_rows<2, 2, S>(L, nbr, taps, in, out, k, st);
+    launch_blur_rows<4, 2, 2, S>(L, nbr, taps, in, out, k, st);
   } else if (k % 4 == 0 && k / 4 <= kThreads) {
-    launch_blur_rows<1, 2, S>(L, nbr, taps, in, out, k, st);
+    launch_blur_rows<4, 1, 2, S>(L, nbr, taps, in, out, k, st);
+  } else if (k == 2) {
+    launch_blur_rows<2, 1, 2, S>(L, nbr, taps, in, out, k, st);
+  } else if (k == 1) {
+    launch_blur_rows<1, 1, 2, S>(L, nbr, taps, in, out, k, st);
   } else {
     launch_pdl(k_blur<S>, (unsigned)ceil_div(L->m * k, kThreads), kThreads, st, L->m, k, L->r, taps, nbr,
                                                                           in, out);
@@ -529,28 +565,22 @@ void launch_blur_t(const Lattice* L, int j, const Taps& taps, const S* in, S* ou
   note_launches(1);
 }
 
+// out = alpha W lat + beta Vp (Vp in locality order, rows of kp).  PERM: out is the caller's
+// [n][k]; else [n][kp] in locality order.
 template <bool PERM, class S>
-void launch_slice_t(const Lattice* L, const S* lat, const float* V, int k, float alpha,
+void launch_slice_t(const Lattice* L, const S* lat, const float* Vp, int k, int kp, float alpha,
                     float beta, float* out, cudaStream_t st) {
-  const bool v4 = vec4_ok(k, out, V ? (const void*)V : (const void*)out);
-  const int G = v4 ? k / 4 : k;
-  const unsigned grid = (unsigned)ceil_div(L->n * G, kThreads);
-  const bool use_beta = beta != 0.f && V != nullptr;
-  if (v4) {
-    if (use_beta)
-      launch_pdl(k_slice<4, true, PERM, S>, grid, kThreads, st, L->n, G, k, L->D, L->perm, L->idx, L->w,
-                                                           lat, V, alpha, beta, out);
+  const RowShape q = row_shape(L->n, kp);
+  if (!Vp) beta = 0.f;
+  by_vec(q.vec, [&](auto vec) {
+    constexpr int VEC = decltype(vec)::value;
+    if (!PERM || wide_ok(k, kp, out))
+      launch_pdl(k_slice<VEC, PERM, true, S>, q.blocks, q.threads, st, L->n, q.G, kp, k, L->D,
+                 L->perm, L->idx, L->w, lat, Vp, alpha, beta, out);
     else
-      launch_pdl(k_slice<4, false, PERM, S>, grid, kThreads, st, L->n, G, k, L->D, L->perm, L->idx,
-                                                            L->w, lat, V, alpha, beta, out);
-  } else {
-    if (use_beta)
-      launch_pdl(k_slice<1, true, PERM, S>, grid, kThreads, st, L->n, G, k, L->D, L->perm, L->idx, L->w,
-                                                           lat, V, alpha, beta, out);
-    else
-      launch_pdl(k_slice<1, false, PERM, S>, grid, kThreads, st, L->n, G, k, L->D, L->perm, L->idx,
-                                                            L->w, lat, V, alpha, beta, out);
-  }
+      launch_pdl(k_slice<VEC, PERM, false, S>, q.blocks, q.threads, st, L->n, q.G, kp, k, L->D,
+                 L->perm, L->idx, L->w, lat, Vp, alpha, beta, out);
+  });
   note_launches(1);
 }
 
@@ -569,15 +599,15 @@ void launch_slice_dot(const Lattice* L, const S* lat, const float* V, int k, flo
   note_launches(1);
 }
 
-void launch_permute(const Lattice* L, const float* V, int k, float* Vp, cudaStream_t st) {
-  if (vec4_ok(k, V, Vp)) {
-    const int G = k / 4;
-    launch_pdl(k_permute_rows<4>, (unsigned)ceil_div(L->n * G, kThreads), kThreads, st, 
-        L->n, G, k, L->perm, V, Vp);
-  } else {
-    launch_pdl(k_permute_rows<1>, (unsigned)ceil_div(L->n * k, kThreads), kThreads, st, 
-        L->n, k, k, L->perm, V, Vp);
-  }
+void launch_permute(const Lattice* L, const float* V, int k, int kp, float* Vp, cudaStream_t st) {
+  const RowShape q = row_shape(L->n, kp);
+  by_vec(q.vec, [&](auto vec) {
+    constexpr int VEC = decltype(vec)::value;
+    if (wide_ok(k, kp, V))
+      launch_pdl(k_permute_rows<VEC, true>, q.blocks, q.threads, st, L->n, q.G, kp, k, L->perm, V, Vp);
+    else
+      launch_pdl(k_permute_rows<VEC, false>, q.blocks, q.threads, st, L->n, q.G, kp, k, L->perm, V, Vp);
+  });
   note_launches(1);
 }
 
@@ -614,69 +644,67 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
   }
   // sparse: lazy centre-tap factors (none when the centre tap is 1)
   const float* pw = tp.t[0] == 1.f ? nullptr : L->g0pow;
-  const bool v4 = k % 4 == 0;
-  const int G = v4 ? k / 4 : k;
   if (pw) cudaMemsetAsync(L->epoch, 0, (size_t)L->m * sizeof(int32_t), st);
   S* tmp = static_cast<S*>(L->act_tmp);
-  for (int t = 0; t < P; ++t) {
-    const int j = dir(t);
-    const int64_t count = L->act_off[j + 1] - L->act_off[j];
-    if (count == 0) continue;
-    const int32_t* act = L->act + L->act_off[j];
-    const int32_t* nbr_j = L->nbr + (size_t)j * L->r * 2 * L->m;
-    const unsigned grid = (unsigned)ceil_div(count * G, kThreads);
-    if (v4) {
-      launch_pdl(k_sparse_blur<4, S>, grid, kThreads, st, count, G, k, L->r, tp, t, act, nbr_j, L->m,
-                                                     L->epoch, pw, lat0, tmp);
-      launch_pdl(k_sparse_store<4, S>, grid, kThreads, st, count, G, k, t, act, tmp, lat0, L->epoch);
-    } else {
-      launch_pdl(k_sparse_blur<1, S>, grid, kThreads, st, count, G, k, L->r, tp, t, act, nbr_j, L->m,
-                                                     L->epoch, pw, lat0, tmp);
-      launch_pdl(k_sparse_store<1, S>, grid, kThreads, st, count, G, k, t, act, tmp, lat0, L->epoch);
+  by_vec(row_shape(1, k).vec, [&](auto vec) {
+    constexpr int VEC = decltype(vec)::value;
+    for (int t = 0; t < P; ++t) {
+      const int j = dir(t);
+      const int64_t count = L->act_off[j + 1] - L->act_off[j];
+      if (count == 0) continue;
+      const int32_t* act = L->act + L->act_off[j];
+      const int32_t* nbr_j = L->nbr + (size_t)j * L->r * 2 * L->m;
+      const RowShape q = row_shape(count, k);
+      launch_pdl(k_sparse_blur<VEC, S>, q.blocks, q.threads, st, count, q.G, k, L->r, tp, t, act,
+                 nbr_j, L->m, L->epoch, pw, lat0, tmp);
+      launch_pdl(k_sparse_store<VEC, S>, q.blocks, q.threads, st, count, q.G, k, t, act, tmp, lat0,
+                 L->epoch);
+      note_launches(2);
     }
-    note_launches(2);
-  }
-  if (pw) {
-    const unsigned grid = (unsigned)ceil_div(L->m * G, kThreads);
-    if (v4) launch_pdl(k_sparse_finish<4, S>, grid, kThreads, st, L->m, G, k, P, L->epoch, pw, lat0);
-    else launch_pdl(k_sparse_finish<1, S>, grid, kThreads, st, L->m, G, k, P, L->epoch, pw, lat0);
-    note_launches(1);
-  }
+    if (pw) {
+      const RowShape q = row_shape(L->m, k);
+      launch_pdl(k_sparse_finish<VEC, S>, q.blocks, q.threads, st, L->m, q.G, k, P, L->epoch, pw,
+                 lat0);
+      note_launches(1);
+    }
+  });
   return lat0;
 }
 
-// The whole operator with explicit buffers.  internal: V and out in locality order;
-// else V and out are in the caller's order and V is first gathered into `vperm`.
+// The whole operator with explicit buffers, whose rows have kp columns.  internal: V and out
+// are [n][kp] in locality order; else V and out are the caller's [n][k] and V is first
+// gathered into `vperm`.  kt: see launch_splat_t.
 template <class S>
-int enqueue_t(const Lattice* L, const float* V, int k, int blur, float alpha, float beta,
-              float* out, S* lat0, S* lat1, float* partial, float* vperm, cudaStream_t st,
-              cudaEvent_t* ev, bool internal, double* dot_partial = nullptr,
+int enqueue_t(const Lattice* L, const float* V, int k, int kp, int kt, int blur, float alpha,
+              float beta, float* out, S* lat0, S* lat1, float* partial, float* vperm,
+              cudaStream_t st, cudaEvent_t* ev, bool internal, double* dot_partial = nullptr,
               bool dense = false) {
   const float* src = V;
   if (!internal) {
-    launch_permute(L, V, k, vperm, st);
+    launch_permute(L, V, k, kp, vperm, st);
     src = vperm;
   }
   if (ev) cudaEventRecordWithFlags(ev[2], st, cudaEventRecordExternal);
-  launch_splat_t<S>(L, src, k, lat0, partial, st);
+  launch_splat_t<S>(L, src, kp, kt, lat0, partial, st);
   // External: inside a stream capture this becomes an event-record node of the graph
   if (ev) cudaEventRecordWithFlags(ev[0], st, cudaEventRecordExternal);
   int passes = 0;
-  S* a = blur_passes_t<S>(L, blur, lat0, lat1, k, st, &passes, dense);
+  S* a = blur_passes_t<S>(L, blur, lat0, lat1, kp, st, &passes, dense);
   if (ev) cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal);
-  if (internal && dot_partial) launch_slice_dot<S>(L, a, V, k, alpha, beta, out, dot_partial, st);
-  else if (internal) launch_slice_t<false, S>(L, a, V, k, alpha, beta, out, st);
-  else launch_slice_t<true, S>(L, a, V, k, alpha, beta, out, st);
+  if (internal && dot_partial) launch_slice_dot<S>(L, a, V, kp, alpha, beta, out, dot_partial, st);
+  else if (internal) launch_slice_t<false, S>(L, a, V, kp, kp, alpha, beta, out, st);
+  else launch_slice_t<true, S>(L, a, src, k, kp, alpha, beta, out, st);
   if (ev) cudaEventRecordWithFlags(ev[3], st, cudaEventRecordExternal);
   return passes;
 }
 
-// Splat (locality-ordered input) and blur only; returns the buffer holding the result.
+// Splat (locality-ordered input, rows of kp) and blur only; returns the buffer holding the
+// result.
 template <class S>
-S* splat_blur_t(const Lattice* L, const float* Vp, int k, int blur, S* lat0, S* lat1,
+S* splat_blur_t(const Lattice* L, const float* Vp, int kp, int kt, int blur, S* lat0, S* lat1,
                 float* partial, cudaStream_t st) {
-  launch_splat_t<S>(L, Vp, k, lat0, partial, st);
-  return blur_passes_t<S>(L, blur, lat0, lat1, k, st, nullptr, false);
+  launch_splat_t<S>(L, Vp, kp, kt, lat0, partial, st);
+  return blur_passes_t<S>(L, blur, lat0, lat1, kp, st, nullptr, false);
 }
 
 size_t value_size(const Lattice* L) {
@@ -728,18 +756,21 @@ sgp_status ensure_lattice_values(Lattice* L, int k, cudaStream_t st) {
 }
 
 int enqueue_mvm(const Lattice* L, const float* V, int k, int blur, float alpha, float beta,
-                float* out, cudaStream_t st, cudaEvent_t* ev, bool internal, double* dot_partial) {
+                float* out, cudaStream_t st, cudaEvent_t* ev, bool internal, double* dot_partial,
+                int tree_k) {
+  const int kp = internal ? k : value_cols(L, k);
+  const int kt = tree_k > 0 ? tree_k : k;
   if (L->value_dtype == SGP_VALUES_BF16)
-    return enqueue_t<bf16>(L, V, k, blur, alpha, beta, out, (bf16*)L->lat[0], (bf16*)L->lat[1],
-                           L->partial, L->vperm, st, ev, internal, dot_partial);
-  return enqueue_t<float>(L, V, k, blur, alpha, beta, out, (float*)L->lat[0], (float*)L->lat[1],
-                          L->partial, L->vperm, st, ev, internal, dot_partial);
+    return enqueue_t<bf16>(L, V, k, kp, kt, blur, alpha, beta, out, (bf16*)L->lat[0],
+                           (bf16*)L->lat[1], L->partial, L->vperm, st, ev, internal, dot_partial);
+  return enqueue_t<float>(L, V, k, kp, kt, blur, alpha, beta, out, (float*)L->lat[0],
+                          (float*)L->lat[1], L->partial, L->vperm, st, ev, internal, dot_partial);
 }
 
 void enqueue_mvm_bf16_values(const Lattice* L, const float* V, int k, int blur, float alpha,
                              float* out, cudaStream_t st) {
-  enqueue_t<bf16>(L, V, k, blur, alpha, 0.f, out, (bf16*)L->lat[0], (bf16*)L->lat[1], L->partial,
-                  L->vperm, st, nullptr, /*internal=*/true);
+  enqueue_t<bf16>(L, V, k, k, k, blur, alpha, 0.f, out, (bf16*)L->lat[0], (bf16*)L->lat[1],
+                  L->partial, L->vperm, st, nullptr, /*internal=*/true);
 }
 
 int64_t slice_dot_blocks(const Lattice* L, int k) {
@@ -776,37 +807,50 @@ void enqueue_mvm_into(const Lattice* L, const float* V_user, int k, int blur, fl
   float* vperm = reinterpret_cast<float*>(w + 2 * vb + round256((size_t)L->nslots * k * sizeof(float)));
   // the fixed work area holds no direction-list buffers: dense passes
   if (L->value_dtype == SGP_VALUES_BF16)
-    enqueue_t<bf16>(L, V_user, k, blur, alpha, beta, out, (bf16*)lat0, (bf16*)lat1, partial, vperm,
+    enqueue_t<bf16>(L, V_user, k, k, k, blur, alpha, beta, out, (bf16*)lat0, (bf16*)lat1, partial, vperm,
                     st, nullptr, false, nullptr, /*dense=*/true);
   else
-    enqueue_t<float>(L, V_user, k, blur, alpha, beta, out, (float*)lat0, (float*)lat1, partial,
+    enqueue_t<float>(L, V_user, k, k, k, blur, alpha, beta, out, (float*)lat0, (float*)lat1, partial,
                      vperm, st, nullptr, false, nullptr, /*dense=*/true);
 }
 
-void* enqueue_splat_blur(const Lattice* L, const float* Vp, int k, int blur, void* lat0,
+void* enqueue_splat_blur(const Lattice* L, const float* Vp, int kp, int kt, int blur, void* lat0,
                          void* lat1, float* partial, cudaStream_t st) {
   if (L->value_dtype == SGP_VALUES_BF16)
-    return splat_blur_t<bf16>(L, Vp, k, blur, (bf16*)lat0, (bf16*)lat1, partial, st);
-  return splat_blur_t<float>(L, Vp, k, blur, (float*)lat0, (float*)lat1, partial, st);
+    return splat_blur_t<bf16>(L, Vp, kp, kt, blur, (bf16*)lat0, (bf16*)lat1, partial, st);
+  return splat_blur_t<float>(L, Vp, kp, kt, blur, (float*)lat0, (float*)lat1, partial, st);
 }
 
-void enqueue_permute(const Lattice* L, const float* V, int k, float* Vp, cudaStream_t st) {
-  launch_permute(L, V, k, Vp, st);
+void enqueue_permute(const Lattice* L, const float* V, int k, int kp, float* Vp, cudaStream_t st) {
+  launch_permute(L, V, k, kp, Vp, st);
 }
 
-void enqueue_slice_caller(const Lattice* L, const void* lat, int k, float alpha, float* out,
+void enqueue_slice_caller(const Lattice* L, const void* lat, int k, int kp, float alpha, float* out,
                           cudaStream_t st) {
   if (L->value_dtype == SGP_VALUES_BF16)
-    launch_slice_t<true, bf16>(L, (const bf16*)lat, nullptr, k, alpha, 0.f, out, st);
+    launch_slice_t<true, bf16>(L, (const bf16*)lat, nullptr, k, kp, alpha, 0.f, out, st);
   else
-    launch_slice_t<true, float>(L, (const float*)lat, nullptr, k, alpha, 0.f, out, st);
+    launch_slice_t<true, float>(L, (const float*)lat, nullptr, k, kp, alpha, 0.f, out, st);
 }
 
 size_t lattice_value_bytes(const Lattice* L, int k) { return (size_t)L->m * k * value_size(L); }
 
+int padded_cols(int k) { return k <= 2 ? k : (k + 3) / 4 * 4; }
+
+int value_cols(const Lattice* L, int k) { return L->tight_cols ? k : padded_cols(k); }
+
+sgp_status ensure_product(Lattice* L, int k, cudaStream_t st) {
+  sgp_status s = ensure_lattice_values(L, value_cols(L, k), st);
+  if (s == SGP_ERR_OOM && !L->tight_cols && padded_cols(k) != k) {
+    L->tight_cols = true;  // no room for zero columns: products of this lattice go without
+    s = ensure_lattice_values(L, k, st);
+  }
+  return s;
+}
+
 sgp_status run_mvm(Lattice* L, const float* V, int k, int blur, float alpha, float beta,
                    float* out) {
-  sgp_status s = ensure_lattice_values(L, k, L->stream);
+  sgp_status s = ensure_product(L, k, L->stream);
   if (s != SGP_OK) return s;
   enqueue_mvm(L, V, k, blur, alpha, beta, out, L->stream);
   cudaError_t e = cudaGetLastError();

@@ -108,6 +108,7 @@ struct sgp_lattice {
   size_t lat_elems = 0;
   size_t lat_bytes = 0;  // value buffers + splat partials + permuted input
   size_t vperm_elems = 0;
+  bool tight_cols = false;  // products use unpadded rows (value_cols): memory was short
 
   // Optional blur timing: events bracket the blur passes of one MVM inside the CG graph
   // and are read at every flag check (sgp_profile_blur / sgp_profile_read).
@@ -144,13 +145,15 @@ cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t st);
 
 // ---- programmatic dependent launch ----
 // Back-to-back dependent kernels on one stream start about 4.1 us apart on GB300 when each
-// launch waits for the previous grid to drain, and 1.4-1.6 us apart when the next grid is
-// already resident and only waits for the data (measured: 200 dependent kernels of 152
-// blocks, legacy and created streams; inside a graph 1.15 and 0.94 us).  launch_pdl marks a
-// launch as such a dependent; every kernel launched with it starts with pdl_enter(), which
-// lets the next grid in early and then waits until all work before this grid has completed
-// and is visible.  Nothing is read or written before that wait, so ordering is as with
-// ordinary launches.
+// launch waits for the previous grid to drain, and 1.4-1.6 us apart when it is set up
+// beforehand and only waits for the data (measured: 200 dependent kernels of 152 blocks,
+// legacy and created streams; inside a graph 1.15 and 0.94 us).  launch_pdl marks a launch as
+// such a dependent; every kernel launched with it starts with pdl_enter(), which waits until
+// all work before this grid has completed and is visible.  Nothing is read or written
+// before that wait, so ordering is as with ordinary launches.  No kernel lets its dependents
+// in early (griddepcontrol.launch_dependents): their waiting blocks take slots from the
+// running grid (a product at n = 50k, d = 8, k = 9: 63 us without, 78 us with it at the top
+// of each kernel; eight CG iterations at n = 86k, d = 8: 998 and 1154 us).
 template <class... P, class... A>
 inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... args) {
   cudaLaunchAttribute at{};
@@ -165,7 +168,6 @@ inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t
   (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);  // read by cudaGetLastError
 }
 __device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -194,14 +196,22 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls);
 // Make sure the lattice value buffers, splat partials and permuted-input buffer hold
 // what a k-column product needs (allocated on `st`).
 sgp_status ensure_lattice_values(Lattice* L, int k, cudaStream_t st);
-// Enqueue out = alpha * W B W^T V + beta * V on `st` (buffers must be ready).  With
-// internal = false, V and out are in the caller's point order (V is first permuted into
-// locality order); with internal = true both are already in locality order (CG).  When
-// `ev` is given, ev[0] / ev[1] are recorded around the blur passes.  Returns the number
-// of blur passes.
+// Columns of a row inside the operator for a caller's k (zero columns appended), and what
+// this lattice uses (k itself once the padded buffers did not fit).
+int padded_cols(int k);
+int value_cols(const Lattice* L, int k);
+// ensure_lattice_values for a public k-column product (value_cols columns).
+sgp_status ensure_product(Lattice* L, int k, cudaStream_t st);
+// Enqueue out = alpha * W B W^T V + beta * V on `st` (buffers must be ready: ensure_product,
+// or ensure_lattice_values when internal).  With internal = false, V and out are the
+// caller's [n][k] in the caller's point order (V is first permuted into locality order);
+// with internal = true both are [n][k] in locality order (CG; 16-byte aligned rows or k <=
+// 2).  When `ev` is given, ev[0] / ev[1] are recorded around the blur passes.  tree_k > 0:
+// the column count that shapes the huge vertices' sums (k otherwise).  Returns the number of
+// blur passes.
 int enqueue_mvm(const Lattice* L, const float* V, int k, int blur, float alpha, float beta,
                 float* out, cudaStream_t st, cudaEvent_t* ev = nullptr, bool internal = false,
-                double* dot_partial = nullptr);
+                double* dot_partial = nullptr, int tree_k = 0);
 // out = alpha K V (V and out in locality order) with the lattice values held in bf16 whatever
 // the lattice's value type, in the lattice's own value buffers, which
 // ensure_lattice_values(L, k) must have sized (a bf16 value takes half the room of an fp32
@@ -219,13 +229,14 @@ size_t mvm_work_bytes(const Lattice* L, int k);
 // (mvm_work_bytes(L, k) bytes, 256-byte aligned); allocates nothing.
 void enqueue_mvm_into(const Lattice* L, const float* V, int k, int blur, float alpha,
                       float beta, float* out, void* work, cudaStream_t st);
-// Pieces of the operator for the backward: splat a locality-ordered Vp and blur it (the
-// result ends in the returned buffer, lat0 or lat1, of the handle's value type); gather
-// the caller's rows into locality order; out (caller's order) = alpha W lat.
-void* enqueue_splat_blur(const Lattice* L, const float* Vp, int k, int blur, void* lat0,
+// Pieces of the operator for the backward: splat a locality-ordered Vp (rows of kp) and blur
+// it (the result ends in the returned buffer, lat0 or lat1, of the handle's value type; kt
+// as enqueue_mvm's tree_k); gather the caller's rows of k into locality-ordered rows of kp;
+// out (caller's order, rows of k) = alpha W lat.
+void* enqueue_splat_blur(const Lattice* L, const float* Vp, int kp, int kt, int blur, void* lat0,
                          void* lat1, float* partial, cudaStream_t st);
-void enqueue_permute(const Lattice* L, const float* V, int k, float* Vp, cudaStream_t st);
-void enqueue_slice_caller(const Lattice* L, const void* lat, int k, float alpha, float* out,
+void enqueue_permute(const Lattice* L, const float* V, int k, int kp, float* Vp, cudaStream_t st);
+void enqueue_slice_caller(const Lattice* L, const void* lat, int k, int kp, float alpha, float* out,
                           cudaStream_t st);
 size_t lattice_value_bytes(const Lattice* L, int k);
 // Full operator on the handle's stream, allocating value buffers when needed.
@@ -297,7 +308,7 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
 
 // ---- CG (cg.cu) ----
 // Device buffers that receive the CG coefficients of every column for the Lanczos
-// quadrature: alpha_j / beta_j of column c at [j][k] for j < cap, ||b_c|| and the
+// quadrature: alpha_j / beta_j of column c at [j][padded_cols(k)] for j < cap, ||b_c|| and the
 // iteration count per column.
 struct LanczosRecord {
   double* alpha;

@@ -32,6 +32,15 @@ struct Store<float> {
     reinterpret_cast<float4*>(p)[0] = a;
     reinterpret_cast<float4*>(p)[1] = b;
   }
+  static __device__ __forceinline__ float2 ld2(const float* p) {
+    return *reinterpret_cast<const float2*>(p);
+  }
+  static __device__ __forceinline__ float2 ldg2(const float* p) {
+    return __ldg(reinterpret_cast<const float2*>(p));
+  }
+  static __device__ __forceinline__ void st2(float* p, float2 v) {
+    *reinterpret_cast<float2*>(p) = v;
+  }
   static __device__ __forceinline__ float ld1(const float* p) { return *p; }
   static __device__ __forceinline__ void st1(float* p, float v) { *p = v; }
 };
@@ -72,6 +81,15 @@ struct Store<bf16> {
     *reinterpret_cast<uint4*>(p) =
         make_uint4(pack2(a.x, a.y), pack2(a.z, a.w), pack2(b.x, b.y), pack2(b.z, b.w));
   }
+  static __device__ __forceinline__ float2 ld2(const bf16* p) {
+    return unpack2(*reinterpret_cast<const uint32_t*>(p));
+  }
+  static __device__ __forceinline__ float2 ldg2(const bf16* p) {
+    return unpack2(__ldg(reinterpret_cast<const uint32_t*>(p)));
+  }
+  static __device__ __forceinline__ void st2(bf16* p, float2 v) {
+    *reinterpret_cast<uint32_t*>(p) = pack2(v.x, v.y);
+  }
   static __device__ __forceinline__ float ld1(const bf16* p) { return __bfloat162float(*p); }
   static __device__ __forceinline__ void st1(bf16* p, float v) { *p = __float2bfloat16_rn(v); }
 };
@@ -86,7 +104,7 @@ __device__ __forceinline__ void split3(float x, bf16& a, bf16& b, bf16& c) {
   c = __float2bfloat16_rn(r1 - __bfloat162float(b));
 }
 
-// ---- fp32 register vectors of VEC = 4 or 1 columns ----------------------------------
+// ---- fp32 register vectors of VEC = 4, 2 or 1 columns -------------------------------
 template <int VEC>
 struct Vec;
 template <>
@@ -113,6 +131,27 @@ struct Vec<4> {
   static __device__ __forceinline__ T scale(float a, T x) {
     return make_float4(a * x.x, a * x.y, a * x.z, a * x.w);
   }
+};
+template <>
+struct Vec<2> {
+  using T = float2;
+  static __device__ __forceinline__ T zero() { return make_float2(0.f, 0.f); }
+  static __device__ __forceinline__ T ld(const float* p) { return *reinterpret_cast<const float2*>(p); }
+  static __device__ __forceinline__ void st(float* p, T v) { *reinterpret_cast<float2*>(p) = v; }
+  static __device__ __forceinline__ T ldg(const float* p) {
+    return __ldg(reinterpret_cast<const float2*>(p));
+  }
+  template <class S>
+  static __device__ __forceinline__ T lds(const S* p) { return Store<S>::ld2(p); }
+  template <class S>
+  static __device__ __forceinline__ T ldgs(const S* p) { return Store<S>::ldg2(p); }
+  template <class S>
+  static __device__ __forceinline__ void sts(S* p, T v) { Store<S>::st2(p, v); }
+  static __device__ __forceinline__ T fma(float a, T x, T y) {
+    return make_float2(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y));
+  }
+  static __device__ __forceinline__ T add(T x, T y) { return make_float2(x.x + y.x, x.y + y.y); }
+  static __device__ __forceinline__ T scale(float a, T x) { return make_float2(a * x.x, a * x.y); }
 };
 template <>
 struct Vec<1> {
