@@ -92,34 +92,284 @@ __device__ __forceinline__ bool entry_has_key(uint32_t e, const int* key, int d,
 // ---------------------------------------------------------------------------------
 // 1. Elevation, enclosing simplex, barycentric weights.
 // ---------------------------------------------------------------------------------
+// FP64 issues at about 2 results per SM and clock on this part, so the elevation is bound by
+// its count of fp64 operations (comparisons and conversions included).  Where the result is
+// the same, divisions become a multiplication with an exact correction, conversions become
+// integer operations on the bits, and the rounding to a multiple of D starts from a fp32
+// guess that a fp64 residual confirms: 14 fp64 operations a coordinate.
+
+// Correctly rounded a / b from rb = RN(1 / b) (one Newton correction with an exact remainder;
+// Markstein, "Computation of elementary functions on the IBM RISC System/6000", 1990).  With
+// q0 = RN(a rb), |q0 - a/b| <= 2 ulp(q0).  Here b has at most 24 significant bits (a
+// lengthscale, or D) and a is a float or a difference of magnitude |q0 b|, so a - q0 b is a
+// multiple of ulp(q0) ulp(b) below 2^26 of them: exact in one fma.  Then q0 + r rb differs from
+// a/b by at most 2^-51 ulp(q0), while a/b is at least 2^-25 ulp(q0) away from every
+// rounding boundary (a - M b is a non-zero multiple of ulp(b) ulp(q0) / 2 for a 54-bit M, and
+// M b = a would need more bits than a has), so the last fma rounds to RN(a/b).  a = 0 keeps
+// its sign through q0.
+__device__ __forceinline__ double div_rn(double a, double b, double rb) {
+  const double q0 = __dmul_rn(a, rb);
+  const double q = __fma_rn(__fma_rn(-q0, b, a), rb, q0);
+  return (__double_as_longlong(a) << 1) == 0 ? q0 : q;
+}
+
+// (double)x, and x to 22 bits or more as a float (0 below 2^-126; callers bound it above).
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), e = (u >> 23) & 255u;
+  if (e == 0u || e == 255u) return (double)x;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))),
+                          (int)(u << 29));
+}
+__device__ __forceinline__ float narrow(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), m = hi & 0x7fffffffu;
+  if (m < (897u << 20)) return 0.f;
+  return __uint_as_float((hi & 0x80000000u) | ((m - (896u << 20)) << 3) |
+                         ((uint32_t)__double2loint(x) >> 29));
+}
+
+constexpr int kElevT = 128;  // points per block
+
+// Order-preserving integer image of a residual's fp64 bits (-0 taken as +0, no NaN here).
+__device__ __forceinline__ long long rank_key(double x) {
+  long long bits = __double_as_longlong(x);
+  if (bits == (long long)0x8000000000000000ull) bits = 0;
+  return bits ^ ((bits >> 63) & 0x7fffffffffffffffLL);
+}
+
+// (double) of an integer below 2^24 in magnitude.
+__device__ __forceinline__ double exact_int(int x) {
+  return x == 0 ? 0.0 : widen((float)x);
+}
+
+// Nearest multiple of D to y (ties go down) as an integer, and y minus it.  False when the
+// multiple lies beyond +-32000 (NaN included).
+__device__ __noinline__ bool nearest_multiple_exact(double y, int D, int& r0, double& delta) {
+  const double q = __ddiv_rn(y, (double)D);
+  if (!(fabs(q) < 40000.0)) return false;
+  const int lo = __double2int_rd(q) * D;
+  const double below = __dsub_rn(y, (double)lo);            // y - down
+  const double above = __dsub_rn((double)(lo + D), y);      // up - y
+  const bool up = above < below;
+  r0 = up ? lo + D : lo;
+  delta = up ? -above : below;
+  return r0 <= 32000 && r0 >= -32000;
+}
+// The same: a multiple whose residual is below D / 2 is the nearest one, however it was
+// guessed.  The test compares the high words (2^-20 short of D / 2 at most); what it does
+// not pass, ties and values beyond the range included, takes the exact path.
+__device__ __forceinline__ bool nearest_multiple(double y, int D, float rD, int half_hi, int& r0,
+                                                 double& delta) {
+  const int y_hi = __double2hiint(y) & 0x7fffffff;
+  if (y_hi < __double2hiint(32000.0)) {
+    const int guess = __float2int_rn(narrow(y) * rD) * D;
+    delta = __dsub_rn(y, exact_int(guess));
+    if ((__double2hiint(delta) & 0x7fffffff) < half_hi && guess <= 32000 && guess >= -32000) {
+      r0 = guess;
+      return true;
+    }
+  }
+  return nearest_multiple_exact(y, D, r0, delta);
+}
+
+// Range of rem0 / D per coordinate over all points, the caller's warps arriving converged;
+// the plain read spares the atomic where the value would not change.
+__device__ __forceinline__ void note_range(int q, int c, int* qmin, int* qmax, unsigned active,
+                                           bool leader) {
+  const int lo = __reduce_min_sync(active, q), hi = __reduce_max_sync(active, q);
+  if (!leader) return;
+  if (lo < __ldcg(qmin + c)) atomicMin(qmin + c, lo);
+  if (hi > __ldcg(qmax + c)) atomicMax(qmax + c, hi);
+}
+
+// D <= MAXD <= 16: one thread per point, all per-coordinate values in registers (fully
+// unrolled loops), the inputs and outputs of a block staged in shared memory so that global
+// rows move coalesced, the rank-indexed weights through a conflict-free shared column.
+// n = 2M, d = 11: 0.91 ms, against 2.05 ms with per-thread local arrays and fp64 divisions.
 template <int MAXD>
-__global__ void __launch_bounds__(128) k_elevate(const float* __restrict__ X,
-                                                 const float* __restrict__ ls,
-                                                 const double* __restrict__ f, int64_t n,
-                                                 int d, int16_t* __restrict__ rem0_out,
-                                                 uint8_t* __restrict__ rank_out,
-                                                 float* __restrict__ w_out,
-                                                 int* __restrict__ qmin, int* __restrict__ qmax,
-                                                 unsigned* __restrict__ err, int inject_nan) {
+__global__ void __launch_bounds__(kElevT) k_elevate_small(
+    const float* __restrict__ X, const float* __restrict__ ls, const double* __restrict__ f,
+    int64_t n, int d, int16_t* __restrict__ rem0_out, uint8_t* __restrict__ rank_out,
+    float* __restrict__ w_out, int* __restrict__ qmin, int* __restrict__ qmax,
+    unsigned* __restrict__ err, int inject_nan) {
   pdl_enter();
+  __shared__ double s_l[MAXD], s_rl[MAXD], s_f[MAXD];
+  __shared__ int s_bad;  // a lengthscale is not finite and positive
+  __shared__ double s_v[MAXD][kElevT];  // then the block's outputs
+  __shared__ float s_x[kElevT * MAXD];
+  const int tid = threadIdx.x;
+  const int D = d + 1;
+  const double Dd = (double)D, rD = __drcp_rn(Dd);
+  const float rDf = 1.f / (float)D;
+  const int half_hi = __double2hiint(0.5 * Dd);
+  const int64_t i0 = (int64_t)blockIdx.x * kElevT;
+  const int pts = (int)min((int64_t)kElevT, n - i0);
+  if (tid == 0) s_bad = 0;
+  __syncthreads();
+  if (tid < d) {
+    const float lv = ls[tid];
+    const double l = (double)lv;
+    if (!isfinite(lv) || !(lv > 0.f)) s_bad = 1;
+    s_l[tid] = l;
+    s_rl[tid] = __drcp_rn(l);
+    s_f[tid] = f[tid];
+  }
+  for (int q = tid; q < pts * d; q += kElevT) s_x[q] = X[i0 * d + q];
+  __syncthreads();
+  const bool live = tid < pts;
+  bool bad = s_bad != 0;
+  double y[MAXD];
+  double sm = 0.0;
+#pragma unroll
+  for (int c = MAXD - 1; c >= 1; --c) {
+    y[c] = 0.0;
+    if (c > d) continue;
+    const float xv = live ? s_x[tid * d + (c - 1)] : 0.f;
+    if (!isfinite(xv)) bad = true;
+    const double cf = __dmul_rn(div_rn(widen(xv), s_l[c - 1], s_rl[c - 1]), s_f[c - 1]);
+    y[c] = __dsub_rn(sm, __dmul_rn((double)c, cf));
+    sm = __dadd_rn(sm, cf);
+  }
+  y[0] = sm;
+  if (inject_nan && i0 + tid == 0) bad = true;  // SGP_FAULT=nan_input
+  if (bad) {
+    if (live) atomicOr(err, ERRBIT_NONFINITE);
+#pragma unroll
+    for (int c = 0; c < MAXD; ++c) y[c] = 0.0;
+  }
+  int rem0[MAXD], rank[MAXD];
+  long long key[MAXD];
+  int sum = 0;
+  bool range = false;
+#pragma unroll
+  for (int c = 0; c < MAXD; ++c) {
+    rem0[c] = 0;
+    key[c] = 0;
+    if (c >= D) continue;
+    double delta = 0.0;
+    if (!nearest_multiple(y[c], D, rDf, half_hi, rem0[c], delta)) range = true;
+    key[c] = rank_key(delta);
+    sum += rem0[c];
+  }
+  if (range) {  // keep the rest of the computation in bounds; the build reports the error
+    if (live) atomicOr(err, ERRBIT_RANGE);
+    sum = 0;
+#pragma unroll
+    for (int c = 0; c < MAXD; ++c) {
+      y[c] = 0.0;
+      rem0[c] = 0;
+      key[c] = 0;
+    }
+  }
+  // rank: strictly larger residuals, plus equal residuals at a lower index; then move rem0
+  // onto H_d (coordinate sum 0)
+  const int h = sum / D;
+#pragma unroll
+  for (int c = 0; c < MAXD; ++c) {
+    rank[c] = 0;
+    if (c >= D) continue;
+    int rk = h;
+#pragma unroll
+    for (int c2 = 0; c2 < MAXD; ++c2) {
+      if (c2 == c || c2 >= D) continue;
+      rk += (c2 < c ? key[c2] >= key[c] : key[c2] > key[c]) ? 1 : 0;
+    }
+    if (rk < 0) {
+      rk += D;
+      rem0[c] += D;
+    } else if (rk > d) {
+      rk -= D;
+      rem0[c] -= D;
+    }
+    rank[c] = min(max(rk, 0), d);  // already true when sum(y) = 0; guards the indexing
+    s_v[rank[c]][tid] = div_rn(__dsub_rn(y[c], exact_int(rem0[c])), Dd, rD);
+  }
+#pragma unroll
+  for (int c = 0; c < MAXD; ++c) {
+    if (c >= D) continue;
+    // rem0 is a multiple of D: exact; idle threads repeat their warp's first point, if any
+    const int first = __shfl_sync(0xffffffffu, rem0[c], 0);
+    note_range((live ? rem0[c] : first) / D, c, qmin, qmax, 0xffffffffu,
+               (tid & 31) == 0 && tid < pts);
+  }
+  // w[t] = v of rank d - t minus v of rank D - t (w[0]: plus one)
+  float w[MAXD];
+  {
+    const double first = s_v[d][tid], last = s_v[0][tid];
+    w[0] = __double2float_rn(__dadd_rn(first, __dadd_rn(1.0, -last)));
+#pragma unroll
+    for (int t = 1; t < MAXD; ++t)
+      if (t < D) w[t] = __double2float_rn(__dsub_rn(s_v[d - t][tid], s_v[D - t][tid]));
+  }
+  __syncthreads();
+  float* o_w = s_x;  // reuse: kElevT * D floats, then ranks and rem0 in the s_v area
+  int16_t* o_r = reinterpret_cast<int16_t*>(&s_v[0][0]);
+  uint8_t* o_k = reinterpret_cast<uint8_t*>(o_r + kElevT * MAXD);
+  if (live) {
+#pragma unroll
+    for (int c = 0; c < MAXD; ++c) {
+      if (c >= D) continue;
+      o_w[tid * D + c] = w[c];
+      o_r[tid * D + c] = (int16_t)rem0[c];
+      o_k[tid * D + c] = (uint8_t)rank[c];
+    }
+  }
+  __syncthreads();
+  const int64_t e0 = i0 * D;  // a multiple of 128: 4-byte words of every output stay aligned
+  const int count = pts * D;
+  for (int q = tid; q < count; q += kElevT) w_out[e0 + q] = o_w[q];
+  for (int q = 2 * tid; q < count; q += 2 * kElevT) {
+    if (q + 1 < count) *reinterpret_cast<uint32_t*>(rem0_out + e0 + q) = *reinterpret_cast<uint32_t*>(o_r + q);
+    else rem0_out[e0 + q] = o_r[q];
+  }
+  for (int q = 4 * tid; q < count; q += 4 * kElevT) {
+    if (q + 3 < count) *reinterpret_cast<uint32_t*>(rank_out + e0 + q) = *reinterpret_cast<uint32_t*>(o_k + q);
+    else
+      for (int z = q; z < count; ++z) rank_out[e0 + z] = o_k[z];
+  }
+}
+
+// Any D <= MAXD: one thread per point, per-coordinate values in local memory (n = 500k, d =
+// 20: 0.46 ms, before 0.96; n = 60k, d = 50: 0.33 ms, before 0.48).
+template <int MAXD>
+__global__ void __launch_bounds__(kElevT) k_elevate(const float* __restrict__ X,
+                                                    const float* __restrict__ ls,
+                                                    const double* __restrict__ f, int64_t n,
+                                                    int d, int16_t* __restrict__ rem0_out,
+                                                    uint8_t* __restrict__ rank_out,
+                                                    float* __restrict__ w_out,
+                                                    int* __restrict__ qmin, int* __restrict__ qmax,
+                                                    unsigned* __restrict__ err, int inject_nan) {
+  pdl_enter();
+  __shared__ double s_l[MAXD], s_rl[MAXD], s_f[MAXD];
+  __shared__ int s_bad;  // a lengthscale is not finite and positive
+  const int D = d + 1;
+  if (threadIdx.x == 0) s_bad = 0;
+  __syncthreads();
+  for (int c = threadIdx.x; c < d; c += kElevT) {
+    const float lv = ls[c];
+    const double l = (double)lv;
+    if (!isfinite(lv) || !(lv > 0.f)) s_bad = 1;
+    s_l[c] = l;
+    s_rl[c] = __drcp_rn(l);
+    s_f[c] = f[c];
+  }
+  __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int D = d + 1;
-  const double Dd = (double)D;
-  double y[MAXD];
+  const double Dd = (double)D, rD = __drcp_rn(Dd);
+  const float rDf = 1.f / (float)D;
+  const int half_hi = __double2hiint(0.5 * Dd);
+  double y[MAXD];  // then the weights' differences by rank
   int rem0[MAXD];
   int rank[MAXD];
-  double b[MAXD + 1];
-  bool bad = false;
+  bool bad = s_bad != 0;
   // y = E z, E's column j is (1, .., 1, -(j+1), 0, ..) / sqrt((j+1)(j+2)) times the scale;
   // f[j] already holds scale / sqrt((j+1)(j+2)).
   double sm = 0.0;
   for (int c = d; c >= 1; --c) {
     const float xv = X[i * d + (c - 1)];
-    const float lv = ls[c - 1];
-    if (!isfinite(xv) || !isfinite(lv) || !(lv > 0.f)) bad = true;
-    const double z = __ddiv_rn((double)xv, (double)lv);
-    const double cf = __dmul_rn(z, f[c - 1]);
+    if (!isfinite(xv)) bad = true;
+    const double cf = __dmul_rn(div_rn(widen(xv), s_l[c - 1], s_rl[c - 1]), s_f[c - 1]);
     y[c] = __dsub_rn(sm, __dmul_rn((double)c, cf));
     sm = __dadd_rn(sm, cf);
   }
@@ -132,35 +382,26 @@ __global__ void __launch_bounds__(128) k_elevate(const float* __restrict__ X,
   // nearest remainder-0 point coordinate by coordinate (ties go down)
   int sum = 0;
   bool range = false;
+  long long key[MAXD];
   for (int c = 0; c < D; ++c) {
-    const double q = __ddiv_rn(y[c], Dd);
-    const double lo = floor(q);
-    const double down = __dmul_rn(lo, Dd);
-    const double up = __dadd_rn(down, Dd);
-    const double r0 = (__dsub_rn(up, y[c]) < __dsub_rn(y[c], down)) ? up : down;
-    if (!(fabs(r0) <= 32000.0)) {
-      range = true;
-      rem0[c] = 0;
-    } else {
-      rem0[c] = (int)r0;
-    }
-    sum += rem0[c];
+    double delta = 0.0;
+    int r0 = 0;
+    if (!nearest_multiple(y[c], D, rDf, half_hi, r0, delta)) range = true;
+    rem0[c] = r0;
+    key[c] = rank_key(delta);
+    sum += r0;
   }
   if (range) {  // keep the rest of the computation in bounds; the build reports the error
+    atomicOr(err, ERRBIT_RANGE);
     sum = 0;
     for (int c = 0; c < D; ++c) {
       y[c] = 0.0;
       rem0[c] = 0;
+      key[c] = 0;
     }
   }
-  // rank: strictly larger residuals, plus equal residuals at a lower index.  The residuals
-  // are compared through an order-preserving integer image of their fp64 bits (-0 taken as
-  // +0, no NaN here), the same order as the fp64 comparison at integer-compare cost.
-  long long key[MAXD];
-  for (int c = 0; c < D; ++c) {
-    const long long bits = __double_as_longlong(__dadd_rn(__dsub_rn(y[c], (double)rem0[c]), 0.0));
-    key[c] = bits ^ ((bits >> 63) & 0x7fffffffffffffffLL);
-  }
+  // rank: strictly larger residuals, plus equal residuals at a lower index (compared through
+  // their integer images, the same order at integer-compare cost)
   for (int c = 0; c < D; ++c) {
     const long long kc = key[c];
     int rk = 0;
@@ -168,44 +409,32 @@ __global__ void __launch_bounds__(128) k_elevate(const float* __restrict__ X,
     for (int c2 = c + 1; c2 < D; ++c2) rk += key[c2] > kc ? 1 : 0;
     rank[c] = rk;
   }
-  // move rem0 onto H_d (coordinate sum 0)
+  // move rem0 onto H_d (coordinate sum 0); b holds the weights' terms by rank
   const int h = sum / D;
+  double b[MAXD];
   for (int c = 0; c < D; ++c) {
-    rank[c] += h;
-    if (rank[c] < 0) {
-      rank[c] += D;
+    int rk = rank[c] + h;
+    if (rk < 0) {
+      rk += D;
       rem0[c] += D;
-    } else if (rank[c] > d) {
-      rank[c] -= D;
+    } else if (rk > d) {
+      rk -= D;
       rem0[c] -= D;
     }
-    rank[c] = min(max(rank[c], 0), d);  // already true when sum(y) = 0; guards the indexing
+    rk = min(max(rk, 0), d);  // already true when sum(y) = 0; guards the indexing
+    rank[c] = rk;
+    b[rk] = div_rn(__dsub_rn(y[c], exact_int(rem0[c])), Dd, rD);
   }
-  for (int c = 0; c <= D; ++c) b[c] = 0.0;
-  for (int c = 0; c < D; ++c) {
-    const double v = __ddiv_rn(__dsub_rn(y[c], (double)rem0[c]), Dd);
-    b[d - rank[c]] = __dadd_rn(b[d - rank[c]], v);
-    b[D - rank[c]] = __dsub_rn(b[D - rank[c]], v);
-  }
-  b[0] = __dadd_rn(b[0], __dadd_rn(1.0, b[D]));
-  if (range) atomicOr(err, ERRBIT_RANGE);
   for (int c = 0; c < D; ++c) {
     rem0_out[i * D + c] = (int16_t)rem0[c];
     rank_out[i * D + c] = (uint8_t)rank[c];
-    w_out[i * D + c] = __double2float_rn(b[c]);
+    const double w = c == 0 ? __dadd_rn(b[d], __dadd_rn(1.0, -b[0])) : __dsub_rn(b[d - c], b[D - c]);
+    w_out[i * D + c] = __double2float_rn(w);
   }
   const unsigned active = __activemask();
-  const int lane = threadIdx.x & 31;
-  const bool leader = lane == __ffs(active) - 1;
-  for (int c = 0; c < d; ++c) {
-    const int q = rem0[c] / D;  // rem0 is a multiple of D: exact
-    const int qlo = __reduce_min_sync(active, q);
-    const int qhi = __reduce_max_sync(active, q);
-    if (leader) {
-      atomicMin(&qmin[c], qlo);
-      atomicMax(&qmax[c], qhi);
-    }
-  }
+  const bool leader = (int)(threadIdx.x & 31) == __ffs(active) - 1;
+  for (int c = 0; c < D; ++c)  // rem0 is a multiple of D: exact
+    note_range(rem0[c] / D, c, qmin, qmax, active, leader);
 }
 
 // ---------------------------------------------------------------------------------
@@ -736,9 +965,20 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   }
   SGP_CHECK(cudaMemsetAsync(L->err, 0, sizeof(unsigned), st), "memset err");
   {
-    const int B = 128;
-    SGP_DISPATCH_D(D, k_elevate, (unsigned)ceil_div(n, B), B, st, X, ls, f, n, d, rem0, rank,
-                   w_user, qmm, qmm + D, L->err, L->fault == FAULT_NAN_INPUT ? 1 : 0);
+    const unsigned grid = (unsigned)ceil_div(n, kElevT);
+    const int nan = L->fault == FAULT_NAN_INPUT ? 1 : 0;
+    auto go = [&](auto kernel) {
+      launch_pdl(kernel, grid, kElevT, st, X, ls, f, n, d, rem0, rank, w_user, qmm, qmm + D, L->err,
+                 nan);
+    };
+    if (D <= 4) go(k_elevate_small<4>);
+    else if (D <= 8) go(k_elevate_small<8>);
+    else if (D <= 12) go(k_elevate_small<12>);
+    else if (D <= 16) go(k_elevate_small<16>);
+    else if (D <= 32) go(k_elevate<32>);
+    else if (D <= 64) go(k_elevate<64>);
+    else go(k_elevate<128>);
+    note_launches(1);
     SGP_CHECK(cudaGetLastError(), "k_elevate");
   }
   unsigned herr = 0;
