@@ -15,7 +15,8 @@
 //                    atomicMin keeps the earliest entry as owner.
 //  4. numbering      vertex ids = first occurrence in locality order (owner flags +
 //                    exclusive scan).
-//  5. k_neighbours   per vertex and direction j: ids of v +- t u_j, u_j = (d+1) e_j - 1.
+//  5. k_neighbours   per vertex and direction j: ids of v +- t u_j, u_j = (d+1) e_j - 1, by
+//                    looking the shifted linear hashes up in the sorted vertex hashes.
 //  6. splat lists    (vertex, entry) pairs sorted stably by vertex id (radix sort) give
 //                    each vertex the list of (point, weight) it gathers.
 #include <algorithm>
@@ -38,11 +39,6 @@ __device__ __forceinline__ uint64_t mix64(uint64_t h) {
   h ^= h >> 33;
   return h;
 }
-// Vertex-filter bit of a linear hash: its upper half (the linear hash's high bits mix every
-// coordinate through the odd 64-bit multipliers), cheap for the filter test that every
-// (vertex, direction) candidate makes; the table's slot and tag still come from mix64.
-__device__ __forceinline__ uint32_t filter_hash(uint64_t h) { return (uint32_t)(h >> 32); }
-
 uint64_t host_mix64(uint64_t h) {
   h ^= h >> 33;
   h *= 0xff51afd7ed558ccdull;
@@ -517,8 +513,7 @@ __global__ void k_assign_ids(const uint32_t* __restrict__ scanned,
                              const int32_t* __restrict__ perm, const int16_t* __restrict__ rem0,
                              const uint8_t* __restrict__ rank, int64_t nD, int d,
                              int32_t* __restrict__ slot_id, int16_t* __restrict__ keys,
-                             uint64_t* __restrict__ vhash, int2* __restrict__ vrange,
-                             uint32_t* __restrict__ bloom, uint64_t bloom_mask) {
+                             uint64_t* __restrict__ vhash, uint32_t* __restrict__ owner) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nD) return;
@@ -527,10 +522,10 @@ __global__ void k_assign_ids(const uint32_t* __restrict__ scanned,
   const int D = d + 1;
   const uint32_t id = scanned[e];
   slot_id[s] = (int32_t)id;
+  owner[id] = (uint32_t)e;
   const int64_t i = perm[e / D];
   const int k = (int)(e % D);
   uint64_t h = 0;
-  int lo = 1 << 30, hi = -(1 << 30);
   int16_t* row = keys + (int64_t)id * D;
   // the row's coordinates, stored two per 4-byte word where the row is 4-byte aligned
   int c = 0;
@@ -538,8 +533,6 @@ __global__ void k_assign_ids(const uint32_t* __restrict__ scanned,
     const int x = vertex_coord(rem0 + i * D, rank + i * D, d, k, 0);
     row[0] = (int16_t)x;
     h += coord_mult(0) * (uint64_t)(int64_t)x;
-    lo = min(lo, x);
-    hi = max(hi, x);
     c = 1;
   }
   for (; c + 1 < D; c += 2) {
@@ -548,20 +541,13 @@ __global__ void k_assign_ids(const uint32_t* __restrict__ scanned,
     *reinterpret_cast<uint32_t*>(row + c) =
         (uint32_t)(uint16_t)(int16_t)x0 | ((uint32_t)(uint16_t)(int16_t)x1 << 16);
     h += coord_mult(c) * (uint64_t)(int64_t)x0 + coord_mult(c + 1) * (uint64_t)(int64_t)x1;
-    lo = min(lo, min(x0, x1));
-    hi = max(hi, max(x0, x1));
   }
   if (c < D) {
     const int x = vertex_coord(rem0 + i * D, rank + i * D, d, k, c);
     row[c] = (int16_t)x;
     h += coord_mult(c) * (uint64_t)(int64_t)x;
-    lo = min(lo, x);
-    hi = max(hi, x);
   }
   vhash[id] = h;
-  vrange[id] = make_int2(lo, hi);
-  const uint64_t b = filter_hash(h) & bloom_mask;  // the vertex's filter bit
-  atomicOr(&bloom[b >> 5], 1u << (b & 31));
 }
 
 __global__ void k_entry_ids(const int32_t* __restrict__ entry_slot,
@@ -583,123 +569,244 @@ __global__ void k_entry_ids(const int32_t* __restrict__ entry_slot,
 // ---------------------------------------------------------------------------------
 // 5. Neighbour table.
 // ---------------------------------------------------------------------------------
-// Does the vertex of entry `e` equal keys[v] + step u_j?  (the owner entry's key is
-// recomputed from its point's rem0 and rank)
-__device__ __forceinline__ bool entry_is_neighbour(uint32_t e, const int16_t* __restrict__ kv,
-                                                   int j, int step, int d,
-                                                   const int32_t* __restrict__ perm,
-                                                   const int16_t* __restrict__ rem0,
-                                                   const uint8_t* __restrict__ rank) {
+// A lattice step u_j moves the linear hash by a constant delta_j, so the vertices in hash
+// order have their candidates v + t u_j in hash order too: a warp's 32 lookups of one
+// direction fall into a few neighbouring buckets of the sorted hashes and read a few
+// consecutive sectors, where probing a hash table (or a bit filter) in any other order
+// touches a sector of its own for every candidate.  The index holds 32 bits of each hash
+// beside its bucket, so that it stays in L2 up to some 15M vertices.  One side is looked up;
+// a match is confirmed on the keys and written on both (u is v + t u_j, v is u - t u_j).
+// Consecutive vertices of a simplex are one step apart (vertex k + 1 is vertex k minus u_c, c
+// the coordinate of rank d - k, cyclically), so every vertex starts with the two links its
+// own simplex gives it, and those need no confirmation.
+// Measured, all steps of the table (the filter and table probes of every candidate that this
+// replaced in brackets): n = 500k, d = 20 (m = 10.5M) 1.9 ms (5.1); n = 60k, d = 50 (m = 3.1M)
+// 1.1 ms (5.0); n = 2M, d = 11 (m = 1.6M) 0.75 ms (1.4).
+
+// nbr[j][t][side][v]: the links of v's owner simplex, -1 elsewhere; up[v]: the direction along
+// which v's link upwards lies.  owner[v]: its entry.
+__global__ void __launch_bounds__(256) k_nbr_init(const uint32_t* __restrict__ owner,
+                                                  const int32_t* __restrict__ idx,
+                                                  const uint8_t* __restrict__ rank, int64_t m, int d,
+                                                  int r, int32_t* __restrict__ nbr,
+                                                  uint8_t* __restrict__ up) {
+  pdl_enter();
+  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= m) return;
   const int D = d + 1;
-  const int64_t i = perm[e / D];
-  const int k = (int)(e % D);
-  for (int c = 0; c < D; ++c) {
-    const int want = (int)kv[c] + step * ((c == j ? D : 0) - 1);
-    if (vertex_coord(rem0 + i * D, rank + i * D, d, k, c) != want) return false;
+  const uint32_t e = owner[v];
+  const uint32_t p = e / (uint32_t)D;
+  const int k = (int)(e - p * (uint32_t)D);
+  const int64_t row = (int64_t)p * D;
+  // v - u_c, c of rank d - k, is vertex k + 1 (0 after d); v + u_c, c of rank d - k + 1 (0
+  // for k = 0), is vertex k - 1 (d before 0)
+  const int below = idx[row + (k == d ? 0 : k + 1)], above = idx[row + (k == 0 ? d : k - 1)];
+  const int rk_below = d - k, rk_above = k == 0 ? 0 : d - k + 1;
+  int dir = 0;
+  for (int j = 0; j < D; ++j) {
+    const int rk = rank[row + j];
+    if (rk == rk_above) dir = j;
+    int32_t* q = nbr + (int64_t)j * r * 2 * m + v;
+    __stcs(q, rk == rk_below ? below : -1);
+    __stcs(q + m, rk == rk_above ? above : -1);
+    for (int t = 2; t <= r; ++t) {
+      __stcs(q + (int64_t)(2 * t - 2) * m, -1);
+      __stcs(q + (int64_t)(2 * t - 1) * m, -1);
+    }
   }
-  return true;
+  up[v] = (uint8_t)dir;
 }
 
-// One thread per vertex, all directions j: ids of v -+ t u_j, t = 1..r, and hasnb[j / 32]
-// [v] bit j % 32: whether v has a neighbour along j.  The neighbour's
-// hash comes from the vertex's linear hash in O(1) (sum_A = sum_c A_c); most absent
-// neighbours stop at the vertex filter (one bit per hash, sized to stay in L2); the key
-// itself is read only to confirm a tag match.  The filter words of kNbrGroup directions
-// (both signs) are loaded together before any of them is tested, so that their latencies
-// overlap.  A neighbour outside the int16 key range does not exist.  counts[j]
-// accumulates the vertices with a neighbour along j.
-constexpr int kNbrGroup = 8;
-__global__ void __launch_bounds__(256) k_neighbours(
-    const int16_t* __restrict__ keys, const uint64_t* __restrict__ vhash,
-    const int2* __restrict__ vrange, int64_t m, int d, int r, uint64_t sum_A,
-    const unsigned long long* __restrict__ table, uint64_t mask,
-    const int32_t* __restrict__ slot_id, const int32_t* __restrict__ perm,
-    const int16_t* __restrict__ rem0, const uint8_t* __restrict__ rank,
-    const uint32_t* __restrict__ bloom, uint64_t bloom_mask, int32_t* __restrict__ nbr,
-    unsigned long long* __restrict__ counts, uint32_t* __restrict__ hasnb) {
+// The other ends of those links, where they belong to another simplex and so did not write
+// theirs.  (Several simplices may write one link; they write the same id.)
+__global__ void __launch_bounds__(256) k_nbr_close(const uint32_t* __restrict__ owner,
+                                                   const int32_t* __restrict__ idx,
+                                                   const uint8_t* __restrict__ rank, int64_t m,
+                                                   int d, int r, int32_t* __restrict__ nbr) {
   pdl_enter();
-  __shared__ unsigned block_count[kMaxD];  // this block's vertices with a neighbour along j
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= m) return;
   const int D = d + 1;
-  for (int j = threadIdx.x; j < D; j += blockDim.x) block_count[j] = 0;
+  const uint32_t e = owner[v];
+  const uint32_t p = e / (uint32_t)D;
+  const int k = (int)(e - p * (uint32_t)D);
+  const int64_t row = (int64_t)p * D;
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {  // 0: the link below v, 1: the link above
+    const int other = side == 0 ? (k == d ? 0 : k + 1) : (k == 0 ? d : k - 1);
+    const int u = idx[row + other];
+    if (owner[u] == (uint32_t)(row + other)) continue;
+    const int rk = side == 0 ? d - k : (k == 0 ? 0 : d - k + 1);
+    int j = 0;
+    while (rank[row + j] != rk) ++j;  // ranks are a permutation of 0..d
+    nbr[((int64_t)j * r * 2 + (side == 0 ? 1 : 0)) * m + u] = (int32_t)v;
+  }
+}
+
+// Sort keys: the top bits of the vertex hashes.
+__global__ void k_hash_keys(const uint64_t* __restrict__ vhash, int64_t m, int shift,
+                            uint32_t* __restrict__ key, uint32_t* __restrict__ val) {
+  pdl_enter();
+  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= m) return;
+  key[v] = (uint32_t)(vhash[v] >> shift);
+  val[v] = (uint32_t)v;
+}
+
+// Of the i-th vertex in bucket order: its hash (low and high half) and its direction up;
+// start[b] = first i of bucket b (b <= buckets).
+__global__ void k_hash_index(const uint32_t* __restrict__ key, const uint32_t* __restrict__ ord,
+                             const uint64_t* __restrict__ vhash, const uint8_t* __restrict__ up,
+                             int64_t m, int64_t buckets, uint32_t* __restrict__ low,
+                             uint32_t* __restrict__ high, uint8_t* __restrict__ up_sorted,
+                             uint32_t* __restrict__ start) {
+  pdl_enter();
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= m) return;
+  const uint64_t h = vhash[ord[i]];
+  low[i] = (uint32_t)h;
+  high[i] = (uint32_t)(h >> 32);
+  up_sorted[i] = up[ord[i]];
+  const int64_t own = key[i];
+  for (int64_t b = i == 0 ? 0 : (int64_t)key[i - 1] + 1; b <= own; ++b) start[b] = (uint32_t)i;
+  if (i == m - 1)
+    for (int64_t b = own + 1; b <= buckets; ++b) start[b] = (uint32_t)m;
+}
+
+// Does coordinate c of u equal that of v + t u_j?  Coordinates stay within +-32255 (rem0 within
+// 32000, the sum fix and the vertex offset add less than 2 D), so no sum leaves int16.
+__device__ __forceinline__ bool steps_to(int16_t v, int16_t u, int c, int j, int t, int D) {
+  return (int)u == (int)v + t * ((c == j ? D : 0) - 1);
+}
+
+// Thread i: the i-th vertex in hash order, all directions but the one its simplex gave.  The
+// bucket bounds of kNbrGroup directions are loaded together, then their first hashes, so
+// that their latencies overlap; a lane walks its bucket on its own.  Matches are confirmed on
+// the keys by the thread itself for D <= 16 (every row load in flight at once), by the whole
+// warp, one after another, above (a lane alone would walk a row of D loads while 31 wait).
+// *hits receives the number of pairs (v, v + u_j).
+constexpr int kNbrGroup = 4;
+template <bool WARP>
+__global__ void __launch_bounds__(256) k_neighbours(
+    const int16_t* __restrict__ keys, const uint32_t* __restrict__ low,
+    const uint32_t* __restrict__ high, const uint8_t* __restrict__ up,
+    const uint32_t* __restrict__ ord, const uint32_t* __restrict__ start, int shift, int64_t m,
+    int d, int r, uint64_t sum_A, int32_t* __restrict__ nbr, unsigned long long* __restrict__ hits) {
+  pdl_enter();
+  __shared__ uint64_t delta[kMaxD];  // hash of u_j
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int D = d + 1, lane = (int)(threadIdx.x & 31);
+  for (int j = threadIdx.x; j < D; j += blockDim.x) delta[j] = (uint64_t)D * coord_mult(j) - sum_A;
   __syncthreads();
-  const bool live = v < m;
-  const uint64_t hv = live ? vhash[v] : 0;
-  const int2 rg = live ? vrange[v] : make_int2(0, 0);
-  const int16_t* kv = keys + (live ? v : 0) * D;
-  uint32_t word = 0;  // bits j % 32 of the directions with a neighbour, 32 at a time
+  const bool live = i < m;
+  const uint64_t h = live ? (uint64_t)high[i] << 32 | low[i] : 0;
+  const int given = live ? up[i] : 0;
+  unsigned found = live ? 1u : 0u;  // the given pair
   for (int j0 = 0; j0 < D; j0 += kNbrGroup) {
-    uint32_t any = 0;  // bit q: a neighbour along j0 + q
     for (int t = 1; t <= r; ++t) {
-      // filter bits of the group's 2 kNbrGroup candidates: bit 2 q + sg
-      uint32_t hits = 0;
+      uint32_t want[kNbrGroup], at[kNbrGroup], p[kNbrGroup], end[kNbrGroup];
+#pragma unroll
+      for (int q = 0; q < kNbrGroup; ++q) {
+        const uint64_t x = h + (uint64_t)t * delta[min(j0 + q, D - 1)];
+        const uint32_t* s = start + (x >> shift);
+        const bool on = live && j0 + q < D && (t > 1 || j0 + q != given);
+        want[q] = (uint32_t)x;
+        p[q] = on ? __ldg(s) : 0u;
+        end[q] = on ? __ldg(s + 1) : 0u;
+      }
+#pragma unroll
+      for (int q = 0; q < kNbrGroup; ++q) at[q] = p[q] < end[q] ? __ldg(low + p[q]) : 0u;
 #pragma unroll
       for (int q = 0; q < kNbrGroup; ++q) {
         const int j = j0 + q;
-        // t lin(u_j): the hash moves by -t lin(u_j) (sg = 0) or + t lin(u_j) (sg = 1)
-        const uint64_t tdj = (uint64_t)t * ((uint64_t)D * coord_mult(j < D ? j : 0) - sum_A);
+        int32_t* plane = nbr + ((int64_t)j * r + (t - 1)) * 2 * m;
+        bool more = true;
+        while (more) {
+          while (p[q] < end[q] && at[q] != want[q])
+            if (++p[q] < end[q]) at[q] = __ldg(low + p[q]);
+          __syncwarp();
+          const bool match = p[q] < end[q];
+          unsigned todo = __ballot_sync(0xffffffffu, match);
+          if (!todo) break;
+          uint32_t u = 0, v = 0;
+          if (match) {
+            u = __ldg(ord + p[q]);
+            v = __ldg(ord + i);
+          }
+          bool ok = false;
+          if (WARP) {
+            while (todo) {
+              const int src = __ffs(todo) - 1;
+              todo &= todo - 1;
+              const int16_t* kv = keys + (int64_t)__shfl_sync(0xffffffffu, v, src) * D;
+              const int16_t* ku = keys + (int64_t)__shfl_sync(0xffffffffu, u, src) * D;
+              bool same = true;
 #pragma unroll
-        for (int sg = 0; sg < 2; ++sg) {
-          const uint64_t b = filter_hash(sg ? hv + tdj : hv - tdj) & bloom_mask;
-          const uint32_t word = (live && j < D) ? __ldg(bloom + (b >> 5)) : 0u;
-          hits |= ((word >> (b & 31)) & 1u) << (2 * q + sg);
-        }
-      }
-      // absent unless a filter hit is confirmed in the table (streaming stores: the table
-      // is written once, and the vertex filter should keep its place in L2)
-      if (live) {
-        const int64_t sj = (int64_t)2 * r * m;  // from direction j to j + 1
-        int32_t* p0 = nbr + ((int64_t)j0 * 2 * r + 2 * (t - 1)) * m + v;
+              for (int c0 = 0; c0 < kMaxD; c0 += 32)
+                if (c0 < D && c0 + lane < D)
+                  same = same & steps_to(__ldg(kv + c0 + lane), __ldg(ku + c0 + lane), c0 + lane, j, t, D);
+              same = __all_sync(0xffffffffu, same);
+              ok = ok || (same && lane == src);
+            }
+          } else if (match) {
+            const int16_t *kv = keys + (int64_t)v * D, *ku = keys + (int64_t)u * D;
+            ok = true;
 #pragma unroll
-        for (int q = 0; q < kNbrGroup; ++q)
-          if (j0 + q < D) {
-            __stcs(p0 + q * sj, -1);
-            __stcs(p0 + q * sj + m, -1);
+            for (int c = 0; c < 16; ++c)
+              if (c < D) ok = ok & steps_to(__ldg(kv + c), __ldg(ku + c), c, j, t, D);
           }
-      }
-      while (hits) {
-        const int bit = __ffs(hits) - 1;
-        hits &= hits - 1;
-        const int q = bit >> 1, sg = bit & 1, j = j0 + q;
-        const int step = sg ? t : -t;
-        // every coordinate moves by -step except j, which moves by d step
-        bool in_range = rg.x - t * d >= -32768 && rg.y + t * d <= 32767;
-        if (!in_range) {
-          in_range = true;
-          for (int c = 0; c < D; ++c) {
-            const int x = (int)kv[c] + step * ((c == j ? D : 0) - 1);
-            in_range = in_range && x >= -32768 && x <= 32767;
+          if (ok) {
+            plane[u] = (int32_t)v;
+            plane[m + v] = (int32_t)u;
+            found += t == 1 ? 1u : 0u;
+            p[q] = end[q];
+          } else if (match && ++p[q] < end[q]) {  // another vertex with these hash bits
+            at[q] = __ldg(low + p[q]);
           }
-        }
-        if (!in_range) continue;
-        const uint64_t tdj = (uint64_t)t * ((uint64_t)D * coord_mult(j) - sum_A);
-        const uint64_t h = mix64(sg ? hv + tdj : hv - tdj);
-        const uint32_t tag = (uint32_t)(h >> 33);
-        uint64_t slot = h & mask;
-        for (uint64_t probe = 0; probe <= mask; ++probe) {
-          const unsigned long long cur = table[slot];
-          if (cur == kEmpty) break;
-          if ((uint32_t)(cur >> 32) == tag &&
-              entry_is_neighbour((uint32_t)cur, kv, j, step, d, perm, rem0, rank)) {
-            nbr[(((int64_t)j * r + (t - 1)) * 2 + sg) * m + v] = slot_id[slot];
-            any |= 1u << q;
-            break;
-          }
-          slot = (slot + 1) & mask;
+          more = __any_sync(0xffffffffu, p[q] < end[q]);
         }
       }
     }
-    // vertices with a neighbour along j: one shared-memory add per warp, one global add
-    // per block at the end
+  }
+  found = __reduce_add_sync(0xffffffffu, found);
+  if (lane == 0 && found) atomicAdd(hits, (unsigned long long)found);
+}
+
+// hasnb[j / 32][v] bit j % 32: whether v has a neighbour along j; counts[j]: the vertices that
+// have one.  Run only for lattices that may be sparse.
+__global__ void __launch_bounds__(256) k_active_flags(const int32_t* __restrict__ nbr, int64_t m,
+                                                      int D, int r, uint32_t* __restrict__ hasnb,
+                                                      unsigned long long* __restrict__ counts) {
+  pdl_enter();
+  __shared__ unsigned block_count[kMaxD];  // this block's vertices with a neighbour along j
+  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (int j = threadIdx.x; j < D; j += blockDim.x) block_count[j] = 0;
+  __syncthreads();
+  const bool live = v < m;
+  uint32_t word = 0;  // bits j % 32 of the directions with a neighbour, 32 at a time
+  constexpr int kGroup = 8;  // directions whose loads are in flight together
+  for (int j0 = 0; j0 < D; j0 += kGroup) {
+    int any[kGroup];
 #pragma unroll
-    for (int q = 0; q < kNbrGroup; ++q) {
-      if (j0 + q >= D) break;
-      const unsigned with = __ballot_sync(0xffffffffu, (any >> q) & 1u);
+    for (int q = 0; q < kGroup; ++q) any[q] = -1;
+    for (int z = 0; z < r; ++z) {
+      int a[kGroup][2];
+#pragma unroll
+      for (int q = 0; q < kGroup; ++q)
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg)
+          a[q][sg] = live && j0 + q < D ? __ldcs(nbr + (((int64_t)(j0 + q) * r + z) * 2 + sg) * m + v) : -1;
+#pragma unroll
+      for (int q = 0; q < kGroup; ++q) any[q] = max(any[q], max(a[q][0], a[q][1]));
+    }
+#pragma unroll
+    for (int q = 0; q < kGroup; ++q) {
+      const unsigned with = __ballot_sync(0xffffffffu, any[q] >= 0);
       if (with && (int)(threadIdx.x & 31) == __ffs(with) - 1)
         atomicAdd(&block_count[j0 + q], (unsigned)__popc(with));
+      word |= (any[q] >= 0 ? 1u : 0u) << ((j0 + q) & 31);
     }
-    word |= any << (j0 & 31);
-    if (((j0 + kNbrGroup) & 31) == 0 || j0 + kNbrGroup >= D) {
+    if (((j0 + kGroup) & 31) == 0 || j0 + kGroup >= D) {
       if (live) hasnb[(int64_t)(j0 >> 5) * m + v] = word;
       word = 0;
     }
@@ -998,6 +1105,14 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     return SGP_ERR_RANGE;
   }
 
+  // sort buffers, used in turn for the points, the vertex hashes and the splat lists
+  uint32_t *ka, *va, *kb, *vb, *rt;
+  SGP_CHECK(tmp.get(&ka, nD), "alloc sort");
+  SGP_CHECK(tmp.get(&va, nD), "alloc sort");
+  SGP_CHECK(tmp.get(&kb, nD), "alloc sort");
+  SGP_CHECK(tmp.get(&vb, nD), "alloc sort");
+  SGP_CHECK(tmp.get(&rt, radix_temp_elems(nD)), "alloc sort");
+
   // 2. locality order
   CellPack pk{};
   {
@@ -1010,12 +1125,6 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
       used += b;
       pk.shift[c] = b > 0 ? 32 - used : 0;  // a single-valued coordinate packs to 0
     }
-    uint32_t *ka, *va, *kb, *vb, *rt;
-    SGP_CHECK(tmp.get(&ka, n), "alloc sort");
-    SGP_CHECK(tmp.get(&va, n), "alloc sort");
-    SGP_CHECK(tmp.get(&kb, n), "alloc sort");
-    SGP_CHECK(tmp.get(&vb, n), "alloc sort");
-    SGP_CHECK(tmp.get(&rt, radix_temp_elems(n)), "alloc sort");
     launch_pdl(k_point_key, (unsigned)ceil_div(n, 256), 256, st, rem0, n, D, pk, ka, va);
     note_launches(1);
     // the packed cell occupies the top `used` bits; bits below are zero
@@ -1065,18 +1174,11 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   SGP_CHECK(dalloc(&L->keys, m * D, st), "alloc keys");
   L->bytes += m * D * sizeof(int16_t);
   uint64_t* vhash = nullptr;
-  int2* vrange = nullptr;
   SGP_CHECK(tmp.get(&vhash, m), "alloc vertex hashes");
-  SGP_CHECK(tmp.get(&vrange, m), "alloc vertex ranges");
-  // vertex filter: about 8 bits per vertex, 2^16 .. 2^29 bits
-  uint64_t bloom_bits = 1ull << 16;
-  while (bloom_bits < 8ull * (uint64_t)m && bloom_bits < (1ull << 29)) bloom_bits <<= 1;
-  uint32_t* bloom = nullptr;
-  SGP_CHECK(tmp.get(&bloom, bloom_bits / 32), "alloc vertex filter");
-  SGP_CHECK(cudaMemsetAsync(bloom, 0, bloom_bits / 8, st), "clear vertex filter");
+  uint32_t* owner = nullptr;  // [m] first entry of each vertex
+  SGP_CHECK(tmp.get(&owner, m), "alloc owners");
   launch_pdl(k_assign_ids, (unsigned)ceil_div(nD, 256), 256, st, flags, entry_slot, table, L->perm,
-                                                           rem0, rank, nD, d, slot_id, L->keys,
-                                                           vhash, vrange, bloom, bloom_bits - 1);
+             rem0, rank, nD, d, slot_id, L->keys, vhash, owner);
   note_launches(1);
   SGP_CHECK(dalloc(&L->idx, nD, st), "alloc idx");
   SGP_CHECK(dalloc(&L->w, nD, st), "alloc w");
@@ -1088,32 +1190,42 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   SGP_CHECK(cudaGetLastError(), "numbering");
 
   // 5. neighbour table
-  SGP_CHECK(dalloc(&L->nbr, (size_t)D * r * 2 * m, st), "alloc nbr");
-  L->bytes += (size_t)D * r * 2 * m * sizeof(int32_t);
-  unsigned long long* counts = nullptr;
-  SGP_CHECK(tmp.get(&counts, 2 * D), "alloc counts");
-  SGP_CHECK(cudaMemsetAsync(counts, 0, 2 * D * sizeof(unsigned long long), st), "clear counts");
-  uint32_t* hasnb = nullptr;  // [ceil(D / 32)][m] neighbour bits per direction
-  SGP_CHECK(tmp.get(&hasnb, (int64_t)((D + 31) / 32) * m), "alloc neighbour bits");
-  {
+  const size_t nbr_count = (size_t)D * r * 2 * m;
+  SGP_CHECK(dalloc(&L->nbr, nbr_count, st), "alloc nbr");
+  L->bytes += nbr_count * sizeof(int32_t);
+  unsigned long long* counts = nullptr;  // [D] vertices per direction, [D] fill, pairs (v, v + u_j)
+  SGP_CHECK(tmp.get(&counts, 2 * D + 1), "alloc counts");
+  SGP_CHECK(cudaMemsetAsync(counts, 0, (2 * D + 1) * sizeof(unsigned long long), st), "clear counts");
+  if (m > 0) {
+    // one to two vertices per bucket on average
+    const int bits = std::min(31, std::max(1, bits_for((uint64_t)(m - 1)) - 1));
+    const int64_t buckets = (int64_t)1 << bits;
+    uint32_t *low = nullptr, *high = nullptr, *start = nullptr;
+    uint8_t *up = nullptr, *up_sorted = nullptr;
+    SGP_CHECK(tmp.get(&low, m), "alloc sorted hashes");
+    SGP_CHECK(tmp.get(&high, m), "alloc sorted hashes");
+    SGP_CHECK(tmp.get(&up, m), "alloc links");
+    SGP_CHECK(tmp.get(&up_sorted, m), "alloc links");
+    SGP_CHECK(tmp.get(&start, buckets + 1), "alloc hash buckets");
+    const unsigned grid = (unsigned)ceil_div(m, 256);
+    launch_pdl(k_nbr_init, grid, 256, st, owner, L->idx, L->rank, m, d, r, L->nbr, up);
+    launch_pdl(k_nbr_close, grid, 256, st, owner, L->idx, L->rank, m, d, r, L->nbr);
+    launch_pdl(k_hash_keys, grid, 256, st, vhash, m, 64 - bits, ka, va);
+    const bool in_alt = radix_sort_pairs(ka, va, kb, vb, m, bits, rt, st);
+    const uint32_t* ord = in_alt ? vb : va;
+    launch_pdl(k_hash_index, grid, 256, st, in_alt ? kb : ka, ord, vhash, up, m, buckets,
+               low, high, up_sorted, start);
     // sum_c A_c over the D coordinates, as the kernels compute A_c
     uint64_t sum_A = 0;
     for (int c = 0; c < D; ++c) sum_A += host_coord_mult(c);
-    launch_pdl(k_neighbours, (unsigned)ceil_div(m, 256), 256, st, 
-        L->keys, vhash, vrange, m, d, r, sum_A, table, mask, slot_id, L->perm, rem0, rank,
-        bloom, bloom_bits - 1, L->nbr, counts, hasnb);
-    note_launches(1);
+    launch_pdl(D <= 16 ? k_neighbours<false> : k_neighbours<true>, grid, 256, st, L->keys, low, high,
+               up_sorted, ord, start, 64 - bits, m, d, r, sum_A, L->nbr, counts + 2 * D);
+    note_launches(5);
   }
   SGP_CHECK(cudaGetLastError(), "k_neighbours");
 
   // 6. splat lists: (vertex id, entry) sorted by id, stable in entry order
   {
-    uint32_t *ka, *va, *kb, *vb, *rt;
-    SGP_CHECK(tmp.get(&ka, nD), "alloc csr");
-    SGP_CHECK(tmp.get(&va, nD), "alloc csr");
-    SGP_CHECK(tmp.get(&kb, nD), "alloc csr");
-    SGP_CHECK(tmp.get(&vb, nD), "alloc csr");
-    SGP_CHECK(tmp.get(&rt, radix_temp_elems(nD)), "alloc csr");
     SGP_CHECK(cudaMemcpyAsync(ka, L->idx, nD * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st),
               "copy ids");
     launch_pdl(k_iota, (unsigned)ceil_div(nD, 256), 256, st, va, nD);
@@ -1134,6 +1246,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   }
 
   // 7. splat segments (load balance)
+  unsigned long long pairs = 0;  // (v, v + u_j) pairs: at least as many active vertices
   {
     uint32_t *cnt, *slots, *med, *huge, *tot, *stmp;
     SGP_CHECK(tmp.get(&cnt, m), "alloc seg");
@@ -1150,6 +1263,8 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     exclusive_scan_u32(huge, m, tot + 3, stmp, st);
     uint32_t ht[4];
     SGP_CHECK(cudaMemcpyAsync(ht, tot, sizeof(ht), cudaMemcpyDeviceToHost, st), "read seg");
+    SGP_CHECK(cudaMemcpyAsync(&pairs, counts + 2 * D, sizeof(pairs), cudaMemcpyDeviceToHost, st),
+              "read pairs");
     SGP_CHECK(cudaStreamSynchronize(st), "sync seg");
     L->nseg = ht[0];
     L->nslots = ht[1];
@@ -1170,8 +1285,13 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     note_launches(2);
     SGP_CHECK(cudaGetLastError(), "splat segments");
   }
-  // 8. direction lists of a sparse lattice (counts from k_neighbours)
-  {
+  // 8. direction lists of a sparse lattice
+  if ((double)pairs <= kSparseFrac * (double)D * (double)m) {
+    uint32_t* hasnb = nullptr;  // [ceil(D / 32)][m] neighbour bits per direction
+    SGP_CHECK(tmp.get(&hasnb, (int64_t)((D + 31) / 32) * m), "alloc neighbour bits");
+    launch_pdl(k_active_flags, (unsigned)std::max<int64_t>(1, ceil_div(m, 256)), 256, st, L->nbr, m,
+               D, r, hasnb, counts);
+    note_launches(1);
     std::vector<unsigned long long> hc(D);
     SGP_CHECK(cudaMemcpyAsync(hc.data(), counts, D * sizeof(unsigned long long),
                               cudaMemcpyDeviceToHost, st),
