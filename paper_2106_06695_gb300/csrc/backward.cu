@@ -265,14 +265,17 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
     BW_CHECK(w.get(&Vp, (size_t)n * kp * sizeof(float)), "alloc V");
     BW_CHECK(w.get(&Gp, (size_t)n * kp * sizeof(float)), "alloc G");
     enqueue_permute(L, G, k, kp, Gp, st);
-    // B^T W^T G into (b0, b1), B W^T V into the handle's buffers
+    // B^T W^T G into (b0, b1), B W^T V into the handle's buffers, each over its factor (both
+    // blurs have as many passes and the same centre tap: one factor)
+    double scale = 1.0;
     const void* BS = enqueue_splat_blur(L, Gp, kp, k, transpose_blur(blur), b0, b1, L->partial,
-                                        st);
+                                        st, &scale);
+    alpha = (float)(alpha * scale);
     if (dV) enqueue_slice_caller(L, BS, k, kp, alpha, dV, st);
     if (want_x) {
       enqueue_permute(L, V, k, kp, Vp, st);
       const void* BU = enqueue_splat_blur(L, Vp, kp, k, blur, L->lat[0], L->lat[1],
-                                          L->partial, st);
+                                          L->partial, st, &scale);
       const double scale = std::sqrt((double)(d * (d + 1))) / L->s;
       std::vector<double> hf(d);
       for (int j = 0; j < d; ++j) hf[j] = scale / std::sqrt((double)((j + 1) * (j + 2)));

@@ -581,7 +581,14 @@ __global__ void k_entry_ids(const int32_t* __restrict__ entry_slot,
 // own simplex gives it, and those need no confirmation.
 // Measured, all steps of the table (the filter and table probes of every candidate that this
 // replaced in brackets): n = 500k, d = 20 (m = 10.5M) 1.9 ms (5.1); n = 60k, d = 50 (m = 3.1M)
-// 1.1 ms (5.0); n = 2M, d = 11 (m = 1.6M) 0.75 ms (1.4).
+// 1.2 ms (5.0); n = 2M, d = 11 (m = 1.6M) 0.75 ms (1.4).
+
+// Bit j % 32 of above[j / 32][v] / below[j / 32][v]: v has a neighbour v + u_j / v - u_j
+// (stencil order 1).  Null: not recorded.
+struct LinkBits {
+  uint32_t* above;
+  uint32_t* below;
+};
 
 // nbr[j][t][side][v]: the links of v's owner simplex, -1 elsewhere; up[v]: the direction along
 // which v's link upwards lies.  owner[v]: its entry.
@@ -589,7 +596,7 @@ __global__ void __launch_bounds__(256) k_nbr_init(const uint32_t* __restrict__ o
                                                   const int32_t* __restrict__ idx,
                                                   const uint8_t* __restrict__ rank, int64_t m, int d,
                                                   int r, int32_t* __restrict__ nbr,
-                                                  uint8_t* __restrict__ up) {
+                                                  uint8_t* __restrict__ up, LinkBits lb) {
   pdl_enter();
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= m) return;
@@ -603,9 +610,17 @@ __global__ void __launch_bounds__(256) k_nbr_init(const uint32_t* __restrict__ o
   const int below = idx[row + (k == d ? 0 : k + 1)], above = idx[row + (k == 0 ? d : k - 1)];
   const int rk_below = d - k, rk_above = k == 0 ? 0 : d - k + 1;
   int dir = 0;
+  uint32_t has_above = 0, has_below = 0;
   for (int j = 0; j < D; ++j) {
     const int rk = rank[row + j];
     if (rk == rk_above) dir = j;
+    has_above |= (rk == rk_above ? 1u : 0u) << (j & 31);
+    has_below |= (rk == rk_below ? 1u : 0u) << (j & 31);
+    if (lb.above && ((j & 31) == 31 || j == d)) {
+      lb.above[(int64_t)(j >> 5) * m + v] = has_above;
+      lb.below[(int64_t)(j >> 5) * m + v] = has_below;
+      has_above = has_below = 0;
+    }
     int32_t* q = nbr + (int64_t)j * r * 2 * m + v;
     __stcs(q, rk == rk_below ? below : -1);
     __stcs(q + m, rk == rk_above ? above : -1);
@@ -622,7 +637,8 @@ __global__ void __launch_bounds__(256) k_nbr_init(const uint32_t* __restrict__ o
 __global__ void __launch_bounds__(256) k_nbr_close(const uint32_t* __restrict__ owner,
                                                    const int32_t* __restrict__ idx,
                                                    const uint8_t* __restrict__ rank, int64_t m,
-                                                   int d, int r, int32_t* __restrict__ nbr) {
+                                                   int d, int r, int32_t* __restrict__ nbr,
+                                                   LinkBits lb) {
   pdl_enter();
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= m) return;
@@ -640,6 +656,7 @@ __global__ void __launch_bounds__(256) k_nbr_close(const uint32_t* __restrict__ 
     int j = 0;
     while (rank[row + j] != rk) ++j;  // ranks are a permutation of 0..d
     nbr[((int64_t)j * r * 2 + (side == 0 ? 1 : 0)) * m + u] = (int32_t)v;
+    if (lb.above) atomicOr((side == 0 ? lb.above : lb.below) + (int64_t)(j >> 5) * m + u, 1u << (j & 31));
   }
 }
 
@@ -691,7 +708,8 @@ __global__ void __launch_bounds__(256) k_neighbours(
     const int16_t* __restrict__ keys, const uint32_t* __restrict__ low,
     const uint32_t* __restrict__ high, const uint8_t* __restrict__ up,
     const uint32_t* __restrict__ ord, const uint32_t* __restrict__ start, int shift, int64_t m,
-    int d, int r, uint64_t sum_A, int32_t* __restrict__ nbr, unsigned long long* __restrict__ hits) {
+    int d, int r, uint64_t sum_A, int32_t* __restrict__ nbr, unsigned long long* __restrict__ hits,
+    LinkBits lb) {
   pdl_enter();
   __shared__ uint64_t delta[kMaxD];  // hash of u_j
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -758,6 +776,10 @@ __global__ void __launch_bounds__(256) k_neighbours(
           if (ok) {
             plane[u] = (int32_t)v;
             plane[m + v] = (int32_t)u;
+            if (lb.above) {
+              atomicOr(lb.above + (int64_t)(j >> 5) * m + v, 1u << (j & 31));
+              atomicOr(lb.below + (int64_t)(j >> 5) * m + u, 1u << (j & 31));
+            }
             found += t == 1 ? 1u : 0u;
             p[q] = end[q];
           } else if (match && ++p[q] < end[q]) {  // another vertex with these hash bits
@@ -772,48 +794,52 @@ __global__ void __launch_bounds__(256) k_neighbours(
   if (lane == 0 && found) atomicAdd(hits, (unsigned long long)found);
 }
 
-// hasnb[j / 32][v] bit j % 32: whether v has a neighbour along j; counts[j]: the vertices that
-// have one.  Run only for lattices that may be sparse.
-__global__ void __launch_bounds__(256) k_active_flags(const int32_t* __restrict__ nbr, int64_t m,
-                                                      int D, int r, uint32_t* __restrict__ hasnb,
-                                                      unsigned long long* __restrict__ counts) {
+// The link bits read off the table, where they were not recorded while it was made; for r > 1,
+// above = any neighbour along the direction and below = 0.
+__global__ void __launch_bounds__(256) k_link_bits(const int32_t* __restrict__ nbr, int64_t m,
+                                                   int D, int r, LinkBits lb) {
   pdl_enter();
-  __shared__ unsigned block_count[kMaxD];  // this block's vertices with a neighbour along j
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (int j = threadIdx.x; j < D; j += blockDim.x) block_count[j] = 0;
-  __syncthreads();
-  const bool live = v < m;
-  uint32_t word = 0;  // bits j % 32 of the directions with a neighbour, 32 at a time
-  constexpr int kGroup = 8;  // directions whose loads are in flight together
-  for (int j0 = 0; j0 < D; j0 += kGroup) {
-    int any[kGroup];
-#pragma unroll
-    for (int q = 0; q < kGroup; ++q) any[q] = -1;
-    for (int z = 0; z < r; ++z) {
-      int a[kGroup][2];
-#pragma unroll
-      for (int q = 0; q < kGroup; ++q)
-#pragma unroll
-        for (int sg = 0; sg < 2; ++sg)
-          a[q][sg] = live && j0 + q < D ? __ldcs(nbr + (((int64_t)(j0 + q) * r + z) * 2 + sg) * m + v) : -1;
-#pragma unroll
-      for (int q = 0; q < kGroup; ++q) any[q] = max(any[q], max(a[q][0], a[q][1]));
+  if (v >= m) return;
+  for (int j0 = 0; j0 < D; j0 += 32) {
+    uint32_t hi = 0, lo = 0;
+    for (int j = j0; j < min(j0 + 32, D); ++j) {
+      const int32_t* p = nbr + (int64_t)j * 2 * r * m + v;
+      if (r == 1) {
+        lo |= (__ldcs(p) >= 0 ? 1u : 0u) << (j & 31);
+        hi |= (__ldcs(p + m) >= 0 ? 1u : 0u) << (j & 31);
+      } else {
+        int any = -1;
+        for (int q = 0; q < 2 * r; ++q) any = max(any, __ldcs(p + (int64_t)q * m));
+        hi |= (any >= 0 ? 1u : 0u) << (j & 31);
+      }
     }
-#pragma unroll
-    for (int q = 0; q < kGroup; ++q) {
-      const unsigned with = __ballot_sync(0xffffffffu, any[q] >= 0);
-      if (with && (int)(threadIdx.x & 31) == __ffs(with) - 1)
-        atomicAdd(&block_count[j0 + q], (unsigned)__popc(with));
-      word |= (any[q] >= 0 ? 1u : 0u) << ((j0 + q) & 31);
-    }
-    if (((j0 + kGroup) & 31) == 0 || j0 + kGroup >= D) {
-      if (live) hasnb[(int64_t)(j0 >> 5) * m + v] = word;
-      word = 0;
-    }
+    lb.above[(int64_t)(j0 >> 5) * m + v] = hi;
+    lb.below[(int64_t)(j0 >> 5) * m + v] = lo;
   }
+}
+
+// counts[j]: the vertices with a neighbour along j; heads[j]: those that head a chain along j
+// (one above and none below).
+__global__ void __launch_bounds__(256) k_link_counts(LinkBits lb, int64_t m, int D,
+                                                     unsigned long long* __restrict__ counts,
+                                                     unsigned long long* __restrict__ heads) {
+  pdl_enter();
+  __shared__ unsigned block_count[kMaxD], block_heads[kMaxD];
+  for (int j = threadIdx.x; j < D; j += blockDim.x) block_count[j] = block_heads[j] = 0;
   __syncthreads();
-  for (int j = threadIdx.x; j < D; j += blockDim.x)
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < m;
+       v += (int64_t)gridDim.x * blockDim.x)
+    for (int w = 0; w * 32 < D; ++w) {
+      const uint32_t hi = lb.above[(int64_t)w * m + v], lo = lb.below[(int64_t)w * m + v];
+      for (uint32_t x = hi | lo; x; x &= x - 1) atomicAdd(&block_count[w * 32 + __ffs(x) - 1], 1u);
+      for (uint32_t x = hi & ~lo; x; x &= x - 1) atomicAdd(&block_heads[w * 32 + __ffs(x) - 1], 1u);
+    }
+  __syncthreads();
+  for (int j = threadIdx.x; j < D; j += blockDim.x) {
     if (block_count[j]) atomicAdd(&counts[j], (unsigned long long)block_count[j]);
+    if (block_heads[j]) atomicAdd(&heads[j], (unsigned long long)block_heads[j]);
+  }
 }
 
 // Direction lists: thread per vertex, reading its direction bits (32 directions per word).
@@ -868,6 +894,66 @@ __global__ void __launch_bounds__(kFillThreads) k_active_fill(
       if (on) act[off[j] + wpos[warp][j] + __popc(with & ((1u << lane) - 1u))] = (int32_t)v;
     }
   }
+}
+
+// The same lists in chain order (stencil order 1): thread per vertex, for the directions in
+// which it heads a chain.  Every head walks its chain for the length (all lanes at once: the
+// walks are chains of dependent loads), the block takes one range of list slots and one of
+// chain slots per direction, and each head walks again to write its chain.  The order of
+// the chains is immaterial.  *longest: the longest chain.
+__global__ void __launch_bounds__(kFillThreads) k_chain_fill(
+    LinkBits lb, const int32_t* __restrict__ nbr, int64_t m, int D,
+    const int64_t* __restrict__ off, const int64_t* __restrict__ chain_off,
+    unsigned long long* __restrict__ fill, unsigned long long* __restrict__ chain_fill,
+    int32_t* __restrict__ act, uint2* __restrict__ chain, int* __restrict__ longest) {
+  pdl_enter();
+  __shared__ unsigned slen[kMaxD], scnt[kMaxD];  // this block's sums, then running positions
+  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool live = v < m;
+  for (int j = threadIdx.x; j < D; j += blockDim.x) slen[j] = scnt[j] = 0;
+  __syncthreads();
+  auto heads = [&](int w) {
+    return live ? lb.above[(int64_t)w * m + v] & ~lb.below[(int64_t)w * m + v] : 0u;
+  };
+  // length of the chain v heads along j (at most m steps: a line visits no vertex twice)
+  auto length = [&](int j) {
+    const int32_t* above = nbr + ((int64_t)j * 2 + 1) * m;
+    unsigned len = 1;
+    for (int32_t x = above[v]; x >= 0 && len < (unsigned)m; x = above[x]) ++len;
+    return len;
+  };
+  int most = 0;
+  for (int w = 0; w * 32 < D; ++w)
+    for (uint32_t x = heads(w); x; x &= x - 1) {
+      const int j = w * 32 + __ffs(x) - 1;
+      const unsigned len = length(j);
+      most = max(most, (int)len);
+      atomicAdd(&slen[j], len);
+      atomicAdd(&scnt[j], 1u);
+    }
+  most = __reduce_max_sync(0xffffffffu, most);
+  if ((threadIdx.x & 31) == 0 && most > __ldcg(longest)) atomicMax(longest, most);
+  __syncthreads();
+  for (int j = threadIdx.x; j < D; j += blockDim.x) {
+    if (scnt[j] == 0) continue;
+    slen[j] = (unsigned)atomicAdd(&fill[j], (unsigned long long)slen[j]);
+    scnt[j] = (unsigned)atomicAdd(&chain_fill[j], (unsigned long long)scnt[j]);
+  }
+  __syncthreads();
+  for (int w = 0; w * 32 < D; ++w)
+    for (uint32_t x = heads(w); x; x &= x - 1) {
+      const int j = w * 32 + __ffs(x) - 1;
+      const unsigned len = length(j);
+      const int64_t at = off[j] + atomicAdd(&slen[j], len);
+      const int64_t c = chain_off[j] + atomicAdd(&scnt[j], 1u);
+      const int32_t* above = nbr + ((int64_t)j * 2 + 1) * m;
+      int32_t y = (int32_t)v;
+      for (unsigned q = 0; q < len; ++q) {
+        act[at + q] = y;
+        y = above[y];
+      }
+      chain[c] = make_uint2((uint32_t)at, (uint32_t)(at + len));
+    }
 }
 
 // ---------------------------------------------------------------------------------
@@ -1193,10 +1279,21 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   const size_t nbr_count = (size_t)D * r * 2 * m;
   SGP_CHECK(dalloc(&L->nbr, nbr_count, st), "alloc nbr");
   L->bytes += nbr_count * sizeof(int32_t);
-  unsigned long long* counts = nullptr;  // [D] vertices per direction, [D] fill, pairs (v, v + u_j)
-  SGP_CHECK(tmp.get(&counts, 2 * D + 1), "alloc counts");
-  SGP_CHECK(cudaMemsetAsync(counts, 0, (2 * D + 1) * sizeof(unsigned long long), st), "clear counts");
+  // [D] vertices per direction, [D] list fill, pairs (v, v + u_j), [D] chains, [D] chain fill,
+  // longest chain
+  unsigned long long* counts = nullptr;
+  SGP_CHECK(tmp.get(&counts, 4 * D + 2), "alloc counts");
+  SGP_CHECK(cudaMemsetAsync(counts, 0, (4 * D + 2) * sizeof(unsigned long long), st), "clear counts");
+  LinkBits lb{nullptr, nullptr};
   if (m > 0) {
+    // few vertices belong to several simplices: the lattice is probably sparse, so record the
+    // links while they are found (two atomics a link; sparse ones have few beyond their own
+    // simplex's).  Otherwise k_link_bits reads them off the table if it turns out sparse.
+    if (r == 1 && m >= nD / 4) {
+      const int64_t words = (int64_t)((D + 31) / 32) * m;
+      SGP_CHECK(tmp.get(&lb.above, words), "alloc link bits");
+      SGP_CHECK(tmp.get(&lb.below, words), "alloc link bits");
+    }
     // one to two vertices per bucket on average
     const int bits = std::min(31, std::max(1, bits_for((uint64_t)(m - 1)) - 1));
     const int64_t buckets = (int64_t)1 << bits;
@@ -1208,8 +1305,9 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     SGP_CHECK(tmp.get(&up_sorted, m), "alloc links");
     SGP_CHECK(tmp.get(&start, buckets + 1), "alloc hash buckets");
     const unsigned grid = (unsigned)ceil_div(m, 256);
-    launch_pdl(k_nbr_init, grid, 256, st, owner, L->idx, L->rank, m, d, r, L->nbr, up);
-    launch_pdl(k_nbr_close, grid, 256, st, owner, L->idx, L->rank, m, d, r, L->nbr);
+    launch_pdl(k_nbr_init, grid, 256, st, owner, L->idx, L->rank, m, d, r, L->nbr, up, lb);
+    launch_pdl(k_nbr_close, grid, 256, st, owner, L->idx, L->rank, m, d, r, L->nbr,
+               lb);
     launch_pdl(k_hash_keys, grid, 256, st, vhash, m, 64 - bits, ka, va);
     const bool in_alt = radix_sort_pairs(ka, va, kb, vb, m, bits, rt, st);
     const uint32_t* ord = in_alt ? vb : va;
@@ -1219,7 +1317,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     uint64_t sum_A = 0;
     for (int c = 0; c < D; ++c) sum_A += host_coord_mult(c);
     launch_pdl(D <= 16 ? k_neighbours<false> : k_neighbours<true>, grid, 256, st, L->keys, low, high,
-               up_sorted, ord, start, 64 - bits, m, d, r, sum_A, L->nbr, counts + 2 * D);
+               up_sorted, ord, start, 64 - bits, m, d, r, sum_A, L->nbr, counts + 2 * D, lb);
     note_launches(5);
   }
   SGP_CHECK(cudaGetLastError(), "k_neighbours");
@@ -1287,13 +1385,19 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   }
   // 8. direction lists of a sparse lattice
   if ((double)pairs <= kSparseFrac * (double)D * (double)m) {
-    uint32_t* hasnb = nullptr;  // [ceil(D / 32)][m] neighbour bits per direction
-    SGP_CHECK(tmp.get(&hasnb, (int64_t)((D + 31) / 32) * m), "alloc neighbour bits");
-    launch_pdl(k_active_flags, (unsigned)std::max<int64_t>(1, ceil_div(m, 256)), 256, st, L->nbr, m,
-               D, r, hasnb, counts);
+    const unsigned vgrid = (unsigned)std::max<int64_t>(1, ceil_div(m, 256));
+    if (!lb.above) {
+      const int64_t words = (int64_t)((D + 31) / 32) * m;
+      SGP_CHECK(tmp.get(&lb.above, words), "alloc link bits");
+      SGP_CHECK(tmp.get(&lb.below, words), "alloc link bits");
+      launch_pdl(k_link_bits, vgrid, 256, st, L->nbr, m, D, r, lb);
+      note_launches(1);
+    }
+    launch_pdl(k_link_counts, std::min(vgrid, 8u * 152u), 256, st, lb, m, D, counts,
+               counts + 2 * D + 1);
     note_launches(1);
-    std::vector<unsigned long long> hc(D);
-    SGP_CHECK(cudaMemcpyAsync(hc.data(), counts, D * sizeof(unsigned long long),
+    std::vector<unsigned long long> hc(4 * D + 2);
+    SGP_CHECK(cudaMemcpyAsync(hc.data(), counts, hc.size() * sizeof(unsigned long long),
                               cudaMemcpyDeviceToHost, st),
               "read counts");
     SGP_CHECK(cudaStreamSynchronize(st), "sync counts");
@@ -1302,7 +1406,8 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
       total += (int64_t)hc[j];
       largest = std::max<int64_t>(largest, (int64_t)hc[j]);
     }
-    if (m > 0 && (double)total <= kSparseFrac * (double)D * (double)m) {
+    if (m > 0 && (double)total <= kSparseFrac * (double)D * (double)m &&
+        total <= (int64_t)0xffffffff) {  // chains hold 32-bit positions
       L->sparse = true;
       L->act_max = largest;
       L->act_off.assign(D + 1, 0);
@@ -1310,12 +1415,28 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
       SGP_CHECK(dalloc(&L->act, std::max<int64_t>(total, 1), st), "alloc direction lists");
       SGP_CHECK(dalloc(&L->epoch, m, st), "alloc epochs");
       L->bytes += (size_t)total * sizeof(int32_t) + (size_t)m * sizeof(int32_t);
-      SGP_CHECK(dalloc(&L->act_off_dev, D + 1, st), "alloc list offsets");
-      SGP_CHECK(cudaMemcpyAsync(L->act_off_dev, L->act_off.data(), (D + 1) * sizeof(int64_t),
+      SGP_CHECK(dalloc(&L->act_off_dev, 2 * (D + 1), st), "alloc list offsets");
+      std::vector<int64_t> offsets(L->act_off);  // then the chains' offsets
+      offsets.resize(2 * (D + 1), 0);
+      for (int j = 0; j < D; ++j) offsets[D + 2 + j] = offsets[D + 1 + j] + (int64_t)hc[2 * D + 1 + j];
+      SGP_CHECK(cudaMemcpyAsync(L->act_off_dev, offsets.data(), offsets.size() * sizeof(int64_t),
                                 cudaMemcpyHostToDevice, st),
                 "copy list offsets");
-      launch_pdl(k_active_fill, (unsigned)ceil_div(m, kFillThreads), kFillThreads, st, 
-          hasnb, m, D, L->act_off_dev, counts + D, L->act);
+      const unsigned grid = (unsigned)ceil_div(m, kFillThreads);
+      if (r == 1) {
+        L->chain_off.assign(offsets.begin() + D + 1, offsets.end());
+        const int64_t chains = L->chain_off.back();
+        SGP_CHECK(dalloc(&L->chain, std::max<int64_t>(chains, 1), st), "alloc chains");
+        L->bytes += (size_t)chains * sizeof(uint2);
+        int* longest = reinterpret_cast<int*>(counts + 4 * D + 1);
+        launch_pdl(k_chain_fill, grid, kFillThreads, st, lb, L->nbr, m, D, L->act_off_dev,
+                   L->act_off_dev + D + 1, counts + D, counts + 3 * D + 1, L->act, L->chain, longest);
+        SGP_CHECK(cudaMemcpyAsync(&L->chain_max, longest, sizeof(int), cudaMemcpyDeviceToHost, st),
+                  "read chains");
+      } else {
+        launch_pdl(k_active_fill, grid, kFillThreads, st, lb.above, m, D, L->act_off_dev, counts + D,
+                   L->act);
+      }
       note_launches(1);
       // powers of the symmetric blur's centre tap g_0 (stored rows are rescaled lazily)
       std::vector<float> pw(2 * D + 1);

@@ -19,6 +19,7 @@
 // consecutive columns of a row, the pipelined blur 8.  At n = 50k, d = 8, k = 9 a product
 // with 9 scalar columns took 100 us, with 12 padded ones 77.5 us (launches alike).
 #include <atomic>
+#include <cmath>
 #include <type_traits>
 
 #include <cuda_bf16.h>
@@ -283,12 +284,66 @@ int blur_pipe_blocks() {
 }
 
 // ---- sparse blur (lattices whose direction lists are short) ------------------------------
-// Stored rows carry a lazy factor: the value of vertex x before pass t is
-// g0^(t - epoch[x]) stored[x] (g0 = the pass's centre tap), since a vertex without a
-// neighbour along a pass's direction is only scaled by the centre tap.  Pass t (direction
-// j) computes the new rows of the vertices on list j into tmp; a second kernel stores them
-// and sets their epoch to t + 1.  After the last pass, k_sparse_finish applies the
-// remaining factors.
+// A vertex without a neighbour along a pass's direction is only scaled by the centre tap g0.
+// With the values kept as y = x / g0^t after t passes such vertices do not change, a pass is
+// y[v] += (g1 / g0) (y[v - u_j] + y[v + u_j]) on the others, and the factor g0^passes is
+// applied once at the end (by the caller, through its alpha).
+//
+// One thread-group of G threads per chain v, v + u_j, v + 2 u_j, ...: it reads every row of the
+// chain once and writes it back in place, which no other group reads (chains are maximal).
+// Chains have two vertices as a rule, so the first kChainRows rows are loaded together.
+// Bound by memory: per active vertex one row read and written and a 4-byte id, per chain 8
+// bytes.  n = 500k, d = 20, k = 8 (m = 10.5M, 1M active vertices a pass): 22 us a pass, 64.8
+// with per-vertex epochs, a buffer of new rows and a store kernel (k_sparse_blur, below).
+constexpr int kChainRows = 4;
+template <int VEC, class S>
+__global__ void __launch_bounds__(kThreads) k_chain_blur(int64_t chains, int G, int k, float tap,
+                                                         const uint2* __restrict__ chain,
+                                                         const int32_t* __restrict__ act,
+                                                         S* __restrict__ vals) {
+  pdl_enter();
+  using Vt = Vec<VEC>;
+  using T = typename Vt::T;
+  const int64_t q = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
+  if (q >= chains) return;
+  const int col = (int)(threadIdx.x % G) * VEC;
+  const uint2 ch = __ldg(chain + q);
+  T prev = Vt::zero();  // the row below the current one, before this pass
+  for (int64_t p0 = ch.x; p0 < (int64_t)ch.y; p0 += kChainRows) {
+    S* at[kChainRows + 1];
+    T row[kChainRows + 1];  // the last one only as a neighbour
+#pragma unroll
+    for (int e = 0; e <= kChainRows; ++e) {
+      at[e] = p0 + e < (int64_t)ch.y ? vals + (int64_t)__ldg(act + p0 + e) * k + col : nullptr;
+      row[e] = Vt::zero();
+    }
+#pragma unroll
+    for (int e = 0; e <= kChainRows; ++e)
+      if (at[e]) row[e] = Vt::lds(at[e]);
+#pragma unroll
+    for (int e = 0; e < kChainRows; ++e) {
+      if (at[e]) Vt::sts(at[e], Vt::fma(tap, Vt::add(prev, row[e + 1]), row[e]));
+      prev = row[e];
+    }
+  }
+}
+
+template <int VEC, class S>
+__global__ void __launch_bounds__(kThreads) k_rescale(int64_t m, int G, int k, float f,
+                                                      S* __restrict__ vals) {
+  pdl_enter();
+  using Vt = Vec<VEC>;
+  const int64_t v = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
+  if (v >= m) return;
+  S* p = vals + v * k + (int)(threadIdx.x % G) * VEC;
+  Vt::sts(p, Vt::scale(f, Vt::lds(p)));
+}
+
+// The general form (stencil orders above 1, chains longer than kMaxChain): stored rows carry
+// a lazy factor, the value of vertex x before pass t being g0^(t - epoch[x]) stored[x].  Pass
+// t (direction j) computes the new rows of the vertices on list j into tmp; a second kernel
+// stores them and sets their epoch to t + 1.  After the last pass, k_sparse_finish applies
+// the remaining factors.
 template <int VEC, class S>
 __global__ void __launch_bounds__(kThreads) k_sparse_blur(int64_t count, int G, int k, int r,
                                                           Taps tp, int t,
@@ -611,12 +666,16 @@ void launch_permute(const Lattice* L, const float* V, int k, int kp, float* Vp, 
   note_launches(1);
 }
 
+// Sparse blurs run on chains (else on the direction lists).
+bool chains_ok(const Lattice* L) { return L->chain_max > 0 && L->chain_max <= kMaxChain; }
+
 // The blur passes of `blur` on the splatted values in lat0 (lat1: ping-pong buffer);
-// returns the buffer that holds the result.  Sparse lattices use the direction lists
-// (lat1 unused) unless `dense` is set.
+// returns the buffer that holds the result divided by *scale.  Sparse lattices use their
+// chains or direction lists (lat1 unused) unless `dense` is set.
 template <class S>
 S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream_t st,
-                 int* passes_out, bool dense) {
+                 int* passes_out, bool dense, double* scale) {
+  *scale = 1.0;
   Taps c{}, g{};
   for (int t = 0; t <= L->r; ++t) {
     c.t[t] = (float)L->coef[t];
@@ -641,6 +700,36 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
       b = x;
     }
     return a;
+  }
+  if (chains_ok(L)) {
+    const double g0 = blur == SGP_BLUR_SYMMETRIC ? L->half[0] : L->coef[0];
+    const double g1 = blur == SGP_BLUR_SYMMETRIC ? L->half[1] : L->coef[1];
+    // y / x = g0^-t grows with the passes: bring it back every kRescale passes (never for D
+    // <= 64) so that it stays far from the end of the exponent range
+    constexpr int kRescale = 64;
+    int owed = 0;  // passes whose factor has not been applied
+    by_vec(row_shape(1, k).vec, [&](auto vec) {
+      constexpr int VEC = decltype(vec)::value;
+      for (int t = 0; t < P; ++t) {
+        const int j = dir(t);
+        const int64_t count = L->chain_off[j + 1] - L->chain_off[j];
+        if (g0 != 1.0 && P > 2 * kRescale && owed == kRescale) {
+          const RowShape q = row_shape(L->m, k);
+          launch_pdl(k_rescale<VEC, S>, q.blocks, q.threads, st, L->m, q.G, k,
+                     (float)std::pow(g0, kRescale), lat0);
+          note_launches(1);
+          owed = 0;
+        }
+        ++owed;
+        if (count == 0) continue;
+        const RowShape q = row_shape(count, k);
+        launch_pdl(k_chain_blur<VEC, S>, q.blocks, q.threads, st, count, q.G, k, (float)(g1 / g0),
+                   L->chain + L->chain_off[j], L->act, lat0);
+        note_launches(1);
+      }
+    });
+    *scale = std::pow(g0, owed);
+    return lat0;
   }
   // sparse: lazy centre-tap factors (none when the centre tap is 1)
   const float* pw = tp.t[0] == 1.f ? nullptr : L->g0pow;
@@ -689,7 +778,9 @@ int enqueue_t(const Lattice* L, const float* V, int k, int kp, int kt, int blur,
   // External: inside a stream capture this becomes an event-record node of the graph
   if (ev) cudaEventRecordWithFlags(ev[0], st, cudaEventRecordExternal);
   int passes = 0;
-  S* a = blur_passes_t<S>(L, blur, lat0, lat1, kp, st, &passes, dense);
+  double scale = 1.0;
+  S* a = blur_passes_t<S>(L, blur, lat0, lat1, kp, st, &passes, dense, &scale);
+  alpha = (float)(alpha * scale);
   if (ev) cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal);
   if (internal && dot_partial) launch_slice_dot<S>(L, a, V, kp, alpha, beta, out, dot_partial, st);
   else if (internal) launch_slice_t<false, S>(L, a, V, kp, kp, alpha, beta, out, st);
@@ -702,9 +793,9 @@ int enqueue_t(const Lattice* L, const float* V, int k, int kp, int kt, int blur,
 // result.
 template <class S>
 S* splat_blur_t(const Lattice* L, const float* Vp, int kp, int kt, int blur, S* lat0, S* lat1,
-                float* partial, cudaStream_t st) {
+                float* partial, cudaStream_t st, double* scale) {
   launch_splat_t<S>(L, Vp, kp, kt, lat0, partial, st);
-  return blur_passes_t<S>(L, blur, lat0, lat1, kp, st, nullptr, false);
+  return blur_passes_t<S>(L, blur, lat0, lat1, kp, st, nullptr, false, scale);
 }
 
 size_t value_size(const Lattice* L) {
@@ -721,7 +812,8 @@ size_t mvm_work_bytes(const Lattice* L, int k) {
 }
 
 sgp_status ensure_lattice_values(Lattice* L, int k, cudaStream_t st) {
-  if (L->sparse && L->act_tmp_elems < (size_t)L->act_max * k) {
+  if (L->sparse && (!chains_ok(L) || L->table_blur) &&
+      L->act_tmp_elems < (size_t)L->act_max * k) {
     if (L->act_tmp) cudaFreeAsync(L->act_tmp, st);
     L->act_tmp = nullptr;
     const size_t bytes = std::max<size_t>((size_t)L->act_max * k * value_size(L), 16);
@@ -815,10 +907,10 @@ void enqueue_mvm_into(const Lattice* L, const float* V_user, int k, int blur, fl
 }
 
 void* enqueue_splat_blur(const Lattice* L, const float* Vp, int kp, int kt, int blur, void* lat0,
-                         void* lat1, float* partial, cudaStream_t st) {
+                         void* lat1, float* partial, cudaStream_t st, double* scale) {
   if (L->value_dtype == SGP_VALUES_BF16)
-    return splat_blur_t<bf16>(L, Vp, kp, kt, blur, (bf16*)lat0, (bf16*)lat1, partial, st);
-  return splat_blur_t<float>(L, Vp, kp, kt, blur, (float*)lat0, (float*)lat1, partial, st);
+    return splat_blur_t<bf16>(L, Vp, kp, kt, blur, (bf16*)lat0, (bf16*)lat1, partial, st, scale);
+  return splat_blur_t<float>(L, Vp, kp, kt, blur, (float*)lat0, (float*)lat1, partial, st, scale);
 }
 
 void enqueue_permute(const Lattice* L, const float* V, int k, int kp, float* Vp, cudaStream_t st) {

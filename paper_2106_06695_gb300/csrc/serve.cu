@@ -1475,6 +1475,7 @@ sgp_status setup(sgp_server* S, Request* R, cudaStream_t st, Table& t1) {
   }
   Lattice* L = R->L;
   R->st.m = L->m;
+  L->table_blur = true;
   s = ensure_lattice_values(L, kp, st);
   if (s != SGP_OK) return s;
   R->l = R->ld = 0;

@@ -39,6 +39,9 @@ constexpr int kSplatMedSegs = 16;  // segments a single thread-group sums in the
 // A lattice blurs in sparse mode when the direction lists hold at most this fraction of
 // the D m (vertex, direction) pairs.
 constexpr double kSparseFrac = 0.3;
+// Chains longer than this are not walked by one thread group: the lattice is blurred through
+// the direction lists then.
+constexpr int kMaxChain = 64;
 
 // Stencil taps passed by value to the blur kernels.
 struct Taps {
@@ -96,6 +99,12 @@ struct sgp_lattice {
   std::vector<int64_t> act_off;  // [D + 1], host
   int64_t* act_off_dev = nullptr;  // [D + 1], device copy
   int64_t act_max = 0;           // largest list
+  // Stencil order 1: each list is ordered by chains (maximal runs v, v + u_j, v + 2 u_j, ...);
+  // chain[chain_off[j] .. chain_off[j+1]) holds (begin, end) of direction j's chains in act.
+  uint2* chain = nullptr;
+  std::vector<int64_t> chain_off;  // [D + 1], host
+  int chain_max = 0;             // longest chain; 0: no chains (order > 1)
+  bool table_blur = false;       // blurred by the server's table kernels too (needs act_tmp)
   int32_t* epoch = nullptr;      // [m] pass after which a vertex's stored row was written
   void* act_tmp = nullptr;       // [act_max][k] new values of one pass
   size_t act_tmp_elems = 0;
@@ -231,10 +240,11 @@ void enqueue_mvm_into(const Lattice* L, const float* V, int k, int blur, float a
                       float beta, float* out, void* work, cudaStream_t st);
 // Pieces of the operator for the backward: splat a locality-ordered Vp (rows of kp) and blur
 // it (the result ends in the returned buffer, lat0 or lat1, of the handle's value type; kt
-// as enqueue_mvm's tree_k); gather the caller's rows of k into locality-ordered rows of kp;
+// as enqueue_mvm's tree_k; the blurred values are *scale times what the buffer holds); gather
+// the caller's rows of k into locality-ordered rows of kp;
 // out (caller's order, rows of k) = alpha W lat.
 void* enqueue_splat_blur(const Lattice* L, const float* Vp, int kp, int kt, int blur, void* lat0,
-                         void* lat1, float* partial, cudaStream_t st);
+                         void* lat1, float* partial, cudaStream_t st, double* scale);
 void enqueue_permute(const Lattice* L, const float* V, int k, int kp, float* Vp, cudaStream_t st);
 void enqueue_slice_caller(const Lattice* L, const void* lat, int k, int kp, float alpha, float* out,
                           cudaStream_t st);
