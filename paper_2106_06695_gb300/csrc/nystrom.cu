@@ -51,6 +51,7 @@ __device__ __forceinline__ float to_f(float x) { return x; }
 template <bool OMEGA, class TX>
 __global__ void k_gram(const TX* __restrict__ X, int ld, const int32_t* __restrict__ perm,
                        int64_t n, int l, uint64_t seed, double* __restrict__ partial) {
+  pdl_enter();
   extern __shared__ float sh[];
   float* xs = sh;                               // [kRowsPerStage][l]
   float* ls = sh + kRowsPerStage * l;           // [kRowsPerStage][l] (OMEGA only)
@@ -93,6 +94,7 @@ __global__ void k_gram(const TX* __restrict__ X, int ld, const int32_t* __restri
 // out[e] = sum over blocks of partial[b][e], in block order.
 __global__ void k_sum_blocks(const double* __restrict__ partial, int nblk, int count,
                              double* __restrict__ out) {
+  pdl_enter();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= count) return;
   double t = 0.0;
@@ -105,6 +107,7 @@ __global__ void k_sum_blocks(const double* __restrict__ partial, int nblk, int c
 // triangle is zeroed.  *status = 1 when a pivot is not positive.
 __global__ void k_cholesky(double* __restrict__ A, int l, double shift, double rel_shift,
                            int* __restrict__ status) {
+  pdl_enter();
   __shared__ double piv, dmax;
   for (int e = threadIdx.x; e < l * l; e += blockDim.x) {
     const int i = e / l, j = e % l;
@@ -151,6 +154,7 @@ __global__ void k_cholesky(double* __restrict__ A, int l, double shift, double r
 // thread c solves R x = e_c by forward substitution.
 __global__ void k_tri_inv_t(const double* __restrict__ R, int l, double* __restrict__ work,
                             float* __restrict__ T) {
+  pdl_enter();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= l) return;
   double* x = work + (int64_t)c * l;
@@ -166,6 +170,7 @@ __global__ void k_tri_inv_t(const double* __restrict__ R, int l, double* __restr
 // column (thread c), then Minv = W^T W.  `work` holds W ([l][l]).
 __global__ void k_inv_from_cholesky(const double* __restrict__ Q, int l, double* __restrict__ W,
                                     double* __restrict__ Minv) {
+  pdl_enter();
   for (int c = threadIdx.x; c < l; c += blockDim.x) {
     for (int i = 0; i < l; ++i) {
       double s = (i == c) ? 1.0 : 0.0;
@@ -186,6 +191,7 @@ __global__ void k_inv_from_cholesky(const double* __restrict__ Q, int l, double*
 // on training rows (perm[p] < n_train) and columns c0 + c < l, else 0.
 __global__ void k_fill_sketch_chunk(const int32_t* __restrict__ perm, int64_t n, int64_t n_train,
                                     int l, int c0, int kp, uint64_t seed, float* __restrict__ V) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n * kp) return;
   const int64_t p = e / kp;
@@ -199,6 +205,7 @@ __global__ void k_fill_sketch_chunk(const int32_t* __restrict__ perm, int64_t n,
 __global__ void k_gather_chunk(const int32_t* __restrict__ perm, int64_t n, int64_t n_train,
                                int l, int ld, int c0, int kp, uint64_t seed, float nu,
                                const float* __restrict__ KV, float* __restrict__ Y) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n * kp) return;
   const int64_t p = e / kp;
@@ -215,6 +222,7 @@ __global__ void k_gather_chunk(const int32_t* __restrict__ perm, int64_t n, int6
 // stages its rows before it writes any of them, and no other block touches those rows.
 __global__ void k_rows_times_inplace(float* Y, const float* __restrict__ T, int64_t n, int l,
                                      int ld) {
+  pdl_enter();
   extern __shared__ float sh[];
   float* ts = sh;              // [l][l]
   float* ys = sh + l * l;      // [rows_per_block][l]
@@ -278,29 +286,29 @@ sgp_status nystrom_build_masked(Lattice* L, int64_t n_train, int l, int ld, uint
   const float nu = 1e-3f * noise;
   const unsigned g = (unsigned)ceil_div(n * kp, 256);
   for (int c0 = 0; c0 < ld; c0 += kp) {
-    k_fill_sketch_chunk<<<g, 256, 0, st>>>(L->perm, n, n_train, l, c0, kp, seed, V);
+    launch_pdl(k_fill_sketch_chunk, g, 256, st, L->perm, n, n_train, l, c0, kp, seed, V);
     enqueue_mvm(L, V, kp, SGP_BLUR_SYMMETRIC, L->outputscale, 0.f, KV, st, nullptr,
                 /*internal=*/true);
-    k_gather_chunk<<<g, 256, 0, st>>>(L->perm, n, n_train, l, ld, c0, kp, seed, nu, KV, Bh);
+    launch_pdl(k_gather_chunk, g, 256, st, L->perm, n, n_train, l, ld, c0, kp, seed, nu, KV, Bh);
     note_launches(2);
   }
   // C = Omega^T Y (masked rows of Y are zero), Cholesky C = R R^T, B = Y R^-T in place
   const size_t gram_smem = 2 * (size_t)kRowsPerStage * l * sizeof(float);
-  k_gram<true, float><<<tall, 256, gram_smem, st>>>(Bh, ld, L->perm, n, l, seed, partial);
-  k_sum_blocks<<<(unsigned)ceil_div(l * l, 256), 256, 0, st>>>(partial, tall, l * l, C);
+  launch_pdl_smem(k_gram<true, float>, tall, 256, gram_smem, st, Bh, ld, L->perm, n, l, seed, partial);
+  launch_pdl(k_sum_blocks, (unsigned)ceil_div(l * l, 256), 256, st, partial, tall, l * l, C);
   // BF16 lattice values perturb A Omega by ~2^-8 relative: a relative diagonal shift keeps
   // C positive definite (any shift leaves P = B B^T + noise I positive definite)
   const double rel = L->value_dtype == SGP_VALUES_BF16 ? 1e-2 : 0.0;
-  k_cholesky<<<1, 1024, 0, st>>>(C, l, 0.0, rel, status_dev);
-  k_tri_inv_t<<<1, 128, 0, st>>>(C, l, work, T);
+  launch_pdl(k_cholesky, 1, 1024, st, C, l, 0.0, rel, status_dev);
+  launch_pdl(k_tri_inv_t, 1, 128, st, C, l, work, T);
   const int rows = std::max(1, 1024 / l);
   const size_t rt_smem = ((size_t)l * l + (size_t)rows * l) * sizeof(float);
-  k_rows_times_inplace<<<tall, rows * l, rt_smem, st>>>(Bh, T, n, l, ld);
+  launch_pdl_smem(k_rows_times_inplace, tall, rows * l, rt_smem, st, Bh, T, n, l, ld);
   // M = noise I + B^T B from the stored B, Cholesky M = Q Q^T, Minv = M^-1
-  k_gram<false, float><<<tall, 256, gram_smem, st>>>(Bh, ld, L->perm, n, l, seed, partial);
-  k_sum_blocks<<<(unsigned)ceil_div(l * l, 256), 256, 0, st>>>(partial, tall, l * l, Q);
-  k_cholesky<<<1, 1024, 0, st>>>(Q, l, (double)noise, 0.0, status_dev);
-  k_inv_from_cholesky<<<1, 128, 0, st>>>(Q, l, work, Minv);
+  launch_pdl_smem(k_gram<false, float>, tall, 256, gram_smem, st, Bh, ld, L->perm, n, l, seed, partial);
+  launch_pdl(k_sum_blocks, (unsigned)ceil_div(l * l, 256), 256, st, partial, tall, l * l, Q);
+  launch_pdl(k_cholesky, 1, 1024, st, Q, l, (double)noise, 0.0, status_dev);
+  launch_pdl(k_inv_from_cholesky, 1, 128, st, Q, l, work, Minv);
   note_launches(9);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e, "building the masked Nystrom factor");

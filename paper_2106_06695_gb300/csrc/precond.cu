@@ -67,6 +67,7 @@ __device__ __forceinline__ float sketch_sign(uint64_t seed, int64_t i, int j, in
 // and below the diagonal, mirrored above it.
 __global__ void k_sum_splits(const float* __restrict__ partial, int splits, int ldp,
                              double* __restrict__ G) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t count = (int64_t)ldp * ldp;
   if (e >= count) return;
@@ -110,6 +111,7 @@ constexpr int kTcThreads = 160;               // warp 0: issue; warps 1-4: epilo
 // first 16 columns' split itself; this kernel serves the CG start and further chunks.)
 __global__ void k_split_r(const float* __restrict__ rh, const float* __restrict__ rl, int k,
                           int c_off, int kc, int64_t n, __nv_bfloat16* __restrict__ r3) {
+  pdl_enter();
   const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= n) return;
   uint32_t w[3][8];
@@ -141,6 +143,7 @@ __global__ void k_split_r(const float* __restrict__ rh, const float* __restrict_
 // The loads of eight splits are issued together (they are independent) before their sums.
 __global__ void k_sum_t(const float* __restrict__ tpart, int splits, int ld,
                         float* __restrict__ t) {
+  pdl_enter();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= ld * 16) return;
   const size_t stride = (size_t)ld * 16;
@@ -162,6 +165,7 @@ __global__ void k_sum_t(const float* __restrict__ tpart, int splits, int ld,
 __global__ void __launch_bounds__(256) k_minv_u(const float* __restrict__ Minv, int ld,
                                                 const float* __restrict__ t,
                                                 __nv_bfloat16* __restrict__ u3) {
+  pdl_enter();
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= ld) return;
   const float* row = Minv + (size_t)i * ld;
@@ -286,6 +290,7 @@ using BtRing = TcRing<kTcStages, kBtStage>;       // B^T r
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_bt_tc(const __grid_constant__ CUtensorMap mapBt, const __grid_constant__ CUtensorMap mapR,
             int64_t n, int64_t rows_per_split, float* __restrict__ tpart, int* __restrict__ err) {
+  pdl_enter();
   extern __shared__ uint8_t tc_raw[];
   const BtRing R = tc_ring<BtRing>(tc_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -402,6 +407,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
            const float* __restrict__ rh, int k, int c_off, int kc, int64_t n, int ld,
            float inv_tau, float* __restrict__ z, double* __restrict__ dot,
            int* __restrict__ err) {
+  pdl_enter();
   extern __shared__ uint8_t tc_raw[];
   __shared__ double red[2][4][16];
   const ApplyRing R = tc_ring<ApplyRing>(tc_raw);
@@ -580,6 +586,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // Eight columns per thread (16-byte stores).
 __global__ void k_fill_sketch3(const int32_t* __restrict__ perm, int64_t n, int l, int ld,
                                uint64_t seed, __nv_bfloat16* __restrict__ P3) {
+  pdl_enter();
   const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
   const int64_t plane = n * ld;
   if (e >= plane) return;
@@ -603,6 +610,7 @@ __global__ void k_fill_sketch3(const int32_t* __restrict__ perm, int64_t n, int 
 // columns per thread (16-byte plane accesses, two float4 of dense).
 __global__ void k_cols3(__nv_bfloat16* __restrict__ P3, int ld, int c0, float* __restrict__ dense,
                         int kc, int64_t n, bool to_panel) {
+  pdl_enter();
   const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
   if (e >= n * kc) return;
   const int64_t p = e / kc;
@@ -650,6 +658,7 @@ __global__ void k_cols3(__nv_bfloat16* __restrict__ P3, int ld, int c0, float* _
 // zero elsewhere in [ld][ld].
 __global__ void k_split3_pad(const double* __restrict__ A, int lda, int l, int ld,
                              __nv_bfloat16* __restrict__ T3) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t plane = (int64_t)ld * ld;
   if (e >= plane) return;
@@ -684,6 +693,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     k_gram5(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY,
             int64_t n, int64_t rows_per_split, int ldp, float* __restrict__ partial,
             int* __restrict__ err) {
+  pdl_enter();
   using Cfg = GramCfg<P>;
   using Ring = typename Cfg::Ring;
   extern __shared__ uint8_t tc_raw[];
@@ -806,6 +816,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     k_panel5(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapT,
              int64_t n, int ld, int kdim, bool lower, bool rows_in_y,
              __nv_bfloat16* __restrict__ Z, int* __restrict__ err) {
+  pdl_enter();
   using Ring = PanelCfg::Ring;
   extern __shared__ uint8_t tc_raw[];
   const Ring R = tc_ring<Ring>(tc_raw);
@@ -934,6 +945,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 __global__ void __launch_bounds__(256) k_prepare_spd(const double* __restrict__ src,
                                                      double* __restrict__ dst, int l, int lda,
                                                      double shift, double rel) {
+  pdl_enter();
   __shared__ double red[256];
   double m = 0.0;
   for (int j = threadIdx.x; j < l; j += blockDim.x) m = fmax(m, src[(size_t)j * lda + j]);
@@ -961,6 +973,7 @@ __global__ void __launch_bounds__(256) k_prepare_spd(const double* __restrict__ 
 // c, rows c + t, c + t + 8, ...).
 __global__ void __launch_bounds__(256) k_potrf_diag(double* __restrict__ A, int lda, int kb,
                                                     int nb, int* __restrict__ status) {
+  pdl_enter();
   __shared__ double a[kNB][kNB + 1];
   __shared__ double rinv;
   const int tx = (int)threadIdx.x % kNB, ty = (int)threadIdx.x / kNB;
@@ -1000,6 +1013,7 @@ __global__ void __launch_bounds__(256) k_potrf_diag(double* __restrict__ A, int 
 // orders them); it then updates the columns after it, which are independent of each other.
 __global__ void __launch_bounds__(32) k_trsm_panel(double* __restrict__ A, int lda, int l,
                                                    int kb, int nb) {
+  pdl_enter();
   __shared__ double Lk[kNB][kNB + 1];
   __shared__ double rd[kNB];
   for (int e = threadIdx.x; e < kNB * kNB; e += blockDim.x) {
@@ -1032,6 +1046,7 @@ __global__ void __launch_bounds__(32) k_trsm_panel(double* __restrict__ A, int l
 // s <= j <= i < l, s = kb + nb; one 32 x 32 tile (I >= J) per block, 4 outputs per thread.
 __global__ void __launch_bounds__(256) k_syrk_trailing(double* __restrict__ A, int lda, int l,
                                                         int kb, int nb) {
+  pdl_enter();
   __shared__ double pi[kNB][kNB + 1], pj[kNB][kNB + 1];
   const int s = kb + nb;
   const int b = blockIdx.x;
@@ -1062,6 +1077,7 @@ __global__ void __launch_bounds__(256) k_syrk_trailing(double* __restrict__ A, i
 // column in shared memory); the strict upper part of the block is zero.
 __global__ void k_trtri_diag(const double* __restrict__ L, double* __restrict__ X, int lda,
                              int l) {
+  pdl_enter();
   __shared__ double a[kNB][kNB + 1], x[kNB][kNB + 1];
   const int b0 = blockIdx.x * kNB;
   const int nb = min(kNB, l - b0);
@@ -1106,6 +1122,7 @@ __global__ void __launch_bounds__(256) k_trtri_level(const double* __restrict__ 
                                                       double* __restrict__ X,
                                                       double* __restrict__ S, int lda, int l,
                                                       int b) {
+  pdl_enter();
   __shared__ double at[kNB][kNB + 1], bt[kNB][kNB + 1];
   const int tb = b / kNB;
   const int pair = (int)(blockIdx.x / (unsigned)(tb * tb));
@@ -1154,6 +1171,7 @@ __global__ void __launch_bounds__(256) k_trtri_level(const double* __restrict__ 
 // lower triangle per block (mirrored).  Rows of X below the tiles' columns only.
 __global__ void __launch_bounds__(256) k_xtx(const double* __restrict__ X, int lda, int l,
                                              double* __restrict__ M) {
+  pdl_enter();
   __shared__ double xa[kNB][kNB + 1], xb[kNB][kNB + 1];
   const int b = blockIdx.x;
   int A = (int)((sqrt(8.0 * b + 1.0) - 1.0) * 0.5);
@@ -1195,6 +1213,7 @@ __global__ void __launch_bounds__(256) k_xtx(const double* __restrict__ X, int l
 // y = M v (M symmetric l x l, fp64): one warp per row.
 __global__ void k_symv(const double* __restrict__ M, int lda, int l, const double* __restrict__ v,
                        double* __restrict__ y) {
+  pdl_enter();
   const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= l) return;
@@ -1208,6 +1227,7 @@ __global__ void k_symv(const double* __restrict__ M, int lda, int l, const doubl
 // One block of 1024 threads; v0 != 0 on entry.
 __global__ void k_power_step(double* __restrict__ v, const double* __restrict__ y, int l,
                              double* __restrict__ rq) {
+  pdl_enter();
   __shared__ double s1[1024], s2[1024];
   double a = 0.0, b = 0.0;
   for (int j = threadIdx.x; j < l; j += blockDim.x) {
@@ -1230,6 +1250,7 @@ __global__ void k_power_step(double* __restrict__ v, const double* __restrict__ 
 }
 
 __global__ void k_init_unit(double* __restrict__ v, int l) {
+  pdl_enter();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < l) v[j] = 1.0 / sqrt((double)l) * (1.0 + 0.25 * sin(0.7 * j));
 }
@@ -1237,6 +1258,7 @@ __global__ void k_init_unit(double* __restrict__ v, int l) {
 // out[i][j] = (float)A[i][j] for i, j < l, 0 elsewhere in [ld][ld].
 __global__ void k_to_f32_pad(const double* __restrict__ A, int lda, int l, int ld,
                              float* __restrict__ out) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)ld * ld) return;
   const int i = (int)(e / ld), j = (int)(e % ld);
@@ -1246,6 +1268,7 @@ __global__ void k_to_f32_pad(const double* __restrict__ A, int lda, int l, int l
 // A[i][j] = src[i][j] + d (i == j) on the l x l block.
 __global__ void k_copy_shift(const double* __restrict__ src, double* __restrict__ A, int lda,
                              int l, double d) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)l * l) return;
   const int i = (int)(e / l), j = (int)(e % l);
@@ -1295,13 +1318,13 @@ struct Dense {
     if (err != cudaSuccess) return false;
     for (int kb = 0; kb < l; kb += kNB) {
       const int nb = std::min(kNB, l - kb);
-      k_potrf_diag<<<1, 256, 0, st>>>(A, lda, kb, nb, status);
+      launch_pdl(k_potrf_diag, 1, 256, st, A, lda, kb, nb, status);
       note_launches(1);
       const int rest = l - kb - nb;
       if (rest > 0) {
-        k_trsm_panel<<<(unsigned)ceil_div(rest, 32), 32, 0, st>>>(A, lda, l, kb, nb);
+        launch_pdl(k_trsm_panel, (unsigned)ceil_div(rest, 32), 32, st, A, lda, l, kb, nb);
         const int64_t T = ceil_div(rest, kNB);
-        k_syrk_trailing<<<(unsigned)(T * (T + 1) / 2), 256, 0, st>>>(A, lda, l, kb, nb);
+        launch_pdl(k_syrk_trailing, (unsigned)(T * (T + 1) / 2), 256, st, A, lda, l, kb, nb);
         note_launches(2);
       }
     }
@@ -1317,20 +1340,20 @@ struct Dense {
     cudaError_t e = cudaMemsetAsync(X, 0, (size_t)lda * lda * sizeof(double), st);
     if (e != cudaSuccess) return e;
     const int nblk = (l + kNB - 1) / kNB;
-    k_trtri_diag<<<nblk, kNB, 0, st>>>(L, X, lda, l);
+    launch_pdl(k_trtri_diag, nblk, kNB, st, L, X, lda, l);
     note_launches(1);
     for (int b = kNB; b < l; b *= 2) {
       const int tb = b / kNB;
       const unsigned grid = (unsigned)(ceil_div(l - b, 2 * b) * tb * tb);
-      k_trtri_level<0><<<grid, 256, 0, st>>>(L, X, S, lda, l, b);
-      k_trtri_level<1><<<grid, 256, 0, st>>>(L, X, S, lda, l, b);
+      launch_pdl(k_trtri_level<0>, grid, 256, st, L, X, S, lda, l, b);
+      launch_pdl(k_trtri_level<1>, grid, 256, st, L, X, S, lda, l, b);
       note_launches(2);
     }
     return cudaGetLastError();
   }
   cudaError_t xtx(const double* X, double* M) {
     const int64_t nblk = (l + kNB - 1) / kNB;
-    k_xtx<<<(unsigned)(nblk * (nblk + 1) / 2), 256, 0, st>>>(X, lda, l, M);
+    launch_pdl(k_xtx, (unsigned)(nblk * (nblk + 1) / 2), 256, st, X, lda, l, M);
     note_launches(1);
     return cudaGetLastError();
   }
@@ -1501,13 +1524,13 @@ sgp_status ShiftedNystrom::build(Lattice* L, int rank, uint64_t seed, float nois
   // only fixes the subspace)
   auto product = [&](__nv_bfloat16* src, __nv_bfloat16* dst, bool bf16_values) -> sgp_status {
     for (int c0 = 0; c0 < ld; c0 += kSketchCols) {
-      k_cols3<<<g_chunk, 256, 0, st>>>(src, ld, c0, Vc, kSketchCols, n, false);
+      launch_pdl(k_cols3, g_chunk, 256, st, src, ld, c0, Vc, kSketchCols, n, false);
       if (bf16_values)
         enqueue_mvm_bf16_values(L, Vc, kSketchCols, blur, L->outputscale, KVc, st);
       else
         enqueue_mvm(L, Vc, kSketchCols, blur, L->outputscale, 0.f, KVc, st, nullptr,
                     /*internal=*/true);
-      k_cols3<<<g_chunk, 256, 0, st>>>(dst, ld, c0, KVc, kSketchCols, n, true);
+      launch_pdl(k_cols3, g_chunk, 256, st, dst, ld, c0, KVc, kSketchCols, n, true);
       note_launches(2);
     }
     cudaError_t e = cudaGetLastError();
@@ -1519,12 +1542,12 @@ sgp_status ShiftedNystrom::build(Lattice* L, int rank, uint64_t seed, float nois
     PC_MAP(tc05::make_map_planes(&mx, X, planes, n, ld, ld, planes, 32));
     PC_MAP(tc05::make_map_planes(&my, Y, planes, n, ld, ld, planes, 32));
     if (planes == 3)
-      k_gram5<3><<<dim3(tiles, splits), kTcThreads, GramCfg<3>::Ring::kSmem, st>>>(
+      launch_pdl_smem(k_gram5<3>, dim3(tiles, splits), kTcThreads, GramCfg<3>::Ring::kSmem, st, 
           mx, my, n, rows_per_split, ld, gpart, err);
     else
-      k_gram5<1><<<dim3(tiles, splits), kTcThreads, GramCfg<1>::Ring::kSmem, st>>>(
+      launch_pdl_smem(k_gram5<1>, dim3(tiles, splits), kTcThreads, GramCfg<1>::Ring::kSmem, st, 
           mx, my, n, rows_per_split, ld, gpart, err);
-    k_sum_splits<<<(unsigned)ceil_div((int64_t)ll, 256), 256, 0, st>>>(gpart, splits, ld, out);
+    launch_pdl(k_sum_splits, (unsigned)ceil_div((int64_t)ll, 256), 256, st, gpart, splits, ld, out);
     note_launches(2);
     return SGP_OK;
   };
@@ -1532,7 +1555,7 @@ sgp_status ShiftedNystrom::build(Lattice* L, int rank, uint64_t seed, float nois
   // Z 3-plane, or rounded to bf16 when `round`
   auto panel_times = [&](const __nv_bfloat16* Y, const double* X, void* Z, bool round)
       -> sgp_status {
-    k_split3_pad<<<(unsigned)ceil_div((int64_t)ll, 256), 256, 0, st>>>(X, ld, l, ld, T3);
+    launch_pdl(k_split3_pad, (unsigned)ceil_div((int64_t)ll, 256), 256, st, X, ld, l, ld, T3);
     CUtensorMap my, mt;
     PC_MAP(tc05::make_map_planes(&my, Y, 3, n, ld, ld, 3, 128));
     PC_MAP(tc05::make_map_planes(&mt, T3, 3, ld, ld, ld, 3, 128));
@@ -1543,10 +1566,10 @@ sgp_status ShiftedNystrom::build(Lattice* L, int rank, uint64_t seed, float nois
                                          : dim3((unsigned)row_tiles, ntile);
     const bool rows_in_y = row_tiles <= 65535;
     if (round)
-      k_panel5<true><<<grid, kTcThreads, PanelCfg::Ring::kSmem, st>>>(
+      launch_pdl_smem(k_panel5<true>, grid, kTcThreads, PanelCfg::Ring::kSmem, st, 
           my, mt, n, ld, ld, /*lower=*/true, rows_in_y, static_cast<__nv_bfloat16*>(Z), err);
     else
-      k_panel5<false><<<grid, kTcThreads, PanelCfg::Ring::kSmem, st>>>(
+      launch_pdl_smem(k_panel5<false>, grid, kTcThreads, PanelCfg::Ring::kSmem, st, 
           my, mt, n, ld, ld, /*lower=*/true, rows_in_y, static_cast<__nv_bfloat16*>(Z), err);
     note_launches(2);
     return SGP_OK;
@@ -1560,7 +1583,7 @@ sgp_status ShiftedNystrom::build(Lattice* L, int rank, uint64_t seed, float nois
     raised = false;
     for (int attempt = 0; attempt < 4 && !good; ++attempt, rel *= 100.0) {
       raised = attempt > 0;
-      k_prepare_spd<<<(unsigned)ceil_div((int64_t)ll, 256), 256, 0, st>>>(src, dst, l, ld, 0.0,
+      launch_pdl(k_prepare_spd, (unsigned)ceil_div((int64_t)ll, 256), 256, st, src, dst, l, ld, 0.0,
                                                                           rel);
       note_launches(1);
       cudaError_t err_ = cudaSuccess;
@@ -1573,7 +1596,7 @@ sgp_status ShiftedNystrom::build(Lattice* L, int rank, uint64_t seed, float nois
   // approximation depends only on that range, so one pass suffices while the Gram's first
   // Cholesky succeeds; a second pass restores the orthogonality when its shift had to be
   // raised.
-  k_fill_sketch3<<<g_plane, 256, 0, st>>>(L->perm, n, l, ld, seed, P1);
+  launch_pdl(k_fill_sketch3, g_plane, 256, st, L->perm, n, l, ld, seed, P1);
   note_launches(1);
   __nv_bfloat16* Q = P1;
   __nv_bfloat16* Y = P2;
@@ -1617,12 +1640,12 @@ sgp_status ShiftedNystrom::build(Lattice* L, int rank, uint64_t seed, float nois
     if (!good) return SGP_OK;
     PC_CHECK(dn.trtri(G, Xi), "triangular inverse");
     PC_CHECK(dn.xtx(Xi, M), "inverse");
-    k_init_unit<<<(unsigned)ceil_div(l, 256), 256, 0, st>>>(pv, l);
+    launch_pdl(k_init_unit, (unsigned)ceil_div(l, 256), 256, st, pv, l);
     note_launches(1);
     constexpr int kPowerSteps = 30;
     for (int it = 0; it < kPowerSteps; ++it) {
-      k_symv<<<(unsigned)ceil_div(l, 8), 256, 0, st>>>(M, ld, l, pv, py);
-      k_power_step<<<1, 1024, 0, st>>>(pv, py, l, prq);
+      launch_pdl(k_symv, (unsigned)ceil_div(l, 8), 256, st, M, ld, l, pv, py);
+      launch_pdl(k_power_step, 1, 1024, st, pv, py, l, prq);
       note_launches(2);
     }
     double rq = 0.0;
@@ -1633,7 +1656,7 @@ sgp_status ShiftedNystrom::build(Lattice* L, int rank, uint64_t seed, float nois
   tau = (float)(lam_min + (double)noise);
   // 4. Minv = (tau I + G)^-1 (fp64 Cholesky, inverse factor, product), stored fp32
   {
-    k_copy_shift<<<(unsigned)ceil_div((int64_t)l * l, 256), 256, 0, st>>>(G0, M, ld, l,
+    launch_pdl(k_copy_shift, (unsigned)ceil_div((int64_t)l * l, 256), 256, st, G0, M, ld, l,
                                                                           (double)tau);
     note_launches(1);
     bool good = false;
@@ -1641,7 +1664,7 @@ sgp_status ShiftedNystrom::build(Lattice* L, int rank, uint64_t seed, float nois
     if (!good) return SGP_OK;
     PC_CHECK(dn.trtri(G, Xi), "triangular inverse");
     PC_CHECK(dn.xtx(Xi, M), "inverse");
-    k_to_f32_pad<<<(unsigned)ceil_div((int64_t)ll, 256), 256, 0, st>>>(M, ld, l, ld, Minv);
+    launch_pdl(k_to_f32_pad, (unsigned)ceil_div((int64_t)ll, 256), 256, st, M, ld, l, ld, Minv);
     note_launches(1);
   }
   PC_CHECK(cudaGetLastError(), "building the preconditioner");
@@ -1665,18 +1688,18 @@ void ShiftedNystrom::apply(const float* rh, const float* rl, int k, float* z, do
     const bool mark = ev && c_off == 0;
     if (mark) cudaEventRecordWithFlags(ev[0], st, cudaEventRecordExternal);
     if (!(split_ready && c_off == 0)) {
-      k_split_r<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(rh, rl, k, c_off, kc, n,
+      launch_pdl(k_split_r, (unsigned)ceil_div(n, 256), 256, st, rh, rl, k, c_off, kc, n,
                                                            static_cast<__nv_bfloat16*>(r3));
       note_launches(1);
     }
-    k_bt_tc<<<dim3(ntile, bt_splits), kTcThreads, BtRing::kSmem, st>>>(map_b_mn, map_r, n, bt_rows,
+    launch_pdl_smem(k_bt_tc, dim3(ntile, bt_splits), kTcThreads, BtRing::kSmem, st, map_b_mn, map_r, n, bt_rows,
                                                                   tpart, err);
     if (mark) cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal);
-    k_sum_t<<<(unsigned)ceil_div(ld * 16, 256), 256, 0, st>>>(tpart, bt_splits, ld, tvec);
-    k_minv_u<<<(unsigned)ceil_div(ld, 8), 256, 0, st>>>(Minv, ld, tvec,
+    launch_pdl(k_sum_t, (unsigned)ceil_div(ld * 16, 256), 256, st, tpart, bt_splits, ld, tvec);
+    launch_pdl(k_minv_u, (unsigned)ceil_div(ld, 8), 256, st, Minv, ld, tvec,
                                                          static_cast<__nv_bfloat16*>(u));
     if (mark) cudaEventRecordWithFlags(ev[2], st, cudaEventRecordExternal);
-    k_z_tc<<<z_blocks, kTcThreads, ApplyRing::kSmem, st>>>(map_b_k, map_u, rh, k, c_off, kc, n, ld,
+    launch_pdl_smem(k_z_tc, z_blocks, kTcThreads, ApplyRing::kSmem, st, map_b_k, map_u, rh, k, c_off, kc, n, ld,
                                                   1.f / tau, z, dot, err);
     if (mark) cudaEventRecordWithFlags(ev[3], st, cudaEventRecordExternal);
     note_launches(4);

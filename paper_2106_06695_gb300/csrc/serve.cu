@@ -203,6 +203,7 @@ __device__ __forceinline__ void f4_st(float* p, float4 v) { *reinterpret_cast<fl
 // Splat W^T p into lat0: one thread-group per segment of a vertex's incidence list.
 template <class S>
 __global__ void __launch_bounds__(kST) kb_splat(const Table* __restrict__ T) {
+  pdl_enter();
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
   SLOT_LOOP(U_SPLAT)
@@ -227,6 +228,7 @@ __global__ void __launch_bounds__(kST) kb_splat(const Table* __restrict__ T) {
 // Vertices with 2..kSplatMedSegs segments: one thread-group sums the partials in order.
 template <class S>
 __global__ void __launch_bounds__(kST) kb_splat_med(const Table* __restrict__ T) {
+  pdl_enter();
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
   SLOT_LOOP(U_MED)
@@ -248,6 +250,7 @@ __global__ void __launch_bounds__(kST) kb_splat_med(const Table* __restrict__ T)
 // and a fixed shared-memory tree over the groups.
 template <class S>
 __global__ void __launch_bounds__(kST) kb_splat_huge(const Table* __restrict__ T) {
+  pdl_enter();
   __shared__ float4 red[kST];
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
@@ -282,6 +285,7 @@ __global__ void __launch_bounds__(kST) kb_splat_huge(const Table* __restrict__ T
 // in lat0.  Each thread owns 4 columns of kBlurU rows (ids first, then rows).
 template <int R, class S>
 __global__ void __launch_bounds__(kST) kb_blur(const Table* __restrict__ T, int t) {
+  pdl_enter();
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
   SLOT_LOOP(U_BLUR)
@@ -369,6 +373,7 @@ __global__ void __launch_bounds__(kST) kb_blur(const Table* __restrict__ T, int 
 // Sparse requests, after kb_blur pass t: list rows back into lat0, epoch t + 1.
 template <class S>
 __global__ void __launch_bounds__(kST) kb_sparse_store(const Table* __restrict__ T, int t) {
+  pdl_enter();
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
   SLOT_LOOP(U_BLUR)
@@ -389,6 +394,7 @@ __global__ void __launch_bounds__(kST) kb_sparse_store(const Table* __restrict__
 // Sparse requests, after their 2D passes: the remaining centre-tap factors.
 template <class S>
 __global__ void __launch_bounds__(kST) kb_sparse_finish(const Table* __restrict__ T) {
+  pdl_enter();
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
   SLOT_LOOP(U_VERT)
@@ -410,6 +416,7 @@ __global__ void __launch_bounds__(kST) kb_sparse_finish(const Table* __restrict_
 // A p = outputscale W lat0 + noise p on training rows, 0 on test rows; partials of <p, Ap>.
 template <class S>
 __global__ void __launch_bounds__(kST) kb_slice_dot(const Table* __restrict__ T) {
+  pdl_enter();
   __shared__ double sh[kST * 4];
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
@@ -446,6 +453,7 @@ __global__ void __launch_bounds__(kST) kb_slice_dot(const Table* __restrict__ T)
 
 // alpha = rho / <p, A p> per active column (a non-positive <p, A p> stops the column).
 __global__ void __launch_bounds__(kST) kb_alpha(const Table* __restrict__ T) {
+  pdl_enter();
   __shared__ double red[kST], tot[kMaxServeK];
   const int q = blockIdx.x;
   if (q >= T->nslots) return;
@@ -495,6 +503,7 @@ __device__ __forceinline__ void xr_row(const SlotDev& s, int64_t e, const bool (
 }
 
 __global__ void __launch_bounds__(kST) kb_update_xr(const Table* __restrict__ T) {
+  pdl_enter();
   __shared__ double sh[kST * 4];
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
@@ -523,6 +532,7 @@ __global__ void __launch_bounds__(kST) kb_update_xr(const Table* __restrict__ T)
 // Convergence check and beta = <r, r>_new / <r, r>_old per active column; the request
 // stops when no column is active.  Its state is copied to the host-read flags.
 __global__ void __launch_bounds__(kST) kb_check_beta(const Table* __restrict__ T) {
+  pdl_enter();
   __shared__ double red[kST], trr[kMaxServeK], trz[kMaxServeK];
   const int q = blockIdx.x;
   if (q >= T->nslots) return;
@@ -567,6 +577,7 @@ __global__ void __launch_bounds__(kST) kb_check_beta(const Table* __restrict__ T
 // p = r + beta p on active columns (double-float sum rounded to fp32); p = z + beta p for
 // preconditioned requests (z in ap).
 __global__ void __launch_bounds__(kST) kb_update_p(const Table* __restrict__ T) {
+  pdl_enter();
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
   SLOT_LOOP(U_VEC)
@@ -714,6 +725,7 @@ __device__ __forceinline__ void ring_init(ChunkRing& ring, float* base, uint64_t
 // pass per KC columns (B streamed again).
 template <int KC>
 __global__ void __launch_bounds__(kST, 1) kb_bt(const Table* __restrict__ T) {
+  pdl_enter();
   extern __shared__ __align__(128) float dsm[];
   __shared__ __align__(8) uint64_t bar[kStages];
   __shared__ __align__(16) float red[KC * kMaxLd];  // [c][j]
@@ -800,6 +812,7 @@ __global__ void __launch_bounds__(kST, 1) kb_bt(const Table* __restrict__ T) {
 // First-level sums of the B^T r partials: virtual block (segment g, chunk h) adds the
 // partials g kBtSeg .. g kBtSeg + kBtSeg - 1 of outputs h kST .. h kST + kST - 1 in order.
 __global__ void __launch_bounds__(kST) kb_bt_seg(const Table* __restrict__ T) {
+  pdl_enter();
   const int kp = T->kp;
   SLOT_LOOP(U_BTS)
   if (*s.state == 0 || s.l == 0) continue;
@@ -818,6 +831,7 @@ __global__ void __launch_bounds__(kST) kb_bt_seg(const Table* __restrict__ T) {
 
 // t = B^T r: the segment sums added in order in fp64, one output per thread.
 __global__ void __launch_bounds__(kST) kb_bt_total(const Table* __restrict__ T) {
+  pdl_enter();
   const int kp = T->kp;
   SLOT_LOOP(U_BTT)
   if (*s.state == 0 || s.l == 0) continue;
@@ -834,6 +848,7 @@ __global__ void __launch_bounds__(kST) kb_bt_total(const Table* __restrict__ T) 
 // u = Minv t (fp64) on the first l rows, 0 below; stored fp32 [ld][kp].  Four lanes per
 // output, each a quarter of the dot product, combined by shuffles in a fixed order.
 __global__ void __launch_bounds__(kST) kb_minv(const Table* __restrict__ T) {
+  pdl_enter();
   const int kp = T->kp;
   SLOT_LOOP(U_MINV)
   if (*s.state == 0 || s.l == 0) continue;  // uniform over the block
@@ -882,6 +897,7 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
 // zero B rows and zero r, so z = 0 there.
 template <int NT>
 __global__ void __launch_bounds__(kST, 1) kb_apply_z(const Table* __restrict__ T) {
+  pdl_enter();
   extern __shared__ __align__(128) float dsm[];
   __shared__ __align__(8) uint64_t bar[kStages];
   __shared__ double red[kST / 32][8 * NT];
@@ -1002,10 +1018,10 @@ size_t apply_z_smem_bytes(int kp) { return ring_smem_bytes(kp) + 2 * (size_t)kMa
 void launch_apply_z(int kp, const Table* T, cudaStream_t st) {
   const size_t sm = apply_z_smem_bytes(kp);
   switch ((kp + 7) / 8) {
-    case 1: kb_apply_z<1><<<kRingGrid, kST, sm, st>>>(T); break;
-    case 2: kb_apply_z<2><<<kRingGrid, kST, sm, st>>>(T); break;
-    case 3: kb_apply_z<3><<<kRingGrid, kST, sm, st>>>(T); break;
-    default: kb_apply_z<4><<<kRingGrid, kST, sm, st>>>(T); break;
+    case 1: launch_pdl_smem(kb_apply_z<1>, kRingGrid, kST, sm, st, T); break;
+    case 2: launch_pdl_smem(kb_apply_z<2>, kRingGrid, kST, sm, st, T); break;
+    case 3: launch_pdl_smem(kb_apply_z<3>, kRingGrid, kST, sm, st, T); break;
+    default: launch_pdl_smem(kb_apply_z<4>, kRingGrid, kST, sm, st, T); break;
   }
 }
 cudaError_t apply_z_smem_attributes(int kp) {
@@ -1025,10 +1041,10 @@ cudaError_t apply_z_smem_attributes(int kp) {
 void launch_bt(int kp, const Table* T, cudaStream_t st) {
   const size_t sm = ring_smem_bytes(kp);
   switch (kp < 16 ? kp : 16) {
-    case 4: kb_bt<4><<<kRingGrid, kST, sm, st>>>(T); break;
-    case 8: kb_bt<8><<<kRingGrid, kST, sm, st>>>(T); break;
-    case 12: kb_bt<12><<<kRingGrid, kST, sm, st>>>(T); break;
-    default: kb_bt<16><<<kRingGrid, kST, sm, st>>>(T); break;
+    case 4: launch_pdl_smem(kb_bt<4>, kRingGrid, kST, sm, st, T); break;
+    case 8: launch_pdl_smem(kb_bt<8>, kRingGrid, kST, sm, st, T); break;
+    case 12: launch_pdl_smem(kb_bt<12>, kRingGrid, kST, sm, st, T); break;
+    default: launch_pdl_smem(kb_bt<16>, kRingGrid, kST, sm, st, T); break;
   }
 }
 cudaError_t bt_smem_attributes(int kp) {
@@ -1046,6 +1062,7 @@ cudaError_t bt_smem_attributes(int kp) {
 // ---- per-request set-up and read-out (single-request launches) ------------------------
 // Partials of <r, r> for the initial residual (the same virtual blocks as the iteration).
 __global__ void __launch_bounds__(kST) kb_norm(const Table* __restrict__ T) {
+  pdl_enter();
   __shared__ double sh[kST * 4];
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
@@ -1067,6 +1084,7 @@ __global__ void __launch_bounds__(kST) kb_norm(const Table* __restrict__ T) {
 }
 
 __global__ void __launch_bounds__(kST) kb_init_scalars(const Table* __restrict__ T) {
+  pdl_enter();
   __shared__ double red[kST], trr[kMaxServeK], trz[kMaxServeK];
   const int q = blockIdx.x;
   if (q >= T->nslots) return;
@@ -1099,6 +1117,7 @@ __global__ void __launch_bounds__(kST) kb_init_scalars(const Table* __restrict__
 // the last column (kp - 1 > S) holds 1 on the training rows, for the row sums of K~_XX.
 __global__ void k_probe_fill(float* __restrict__ V, int64_t n_all, int64_t n_train, int kp,
                              int S, uint64_t seed) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_all * kp) return;
   const int64_t i = e / kp;
@@ -1116,6 +1135,7 @@ __global__ void k_probe_fill(float* __restrict__ V, int64_t n_all, int64_t n_tra
 // entries are non-negative, so the float bits order like the values (*out preset to 0).
 __global__ void k_rowsum_max(const float* __restrict__ KZ, int64_t n_train, int kp,
                              int* __restrict__ out) {
+  pdl_enter();
   __shared__ float red[256];
   float m = 0.f;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_train;
@@ -1136,6 +1156,7 @@ __global__ void k_rhs(const int32_t* __restrict__ perm, const float* __restrict_
                       const float* __restrict__ KZ, int64_t n_all, int64_t n_train, int kp,
                       int S, float* __restrict__ xh, float* __restrict__ xl,
                       float* __restrict__ rh, float* __restrict__ rl, float* __restrict__ p) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_all * kp) return;
   const int64_t row = e / kp;
@@ -1152,6 +1173,7 @@ __global__ void k_rhs(const int32_t* __restrict__ perm, const float* __restrict_
 
 __global__ void k_x_sum(const float* __restrict__ xh, const float* __restrict__ xl,
                         float* __restrict__ out, int64_t count) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < count) out[e] = __fadd_rn(xh[e], xl[e]);
 }
@@ -1160,6 +1182,7 @@ __global__ void k_x_sum(const float* __restrict__ xh, const float* __restrict__ 
 __global__ void k_predict(const int32_t* __restrict__ perm, const float* __restrict__ KW,
                           int64_t n_all, int64_t n_train, int kp, int S, uint64_t seed,
                           float outputscale, float* __restrict__ mean, float* __restrict__ var) {
+  pdl_enter();
   const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= n_all) return;
   const int64_t i = perm[row];
@@ -1494,10 +1517,10 @@ sgp_status setup(sgp_server* S, Request* R, cudaStream_t st, Table& t1) {
   SRV_CHECK(tmp.get((void**)&Vz, vec), "alloc probes");
   SRV_CHECK(tmp.get((void**)&KZ, vec), "alloc probes");
   const unsigned g = (unsigned)ceil_div(n_all * kp, 256);
-  k_probe_fill<<<g, 256, 0, st>>>(Vz, n_all, in.n, kp, S->S, in.seed);
+  launch_pdl(k_probe_fill, g, 256, st, Vz, n_all, in.n, kp, S->S, in.seed);
   note_launches(1);
   enqueue_mvm(L, Vz, kp, SGP_BLUR_SYMMETRIC, L->outputscale, 0.f, KZ, st);
-  k_rhs<<<g, 256, 0, st>>>(L->perm, yd, KZ, n_all, in.n, kp, S->S, R->xh, R->xl, R->rh, R->rl,
+  launch_pdl(k_rhs, g, 256, st, L->perm, yd, KZ, n_all, in.n, kp, S->S, R->xh, R->xl, R->rh, R->rl,
                            R->p);
   note_launches(1);
   // Condition estimate (Gershgorin: largest training-row sum of outputscale K~ over
@@ -1508,7 +1531,7 @@ sgp_status setup(sgp_server* S, Request* R, cudaStream_t st, Table& t1) {
     int* rowmax_d = nullptr;
     SRV_CHECK(tmp.get((void**)&rowmax_d, sizeof(int)), "alloc row sum");
     SRV_CHECK(cudaMemsetAsync(rowmax_d, 0, sizeof(int), st), "clear row sum");
-    k_rowsum_max<<<152, 256, 0, st>>>(KZ, in.n, kp, rowmax_d);
+    launch_pdl(k_rowsum_max, 152, 256, st, KZ, in.n, kp, rowmax_d);
     note_launches(1);
     int rowmax_bits = 0;
     SRV_CHECK(cudaMemcpyAsync(&rowmax_bits, rowmax_d, sizeof(int), cudaMemcpyDeviceToHost, st),
@@ -1528,7 +1551,7 @@ sgp_status setup(sgp_server* S, Request* R, cudaStream_t st, Table& t1) {
     s = ensure_lattice_values(L, kp, st);
     if (s != SGP_OK) return s;
     enqueue_mvm(L, Vz, kp, SGP_BLUR_SYMMETRIC, L->outputscale, 0.f, KZ, st);
-    k_rhs<<<g, 256, 0, st>>>(L->perm, yd, KZ, n_all, in.n, kp, S->S, R->xh, R->xl, R->rh,
+    launch_pdl(k_rhs, g, 256, st, L->perm, yd, KZ, n_all, in.n, kp, S->S, R->xh, R->xl, R->rh,
                              R->rl, R->p);
     note_launches(1);
   }
@@ -1585,20 +1608,20 @@ sgp_status setup(sgp_server* S, Request* R, cudaStream_t st, Table& t1) {
   for (int u = 0; u < U_KINDS; ++u) t1.pre[u][1] = R->vb[u];
   SRV_CHECK(cudaMemcpyAsync(R->dtab1, &t1, sizeof(Table), cudaMemcpyHostToDevice, st),
             "copy table");
-  kb_norm<<<kGrid, kST, 0, st>>>(R->dtab1);
+  launch_pdl(kb_norm, kGrid, kST, st, R->dtab1);
   note_launches(1);
   if (R->l) {  // z_0 = P^-1 r_0 (the kernels run for a request whose state is set)
     static const int kOne = 1;
     SRV_CHECK(cudaMemcpyAsync(R->ints + kp, &kOne, sizeof(int), cudaMemcpyHostToDevice, st),
               "mark the request active");
     launch_bt(kp, R->dtab1, st);
-    kb_bt_seg<<<kGrid, kST, 0, st>>>(R->dtab1);
-    kb_bt_total<<<kGrid, kST, 0, st>>>(R->dtab1);
-    kb_minv<<<kGrid, kST, 0, st>>>(R->dtab1);
+    launch_pdl(kb_bt_seg, kGrid, kST, st, R->dtab1);
+    launch_pdl(kb_bt_total, kGrid, kST, st, R->dtab1);
+    launch_pdl(kb_minv, kGrid, kST, st, R->dtab1);
     launch_apply_z(kp, R->dtab1, st);
     note_launches(5);
   }
-  kb_init_scalars<<<1, kST, 0, st>>>(R->dtab1);
+  launch_pdl(kb_init_scalars, 1, kST, st, R->dtab1);
   note_launches(1);
   if (R->l)  // p_0 = z_0
     SRV_CHECK(cudaMemcpyAsync(R->p, R->ap, vec, cudaMemcpyDeviceToDevice, st), "p = z");
@@ -1618,13 +1641,13 @@ sgp_status finish(sgp_server* S, Request* R, cudaStream_t st) {
   const int kp = S->kp;
   const int64_t n_all = L->n;
   const int64_t cnt = n_all * kp;
-  k_x_sum<<<(unsigned)ceil_div(cnt, 256), 256, 0, st>>>(R->xh, R->xl, R->p, cnt);
+  launch_pdl(k_x_sum, (unsigned)ceil_div(cnt, 256), 256, st, R->xh, R->xl, R->p, cnt);
   note_launches(1);
   enqueue_mvm(L, R->p, kp, SGP_BLUR_SYMMETRIC, L->outputscale, 0.f, R->ap, st, nullptr,
               /*internal=*/true);
   float* mean_d = R->outd;
   float* var_d = R->outd + in.ns;
-  k_predict<<<(unsigned)ceil_div(n_all, 256), 256, 0, st>>>(L->perm, R->ap, n_all, in.n, kp,
+  launch_pdl(k_predict, (unsigned)ceil_div(n_all, 256), 256, st, L->perm, R->ap, n_all, in.n, kp,
                                                            S->S, in.seed, L->outputscale,
                                                            mean_d, var_d);
   note_launches(1);
@@ -1702,27 +1725,27 @@ template <int Rr, class Sv>
 int enqueue_iteration_t(Lane* ln, int dmax, bool sparse, bool pre) {
   cudaStream_t st = ln->st;
   const Table* T = ln->dtab;
-  kb_splat<Sv><<<kGrid, kST, 0, st>>>(T);
-  kb_splat_med<Sv><<<kGrid, kST, 0, st>>>(T);
-  kb_splat_huge<Sv><<<kGrid, kST, 0, st>>>(T);
+  launch_pdl(kb_splat<Sv>, kGrid, kST, st, T);
+  launch_pdl(kb_splat_med<Sv>, kGrid, kST, st, T);
+  launch_pdl(kb_splat_huge<Sv>, kGrid, kST, st, T);
   for (int t = 0; t < 2 * dmax; ++t) {
-    kb_blur<Rr, Sv><<<kGrid, kST, 0, st>>>(T, t);
-    if (sparse) kb_sparse_store<Sv><<<kGrid, kST, 0, st>>>(T, t);
+    launch_pdl(kb_blur<Rr, Sv>, kGrid, kST, st, T, t);
+    if (sparse) launch_pdl(kb_sparse_store<Sv>, kGrid, kST, st, T, t);
   }
-  if (sparse) kb_sparse_finish<Sv><<<kGrid, kST, 0, st>>>(T);
-  kb_slice_dot<Sv><<<kGrid, kST, 0, st>>>(T);
-  kb_alpha<<<kMaxSlots, kST, 0, st>>>(T);
-  kb_update_xr<<<kGrid, kST, 0, st>>>(T);
+  if (sparse) launch_pdl(kb_sparse_finish<Sv>, kGrid, kST, st, T);
+  launch_pdl(kb_slice_dot<Sv>, kGrid, kST, st, T);
+  launch_pdl(kb_alpha, kMaxSlots, kST, st, T);
+  launch_pdl(kb_update_xr, kGrid, kST, st, T);
   if (pre) {
     const int kp = ln->htab->kp;
     launch_bt(kp, T, st);
-    kb_bt_seg<<<kGrid, kST, 0, st>>>(T);
-    kb_bt_total<<<kGrid, kST, 0, st>>>(T);
-    kb_minv<<<kGrid, kST, 0, st>>>(T);
+    launch_pdl(kb_bt_seg, kGrid, kST, st, T);
+    launch_pdl(kb_bt_total, kGrid, kST, st, T);
+    launch_pdl(kb_minv, kGrid, kST, st, T);
     launch_apply_z(kp, T, st);
   }
-  kb_check_beta<<<kMaxSlots, kST, 0, st>>>(T);
-  kb_update_p<<<kGrid, kST, 0, st>>>(T);
+  launch_pdl(kb_check_beta, kMaxSlots, kST, st, T);
+  launch_pdl(kb_update_p, kGrid, kST, st, T);
   return 8 + 2 * dmax + (sparse ? 2 * dmax + 1 : 0) + (pre ? 5 : 0);
 }
 

@@ -164,17 +164,23 @@ cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t st);
 // running grid (a product at n = 50k, d = 8, k = 9: 63 us without, 78 us with it at the top
 // of each kernel; eight CG iterations at n = 86k, d = 8: 998 and 1154 us).
 template <class... P, class... A>
-inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... args) {
+inline void launch_pdl_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                            cudaStream_t st, A&&... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);  // read by cudaGetLastError
+}
+template <class... P, class... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... args) {
+  launch_pdl_smem(kernel, grid, block, 0, st, std::forward<A>(args)...);
 }
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
