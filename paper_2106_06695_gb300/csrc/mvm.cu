@@ -18,6 +18,7 @@
 // groups whatever k and however the caller's buffers are aligned; a thread owns 4 (2, 1)
 // consecutive columns of a row, the pipelined blur 8.  At n = 50k, d = 8, k = 9 a product
 // with 9 scalar columns took 100 us, with 12 padded ones 77.5 us (launches alike).
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <type_traits>
@@ -73,35 +74,32 @@ __global__ void __launch_bounds__(kThreads) k_splat(int64_t nseg, int G, int k,
   else Vt::st(partial + (int64_t)sg.w * k + col, acc);
 }
 
-// Fix-up for vertices with 2..kSplatMedSegs segments: one thread-group sums in order.
+// Fix-up of the vertices with several segments, in one launch.  Blocks below `nhuge`: one
+// vertex of more than kSplatMedSegs segments each, in `groups` (a power of two, groups G <=
+// kThreads) strided partial sums and a fixed-shape shared-memory tree over them (the result
+// depends on `groups` only, not on how the threads share the work).  The blocks after them:
+// one thread-group per vertex of 2..kSplatMedSegs segments, summed in order.
 template <int VEC, class S>
-__global__ void __launch_bounds__(kThreads) k_splat_med(int64_t nrows, int G, int k,
-                                                        const int4* __restrict__ rows,
+__global__ void __launch_bounds__(kThreads) k_splat_fix(int nhuge, int64_t nmed, int groups, int G,
+                                                        int k, const int4* __restrict__ huge_rows,
+                                                        const int4* __restrict__ med_rows,
                                                         const float* __restrict__ partial,
                                                         S* __restrict__ lat) {
   pdl_enter();
   using Vt = Vec<VEC>;
-  const int64_t q = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
-  if (q >= nrows) return;
-  const int col = (int)(threadIdx.x % G) * VEC;
-  const int4 rw = rows[q];
-  typename Vt::T acc = Vt::zero();
-  for (int j = 0; j < rw.z; ++j) acc = Vt::add(acc, Vt::ld(partial + (int64_t)(rw.y + j) * k + col));
-  Vt::sts(lat + (int64_t)rw.x * k + col, acc);
-}
-
-// Fix-up for vertices with more segments: one block per vertex.  `groups` (a power of two,
-// groups G <= kThreads) strided partial sums, then a fixed-shape shared-memory tree over
-// them: the result depends on `groups` only, not on how the threads share the work.
-template <int VEC, class S>
-__global__ void __launch_bounds__(kThreads) k_splat_huge(int groups, int G, int k,
-                                                         const int4* __restrict__ rows,
-                                                         const float* __restrict__ partial,
-                                                         S* __restrict__ lat) {
-  pdl_enter();
-  using Vt = Vec<VEC>;
   __shared__ typename Vt::T red[kThreads];
-  const int4 rw = rows[blockIdx.x];
+  if ((int)blockIdx.x >= nhuge) {
+    const int rows = kThreads / G;
+    const int64_t q = (int64_t)((int)blockIdx.x - nhuge) * rows + threadIdx.x / G;
+    if (q >= nmed || (int)threadIdx.x >= rows * G) return;
+    const int col = (int)(threadIdx.x % G) * VEC;
+    const int4 rw = med_rows[q];
+    typename Vt::T acc = Vt::zero();
+    for (int j = 0; j < rw.z; ++j) acc = Vt::add(acc, Vt::ld(partial + (int64_t)(rw.y + j) * k + col));
+    Vt::sts(lat + (int64_t)rw.x * k + col, acc);
+    return;
+  }
+  const int4 rw = huge_rows[blockIdx.x];
   for (int q = threadIdx.x; q < groups * G; q += blockDim.x) {
     typename Vt::T acc = Vt::zero();
     for (int j = q / G; j < rw.z; j += groups)
@@ -150,7 +148,6 @@ __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k,
                                                         const S* __restrict__ in,
                                                         S* __restrict__ out) {
   static_assert(CH == 1 || (CH == 2 && VEC == 4), "one group of columns per thread, or 2 x 4");
-  pdl_enter();
   using Vt = Vec<VEC>;
   using T = typename Vt::T;
   const int rows_per_run = blockDim.x / G;
@@ -166,6 +163,7 @@ __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k,
       ic[u][t] = v[u] < m ? __ldg(nbr + (int64_t)(2 * t + 1) * m + v[u]) : -1;
     }
   }
+  pdl_enter();  // the ids do not change: loaded before the wait
   auto load = [&](int64_t row, T* x) {
     if constexpr (CH == 2) Store<S>::ldg8(in + row * k + col, x[0], x[1]);
     else x[0] = Vt::ldgs(in + row * k + col);
@@ -184,6 +182,7 @@ __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k,
       if (ic[u][t] >= 0) load(ic[u][t], sc[u][t]);
     }
   }
+  pdl_leave();
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     if (v[u] >= m) continue;
@@ -281,6 +280,102 @@ int blur_pipe_blocks() {
   b = std::max(1, per_sm) * std::max(1, sms);
   cache[dev].store(b);
   return b;
+}
+
+// ---- blur of small lattices ---------------------------------------------------------------
+// All passes in one launch: a cluster of thread blocks holds VEC columns of every vertex in
+// its shared memory (two buffers of `rows` rows a block, vertex v in block v / rows), a
+// neighbour's value is read from whichever block holds it (distributed shared memory), and a
+// cluster barrier separates the passes; the column groups are independent clusters.  A pass
+// of its own launch waits for a grid to drain, for the next to start, for the neighbour ids
+// and then for the rows; here the ids of the next pass are loaded before the barrier and
+// the rows come from shared memory.  Same arithmetic as k_blur_rows, values rounded to S after
+// every pass alike (bitwise equal results).
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive;" ::: "memory");
+  asm volatile("barrier.cluster.wait;" ::: "memory");
+}
+// VEC values of type S at shared-memory address `local` of block `rank` of the cluster.
+template <int VEC, class S>
+__device__ __forceinline__ typename Vec<VEC>::T ld_cluster(uint32_t local, uint32_t rank) {
+  uint32_t at;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(local), "r"(rank));
+  constexpr int kBytes = VEC * (int)sizeof(S);
+  alignas(16) uint32_t w[4];
+  if constexpr (kBytes == 16)
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(at) : "memory");
+  else if constexpr (kBytes == 8)
+    asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "r"(at) : "memory");
+  else if constexpr (kBytes == 4)
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(w[0]) : "r"(at) : "memory");
+  else {
+    uint16_t h;
+    asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(h) : "r"(at) : "memory");
+    w[0] = h;
+  }
+  return Vec<VEC>::lds(reinterpret_cast<const S*>(w));
+}
+
+struct ClusterBlur {
+  int m, k, D, passes, blur, rows;  // rows: vertices per block
+  Taps tp;
+  const int32_t* nbr;
+};
+
+// One thread per vertex (rows <= blockDim.x).
+template <int VEC, int R, class S>
+__global__ void __launch_bounds__(1024) k_blur_cluster(ClusterBlur q, S* __restrict__ lat) {
+  using Vt = Vec<VEC>;
+  using T = typename Vt::T;
+  __shared__ __align__(16) S buf[2][1024 * VEC];
+  const uint32_t rank = cluster_rank();
+  const int v0 = (int)rank * q.rows;
+  const int l = (int)threadIdx.x, col = (int)blockIdx.y * VEC;
+  const bool live = l < q.rows && v0 + l < q.m;  // the last blocks may be short or empty
+  S* own = lat + (int64_t)(v0 + l) * q.k + col;
+  int ids[2 * R];
+  auto load_ids = [&](int t) {
+    const int j = q.blur == SGP_BLUR_SEQUENTIAL ? t
+                  : q.blur == SGP_BLUR_TRANSPOSE ? q.D - 1 - t
+                                                 : (t < q.D ? t : 2 * q.D - 1 - t);
+    const int32_t* plane = q.nbr + (int64_t)j * R * 2 * q.m + v0 + l;
+#pragma unroll
+    for (int e = 0; e < 2 * R; ++e) ids[e] = live ? __ldg(plane + (int64_t)e * q.m) : -1;
+  };
+  load_ids(0);  // the table does not change: before the wait
+  pdl_enter();
+  if (live) Vt::sts(buf[0] + l * VEC, Vt::lds(own));
+  cluster_barrier();
+  int cur = 0;
+  for (int t = 0; t < q.passes; ++t) {
+    if (live) {
+      const uint32_t base = (uint32_t)__cvta_generic_to_shared(buf[cur]);
+      T x[2 * R];
+#pragma unroll
+      for (int e = 0; e < 2 * R; ++e) {
+        x[e] = Vt::zero();
+        if (ids[e] >= 0) {
+          const uint32_t b = (uint32_t)ids[e] / (uint32_t)q.rows;
+          x[e] = ld_cluster<VEC, S>(
+              base + ((uint32_t)ids[e] - b * (uint32_t)q.rows) * (uint32_t)(VEC * sizeof(S)), b);
+        }
+      }
+      T acc = Vt::scale(q.tp.t[0], Vt::lds(buf[cur] + l * VEC));
+#pragma unroll
+      for (int e = 0; e < R; ++e) acc = Vt::fma(q.tp.t[e + 1], Vt::add(x[2 * e], x[2 * e + 1]), acc);
+      Vt::sts(buf[cur ^ 1] + l * VEC, acc);
+    }
+    cur ^= 1;
+    if (t + 1 < q.passes) load_ids(t + 1);
+    cluster_barrier();
+  }
+  if (live) Vt::sts(own, Vt::lds(buf[cur] + l * VEC));
 }
 
 // ---- sparse blur (lattices whose direction lists are short) ------------------------------
@@ -438,9 +533,9 @@ __device__ __forceinline__ typename Vec<VEC>::T slice_row(int64_t p, int D, int 
   return acc;
 }
 
-// out = alpha W lat (+ beta Vp, rows of k in locality order, when beta != 0).  PERM: out has
-// the caller's ko columns and row order (row perm[p]), written one value at a time unless
-// WIDE (ko = k, aligned rows); else out is [n][k] in locality order.
+// out = alpha W lat (+ beta V when beta != 0; V's row perm[p] of ko columns if vperm, the caller's, else rows of k in locality order).  PERM: out has the caller's
+// ko columns and row order (row perm[p]), written one value at a time unless WIDE (ko = k,
+// aligned rows); else out is [n][k] in locality order.
 template <int VEC, bool PERM, bool WIDE, class S>
 __global__ void __launch_bounds__(kThreads) k_slice(int64_t n, int G, int k, int ko, int D,
                                                     const int32_t* __restrict__ perm,
@@ -565,18 +660,13 @@ void launch_splat_t(const Lattice* L, const float* V, int kp, int kt, S* lat, fl
     launch_pdl(k_splat<VEC, S>, q.blocks, q.threads, st, L->nseg, q.G, kp, L->seg, L->items, V, lat,
                partial);
     note_launches(1);
-    if (L->nmed > 0) {
-      const RowShape qm = row_shape(L->nmed, kp);
-      launch_pdl(k_splat_med<VEC, S>, qm.blocks, qm.threads, st, L->nmed, qm.G, kp, L->med_rows,
-                 partial, lat);
-      note_launches(1);
-    }
-    if (L->nhuge > 0) {
+    if (L->nmed > 0 || L->nhuge > 0) {
       const int gt = kt % 4 == 0 ? kt / 4 : kt;
       int groups = 1;
       while (groups * 2 * gt <= kThreads) groups *= 2;
-      launch_pdl(k_splat_huge<VEC, S>, (unsigned)L->nhuge, kThreads, st, groups, q.G, kp,
-                 L->huge_rows, partial, lat);
+      const int64_t med_blocks = ceil_div(L->nmed, kThreads / q.G);
+      launch_pdl(k_splat_fix<VEC, S>, (unsigned)(L->nhuge + med_blocks), kThreads, st, (int)L->nhuge,
+                 L->nmed, groups, q.G, kp, L->huge_rows, L->med_rows, partial, lat);
       note_launches(1);
     }
   });
@@ -666,6 +756,57 @@ void launch_permute(const Lattice* L, const float* V, int k, int kp, float* Vp, 
   note_launches(1);
 }
 
+// The cluster blur takes lattices of up to 16 blocks of 1024 vertices and up to 8 column
+// groups (as many clusters are resident at once).  Measured, symmetric product with d = 8, k =
+// 16, clusters of 16 / a launch a pass: m = 5.9k 34 / 55 us, 10.8k (k = 12) 41 / 61 us, 17k (d = 9,
+// k = 2) 52 / 62 us; beyond, remote shared-memory reads cost more than a launch (m = 51k: 107 /
+// 62 us with several vertices a thread).  Blocks of 64 vertices or more: smaller clusters
+// were never faster (m = 1k, d = 4: 38 us with one block, 31 with 16).
+constexpr int kClusterBlocks = 16, kClusterRows = 1024, kClusterGroups = 8;
+
+template <int VEC, int R, class S>
+cudaError_t launch_cluster(const ClusterBlur& q, int blocks, int groups, S* lat, cudaStream_t st) {
+  auto kernel = k_blur_cluster<VEC, R, S>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute at[2]{};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)blocks;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks, (unsigned)groups);
+  cfg.blockDim = (unsigned)(ceil_div(q.rows, 32) * 32);
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, q, lat);
+}
+
+// All passes on lat0 by k_blur_cluster; false when the lattice is not of its size.
+template <class S>
+bool blur_cluster_t(const Lattice* L, int blur, int passes, const Taps& tp, S* lat0, int k,
+                    cudaStream_t st) {
+  const RowShape shape = row_shape(L->m, k);
+  if (L->m > kClusterBlocks * kClusterRows || shape.G > kClusterGroups || L->r > 2) return false;
+  int blocks = 1;
+  while (blocks < kClusterBlocks && L->m > 64 * blocks) blocks *= 2;
+  const ClusterBlur q{(int)L->m, k, L->D, passes, blur, (int)ceil_div(L->m, blocks), tp, L->nbr};
+  cudaError_t e = cudaSuccess;
+  by_vec(shape.vec, [&](auto vec) {
+    constexpr int VEC = decltype(vec)::value;
+    e = L->r == 1 ? launch_cluster<VEC, 1, S>(q, blocks, shape.G, lat0, st)
+                  : launch_cluster<VEC, 2, S>(q, blocks, shape.G, lat0, st);
+  });
+  if (e != cudaSuccess) {  // no room for such a cluster (e.g. a partitioned device)
+    clear_pending_error();
+    return false;
+  }
+  note_launches(1);
+  return true;
+}
+
 // Sparse blurs run on chains (else on the direction lists).
 bool chains_ok(const Lattice* L) { return L->chain_max > 0 && L->chain_max <= kMaxChain; }
 
@@ -691,6 +832,7 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
   const Taps& tp = blur == SGP_BLUR_SYMMETRIC ? g : c;
   if (passes_out) *passes_out = P;
   if (!L->sparse || dense) {
+    if (blur_cluster_t<S>(L, blur, P, tp, lat0, k, st)) return lat0;
     S* a = lat0;
     S* b = lat1;
     for (int t = 0; t < P; ++t) {

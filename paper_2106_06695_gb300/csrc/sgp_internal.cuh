@@ -159,10 +159,11 @@ cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t st);
 // legacy and created streams; inside a graph 1.15 and 0.94 us).  launch_pdl marks a launch as
 // such a dependent; every kernel launched with it starts with pdl_enter(), which waits until
 // all work before this grid has completed and is visible.  Nothing is read or written
-// before that wait, so ordering is as with ordinary launches.  No kernel lets its dependents
-// in early (griddepcontrol.launch_dependents): their waiting blocks take slots from the
-// running grid (a product at n = 50k, d = 8, k = 9: 63 us without, 78 us with it at the top
-// of each kernel; eight CG iterations at n = 86k, d = 8: 998 and 1154 us).
+// before that wait but arrays that do not change after the build (neighbour ids), so ordering is
+// as with ordinary launches.  Dependents are not let in early (griddepcontrol.launch_dependents
+// at the top of each kernel): their waiting blocks take slots from the running grid (a
+// product at n = 50k, d = 8, k = 9: 63 us without, 78 us with it; eight CG iterations at n =
+// 86k, d = 8: 998 and 1154 us).  After the last loads are issued it does no harm (pdl_leave).
 template <class... P, class... A>
 inline void launch_pdl_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                             cudaStream_t st, A&&... args) {
@@ -181,6 +182,10 @@ inline void launch_pdl_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t 
 template <class... P, class... A>
 inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... args) {
   launch_pdl_smem(kernel, grid, block, 0, st, std::forward<A>(args)...);
+}
+// Lets the next grid in: only where this grid has nothing left to load.
+__device__ __forceinline__ void pdl_leave() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
