@@ -109,13 +109,7 @@ __device__ __forceinline__ double div_rn(double a, double b, double rb) {
   return (__double_as_longlong(a) << 1) == 0 ? q0 : q;
 }
 
-// (double)x, and x to 22 bits or more as a float (0 below 2^-126; callers bound it above).
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t u = __float_as_uint(x), e = (u >> 23) & 255u;
-  if (e == 0u || e == 255u) return (double)x;
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))),
-                          (int)(u << 29));
-}
+// x to 22 bits or more as a float (0 below 2^-126; callers bound it above).
 __device__ __forceinline__ float narrow(double x) {
   const uint32_t hi = (uint32_t)__double2hiint(x), m = hi & 0x7fffffffu;
   if (m < (897u << 20)) return 0.f;
@@ -134,7 +128,7 @@ __device__ __forceinline__ long long rank_key(double x) {
 
 // (double) of an integer below 2^24 in magnitude.
 __device__ __forceinline__ double exact_int(int x) {
-  return x == 0 ? 0.0 : widen((float)x);
+  return widen((float)x);
 }
 
 // Nearest multiple of D to y (ties go down) as an integer, and y minus it.  False when the

@@ -23,14 +23,15 @@ namespace {
 
 struct CgState {
   double* partial;  // [blocks][k] per-block column sums
-  double* rho;      // <r, r> of the current residual
-  double* pap;      // <p, A p>
-  double* alpha;
-  double* beta;
+  double* rho;      // <r, r> of the current residual (<r, z> when preconditioned)
+  dfloat* alpha;    // as double-float pairs, the form the vector updates use
+  dfloat* beta;
   double* bnorm;
-  double* relres;
+  double* rr;       // <r, r> after the last iteration of the column
   int* active;
   int* iters;
+  float tol;
+  int max_iter;
   // optional Lanczos record (plain CG): alpha_j, beta_j of column c at [j][k], j < hcap
   double* ha;
   double* hb;
@@ -42,6 +43,137 @@ struct CgState {
   // at 16 p + c), written by the x, r update
   bf16* r3;
 };
+
+// What the totals of a kernel's column sums are used for.
+enum CgEnd {
+  CG_INIT = 0,  // sum = <b, b>: norms, first rho, columns that start stopped
+  CG_ALPHA,     // sum = <p, A p>: step sizes
+  CG_BETA,      // sum = <r, r>: convergence and the next direction's beta (plain CG)
+  CG_CHECK,     // sum = <r, r>: convergence only (preconditioned)
+  CG_RHO_INIT,  // sum = <r, z> at the start
+  CG_BETA_PRE,  // sum = <r, z>: beta (preconditioned)
+};
+
+// Whether ||r|| / ||b|| = sqrt(rr) / bnorm (fp64) is at most tol or not finite.  Decided in
+// fp32 unless the two are within 1e-4 of each other (or out of fp32's range): a square root
+// and a division in fp64 are some 60 dependent operations of a narrow pipe, 2 us.
+__device__ __forceinline__ bool cg_stops(double rr, double bnorm, float tol) {
+  const float r = (float)rr, b = (float)bnorm;
+  const float lim = tol * b * (tol * b);
+  if (r > 1e-30f && r < 1e30f && lim < 1e30f && lim > 1e-30f) {
+    if (r > lim * 1.0002f) return false;
+    if (r < lim * 0.9998f) return true;
+  }
+  const double rel = sqrt(rr) / bnorm;
+  return rel <= (double)tol || !isfinite(rel);
+}
+
+// What one thread holds of a column before its sum is known.
+struct CgColumn {
+  double rho = 0.0, bnorm = 0.0;
+  int active = 0, iters = 0;
+};
+
+__device__ __forceinline__ void cg_end_column(CgEnd what, int c, int k, double sum,
+                                              const CgColumn& col, const CgState& S) {
+  switch (what) {
+    case CG_INIT:
+      S.rho[c] = sum;
+      S.rr[c] = sum;
+      S.bnorm[c] = sqrt(sum);
+      S.iters[c] = 0;
+      S.alpha[c] = S.beta[c] = {0.f, 0.f};
+      S.active[c] = sum != 0.0 && 1.0 > (double)S.tol && S.max_iter > 0 ? 1 : 0;
+      return;
+    case CG_ALPHA: {
+      double alpha = 0.0;
+      if (col.active) {
+        if (sum > 0.0 && isfinite(sum)) {
+          alpha = col.rho / sum;
+          if (S.ha && col.iters < S.hcap) S.ha[(int64_t)col.iters * k + c] = alpha;
+        } else {
+          S.active[c] = 0;  // breakdown: the operator is not positive definite on p
+        }
+      }
+      S.alpha[c] = df_from_double(alpha);
+      return;
+    }
+    case CG_BETA:
+    case CG_CHECK: {
+      if (!col.active) return;
+      const int it = col.iters + 1;
+      S.iters[c] = it;
+      S.rr[c] = sum;
+      if (S.hist && it <= S.hist_cap) S.hist[(int64_t)(it - 1) * k + c] = sqrt(sum) / col.bnorm;
+      if (it >= S.max_iter || cg_stops(sum, col.bnorm, S.tol)) {
+        S.active[c] = 0;
+        return;
+      }
+      if (what == CG_CHECK) return;
+      const double beta = sum / col.rho;
+      S.beta[c] = df_from_double(beta);
+      S.rho[c] = sum;
+      if (S.hb && it - 1 < S.hcap) S.hb[(int64_t)(it - 1) * k + c] = beta;
+      return;
+    }
+    case CG_RHO_INIT:
+      S.rho[c] = sum;
+      if (!(sum > 0.0) || !isfinite(sum)) S.active[c] = 0;
+      return;
+    case CG_BETA_PRE:
+      if (!col.active) return;
+      if (!(sum > 0.0) || !isfinite(sum)) {
+        S.active[c] = 0;
+        return;
+      }
+      S.beta[c] = df_from_double(sum / col.rho);
+      S.rho[c] = sum;
+      return;
+    default:
+      return;
+  }
+}
+
+// Column c's sum over `nblk` block partials and what follows from it.  One warp per column
+// (blockIdx.x = c).  The order of the additions is part of the result (a preconditioned
+// solve of 100 iterations carries a last-place change of one sum to the fifth digit of its
+// answer): 256 strided sums over the blocks, then a tree over them, halves first.  A lane
+// holds eight of the 256 sums, all its loads are in flight together and the tree needs no
+// barrier: a dependent fp64 addition takes some 100 clocks on this part, so the kernel is a
+// chain of latencies (n = 50k: 4.2-5.4 us for the three of an iteration).
+// Letting the last block of the producing kernel do this instead was slower: its twelve
+// columns share one SM's fp64 pipe (slice and sums of n = 50k, k = 12: 27 us, apart 17 us).
+__global__ void __launch_bounds__(32) k_cg_end(CgEnd what, int nblk, int k, CgState S) {
+  pdl_enter();
+  const int lane = (int)threadIdx.x, c = (int)blockIdx.x;
+  CgColumn col;
+  if (lane == 0 && what != CG_INIT) {
+    col.rho = S.rho[c];
+    col.bnorm = S.bnorm[c];
+    col.active = S.active[c];
+    col.iters = S.iters[c];
+  }
+  double v[8];  // sums lane, lane + 32, ..., lane + 224
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v[q] = 0.0;
+#pragma unroll 4
+  for (int b0 = lane; b0 < nblk; b0 += 256) {
+    double x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      x[q] = b0 + 32 * q < nblk ? S.partial[(int64_t)(b0 + 32 * q) * k + c] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] += x[q];
+  }
+#pragma unroll
+  for (int half = 4; half >= 1; half /= 2)
+#pragma unroll
+    for (int q = 0; q < half; ++q) v[q] += v[q + half];
+#pragma unroll
+  for (int half = 16; half >= 1; half /= 2) v[0] += __shfl_down_sync(0xffffffffu, v[0], half);
+  if (lane == 0) cg_end_column(what, c, k, v[0], col, S);
+}
+
 
 // VEC consecutive elements of a row: fp32 (one float4 when VEC = 4) and fp64 (two double2).
 template <int VEC>
@@ -76,7 +208,7 @@ template <int VEC>
 __global__ void k_cg_init(const float* __restrict__ B, int kb, const int32_t* __restrict__ perm,
                           float* __restrict__ xh, float* __restrict__ xl,
                           float* __restrict__ rh, float* __restrict__ rl, float* __restrict__ p,
-                          int64_t n, int k, double* __restrict__ partial) {
+                          int64_t n, int k, CgState S) {
   pdl_enter();
   dfloat acc[VEC];
 #pragma unroll
@@ -100,65 +232,13 @@ __global__ void k_cg_init(const float* __restrict__ B, int kb, const int32_t* __
   double dd[VEC];
 #pragma unroll
   for (int j = 0; j < VEC; ++j) dd[j] = df_to_double(acc[j]);
-  block_column_sums<VEC>(dd, k, partial + (int64_t)blockIdx.x * k);
+  block_column_sums<VEC>(dd, k, S.partial + (int64_t)blockIdx.x * k);
 }
 
-// Column c's sum over `nblk` block partials, in a fixed order (strided per thread, then a
-// shared-memory tree); blockIdx.x = c, blockDim.x = 256.
-__device__ __forceinline__ double column_total(const double* __restrict__ partial, int nblk, int k) {
-  __shared__ double red[256];
-  const int c = blockIdx.x;
-  double t = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) t += partial[(int64_t)b * k + c];
-  red[threadIdx.x] = t;
-  __syncthreads();
-  for (int half = blockDim.x / 2; half >= 1; half /= 2) {
-    if ((int)threadIdx.x < half) red[threadIdx.x] += red[threadIdx.x + half];
-    __syncthreads();
-  }
-  return red[0];
-}
-
-__global__ void k_cg_init_scalars(const double* __restrict__ partial, int nblk, int k,
-                                  float tol, int max_iter, CgState S) {
-  pdl_enter();
-  const double rr = column_total(partial, nblk, k);
-  if (threadIdx.x != 0) return;
-  const int c = blockIdx.x;
-  S.rho[c] = rr;
-  S.bnorm[c] = sqrt(rr);
-  S.iters[c] = 0;
-  S.alpha[c] = 0.0;
-  S.beta[c] = 0.0;
-  if (rr == 0.0) {
-    S.relres[c] = 0.0;
-    S.active[c] = 0;
-  } else {
-    S.relres[c] = 1.0;
-    S.active[c] = (1.0 > (double)tol && max_iter > 0) ? 1 : 0;
-  }
-}
-
-// <p, A p> from the slice's block partials, then alpha = rho / <p, A p>.
-__global__ void k_cg_alpha(int nblk, int k, CgState S) {
-  pdl_enter();
-  const double pap = column_total(S.partial, nblk, k);
-  if (threadIdx.x != 0) return;
-  const int c = blockIdx.x;
-  S.pap[c] = pap;
-  double alpha = 0.0;
-  if (S.active[c]) {
-    if (pap > 0.0 && isfinite(pap)) {
-      alpha = S.rho[c] / pap;
-      if (S.ha && S.iters[c] < S.hcap) S.ha[(int64_t)S.iters[c] * k + c] = alpha;
-    } else {
-      S.active[c] = 0;  // breakdown: the operator is not positive definite on p
-    }
-  }
-  S.alpha[c] = alpha;
-}
-
-// x += alpha p, r -= alpha A p on active columns (double-float); block partials of <r, r>.
+// x += alpha p, r -= alpha A p on active columns (double-float); block partials of
+// <r, r>.  fp64 issues at 2 results per SM and clock, so the step sizes arrive
+// as double-float pairs and the sums leave a thread by integer conversions: n = 50k, k = 12
+// (one row a thread) 10.6 us, 21.2 with both in fp64.
 // With S.r3 (VEC = 4), also the three bf16 parts of r = rh + rl for columns 0..15, the
 // operand of the preconditioner's B^T r (as its split kernel would write them).
 template <int VEC>
@@ -175,7 +255,7 @@ __global__ void k_cg_update_xr(float* __restrict__ xh, float* __restrict__ xl,
     for (int j = 0; j < VEC; ++j) {
       acc[j] = {0.f, 0.f};
       on[j] = S.active[c + j] != 0;
-      a[j] = df_from_double(S.alpha[c + j]);
+      a[j] = S.alpha[c + j];
       na[j] = {-a[j].hi, -a[j].lo};
     }
   }
@@ -226,66 +306,6 @@ __global__ void k_cg_update_xr(float* __restrict__ xh, float* __restrict__ xl,
   block_column_sums<VEC>(dd, k, S.partial + (int64_t)blockIdx.x * k);
 }
 
-__global__ void k_cg_beta(int nblk, int k, float tol, int max_iter, CgState S) {
-  pdl_enter();
-  const double rr = column_total(S.partial, nblk, k);
-  if (threadIdx.x != 0) return;
-  const int c = blockIdx.x;
-  if (!S.active[c]) return;
-  const int it = S.iters[c] + 1;
-  S.iters[c] = it;
-  const double rel = sqrt(rr) / S.bnorm[c];
-  S.relres[c] = rel;
-  if (S.hist && it <= S.hist_cap) S.hist[(int64_t)(it - 1) * k + c] = rel;
-  if (rel <= (double)tol || it >= max_iter || !isfinite(rel)) {
-    S.active[c] = 0;
-    return;
-  }
-  S.beta[c] = rr / S.rho[c];
-  S.rho[c] = rr;
-  if (S.hb && it - 1 < S.hcap) S.hb[(int64_t)(it - 1) * k + c] = S.beta[c];
-}
-
-// Preconditioned CG: convergence check on <r, r> (no beta yet).
-__global__ void k_cg_check(int nblk, int k, float tol, int max_iter, CgState S) {
-  pdl_enter();
-  const double rr = column_total(S.partial, nblk, k);
-  if (threadIdx.x != 0) return;
-  const int c = blockIdx.x;
-  if (!S.active[c]) return;
-  const int it = S.iters[c] + 1;
-  S.iters[c] = it;
-  const double rel = sqrt(rr) / S.bnorm[c];
-  S.relres[c] = rel;
-  if (S.hist && it <= S.hist_cap) S.hist[(int64_t)(it - 1) * k + c] = rel;
-  if (rel <= (double)tol || it >= max_iter || !isfinite(rel)) S.active[c] = 0;
-}
-
-// Preconditioned CG: rho = <r, z> at the start.
-__global__ void k_cg_rho_init(int nblk, int k, CgState S) {
-  pdl_enter();
-  const double rz = column_total(S.partial, nblk, k);
-  if (threadIdx.x != 0) return;
-  const int c = blockIdx.x;
-  S.rho[c] = rz;
-  if (!(rz > 0.0) || !isfinite(rz)) S.active[c] = 0;
-}
-
-// Preconditioned CG: beta = <r, z>_new / <r, z>_old on active columns.
-__global__ void k_cg_beta_pcg(int nblk, int k, CgState S) {
-  pdl_enter();
-  const double rz = column_total(S.partial, nblk, k);
-  if (threadIdx.x != 0) return;
-  const int c = blockIdx.x;
-  if (!S.active[c]) return;
-  if (!(rz > 0.0) || !isfinite(rz)) {
-    S.active[c] = 0;
-    return;
-  }
-  S.beta[c] = rz / S.rho[c];
-  S.rho[c] = rz;
-}
-
 // Preconditioned CG: p = z + beta p on active columns (first == true: p = z).
 template <int VEC, bool FIRST>
 __global__ void k_cg_update_p_z(float* __restrict__ p, const float* __restrict__ z, int64_t n,
@@ -298,7 +318,7 @@ __global__ void k_cg_update_p_z(float* __restrict__ p, const float* __restrict__
 #pragma unroll
     for (int j = 0; j < VEC; ++j) {
       on[j] = S.active[c + j] != 0;
-      b[j] = df_from_double(S.beta[c + j]);
+      b[j] = S.beta[c + j];
     }
   }
   SGP_ROWS_LOOP(row) {
@@ -331,7 +351,7 @@ __global__ void k_cg_update_p(float* __restrict__ p, const float* __restrict__ r
 #pragma unroll
     for (int j = 0; j < VEC; ++j) {
       on[j] = S.active[c + j] != 0;
-      b[j] = df_from_double(S.beta[c + j]);
+      b[j] = S.beta[c + j];
     }
   }
   SGP_ROWS_LOOP(row) {
@@ -422,7 +442,7 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
   const int vec = k % 4 == 0 ? 4 : 1;
   const int T = column_block_threads(k, vec);
   const int64_t rows_per_block = T / (k / vec);
-  const int vblocks = (int)std::min<int64_t>(kVecBlocks, std::max<int64_t>(1, ceil_div(n, rows_per_block)));
+  const unsigned vblocks = (unsigned)std::min<int64_t>(kVecBlocks, std::max<int64_t>(1, ceil_div(n, rows_per_block)));
   const int64_t sblocks = slice_dot_blocks(L, k);
   const bool want_pre = precond_rank > 0 && noise > 0.f && !rec;
   // bounds ShiftedNystrom::dot_blocks (its z blocks: at most one per 128-row tile)
@@ -438,17 +458,18 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
                    sizeof(double)),
            "alloc partial");
   double* scal;
-  CG_CHECK(get((void**)&scal, 6 * (size_t)k * sizeof(double)), "alloc scalars");
+  CG_CHECK(get((void**)&scal, 5 * (size_t)k * sizeof(double)), "alloc scalars");
   S.rho = scal;
-  S.pap = scal + k;
-  S.alpha = scal + 2 * k;
-  S.beta = scal + 3 * k;
-  S.bnorm = scal + 4 * k;
-  S.relres = scal + 5 * k;
+  S.bnorm = scal + k;
+  S.rr = scal + 2 * k;
+  S.alpha = reinterpret_cast<dfloat*>(scal + 3 * k);
+  S.beta = reinterpret_cast<dfloat*>(scal + 4 * k);
   int* flags;
   CG_CHECK(get((void**)&flags, 2 * (size_t)k * sizeof(int)), "alloc flags");
   S.active = flags;
   S.iters = flags + k;
+  S.tol = tol;
+  S.max_iter = max_iter;
   if (rec) {
     S.ha = rec->alpha;
     S.hb = rec->beta;
@@ -480,42 +501,47 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
   }
 
   if (vec == 4)
-    launch_pdl(k_cg_init<4>, vblocks, T, st, B, kb, L->perm, xh, xl, rh, rl, p, n, k, S.partial);
+    launch_pdl(k_cg_init<4>, vblocks, T, st, B, kb, L->perm, xh, xl, rh, rl, p, n, k, S);
   else
-    launch_pdl(k_cg_init<1>, vblocks, T, st, B, kb, L->perm, xh, xl, rh, rl, p, n, k, S.partial);
-  launch_pdl(k_cg_init_scalars, k, 256, st, S.partial, vblocks, k, tol, max_iter, S);
-  note_launches(2);
+    launch_pdl(k_cg_init<1>, vblocks, T, st, B, kb, L->perm, xh, xl, rh, rl, p, n, k, S);
+  auto end = [&](CgEnd what, int64_t blocks) {
+    launch_pdl(k_cg_end, k, 32, st, what, (int)blocks, k, S);
+    note_launches(1);
+  };
+  end(CG_INIT, vblocks);
+  note_launches(1);
   if (use_pre) {  // z = P^-1 r, rho = <r, z>, p = z
     cl.pre.apply(rh, rl, k, z, S.partial, st);
-    launch_pdl(k_cg_rho_init, k, 256, st, (int)cl.pre.dot_blocks(), k, S);
+    end(CG_RHO_INIT, cl.pre.dot_blocks());
     if (vec == 4) launch_pdl(k_cg_update_p_z<4, true>, vblocks, T, st, p, z, n, k, S);
     else launch_pdl(k_cg_update_p_z<1, true>, vblocks, T, st, p, z, n, k, S);
-    note_launches(2);
+    note_launches(1);
   }
   CG_CHECK(cudaGetLastError(), "CG init");
 
   cudaEvent_t* ev = L->profile ? L->prof_ev : nullptr;
   int passes = 0;
+  const CgEnd after_r = use_pre ? CG_CHECK : CG_BETA;
   auto iteration = [&]() {
-    // Ap = outputscale K~ p + noise p, with the slice also summing <p, Ap> per block
+    // Ap = outputscale K~ p + noise p, with the slice also summing <p, Ap>: alpha
     passes = enqueue_mvm(L, p, k, blur, L->outputscale, noise, Ap, st, ev, /*internal=*/true,
                          S.partial, rec ? kb : k);
-    launch_pdl(k_cg_alpha, k, 256, st, (int)sblocks, k, S);
-    if (vec == 4) launch_pdl(k_cg_update_xr<4>, vblocks, T, st, xh, xl, rh, rl, p, Ap, n, k, S);
-    else launch_pdl(k_cg_update_xr<1>, vblocks, T, st, xh, xl, rh, rl, p, Ap, n, k, S);
+    end(CG_ALPHA, sblocks);
+    if (vec == 4)
+      launch_pdl(k_cg_update_xr<4>, vblocks, T, st, xh, xl, rh, rl, p, Ap, n, k, S);
+    else
+      launch_pdl(k_cg_update_xr<1>, vblocks, T, st, xh, xl, rh, rl, p, Ap, n, k, S);
+    end(after_r, vblocks);
     if (use_pre) {
-      launch_pdl(k_cg_check, k, 256, st, vblocks, k, tol, max_iter, S);
       cl.pre.apply(rh, rl, k, z, S.partial, st, ev ? ev + 4 : nullptr, S.r3 != nullptr);
-      launch_pdl(k_cg_beta_pcg, k, 256, st, (int)cl.pre.dot_blocks(), k, S);
+      end(CG_BETA_PRE, cl.pre.dot_blocks());
       if (vec == 4) launch_pdl(k_cg_update_p_z<4, false>, vblocks, T, st, p, z, n, k, S);
       else launch_pdl(k_cg_update_p_z<1, false>, vblocks, T, st, p, z, n, k, S);
-      note_launches(5);
     } else {
-      launch_pdl(k_cg_beta, k, 256, st, vblocks, k, tol, max_iter, S);
       if (vec == 4) launch_pdl(k_cg_update_p<4>, vblocks, T, st, p, rh, rl, n, k, S);
       else launch_pdl(k_cg_update_p<1>, vblocks, T, st, p, rh, rl, n, k, S);
-      note_launches(4);
     }
+    note_launches(2);
   };
 
   std::vector<int> hact(k);
@@ -558,16 +584,21 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
   else launch_pdl(k_cg_store_x<1>, vblocks, T, st, xh, xl, L->perm, X, kb, n, k);
   note_launches(1);
   CG_CHECK(cudaGetLastError(), "CG result");
-  std::vector<double> hrel(k);
+  std::vector<double> hscal(2 * (size_t)k);  // ||b||, <r, r>
   std::vector<int> hit(k);
-  CG_CHECK(cudaMemcpyAsync(hrel.data(), S.relres, k * sizeof(double), cudaMemcpyDeviceToHost, st),
+  CG_CHECK(cudaMemcpyAsync(hscal.data(), S.bnorm, hscal.size() * sizeof(double),
+                           cudaMemcpyDeviceToHost, st),
            "read residuals");
   CG_CHECK(cudaMemcpyAsync(hit.data(), S.iters, k * sizeof(int), cudaMemcpyDeviceToHost, st),
            "read iterations");
   CG_CHECK(cudaStreamSynchronize(st), "sync CG");
   if (use_pre && (s = cl.pre.check(st)) != SGP_OK) return s;
   if (iters) std::copy(hit.begin(), hit.begin() + kb, iters);
-  if (rel_res) std::copy(hrel.begin(), hrel.begin() + kb, rel_res);
+  if (rel_res)
+    for (int c = 0; c < kb; ++c) {  // ||r|| / ||b||; 1 before the first iteration, 0 for b = 0
+      const double b = hscal[c], r = std::sqrt(hscal[k + c]);
+      rel_res[c] = b == 0.0 ? 0.0 : hit[c] == 0 ? 1.0 : r / b;
+    }
   if (S.hist) {  // [max_iter][k] on the device, the caller's [max_iter][kb] on the host
     std::vector<double> h((size_t)max_iter * k);
     CG_CHECK(cudaMemcpyAsync(h.data(), S.hist, h.size() * sizeof(double),

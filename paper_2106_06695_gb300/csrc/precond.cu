@@ -139,21 +139,31 @@ __global__ void k_split_r(const float* __restrict__ rh, const float* __restrict_
   }
 }
 
-// t[i][c] = sum over splits of tpart[s][i][c] (fp64 in split order, stored fp32), i < ld.
-// The loads of eight splits are issued together (they are independent) before their sums.
-__global__ void k_sum_t(const float* __restrict__ tpart, int splits, int ld,
-                        float* __restrict__ t) {
+// t[i][c] = sum over splits of tpart[s][i][c] (fp64 in split order, stored fp32), i < ld.  fp64
+// issues at 2 results per SM and clock, so the outputs are spread over the chip in blocks of
+// one warp; the loads of the next eight splits are in flight while eight are added.  131
+// splits of 256 x 16 outputs: 14.7 us (a chain of 131 fp64 additions), 23.5 with 256 outputs
+// and their conversions on each of 16 SMs.
+__global__ void __launch_bounds__(32) k_sum_t(const float* __restrict__ tpart, int splits, int ld,
+                                              float* __restrict__ t) {
   pdl_enter();
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= ld * 16) return;
+  const int e = blockIdx.x * 32 + threadIdx.x;  // ld * 16 is a multiple of 32
   const size_t stride = (size_t)ld * 16;
+  constexpr int kRun = 8;
+  float v[kRun], next[kRun];
+  auto load = [&](int q0, float (&x)[kRun]) {
+#pragma unroll
+    for (int j = 0; j < kRun; ++j) x[j] = q0 + j < splits ? tpart[(q0 + j) * stride + e] : 0.f;
+  };
+  load(0, v);
   double s = 0.0;
-  for (int q0 = 0; q0 < splits; q0 += 8) {
-    float v[8];
+  for (int q0 = 0; q0 < splits; q0 += kRun) {
+    load(q0 + kRun, next);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = q0 + j < splits ? tpart[(q0 + j) * stride + e] : 0.f;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) s += (double)v[j];
+    for (int j = 0; j < kRun; ++j) {
+      s += widen(v[j]);
+      v[j] = next[j];
+    }
   }
   t[e] = (float)s;
 }
@@ -490,6 +500,27 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     for (int64_t j = 0; j < my_tiles; ++j) {
       const int b = (int)(j & 1);
       const int64_t tile = blockIdx.x + j * (int64_t)gridDim.x;
+      // the tile's rows of r, loaded while its products are made
+      const int64_t row = tile * 128 + 32 * q + lane;
+      const int64_t e0 = row * k + c_off;
+      float rv[16];
+      if (row < n) {
+        if (vec) {
+#pragma unroll
+          for (int c4 = 0; c4 < 4; ++c4)
+            if (4 * c4 < kc) {
+              const float4 h = *reinterpret_cast<const float4*>(rh + e0 + 4 * c4);
+              rv[4 * c4] = h.x;
+              rv[4 * c4 + 1] = h.y;
+              rv[4 * c4 + 2] = h.z;
+              rv[4 * c4 + 3] = h.w;
+            }
+        } else {
+#pragma unroll
+          for (int c = 0; c < 16; ++c)
+            if (c < kc) rv[c] = rh[e0 + c];
+        }
+      }
       bool ok = tc05::mbar_wait(&R.accf[b], (uint32_t)(j >> 1) & 1u, kTcSpin, abort);
       ok = epilogue_and(ok);
       if (!ok) {
@@ -508,35 +539,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       tc05::tmem_wait_ld();
       tc05::fence_before_sync();
       tc05::mbar_arrive(&R.acce[b]);
-      const int64_t row = tile * 128 + 32 * q + lane;
       double pr[16];
 #pragma unroll
       for (int c = 0; c < 16; ++c) pr[c] = 0.0;
       if (row < n) {
-        float rv[16];
-        const int64_t e0 = row * k + c_off;
-        if (vec) {
-#pragma unroll
-          for (int c4 = 0; c4 < 4; ++c4)
-            if (4 * c4 < kc) {
-              const float4 h = *reinterpret_cast<const float4*>(rh + e0 + 4 * c4);
-              rv[4 * c4] = h.x;
-              rv[4 * c4 + 1] = h.y;
-              rv[4 * c4 + 2] = h.z;
-              rv[4 * c4 + 3] = h.w;
-            }
-        } else {
-#pragma unroll
-          for (int c = 0; c < 16; ++c)
-            if (c < kc) rv[c] = rh[e0 + c];
-        }
         float zz[16];
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
           zz[c] = 0.f;
           if (c < kc) {
             zz[c] = (rv[c] - (d1[c] + (d2[c] + d3[c]))) * inv_tau;
-            pr[c] = (double)rv[c] * (double)zz[c];
+            pr[c] = df_to_double(df_two_prod(rv[c], zz[c]));  // the exact product
           }
         }
         if (vec) {
@@ -551,18 +564,21 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (c < kc) z[e0 + c] = zz[c];
         }
       }
-      // column sums over the tile's rows: butterfly within each warp, then the four
-      // quarters in row order
+      // column sums over the tile's rows, within each warp, then the four quarters in row
+      // order.  A butterfly in which lanes also split the columns between them: 16 fp64
+      // additions a lane (80 with every lane summing every column: n = 50k, ld = 256 took 20.9
+      // us, now 12.3).
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        double v = pr[c];
-        v += __shfl_xor_sync(0xffffffffu, v, 16);
-        v += __shfl_xor_sync(0xffffffffu, v, 8);
-        v += __shfl_xor_sync(0xffffffffu, v, 4);
-        v += __shfl_xor_sync(0xffffffffu, v, 2);
-        v += __shfl_xor_sync(0xffffffffu, v, 1);
-        if (lane == 0) red[b][q][c] = v;
+      for (int half = 8; half >= 1; half /= 2) {
+        const bool upper = lane & (2 * half);
+#pragma unroll
+        for (int c = 0; c < half; ++c) {
+          const double give = upper ? pr[c] : pr[c + half], keep = upper ? pr[c + half] : pr[c];
+          pr[c] = keep + __shfl_xor_sync(0xffffffffu, give, 2 * half);
+        }
       }
+      pr[0] += __shfl_xor_sync(0xffffffffu, pr[0], 1);
+      if (!(lane & 1)) red[b][q][lane >> 1] = pr[0];
       epilogue_sync();
       if (warp == 1 && lane < kc)
         blk += ((red[b][0][lane] + red[b][1][lane]) + red[b][2][lane]) + red[b][3][lane];
@@ -1695,7 +1711,7 @@ void ShiftedNystrom::apply(const float* rh, const float* rl, int k, float* z, do
     launch_pdl_smem(k_bt_tc, dim3(ntile, bt_splits), kTcThreads, BtRing::kSmem, st, map_b_mn, map_r, n, bt_rows,
                                                                   tpart, err);
     if (mark) cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal);
-    launch_pdl(k_sum_t, (unsigned)ceil_div(ld * 16, 256), 256, st, tpart, bt_splits, ld, tvec);
+    launch_pdl(k_sum_t, (unsigned)(ld * 16 / 32), 32, st, tpart, bt_splits, ld, tvec);
     launch_pdl(k_minv_u, (unsigned)ceil_div(ld, 8), 256, st, Minv, ld, tvec,
                                                          static_cast<__nv_bfloat16*>(u));
     if (mark) cudaEventRecordWithFlags(ev[2], st, cudaEventRecordExternal);

@@ -355,21 +355,27 @@ __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + 
 // Per-column sums of per-thread fp64 partials inside one block, for kernels whose threads
 // own VEC consecutive columns of one row: thread t owns columns (t % G) VEC .. + VEC - 1
 // of block row t / G, with G = k / VEC threads per row and blockDim.x a multiple of G.
-// The block's column sums go to out[0..k) in a fixed order (deterministic).  Every
-// thread of the block must call it.
+// The block's column sums go to out[0..k), rows in order (the order is part of the CG's
+// results).  Every thread of the block must call it; k <= blockDim.x.
 template <int VEC>
 __device__ __forceinline__ void block_column_sums(const double (&acc)[VEC], int k, double* out) {
   __shared__ double s[256 * VEC];
 #pragma unroll
   for (int j = 0; j < VEC; ++j) s[threadIdx.x * VEC + j] = acc[j];
   __syncthreads();
-  const int G = k / VEC;
-  const int rows = blockDim.x / G;
-  for (int col = threadIdx.x; col < k; col += blockDim.x) {
-    const int chunk = col / VEC, lane = col % VEC;
+  const int rows = (int)blockDim.x / (k / VEC);
+  if ((int)threadIdx.x < k) {
     double t = 0.0;
-    for (int r = 0; r < rows; ++r) t += s[(r * G + chunk) * VEC + lane];
-    out[col] = t;
+    int r = 0;
+    for (; r + 8 <= rows; r += 8) {  // loads ahead of the additions
+      double x[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) x[q] = s[(r + q) * k + threadIdx.x];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) t += x[q];
+    }
+    for (; r < rows; ++r) t += s[r * k + threadIdx.x];
+    out[threadIdx.x] = t;
   }
 }
 
@@ -413,9 +419,17 @@ __device__ __forceinline__ dfloat df_from_double(double x) {
   const float hi = (float)x;
   return {hi, (float)(x - (double)hi)};
 }
-__device__ __forceinline__ double df_to_double(dfloat a) { return (double)a.hi + (double)a.lo; }
+// (double)x by integer operations (conversions share the narrow fp64 pipe).
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), e = (u >> 23) & 255u;
+  if (e - 1u >= 254u) return (u << 1) == 0 ? __hiloint2double((int)u, 0) : (double)x;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))),
+                          (int)(u << 29));
+}
+__device__ __forceinline__ double df_to_double(dfloat a) { return widen(a.hi) + widen(a.lo); }
 
-// Threads per block for the column-owning kernels: a whole number of rows of G threads.
+// Threads per block for the column-owning kernels: a whole number of rows of G threads (k <=
+// 256, so at least k of them).
 inline int column_block_threads(int k, int vec) {
   const int G = k / vec;
   return G * (256 / G);
