@@ -94,16 +94,29 @@ __global__ void __launch_bounds__(kThreads) k_splat_fix(int nhuge, int64_t nmed,
     if (q >= nmed || (int)threadIdx.x >= rows * G) return;
     const int col = (int)(threadIdx.x % G) * VEC;
     const int4 rw = med_rows[q];
-    typename Vt::T acc = Vt::zero();
-    for (int j = 0; j < rw.z; ++j) acc = Vt::add(acc, Vt::ld(partial + (int64_t)(rw.y + j) * k + col));
+    const float* base = partial + (int64_t)rw.y * k + col;
+    typename Vt::T x[kSplatMedSegs], acc = Vt::zero();
+#pragma unroll
+    for (int j = 0; j < kSplatMedSegs; ++j) x[j] = j < rw.z ? Vt::ldg(base + (int64_t)j * k) : Vt::zero();
+#pragma unroll
+    for (int j = 0; j < kSplatMedSegs; ++j)
+      if (j < rw.z) acc = Vt::add(acc, x[j]);
     Vt::sts(lat + (int64_t)rw.x * k + col, acc);
     return;
   }
   const int4 rw = huge_rows[blockIdx.x];
   for (int q = threadIdx.x; q < groups * G; q += blockDim.x) {
+    const float* base = partial + (int64_t)rw.y * k + (q % G) * VEC;
     typename Vt::T acc = Vt::zero();
-    for (int j = q / G; j < rw.z; j += groups)
-      acc = Vt::add(acc, Vt::ld(partial + (int64_t)(rw.y + j) * k + (q % G) * VEC));
+    int j = q / G;
+    for (; j + 15 * groups < rw.z; j += 16 * groups) {  // 16 loads in flight, summed in order
+      typename Vt::T x[16];
+#pragma unroll
+      for (int e = 0; e < 16; ++e) x[e] = Vt::ldg(base + (int64_t)(j + e * groups) * k);
+#pragma unroll
+      for (int e = 0; e < 16; ++e) acc = Vt::add(acc, x[e]);
+    }
+    for (; j < rw.z; j += groups) acc = Vt::add(acc, Vt::ldg(base + (int64_t)j * k));
     red[q] = acc;
   }
   __syncthreads();
