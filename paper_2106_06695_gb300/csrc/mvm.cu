@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(1024) k_blur_cluster(ClusterBlur q, S* __restr
 
 // ---- sparse blur (lattices whose direction lists are short) ------------------------------
 // A vertex without a neighbour along a pass's direction is only scaled by the centre tap g0.
-// With the values kept as y = x / g0^t after t passes such vertices do not change, a pass is
+// With fp32 values kept as y = x / g0^t after t passes such vertices do not change, a pass is
 // y[v] += (g1 / g0) (y[v - u_j] + y[v + u_j]) on the others, and the factor g0^passes is
 // applied once at the end (by the caller, through its alpha).
 //
@@ -403,12 +403,20 @@ __global__ void __launch_bounds__(1024) k_blur_cluster(ClusterBlur q, S* __restr
 // Bound by memory: per active vertex one row read and written and a 4-byte id, per chain 8
 // bytes.  n = 500k, d = 20, k = 8 (m = 10.5M, 1M active vertices a pass): 22 us a pass, 64.8
 // with per-vertex epochs, a buffer of new rows and a store kernel (k_sparse_blur, below).
+//
+// LAZY: the values as k_sparse_blur keeps them, the value of x before pass t being
+// pw[t - e(x)] stored[x], so that BF16 rows round exactly as there (rows kept as y round at
+// other places, 1.6e-3 apart in the product).  Threads of other warps of the group may read an
+// epoch after the pass has set it: the word holds the epoch and, above it, the one before.
 constexpr int kChainRows = 4;
-template <int VEC, class S>
-__global__ void __launch_bounds__(kThreads) k_chain_blur(int64_t chains, int G, int k, float tap,
+constexpr int kEpochMask = 0xffff;
+template <int VEC, class S, bool LAZY>
+__global__ void __launch_bounds__(kThreads) k_chain_blur(int64_t chains, int G, int k, float g0,
+                                                         float tap, int t,
                                                          const uint2* __restrict__ chain,
                                                          const int32_t* __restrict__ act,
-                                                         S* __restrict__ vals) {
+                                                         const float* __restrict__ pw,
+                                                         int32_t* epoch, S* __restrict__ vals) {
   pdl_enter();
   using Vt = Vec<VEC>;
   using T = typename Vt::T;
@@ -420,18 +428,46 @@ __global__ void __launch_bounds__(kThreads) k_chain_blur(int64_t chains, int G, 
   for (int64_t p0 = ch.x; p0 < (int64_t)ch.y; p0 += kChainRows) {
     S* at[kChainRows + 1];
     T row[kChainRows + 1];  // the last one only as a neighbour
+    int32_t* ep[kChainRows + 1];
+    int age[kChainRows + 1];  // LAZY: the epoch before this pass
+    float f[kChainRows + 1];  // and the row's factor
 #pragma unroll
     for (int e = 0; e <= kChainRows; ++e) {
-      at[e] = p0 + e < (int64_t)ch.y ? vals + (int64_t)__ldg(act + p0 + e) * k + col : nullptr;
+      const bool in = p0 + e < (int64_t)ch.y;
+      const int64_t v = in ? __ldg(act + p0 + e) : 0;
+      at[e] = in ? vals + v * k + col : nullptr;
+      ep[e] = epoch + v;
       row[e] = Vt::zero();
     }
 #pragma unroll
     for (int e = 0; e <= kChainRows; ++e)
-      if (at[e]) row[e] = Vt::lds(at[e]);
+      if (at[e]) {
+        row[e] = Vt::lds(at[e]);
+        if constexpr (LAZY) age[e] = *static_cast<volatile int32_t*>(ep[e]);
+      }
+    if constexpr (LAZY) {
+#pragma unroll
+      for (int e = 0; e <= kChainRows; ++e)
+        if (at[e]) {
+          const int now = age[e] & kEpochMask;
+          age[e] = now == t + 1 ? age[e] >> 16 : now;
+          f[e] = __ldg(pw + t - age[e]);
+        }
+    }
 #pragma unroll
     for (int e = 0; e < kChainRows; ++e) {
-      if (at[e]) Vt::sts(at[e], Vt::fma(tap, Vt::add(prev, row[e + 1]), row[e]));
-      prev = row[e];
+      if constexpr (LAZY) {
+        if (at[e]) {
+          const T own = Vt::scale(f[e], row[e]);
+          const T sum = at[e + 1] ? Vt::fma(f[e + 1], row[e + 1], prev) : prev;
+          Vt::sts(at[e], Vt::fma(tap, sum, Vt::scale(g0, own)));
+          if (col == 0) *static_cast<volatile int32_t*>(ep[e]) = (t + 1) | (age[e] << 16);
+          prev = own;
+        }
+      } else {
+        if (at[e]) Vt::sts(at[e], Vt::fma(tap, Vt::add(prev, row[e + 1]), row[e]));
+        prev = row[e];
+      }
     }
   }
 }
@@ -509,7 +545,7 @@ __global__ void __launch_bounds__(kThreads) k_sparse_finish(int64_t m, int G, in
   using Vt = Vec<VEC>;
   const int64_t v = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
   if (v >= m) return;
-  const int e = epoch[v];
+  const int e = epoch[v] & kEpochMask;  // chains keep the epoch before in the upper half
   if (e == P) return;
   const int col = (int)(threadIdx.x % G) * VEC;
   Vt::sts(stored + v * k + col, Vt::scale(pw[P - e], Vt::lds(stored + v * k + col)));
@@ -856,6 +892,18 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
     }
     return a;
   }
+  const float* pw = tp.t[0] == 1.f ? nullptr : L->g0pow;
+  // BF16 chains keep the lazy factors of the direction lists (none when the centre tap is 1)
+  const bool lazy = pw && (!chains_ok(L) || std::is_same_v<S, bf16>);
+  if (lazy) cudaMemsetAsync(L->epoch, 0, (size_t)L->m * sizeof(int32_t), st);
+  auto finish = [&] {
+    const RowShape q = row_shape(L->m, k);
+    by_vec(q.vec, [&](auto vec) {
+      launch_pdl(k_sparse_finish<decltype(vec)::value, S>, q.blocks, q.threads, st, L->m, q.G, k, P,
+                 L->epoch, pw, lat0);
+    });
+    note_launches(1);
+  };
   if (chains_ok(L)) {
     const double g0 = blur == SGP_BLUR_SYMMETRIC ? L->half[0] : L->coef[0];
     const double g1 = blur == SGP_BLUR_SYMMETRIC ? L->half[1] : L->coef[1];
@@ -868,7 +916,7 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
       for (int t = 0; t < P; ++t) {
         const int j = dir(t);
         const int64_t count = L->chain_off[j + 1] - L->chain_off[j];
-        if (g0 != 1.0 && P > 2 * kRescale && owed == kRescale) {
+        if (!lazy && g0 != 1.0 && P > 2 * kRescale && owed == kRescale) {
           const RowShape q = row_shape(L->m, k);
           launch_pdl(k_rescale<VEC, S>, q.blocks, q.threads, st, L->m, q.G, k,
                      (float)std::pow(g0, kRescale), lat0);
@@ -878,17 +926,20 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
         ++owed;
         if (count == 0) continue;
         const RowShape q = row_shape(count, k);
-        launch_pdl(k_chain_blur<VEC, S>, q.blocks, q.threads, st, count, q.G, k, (float)(g1 / g0),
-                   L->chain + L->chain_off[j], L->act, lat0);
+        const uint2* chain = L->chain + L->chain_off[j];
+        auto pass = [&](auto keep, float own, float tap) {
+          launch_pdl(k_chain_blur<VEC, S, decltype(keep)::value>, q.blocks, q.threads, st, count,
+                     q.G, k, own, tap, t, chain, L->act, pw, L->epoch, lat0);
+        };
+        if (lazy) pass(std::is_same<S, bf16>{}, tp.t[0], tp.t[1]);
+        else pass(std::false_type{}, 1.f, (float)(g1 / g0));
         note_launches(1);
       }
     });
-    *scale = std::pow(g0, owed);
+    if (lazy) finish();
+    else *scale = std::pow(g0, owed);
     return lat0;
   }
-  // sparse: lazy centre-tap factors (none when the centre tap is 1)
-  const float* pw = tp.t[0] == 1.f ? nullptr : L->g0pow;
-  if (pw) cudaMemsetAsync(L->epoch, 0, (size_t)L->m * sizeof(int32_t), st);
   S* tmp = static_cast<S*>(L->act_tmp);
   by_vec(row_shape(1, k).vec, [&](auto vec) {
     constexpr int VEC = decltype(vec)::value;
@@ -905,13 +956,8 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
                  L->epoch);
       note_launches(2);
     }
-    if (pw) {
-      const RowShape q = row_shape(L->m, k);
-      launch_pdl(k_sparse_finish<VEC, S>, q.blocks, q.threads, st, L->m, q.G, k, P, L->epoch, pw,
-                 lat0);
-      note_launches(1);
-    }
   });
+  if (pw) finish();
   return lat0;
 }
 
