@@ -1047,8 +1047,8 @@ void launch_bt(int kp, const Table* T, cudaStream_t st) {
     default: launch_pdl_smem(kb_bt<16>, kRingGrid, kST, sm, st, T); break;
   }
 }
-cudaError_t bt_smem_attributes(int kp) {
-  const int sm = (int)ring_smem_bytes(kp);
+cudaError_t bt_smem_attributes() {
+  const int sm = kRingBytes;  // ring_smem_bytes is largest at 28 columns, not at the most
   cudaError_t e = cudaFuncSetAttribute(kb_bt<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kb_bt<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
@@ -2168,7 +2168,7 @@ sgp_status sgp_server_create(const sgp_server_opts* opts, sgp_server** out) {
   }
   SRV_CHECK(cudaGetDevice(&S->device), "cudaGetDevice");
   // the attribute is per kernel, shared by every server: allow the largest kp
-  SRV_CHECK(bt_smem_attributes(kMaxServeK), "shared memory of the preconditioner kernels");
+  SRV_CHECK(bt_smem_attributes(), "shared memory of the preconditioner kernels");
   SRV_CHECK(apply_z_smem_attributes(kMaxServeK), "shared memory of the preconditioner kernels");
   SRV_CHECK(cudaStreamCreateWithFlags(&S->bs, cudaStreamNonBlocking), "stream");
   sgp_server* raw = S.get();
