@@ -54,20 +54,6 @@ enum CgEnd {
   CG_BETA_PRE,  // sum = <r, z>: beta (preconditioned)
 };
 
-// Whether ||r|| / ||b|| = sqrt(rr) / bnorm (fp64) is at most tol or not finite.  Decided in
-// fp32 unless the two are within 1e-4 of each other (or out of fp32's range): a square root
-// and a division in fp64 are some 60 dependent operations of a narrow pipe, 2 us.
-__device__ __forceinline__ bool cg_stops(double rr, double bnorm, float tol) {
-  const float r = (float)rr, b = (float)bnorm;
-  const float lim = tol * b * (tol * b);
-  if (r > 1e-30f && r < 1e30f && lim < 1e30f && lim > 1e-30f) {
-    if (r > lim * 1.0002f) return false;
-    if (r < lim * 0.9998f) return true;
-  }
-  const double rel = sqrt(rr) / bnorm;
-  return rel <= (double)tol || !isfinite(rel);
-}
-
 // What one thread holds of a column before its sum is known.
 struct CgColumn {
   double rho = 0.0, bnorm = 0.0;

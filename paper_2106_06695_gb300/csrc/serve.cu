@@ -14,8 +14,8 @@
 // the rank-l Nystrom factor of App. A.
 //
 // Batching: one CG iteration of every active request is a fixed sequence of kernels
-// (splat, two fix-ups, 2 Dmax blur passes, slice with <p, Ap>, alpha, x/r update; for
-// preconditioned requests B^T r, its two ordered sums, Minv B^T r and z = P^-1 r; then
+// (splat, its fix-ups, 2 Dmax blur passes, slice with <p, Ap>, alpha, x/r update; for
+// preconditioned requests B^T r, its ordered sums, Minv B^T r and z = P^-1 r; then
 // convergence check and beta, p update) with fixed grids.  Each kernel walks "virtual
 // blocks" over a device table of the active requests; a request's virtual blocks cover
 // its own rows in a partition fixed by its own sizes, so its results (and reduction
@@ -25,6 +25,13 @@
 // is such a batch with its own table, stream and CUDA graph of one iteration (captured
 // once per Dmax, sparse blur and preconditioning, then replayed), rewritten
 // (stream-ordered) when requests join or leave, and the lanes run concurrently.
+//
+// An iteration of a small request is a chain of latencies, not of bytes: the kernels read the
+// table (and ids and weights where they can) ahead of the wait for the kernel before, and
+// issue the loads of several rows or items together.  40,000 points, d = 8, 12 columns, rank
+// 100: 142 us an iteration of 30 kernels (blur 18 x 4.4, z 16, B^T r 13, slice 12.5, x/r 11.6,
+// splat 9.9, the others 4.4 to 5.8 each when run apart); 196 with table searches, single loads
+// in flight and 32 kernels.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -64,8 +71,7 @@ constexpr int kSpinLimit = 1 << 20; // bounded mbarrier waits (about a second at
 constexpr double kBf16MaxKappa = 100.0;  // BF16 server: larger condition estimates use fp32
 constexpr uint64_t kPrecondSeedXor = 0x6A09E667F3BCC909ull;  // sketch seed = seed ^ this
 
-enum { U_SPLAT = 0, U_MED, U_HUGE, U_BLUR, U_VEC, U_VERT, U_BT, U_BTS, U_BTT, U_MINV, U_Z,
-       U_KINDS };
+enum { U_SPLAT = 0, U_FIX, U_BLUR, U_VEC, U_VERT, U_BT, U_BTT, U_MINV, U_Z, U_KINDS };
 
 // One active request as the kernels see it.  Row-indexed arrays are in the lattice's
 // locality order p; perm[p] < n_train marks a training row.
@@ -88,7 +94,8 @@ struct SlotDev {
   float* spart;  // splat partials
   float *xh, *xl, *rh, *rl, *p, *ap;  // [n][kp]
   double* dpart;                      // [virtual blocks][kp]
-  double *rho, *bnorm, *relres, *alpha, *beta;  // [kp]
+  double *rho, *bnorm, *rr;           // [kp]; rr = <r, r> of the last check
+  dfloat *alpha, *beta;               // [kp] as the updates use them
   int* active;                        // [kp]
   int* state;                         // [0] request still iterating, [1] iterations done
   int max_iter;
@@ -107,7 +114,6 @@ struct SlotDev {
   const float* Bh;      // [n][ld] fp32, locality order, zero at test rows
   const double* Minv;   // [l][l] (noise I + B^T B)^-1
   float* btpart;        // [U_BT virtual blocks][ld][kp] fp32 partials of B^T r
-  float* bt2;           // [segments][ld][kp] sums of kBtSeg partials
   double* tvec;         // [ld][kp] B^T r
   float* u;             // [ld][kp] Minv B^T r (rows >= l zero)
   double* dpart2;       // [U_Z virtual blocks][kp] partials of <r, z>
@@ -119,32 +125,58 @@ struct Table {
   int* flags;  // [kMaxSlots][2]: state copied by the check kernel, read by the host
   int* err;    // set to 1 when a bulk-copy wait gave up (the round's results are void)
   int wait_limit;  // try_wait polls of the ring's chunk waits (kSpinLimit; 0 under SGP_FAULT)
-  int64_t pre[U_KINDS][kMaxSlots + 1];  // prefix sums of virtual blocks per unit kind
+  // prefix sums of virtual blocks per unit kind, the total repeated after the last request
+  int64_t pre[U_KINDS][kMaxSlots + 1];
   SlotDev s[kMaxSlots];
 };
 
 __host__ __device__ inline int groups_of(int kp) { return kST / (kp / 4); }
+// Column tiles of kb_apply_z: its virtual blocks are (rows, tile) pairs.
+__host__ __device__ inline int z_tiles(int kp) { return (kp + 7) / 8; }
 
-__device__ __forceinline__ int find_slot(const int64_t* pre, int ns, int64_t vb) {
-  int lo = 0, hi = ns - 1;  // largest q with pre[q] <= vb
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (pre[mid] <= vb) lo = mid;
-    else hi = mid - 1;
+// This thread's share of a unit kind's prefix sums: lane i holds entries i and i + 32 (the
+// entries past the last request repeat the total), so the request of a virtual block is one
+// ballot away instead of a chain of table reads (a binary search takes an L2 round trip of
+// some 0.3 us a step, in every kernel of the iteration).
+struct SlotWalk {
+  int64_t total, lo, hi;
+  __device__ __forceinline__ explicit SlotWalk(const int64_t* pre)
+      : total(pre[kMaxSlots]), lo(pre[threadIdx.x & 31]), hi(pre[(threadIdx.x & 31) + 32]) {}
+  // Largest q with pre[q] <= vb < total, and vb's index inside it.  Uniform over the warp.
+  __device__ __forceinline__ int find(int64_t vb, int64_t* local) const {
+    const int q = __popc(__ballot_sync(0xffffffffu, lo <= vb)) +
+                  __popc(__ballot_sync(0xffffffffu, hi <= vb)) - 1;
+    *local = vb - __shfl_sync(0xffffffffu, q < 32 ? lo : hi, q & 31);
+    return q;
   }
-  return lo;
-}
+};
 
 // Walk this block's virtual blocks of one unit kind: q = request, local = its block index.
-#define SLOT_LOOP(KIND)                                                            \
-  const int ns_ = T->nslots;                                                       \
-  const int64_t total_ = T->pre[KIND][ns_];                                        \
-  for (int64_t vb_ = blockIdx.x; vb_ < total_; vb_ += gridDim.x) {                 \
-    const int q = find_slot(T->pre[KIND], ns_, vb_);                               \
-    const SlotDev& s = T->s[q];                                                    \
-    const int64_t local = vb_ - T->pre[KIND][q];
+// The table is constant while a lane's graph runs, so it is read ahead of the wait for the
+// kernel before (SLOT_AHEAD, then pdl_enter()).  A kernel that reads more ahead (ids,
+// weights, the state word) calls pdl_enter() inside the loop, where a second call costs
+// nothing; every block calls it at least once, also one without work.
+#define SLOT_AHEAD(KIND) const SlotWalk walk_(T->pre[KIND])
+#define SLOT_AHEAD_IN_LOOP(KIND)          \
+  SLOT_AHEAD(KIND);                       \
+  if (blockIdx.x >= walk_.total) {        \
+    pdl_enter();                          \
+    return;                               \
+  }
+
+#define SLOT_LOOP                                                                  \
+  for (int64_t vb_ = blockIdx.x; vb_ < walk_.total; vb_ += gridDim.x) {            \
+    int64_t local;                                                                 \
+    const int q = walk_.find(vb_, &local);                                         \
+    const SlotDev& s = T->s[q];
 
 #define SLOT_LOOP_END }
+// The block's last virtual block: once its loads are issued the next kernel may come in.
+#define SLOT_LAST (vb_ + (int64_t)gridDim.x >= walk_.total)
+
+// Whether the request still iterates.  Written by kb_check_beta, so every kernel but the
+// one right after it may ask before its pdl_enter(); from L2, where that write went.
+__device__ __forceinline__ bool slot_on(const SlotDev& s) { return __ldcg(s.state) != 0; }
 
 // SplitMix64 (Steele, Lea & Flood 2014) sign at counter i l + j + 1.
 __device__ __forceinline__ float rademacher_pm(uint64_t seed, int64_t i, int j, int l) {
@@ -166,7 +198,15 @@ __device__ __forceinline__ void vb_column_sums(const dfloat (&d)[4], int kp, dou
   for (int col = threadIdx.x; col < kp; col += blockDim.x) {
     const int chunk = col / 4, lane = col % 4;
     double t = 0.0;
-    for (int r = 0; r < rows; ++r) t += sh[(r * G + chunk) * 4 + lane];
+    int r = 0;
+    for (; r + 8 <= rows; r += 8) {  // loads ahead of the additions
+      double x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = sh[((r + u) * G + chunk) * 4 + lane];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) t += x[u];
+    }
+    for (; r < rows; ++r) t += sh[(r * G + chunk) * 4 + lane];
     out[col] = t;
   }
   __syncthreads();
@@ -175,20 +215,47 @@ __device__ __forceinline__ void vb_column_sums(const dfloat (&d)[4], int kp, dou
 // Totals of all kp columns over a request's nvb virtual-block partials part[b][c], in one
 // coalesced pass: thread t < R kp (R = kST / kp) owns column t % kp and the blocks
 // t / kp, t / kp + R, ... (summed in order), then thread c < kp adds the R sums of its
-// column in order.  out (shared, kp entries); uniform call, trailing barrier.
-__device__ __forceinline__ void slot_cols_total(const double* part, int64_t nvb, int kp,
-                                                double* red, double* out) {
-  const int R = kST / kp;
-  const int t = threadIdx.x;
+// column in order; in the same passes a second set (part2 null: none), whose columns the
+// threads from kST / 2 on add up.  A dependent fp64 addition takes some 0.1 us here, so the
+// two sets' chains run side by side.  out (shared, kp <= kMaxServeK entries); uniform call,
+// trailing barrier.
+__device__ __forceinline__ double slot_col_partial(const double* part, int64_t nvb, int kp) {
+  const int R = kST / kp, t = threadIdx.x;
   double acc = 0.0;
-  if (t < R * kp)
-    for (int64_t b = t / kp; b < nvb; b += R) acc += part[b * kp + t % kp];
-  red[t] = acc;
+  if (t < R * kp) {
+    const double* col = part + t % kp;
+    int64_t b = t / kp;
+    for (; b + 7 * R < nvb; b += 8 * R) {  // loads ahead of the additions
+      double x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = col[(b + u * R) * kp];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc += x[u];
+    }
+    double x[7];
+#pragma unroll
+    for (int u = 0; u < 7; ++u) x[u] = b + u * R < nvb ? col[(b + u * R) * kp] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 7; ++u)
+      if (b + u * R < nvb) acc += x[u];
+  }
+  return acc;
+}
+__device__ __forceinline__ void slot_cols_total(const double* part, int64_t nvb, int kp,
+                                                double* red, double* out,
+                                                const double* part2 = nullptr, int64_t nvb2 = 0,
+                                                double* red2 = nullptr, double* out2 = nullptr) {
+  const int R = kST / kp, t = threadIdx.x;
+  red[t] = slot_col_partial(part, nvb, kp);
+  if (part2) red2[t] = slot_col_partial(part2, nvb2, kp);
   __syncthreads();
-  if (t < kp) {
+  const bool second = t >= kST / 2;
+  const int c = second ? t - kST / 2 : t;
+  if (c < kp && (!second || part2)) {
+    const double* src = second ? red2 : red;
     double v = 0.0;
-    for (int r = 0; r < R; ++r) v += red[r * kp + t];
-    out[t] = v;
+    for (int r = 0; r < R; ++r) v += src[r * kp + c];
+    (second ? out2 : out)[c] = v;
   }
   __syncthreads();
 }
@@ -200,21 +267,40 @@ __device__ __forceinline__ float4 f4_ld(const float* p) { return *reinterpret_ca
 __device__ __forceinline__ void f4_st(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 
 // ---- one CG iteration over the table --------------------------------------------------
-// Splat W^T p into lat0: one thread-group per segment of a vertex's incidence list.
+// Splat W^T p into lat0: one thread-group per segment of a vertex's incidence list, the
+// rows of 8 items in flight and the next 8 items behind them.
 template <class S>
 __global__ void __launch_bounds__(kST) kb_splat(const Table* __restrict__ T) {
+  SLOT_AHEAD(U_SPLAT);
   pdl_enter();
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
-  SLOT_LOOP(U_SPLAT)
-  if (*s.state == 0 || g >= groups) continue;
+  SLOT_LOOP
+  if (!slot_on(s) || g >= groups) continue;
   const int64_t sidx = local * groups + g;
   if (sidx >= s.nseg) continue;
   const int4 sg = s.seg[sidx];
+  const float* p = s.p + col;
+  const int2* items = s.items;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int it = sg.y; it < sg.z; ++it) {
-    const int2 e = s.items[it];
-    acc = f4_fma(__int_as_float(e.y), f4_ld(s.p + (int64_t)e.x * kp + col), acc);
+  int2 e[8];  // past the segment's end the last item is repeated and left out
+  auto load = [&](int it) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) e[u] = items[it + u < sg.z ? it + u : sg.z - 1];
+  };
+  if (sg.y < sg.z) load(sg.y);
+  for (int it = sg.y; it < sg.z; it += 8) {
+    float w[8];
+    float4 x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      w[u] = __int_as_float(e[u].y);
+      x[u] = f4_ld(p + (int64_t)e[u].x * kp);
+    }
+    if (it + 8 < sg.z) load(it + 8);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (it + u < sg.z) acc = f4_fma(w[u], x[u], acc);
   }
   if (sg.w < 0) {
     Store<S>::st4(static_cast<S*>(s.lat0) + (int64_t)sg.x * kp + col, acc);
@@ -225,58 +311,56 @@ __global__ void __launch_bounds__(kST) kb_splat(const Table* __restrict__ T) {
   SLOT_LOOP_END
 }
 
-// Vertices with 2..kSplatMedSegs segments: one thread-group sums the partials in order.
+// Vertices with several segments.  Virtual blocks below nhuge: one vertex of more than
+// kSplatMedSegs segments each, strided partials per group and a fixed shared-memory tree over
+// the groups.  The others: one vertex per thread-group, its partials summed in order.
 template <class S>
-__global__ void __launch_bounds__(kST) kb_splat_med(const Table* __restrict__ T) {
-  pdl_enter();
-  const int kp = T->kp, G = kp / 4, groups = kST / G;
-  const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
-  SLOT_LOOP(U_MED)
-  if (*s.state == 0 || g >= groups) continue;
-  const int64_t ridx = local * groups + g;
-  if (ridx >= s.nmed) continue;
-  const int4 rw = s.med[ridx];
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int j = 0; j < rw.z; ++j) {
-    const float4 v = f4_ld(s.spart + (int64_t)(rw.y + j) * kp + col);
-    acc = make_float4(acc.x + v.x, acc.y + v.y, acc.z + v.z, acc.w + v.w);
-  }
-  Store<S>::st4(static_cast<S*>(s.lat0) + (int64_t)rw.x * kp + col, acc);
-  if (s.sparse && col == 0) s.epoch[rw.x] = 0;
-  SLOT_LOOP_END
-}
-
-// Vertices with more segments: one virtual block per vertex, strided partials per group
-// and a fixed shared-memory tree over the groups.
-template <class S>
-__global__ void __launch_bounds__(kST) kb_splat_huge(const Table* __restrict__ T) {
-  pdl_enter();
+__global__ void __launch_bounds__(kST) kb_splat_fix(const Table* __restrict__ T) {
+  SLOT_AHEAD_IN_LOOP(U_FIX);
   __shared__ float4 red[kST];
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
   int pow2 = 1;
   while (pow2 * 2 <= groups) pow2 *= 2;
-  SLOT_LOOP(U_HUGE)
-  if (*s.state == 0) continue;  // uniform over the block
-  const int4 rw = s.huge[local];
+  SLOT_LOOP
+  const bool on = slot_on(s), whole = local < s.nhuge;  // uniform over the block
+  const int64_t q1 = (local - s.nhuge) * groups + g;
+  int4 rw = make_int4(0, 0, 0, 0);
+  if (on && whole) rw = s.huge[local];
+  else if (on && g < groups && q1 < s.nmed) rw = s.med[q1];
+  pdl_enter();
+  if (!on) continue;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (g < pow2)
-    for (int j = g; j < rw.z; j += pow2) {
-      const float4 v = f4_ld(s.spart + (int64_t)(rw.y + j) * kp + col);
-      acc = make_float4(acc.x + v.x, acc.y + v.y, acc.z + v.z, acc.w + v.w);
+  const float* part = s.spart + (int64_t)rw.y * kp + col;
+  const int j0 = whole ? g : 0, step = whole ? pow2 : 1;
+  if (!whole || g < pow2)
+    for (int j = j0; j < rw.z; j += 8 * step) {
+      float4 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        v[u] = f4_ld(part + (int64_t)(j + u * step < rw.z ? j + u * step : j) * kp);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (j + u * step < rw.z)
+          acc = make_float4(acc.x + v[u].x, acc.y + v[u].y, acc.z + v[u].z, acc.w + v[u].w);
     }
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int half = pow2 / 2; half >= 1; half /= 2) {
-    if (g < half) {
-      const float4 a = red[threadIdx.x], b = red[threadIdx.x + half * G];
-      red[threadIdx.x] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+  if (whole) {
+    red[threadIdx.x] = acc;
+    __syncthreads();
+    for (int half = pow2 / 2; half >= 1; half /= 2) {
+      if (g < half) {
+        const float4 a = red[threadIdx.x], b = red[threadIdx.x + half * G];
+        red[threadIdx.x] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+      }
+      __syncthreads();
     }
+    acc = red[threadIdx.x];
     __syncthreads();
   }
-  if (g == 0) Store<S>::st4(static_cast<S*>(s.lat0) + (int64_t)rw.x * kp + col, red[threadIdx.x]);
-  if (s.sparse && threadIdx.x == 0) s.epoch[rw.x] = 0;
-  __syncthreads();
+  if (rw.z > 0 && (!whole || g == 0)) {
+    Store<S>::st4(static_cast<S*>(s.lat0) + (int64_t)rw.x * kp + col, acc);
+    if (s.sparse && col == 0) s.epoch[rw.x] = 0;
+  }
   SLOT_LOOP_END
 }
 
@@ -285,16 +369,21 @@ __global__ void __launch_bounds__(kST) kb_splat_huge(const Table* __restrict__ T
 // in lat0.  Each thread owns 4 columns of kBlurU rows (ids first, then rows).
 template <int R, class S>
 __global__ void __launch_bounds__(kST) kb_blur(const Table* __restrict__ T, int t) {
-  pdl_enter();
+  SLOT_AHEAD_IN_LOOP(U_BLUR);
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
-  SLOT_LOOP(U_BLUR)
-  if (*s.state == 0 || t >= 2 * s.D || g >= groups) continue;
+  SLOT_LOOP
+  const bool on = slot_on(s);
+  if (!on || t >= 2 * s.D || g >= groups) {
+    pdl_enter();
+    continue;
+  }
   const int j = t < s.D ? t : 2 * s.D - 1 - t;
   if (s.sparse) {  // the vertices of list j: new rows into stmp, lazy factors on reads
     const int64_t base = s.act_off[j], count = s.act_off[j + 1] - base;
     const S* lat = static_cast<const S*>(s.lat0);
     const int32_t* nbr = s.nbr + (int64_t)j * R * 2 * s.m;
+    pdl_enter();
     for (int u = 0; u < kBlurU; ++u) {
       const int64_t e = (local * kBlurU + u) * groups + g;
       if (e >= count) break;
@@ -341,6 +430,7 @@ __global__ void __launch_bounds__(kST) kb_blur(const Table* __restrict__ T, int 
       ic[u][tt] = v[u] < m ? __ldg(nbr + (int64_t)(2 * tt + 1) * m + v[u]) : -1;
     }
   }
+  pdl_enter();
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
   float4 own[kBlurU], sa[kBlurU][R], sc[kBlurU][R];
 #pragma unroll
@@ -352,6 +442,7 @@ __global__ void __launch_bounds__(kST) kb_blur(const Table* __restrict__ T, int 
       sc[u][tt] = ic[u][tt] >= 0 ? Store<S>::ldg4(in + (int64_t)ic[u][tt] * kp + col) : zero;
     }
   }
+  if (SLOT_LAST) pdl_leave();
 #pragma unroll
   for (int u = 0; u < kBlurU; ++u) {
     if (v[u] >= m) continue;
@@ -373,11 +464,12 @@ __global__ void __launch_bounds__(kST) kb_blur(const Table* __restrict__ T, int 
 // Sparse requests, after kb_blur pass t: list rows back into lat0, epoch t + 1.
 template <class S>
 __global__ void __launch_bounds__(kST) kb_sparse_store(const Table* __restrict__ T, int t) {
+  SLOT_AHEAD(U_BLUR);
   pdl_enter();
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
-  SLOT_LOOP(U_BLUR)
-  if (!s.sparse || *s.state == 0 || t >= 2 * s.D || g >= groups) continue;
+  SLOT_LOOP
+  if (!s.sparse || !slot_on(s) || t >= 2 * s.D || g >= groups) continue;
   const int j = t < s.D ? t : 2 * s.D - 1 - t;
   const int64_t base = s.act_off[j], count = s.act_off[j + 1] - base;
   for (int u = 0; u < kBlurU; ++u) {
@@ -394,11 +486,12 @@ __global__ void __launch_bounds__(kST) kb_sparse_store(const Table* __restrict__
 // Sparse requests, after their 2D passes: the remaining centre-tap factors.
 template <class S>
 __global__ void __launch_bounds__(kST) kb_sparse_finish(const Table* __restrict__ T) {
+  SLOT_AHEAD(U_VERT);
   pdl_enter();
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
-  SLOT_LOOP(U_VERT)
-  if (!s.sparse || *s.state == 0 || g >= groups) continue;
+  SLOT_LOOP
+  if (!s.sparse || !slot_on(s) || g >= groups) continue;
   const int P = 2 * s.D;
   for (int u = 0; u < kBlurU; ++u) {
     const int64_t v = (local * kBlurU + u) * groups + g;
@@ -414,115 +507,191 @@ __global__ void __launch_bounds__(kST) kb_sparse_finish(const Table* __restrict_
 }
 
 // A p = outputscale W lat0 + noise p on training rows, 0 on test rows; partials of <p, Ap>.
+// Bound by the latency of its gathers (a 40k-point request has fewer blocks than the chip
+// SMs): the thread's kVecRows rows go together, kSliceC entries of each in flight, ids and
+// weights of the first ones read ahead of the blur's end.
+constexpr int kSliceC = 3;
 template <class S>
-__global__ void __launch_bounds__(kST) kb_slice_dot(const Table* __restrict__ T) {
-  pdl_enter();
+__global__ void __launch_bounds__(kST, 2) kb_slice_dot(const Table* __restrict__ T) {
+  SLOT_AHEAD_IN_LOOP(U_VEC);
   __shared__ double sh[kST * 4];
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
-  SLOT_LOOP(U_VEC)
-  if (*s.state == 0) continue;  // uniform over the block
+  SLOT_LOOP
+  if (!slot_on(s)) {  // uniform over the block
+    pdl_enter();
+    continue;
+  }
   dfloat d[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-  const S* lat = static_cast<const S*>(s.lat0);
+  const S* lat = static_cast<const S*>(s.lat0) + col;
+  const int D = s.D;
+  const int32_t* idx = s.idx;
+  const float* w = s.w;
   if (g < groups) {
+    // rows past the end repeat the last row; their results are left out
+    int64_t row[kVecRows];
+    bool in[kVecRows], train[kVecRows];
+    float4 acc[kVecRows];
+#pragma unroll
     for (int i = 0; i < kVecRows; ++i) {
-      const int64_t row = (local * kVecRows + i) * groups + g;
-      if (row >= s.n) break;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int c = 0; c < s.D; ++c) {
-        const int64_t e = row * s.D + c;
-        acc = f4_fma(s.w[e], Store<S>::ld4(lat + (int64_t)s.idx[e] * kp + col), acc);
-      }
-      const float4 pv = f4_ld(s.p + row * kp + col);
+      const int64_t r = (local * kVecRows + i) * groups + g;
+      in[i] = r < s.n;
+      row[i] = in[i] ? r : s.n - 1;
+      train[i] = s.perm[row[i]] < s.n_train;
+      acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    int id[kVecRows][kSliceC];
+    float wt[kVecRows][kSliceC];
+    auto ids = [&](int c0) {
+#pragma unroll
+      for (int i = 0; i < kVecRows; ++i)
+#pragma unroll
+        for (int u = 0; u < kSliceC; ++u) {
+          const int64_t e = row[i] * D + (c0 + u < D ? c0 + u : D - 1);
+          id[i][u] = idx[e];
+          wt[i][u] = w[e];
+        }
+    };
+    ids(0);
+    pdl_enter();
+    for (int c0 = 0; c0 < D; c0 += kSliceC) {
+      float4 x[kVecRows][kSliceC];
+      float wc[kVecRows][kSliceC];
+#pragma unroll
+      for (int i = 0; i < kVecRows; ++i)
+#pragma unroll
+        for (int u = 0; u < kSliceC; ++u) {
+          x[i][u] = Store<S>::ld4(lat + (int64_t)id[i][u] * kp);
+          wc[i][u] = wt[i][u];
+        }
+      if (c0 + kSliceC < D) ids(c0 + kSliceC);
+#pragma unroll
+      for (int u = 0; u < kSliceC; ++u)
+        if (c0 + u < D)
+#pragma unroll
+          for (int i = 0; i < kVecRows; ++i) acc[i] = f4_fma(wc[i][u], x[i][u], acc[i]);
+    }
+    float4 pv[kVecRows];
+#pragma unroll
+    for (int i = 0; i < kVecRows; ++i) pv[i] = f4_ld(s.p + row[i] * kp + col);
+    const float a = s.outputscale, b = s.noise;
+    float* ap = s.ap + col;
+#pragma unroll
+    for (int i = 0; i < kVecRows; ++i) {
+      if (!in[i]) continue;
       float4 res = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (s.perm[row] < s.n_train) {
-        const float a = s.outputscale, b = s.noise;
-        res = make_float4(fmaf(b, pv.x, a * acc.x), fmaf(b, pv.y, a * acc.y),
-                          fmaf(b, pv.z, a * acc.z), fmaf(b, pv.w, a * acc.w));
-      }
-      f4_st(s.ap + row * kp + col, res);
-      d[0] = df_add(d[0], df_two_prod(pv.x, res.x));
-      d[1] = df_add(d[1], df_two_prod(pv.y, res.y));
-      d[2] = df_add(d[2], df_two_prod(pv.z, res.z));
-      d[3] = df_add(d[3], df_two_prod(pv.w, res.w));
+      if (train[i])
+        res = make_float4(fmaf(b, pv[i].x, a * acc[i].x), fmaf(b, pv[i].y, a * acc[i].y),
+                          fmaf(b, pv[i].z, a * acc[i].z), fmaf(b, pv[i].w, a * acc[i].w));
+      f4_st(ap + row[i] * kp, res);
+      d[0] = df_add(d[0], df_two_prod(pv[i].x, res.x));
+      d[1] = df_add(d[1], df_two_prod(pv[i].y, res.y));
+      d[2] = df_add(d[2], df_two_prod(pv[i].z, res.z));
+      d[3] = df_add(d[3], df_two_prod(pv[i].w, res.w));
     }
   }
+  pdl_enter();
   vb_column_sums(d, kp, s.dpart + local * kp, sh);
   SLOT_LOOP_END
 }
 
 // alpha = rho / <p, A p> per active column (a non-positive <p, A p> stops the column).
 __global__ void __launch_bounds__(kST) kb_alpha(const Table* __restrict__ T) {
-  pdl_enter();
   __shared__ double red[kST], tot[kMaxServeK];
   const int q = blockIdx.x;
-  if (q >= T->nslots) return;
+  if (q >= T->nslots) {
+    pdl_enter();
+    return;
+  }
   const SlotDev& s = T->s[q];
-  if (*s.state == 0) return;
+  const bool on = slot_on(s);
   const int kp = T->kp;
   const int64_t nvb = T->pre[U_VEC][q + 1] - T->pre[U_VEC][q];
-  slot_cols_total(s.dpart, nvb, kp, red, tot);
   const int c = threadIdx.x;
+  const int act = c < kp ? __ldcg(s.active + c) : 0;
+  const double rho = c < kp ? __ldcg(s.rho + c) : 0.0;
+  const double* part = s.dpart;
+  pdl_enter();
+  if (!on) return;
+  slot_cols_total(part, nvb, kp, red, tot);
   if (c < kp) {
     const double pap = tot[c];
     double a = 0.0;
-    if (s.active[c]) {
-      if (pap > 0.0 && isfinite(pap)) a = s.rho[c] / pap;
+    if (act) {
+      if (pap > 0.0 && isfinite(pap)) a = rho / pap;
       else s.active[c] = 0;
     }
-    s.alpha[c] = a;
+    s.alpha[c] = df_from_double(a);
   }
 }
 
-// x += alpha p, r -= alpha A p on active columns (double-float); partials of <r, r>.
-__device__ __forceinline__ void xr_row(const SlotDev& s, int64_t e, const bool (&on)[4],
-                                       const dfloat (&a)[4], const dfloat (&na)[4], dfloat (&d)[4]) {
-  const float4 p4 = f4_ld(s.p + e), q4 = f4_ld(s.ap + e);
-  float4 xh = f4_ld(s.xh + e), xl = f4_ld(s.xl + e), rh = f4_ld(s.rh + e), rl = f4_ld(s.rl + e);
-  float* pv = reinterpret_cast<float*>(const_cast<float4*>(&p4));
-  float* qv = reinterpret_cast<float*>(const_cast<float4*>(&q4));
-  float* xhv = reinterpret_cast<float*>(&xh);
-  float* xlv = reinterpret_cast<float*>(&xl);
-  float* rhv = reinterpret_cast<float*>(&rh);
-  float* rlv = reinterpret_cast<float*>(&rl);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (on[j]) {
-      const dfloat x = df_add({xhv[j], xlv[j]}, df_mul_f(a[j], pv[j]));
-      const dfloat r = df_add({rhv[j], rlv[j]}, df_mul_f(na[j], qv[j]));
-      xhv[j] = x.hi, xlv[j] = x.lo, rhv[j] = r.hi, rlv[j] = r.lo;
-    }
-    dfloat sq = df_two_prod(rhv[j], rhv[j]);
-    sq = df_fast_two_sum(sq.hi, __fmaf_rn(2.f * rhv[j], rlv[j], sq.lo));
-    d[j] = df_add(d[j], sq);
+// x += alpha p, r -= alpha A p on active columns (double-float); partials of <r, r>.  The
+// six vectors of the next row are loaded while this row is updated (the stores would hold
+// the loads back otherwise: a round trip to memory a row).
+struct XrRow {
+  float4 p, q, xh, xl, rh, rl;
+  __device__ __forceinline__ void load(const SlotDev& s, int64_t e) {
+    p = f4_ld(s.p + e), q = f4_ld(s.ap + e);
+    xh = f4_ld(s.xh + e), xl = f4_ld(s.xl + e), rh = f4_ld(s.rh + e), rl = f4_ld(s.rl + e);
   }
-  f4_st(s.xh + e, xh);
-  f4_st(s.xl + e, xl);
-  f4_st(s.rh + e, rh);
-  f4_st(s.rl + e, rl);
-}
+  __device__ __forceinline__ void update(const bool (&on)[4], const dfloat (&a)[4],
+                                         const dfloat (&na)[4], dfloat (&d)[4]) {
+    const float pv[4] = {p.x, p.y, p.z, p.w}, qv[4] = {q.x, q.y, q.z, q.w};
+    float xhv[4] = {xh.x, xh.y, xh.z, xh.w}, xlv[4] = {xl.x, xl.y, xl.z, xl.w};
+    float rhv[4] = {rh.x, rh.y, rh.z, rh.w}, rlv[4] = {rl.x, rl.y, rl.z, rl.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (on[j]) {
+        const dfloat x = df_add({xhv[j], xlv[j]}, df_mul_f(a[j], pv[j]));
+        const dfloat r = df_add({rhv[j], rlv[j]}, df_mul_f(na[j], qv[j]));
+        xhv[j] = x.hi, xlv[j] = x.lo, rhv[j] = r.hi, rlv[j] = r.lo;
+      }
+      dfloat sq = df_two_prod(rhv[j], rhv[j]);
+      sq = df_fast_two_sum(sq.hi, __fmaf_rn(2.f * rhv[j], rlv[j], sq.lo));
+      d[j] = df_add(d[j], sq);
+    }
+    xh = make_float4(xhv[0], xhv[1], xhv[2], xhv[3]), xl = make_float4(xlv[0], xlv[1], xlv[2], xlv[3]);
+    rh = make_float4(rhv[0], rhv[1], rhv[2], rhv[3]), rl = make_float4(rlv[0], rlv[1], rlv[2], rlv[3]);
+  }
+  __device__ __forceinline__ void store(const SlotDev& s, int64_t e) const {
+    f4_st(s.xh + e, xh);
+    f4_st(s.xl + e, xl);
+    f4_st(s.rh + e, rh);
+    f4_st(s.rl + e, rl);
+  }
+};
 
 __global__ void __launch_bounds__(kST) kb_update_xr(const Table* __restrict__ T) {
-  pdl_enter();
+  SLOT_AHEAD_IN_LOOP(U_VEC);
   __shared__ double sh[kST * 4];
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
-  SLOT_LOOP(U_VEC)
-  if (*s.state == 0) continue;
+  SLOT_LOOP
+  const bool run = slot_on(s);
+  pdl_enter();
+  if (!run) continue;
   bool on[4];
   dfloat a[4], na[4];
   dfloat d[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    on[j] = s.active[col + j] != 0;
-    a[j] = df_from_double(s.alpha[col + j]);
-    na[j] = {-a[j].hi, -a[j].lo};
-  }
   if (g < groups) {
+    const int64_t first = local * kVecRows * groups + g;
+    const int64_t n = s.n;
+    XrRow cur, next;
+    if (first < n) cur.load(s, first * kp + col);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      on[j] = s.active[col + j] != 0;
+      a[j] = s.alpha[col + j];
+      na[j] = {-a[j].hi, -a[j].lo};
+    }
+#pragma unroll
     for (int i = 0; i < kVecRows; ++i) {
-      const int64_t row = (local * kVecRows + i) * groups + g;
-      if (row >= s.n) break;
-      xr_row(s, row * kp + col, on, a, na, d);
+      const int64_t row = first + (int64_t)i * groups;
+      if (row >= n) break;
+      if (i + 1 < kVecRows && row + groups < n) next.load(s, (row + groups) * kp + col);
+      cur.update(on, a, na, d);
+      cur.store(s, row * kp + col);
+      cur = next;
     }
   }
   vb_column_sums(d, kp, s.dpart + local * kp, sh);
@@ -532,35 +701,38 @@ __global__ void __launch_bounds__(kST) kb_update_xr(const Table* __restrict__ T)
 // Convergence check and beta = <r, r>_new / <r, r>_old per active column; the request
 // stops when no column is active.  Its state is copied to the host-read flags.
 __global__ void __launch_bounds__(kST) kb_check_beta(const Table* __restrict__ T) {
-  pdl_enter();
-  __shared__ double red[kST], trr[kMaxServeK], trz[kMaxServeK];
+  __shared__ double red[kST], red2[kST], trr[kMaxServeK], trz[kMaxServeK];
   const int q = blockIdx.x;
-  if (q >= T->nslots) return;
+  if (q >= T->nslots) {
+    pdl_enter();
+    return;
+  }
   const SlotDev& s = T->s[q];
-  if (*s.state == 0) {
+  const int c = threadIdx.x, kp = T->kp;
+  const bool on = slot_on(s);
+  const int act = c < kp ? __ldcg(s.active + c) : 0;
+  const double rho = c < kp ? __ldcg(s.rho + c) : 0.0, bnorm = c < kp ? s.bnorm[c] : 0.0;
+  const int it = __ldcg(s.state + 1) + 1;
+  pdl_enter();
+  if (!on) {
     if (threadIdx.x == 0) {
       T->flags[2 * q] = 0;
       T->flags[2 * q + 1] = s.state[1];
     }
     return;
   }
-  const int kp = T->kp;
   const int64_t nvb = T->pre[U_VEC][q + 1] - T->pre[U_VEC][q];
-  const int64_t nvz = T->pre[U_Z][q + 1] - T->pre[U_Z][q];
-  const int it = s.state[1] + 1;
-  slot_cols_total(s.dpart, nvb, kp, red, trr);
+  const int64_t nvz = (T->pre[U_Z][q + 1] - T->pre[U_Z][q]) / z_tiles(kp);
   // preconditioned: beta = <r, z>_new / <r, z>_old; the stopping rule stays on ||r||
-  if (s.l) slot_cols_total(s.dpart2, nvz, kp, red, trz);
-  const int c = threadIdx.x;
+  slot_cols_total(s.dpart, nvb, kp, red, trr, s.l ? s.dpart2 : nullptr, nvz, red2, trz);
   int go = 0;
-  if (c < kp && s.active[c]) {
+  if (act) {
     const double rr = trr[c], rz = s.l ? trz[c] : rr;
-    const double rel = sqrt(rr) / s.bnorm[c];
-    s.relres[c] = rel;
-    if (rel <= (double)s.tol || it >= s.max_iter || !isfinite(rel)) {
+    s.rr[c] = rr;
+    if (it >= s.max_iter || cg_stops(rr, bnorm, s.tol)) {
       s.active[c] = 0;
     } else {
-      s.beta[c] = rz / s.rho[c];
+      s.beta[c] = df_from_double(rz / rho);
       s.rho[c] = rz;
       go = 1;
     }
@@ -577,29 +749,40 @@ __global__ void __launch_bounds__(kST) kb_check_beta(const Table* __restrict__ T
 // p = r + beta p on active columns (double-float sum rounded to fp32); p = z + beta p for
 // preconditioned requests (z in ap).
 __global__ void __launch_bounds__(kST) kb_update_p(const Table* __restrict__ T) {
+  SLOT_AHEAD(U_VEC);
   pdl_enter();
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
-  SLOT_LOOP(U_VEC)
-  if (*s.state == 0 || g >= groups) continue;
+  SLOT_LOOP
+  if (!slot_on(s) || g >= groups) continue;
   const bool pre = s.l > 0;
+  const float* hi = (pre ? s.ap : s.rh) + col;
+  const float* lo = s.rl + col;
+  float* p = s.p + col;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 p4[kVecRows], rh[kVecRows], rl[kVecRows];
+#pragma unroll
+  for (int i = 0; i < kVecRows; ++i) {
+    const int64_t row = (local * kVecRows + i) * groups + g;
+    if (row >= s.n) break;
+    p4[i] = f4_ld(p + row * kp);
+    rh[i] = f4_ld(hi + row * kp);
+    rl[i] = pre ? zero : f4_ld(lo + row * kp);
+  }
   bool on[4];
   dfloat b[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     on[j] = s.active[col + j] != 0;
-    b[j] = df_from_double(s.beta[col + j]);
+    b[j] = s.beta[col + j];
   }
+#pragma unroll
   for (int i = 0; i < kVecRows; ++i) {
     const int64_t row = (local * kVecRows + i) * groups + g;
     if (row >= s.n) break;
-    const int64_t e = row * kp + col;
-    float4 p4 = f4_ld(s.p + e);
-    const float4 rh = pre ? f4_ld(s.ap + e) : f4_ld(s.rh + e);
-    const float4 rl = pre ? make_float4(0.f, 0.f, 0.f, 0.f) : f4_ld(s.rl + e);
-    float* pv = reinterpret_cast<float*>(&p4);
-    const float* rhv = reinterpret_cast<const float*>(&rh);
-    const float* rlv = reinterpret_cast<const float*>(&rl);
+    float pv[4] = {p4[i].x, p4[i].y, p4[i].z, p4[i].w};
+    const float rhv[4] = {rh[i].x, rh[i].y, rh[i].z, rh[i].w};
+    const float rlv[4] = {rl[i].x, rl[i].y, rl[i].z, rl[i].w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       if (on[j]) {
@@ -607,7 +790,7 @@ __global__ void __launch_bounds__(kST) kb_update_p(const Table* __restrict__ T) 
         pv[j] = __fadd_rn(t.hi, t.lo);
       }
     }
-    f4_st(s.p + e, p4);
+    f4_st(p + row * kp, make_float4(pv[0], pv[1], pv[2], pv[3]));
   }
   SLOT_LOOP_END
 }
@@ -713,8 +896,8 @@ __device__ __forceinline__ void ring_init(ChunkRing& ring, float* base, uint64_t
 }
 
 // ---- preconditioner apply z = P^-1 r (requests with l > 0) ----------------------------
-// P^-1 r = (r - B Minv B^T r) / noise (Woodbury), in five table-driven kernels: B^T r
-// partials, two ordered sums, Minv (B^T r), and z with the <r, z> partials.
+// P^-1 r = (r - B Minv B^T r) / noise (Woodbury), in four table-driven kernels: B^T r
+// partials, their ordered sums, Minv (B^T r), and z with the <r, z> partials.
 
 // Per-virtual-block partial of B^T r over kBtVbRows rows, with r taken as its fp32 part
 // rh (the low part rl is below the preconditioner's own rounding): the rows stream through
@@ -725,6 +908,7 @@ __device__ __forceinline__ void ring_init(ChunkRing& ring, float* base, uint64_t
 // pass per KC columns (B streamed again).
 template <int KC>
 __global__ void __launch_bounds__(kST, 1) kb_bt(const Table* __restrict__ T) {
+  SLOT_AHEAD(U_BT);
   pdl_enter();
   extern __shared__ __align__(128) float dsm[];
   __shared__ __align__(8) uint64_t bar[kStages];
@@ -734,8 +918,8 @@ __global__ void __launch_bounds__(kST, 1) kb_bt(const Table* __restrict__ T) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   ChunkRing ring;
   ring_init(ring, dsm, bar, kp, false);
-  SLOT_LOOP(U_BT)
-  if (*s.state == 0 || s.l == 0) continue;  // uniform over the block
+  SLOT_LOOP
+  if (!slot_on(s) || s.l == 0) continue;  // uniform over the block
   const int ld = s.ld;
   const int64_t r0 = local * kBtVbRows;
   const int64_t r1 = r0 + kBtVbRows < s.n ? r0 + kBtVbRows : s.n;
@@ -809,55 +993,74 @@ __global__ void __launch_bounds__(kST, 1) kb_bt(const Table* __restrict__ T) {
   SLOT_LOOP_END
 }
 
-// First-level sums of the B^T r partials: virtual block (segment g, chunk h) adds the
-// partials g kBtSeg .. g kBtSeg + kBtSeg - 1 of outputs h kST .. h kST + kST - 1 in order.
-__global__ void __launch_bounds__(kST) kb_bt_seg(const Table* __restrict__ T) {
+// t = B^T r: the partials of each segment of kBtSeg blocks added in order in fp32, then the
+// segment sums in order in fp64.  A virtual block takes kBtOut outputs, its warps the
+// segments (kBtRound at a time, 16 loads in flight a thread).
+constexpr int kBtOut = 32, kBtRound = 32;
+__global__ void __launch_bounds__(kST) kb_bt_sum(const Table* __restrict__ T) {
+  SLOT_AHEAD(U_BTT);
   pdl_enter();
+  __shared__ float sums[kBtRound][kBtOut];
   const int kp = T->kp;
-  SLOT_LOOP(U_BTS)
-  if (*s.state == 0 || s.l == 0) continue;
+  const int y = threadIdx.x / kBtOut, lane = threadIdx.x % kBtOut;
+  SLOT_LOOP
+  if (!slot_on(s) || s.l == 0) continue;  // uniform over the block
   const int cnt = s.ld * kp;
-  const int nch = (cnt + kST - 1) / kST;
-  const int64_t g = local / nch;
-  const int o = (int)(local - g * nch) * kST + threadIdx.x;
-  if (o >= cnt) continue;
+  const int o = (int)local * kBtOut + lane;
   const int64_t nvb = T->pre[U_BT][q + 1] - T->pre[U_BT][q];
-  const int64_t b0 = g * kBtSeg, b1 = b0 + kBtSeg < nvb ? b0 + kBtSeg : nvb;
-  float t = 0.f;
-  for (int64_t b = b0; b < b1; ++b) t += s.btpart[b * cnt + o];
-  s.bt2[g * cnt + o] = t;
-  SLOT_LOOP_END
-}
-
-// t = B^T r: the segment sums added in order in fp64, one output per thread.
-__global__ void __launch_bounds__(kST) kb_bt_total(const Table* __restrict__ T) {
-  pdl_enter();
-  const int kp = T->kp;
-  SLOT_LOOP(U_BTT)
-  if (*s.state == 0 || s.l == 0) continue;
-  const int cnt = s.ld * kp;
-  const int o = (int)local * kST + threadIdx.x;
-  if (o >= cnt) continue;
-  const int64_t nseg = ceil_div(T->pre[U_BT][q + 1] - T->pre[U_BT][q], kBtSeg);
+  const int64_t nseg = ceil_div(nvb, (int64_t)kBtSeg);
   double t = 0.0;
-  for (int64_t g = 0; g < nseg; ++g) t += (double)s.bt2[g * cnt + o];
-  s.tvec[o] = t;
+  for (int64_t g0 = 0; g0 < nseg; g0 += kBtRound) {
+    if (o < cnt)
+      for (int e = y; e < kBtRound && g0 + e < nseg; e += kST / kBtOut) {
+        const int64_t b0 = (g0 + e) * kBtSeg;
+        const int many = (int)(b0 + kBtSeg < nvb ? kBtSeg : nvb - b0);
+        const float* part = s.btpart + b0 * cnt + o;
+        float x[kBtSeg], v = 0.f;
+#pragma unroll
+        for (int u = 0; u < kBtSeg; ++u) x[u] = u < many ? part[(int64_t)u * cnt] : 0.f;
+#pragma unroll
+        for (int u = 0; u < kBtSeg; ++u) v += x[u];
+        sums[e][lane] = v;
+      }
+    __syncthreads();
+    if (y == 0 && o < cnt)
+      for (int e = 0; e < kBtRound && g0 + e < nseg; ++e) t += (double)sums[e][lane];
+    __syncthreads();
+  }
+  if (y == 0 && o < cnt) s.tvec[o] = t;
   SLOT_LOOP_END
 }
 
 // u = Minv t (fp64) on the first l rows, 0 below; stored fp32 [ld][kp].  Four lanes per
-// output, each a quarter of the dot product, combined by shuffles in a fixed order.
-__global__ void __launch_bounds__(kST) kb_minv(const Table* __restrict__ T) {
+// output, each a quarter of the dot product, combined by shuffles in a fixed order.  Small
+// blocks: fp64 runs at 2 results a clock per SM, so the outputs go over all of them.
+constexpr int kMinvT = 64;
+__global__ void __launch_bounds__(kMinvT) kb_minv(const Table* __restrict__ T) {
+  SLOT_AHEAD(U_MINV);
   pdl_enter();
   const int kp = T->kp;
-  SLOT_LOOP(U_MINV)
-  if (*s.state == 0 || s.l == 0) continue;  // uniform over the block
-  const int o = (int)(local * kST + threadIdx.x) / 4, part = threadIdx.x & 3;
-  const int cnt = s.ld * kp;
+  SLOT_LOOP
+  if (!slot_on(s) || s.l == 0) continue;  // uniform over the block
+  const int o = (int)(local * kMinvT + threadIdx.x) / 4, part = threadIdx.x & 3;
+  const int cnt = s.ld * kp, l = s.l;
   const int j = o / kp, c = o - j * kp;
   double a = 0.0;
-  if (o < cnt && j < s.l)
-    for (int i = part; i < s.l; i += 4) a += s.Minv[j * s.l + i] * s.tvec[i * kp + c];
+  if (o < cnt && j < l) {
+    const double* row = s.Minv + (int64_t)j * l;
+    const double* tv = s.tvec + c;
+    for (int i0 = part; i0 < l; i0 += 4 * 13) {  // 13 terms loaded ahead (l = 100: two rounds)
+      double m[13], t[13];
+#pragma unroll
+      for (int u = 0; u < 13; ++u) {
+        const int i = i0 + 4 * u;
+        m[u] = i < l ? row[i] : 0.0;
+        t[u] = i < l ? tv[i * kp] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 13; ++u) a += m[u] * t[u];
+    }
+  }
   a += __shfl_xor_sync(0xffffffffu, a, 1);
   a += __shfl_xor_sync(0xffffffffu, a, 2);
   if (o < cnt && part == 0) s.u[o] = (float)a;
@@ -888,21 +1091,24 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
 }
 
 // z = (r - B u) / noise, written into ap (free between the x, r update and the next
-// product), and the virtual block's column sums of r z into dpart2.  The block's kZVbRows
-// rows stream through the chunk ring; warp w takes the 16-row tiles w, w + 8, ... of each
-// chunk and forms B u on the tensor cores (m16n8k8, 3xTF32 split, NT tiles of 8 columns),
-// A fragments from the staged B rows, B fragments from u split once into shared memory.  The epilogue
-// reads r from the stage.  The column sums of r z are double-float per lane, combined over
-// the lanes of a column by a fixed butterfly and over the warps in order.  Test rows have
-// zero B rows and zero r, so z = 0 there.
-template <int NT>
+// product), and the virtual block's column sums of r z into dpart2.  A virtual block takes
+// kZVbRows rows and 8 columns: the warp-level TF32 MMAs run at about the rate of plain FMAs
+// here (114 multiply-adds a clock per SM), they are what the kernel spends its time on, and
+// with all columns in one block a 40k-point request fills 70 SMs of 152 (22.6 us; 16 with the
+// columns apart, B read twice, the second time from L2).  The rows stream through the chunk
+// ring; warp w takes the 16-row tiles w, w + 8, ... of each chunk and forms B u on the tensor
+// cores (m16n8k8, 3xTF32 split), A fragments from the staged B rows, B fragments from u split
+// once into shared memory.  The epilogue reads r from the stage.  The column sums of r z are
+// double-float per lane, combined over the lanes of a column by a fixed butterfly and over the
+// warps in order.  Test rows have zero B rows and zero r, so z = 0 there.
 __global__ void __launch_bounds__(kST, 1) kb_apply_z(const Table* __restrict__ T) {
+  SLOT_AHEAD(U_Z);
   pdl_enter();
   extern __shared__ __align__(128) float dsm[];
   __shared__ __align__(8) uint64_t bar[kStages];
-  __shared__ double red[kST / 32][8 * NT];
   constexpr int kWarps = kST / 32;
-  const int kp = T->kp;
+  __shared__ double red[kWarps][8];
+  const int kp = T->kp, tiles = z_tiles(kp);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   // u split once per virtual block: uh = tf32(u), ul = tf32(u - uh), [kMaxLd][kp] each
   uint32_t* uh = reinterpret_cast<uint32_t*>(dsm);
@@ -910,18 +1116,22 @@ __global__ void __launch_bounds__(kST, 1) kb_apply_z(const Table* __restrict__ T
   ChunkRing ring;
   ring_init(ring, dsm + 2 * kMaxLd * kp, bar, kp, true);
   ring.rows = ring.rows / 16 * 16;
-  SLOT_LOOP(U_Z)
-  if (*s.state == 0 || s.l == 0) continue;  // uniform over the block
+  SLOT_LOOP
+  if (!slot_on(s) || s.l == 0) continue;  // uniform over the block
   const int ld = s.ld, ksteps = (ld + 7) / 8;
-  const int64_t r0 = local * kZVbRows;
+  const float inv_noise = s.inv_noise;
+  float* z = s.ap;
+  const int64_t vb = local / tiles;
+  const int nt = (int)(local - vb * tiles);
+  const int64_t r0 = vb * kZVbRows;
   const int64_t r1 = r0 + kZVbRows < s.n ? r0 + kZVbRows : s.n;
   const int nch = (int)ceil_div(r1 - r0, ring.rows);
   if (threadIdx.x == 0)
     for (int k = 0; k < nch && k < kStages; ++k) ring_issue(ring, k, s, kp, r0, r1, k);
-  for (int e = threadIdx.x; e < ld * kp; e += kST) tf32_split(s.u[e], uh[e], ul[e]);
-  dfloat acc[NT][2];
-#pragma unroll
-  for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = {0.f, 0.f};
+  for (int e = threadIdx.x; e < ld * kp; e += blockDim.x) tf32_split(s.u[e], uh[e], ul[e]);
+  dfloat acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
+  const int n = 8 * nt + g, c = 8 * nt + 2 * t;
+  const bool n_in = n < kp, c_in = c < kp;  // kp is a multiple of 4: c + 1 < kp too
   for (int k = 0; k < nch; ++k) {
     const int st = k % kStages;
     const bool ok =
@@ -937,12 +1147,11 @@ __global__ void __launch_bounds__(kST, 1) kb_apply_z(const Table* __restrict__ T
     const float* Hs = Bs + rows * ld;
     const float* Ls = Hs + rows * kp;
     for (int rt = warp * 16; rt < rows; rt += kWarps * 16) {
-      float d[NT][4];
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
+      float d[4] = {0.f, 0.f, 0.f, 0.f};
       // rows past the chunk read stale stage data; their outputs are not stored
       const float* ra = Bs + (rt + g) * ld;
       const float* rb = ra + 8 * ld;
+#pragma unroll 4
       for (int ks = 0; ks < ksteps; ++ks) {
         const int j0 = ks * 8 + t, j1 = j0 + 4;
         const bool in0 = j0 < ld, in1 = j1 < ld;
@@ -951,36 +1160,26 @@ __global__ void __launch_bounds__(kST, 1) kb_apply_z(const Table* __restrict__ T
         tf32_split(in0 ? rb[j0] : 0.f, ah[1], al[1]);
         tf32_split(in1 ? ra[j1] : 0.f, ah[2], al[2]);
         tf32_split(in1 ? rb[j1] : 0.f, ah[3], al[3]);
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          const int n = 8 * nt + g;
-          const bool n_in = n < kp;
-          const uint32_t bh0 = in0 && n_in ? uh[j0 * kp + n] : 0u;
-          const uint32_t bl0 = in0 && n_in ? ul[j0 * kp + n] : 0u;
-          const uint32_t bh1 = in1 && n_in ? uh[j1 * kp + n] : 0u;
-          const uint32_t bl1 = in1 && n_in ? ul[j1 * kp + n] : 0u;
-          mma_tf32(d[nt], ah, bh0, bh1);
-          mma_tf32(d[nt], ah, bl0, bl1);
-          mma_tf32(d[nt], al, bh0, bh1);
-        }
+        const uint32_t bh0 = in0 && n_in ? uh[j0 * kp + n] : 0u;
+        const uint32_t bl0 = in0 && n_in ? ul[j0 * kp + n] : 0u;
+        const uint32_t bh1 = in1 && n_in ? uh[j1 * kp + n] : 0u;
+        const uint32_t bl1 = in1 && n_in ? ul[j1 * kp + n] : 0u;
+        mma_tf32(d, ah, bh0, bh1);
+        mma_tf32(d, ah, bl0, bl1);
+        mma_tf32(d, al, bh0, bh1);
       }
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        const int c = 8 * nt + 2 * t;
-        if (c >= kp) continue;
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          const int row = rt + g + 8 * half;
-          if (row >= rows) continue;
-          const float2 h = *reinterpret_cast<const float2*>(Hs + row * kp + c);
-          const float2 lo = *reinterpret_cast<const float2*>(Ls + row * kp + c);
-          const float x0 = __fadd_rn(h.x, lo.x), x1 = __fadd_rn(h.y, lo.y);
-          const float z0 = (x0 - d[nt][2 * half]) * s.inv_noise;
-          const float z1 = (x1 - d[nt][2 * half + 1]) * s.inv_noise;
-          *reinterpret_cast<float2*>(s.ap + (a0 + row) * kp + c) = make_float2(z0, z1);
-          acc[nt][0] = df_add(acc[nt][0], df_two_prod(x0, z0));
-          acc[nt][1] = df_add(acc[nt][1], df_two_prod(x1, z1));
-        }
+      for (int half = 0; half < 2; ++half) {
+        const int row = rt + g + 8 * half;
+        if (row >= rows || !c_in) continue;
+        const float2 h = *reinterpret_cast<const float2*>(Hs + row * kp + c);
+        const float2 lo = *reinterpret_cast<const float2*>(Ls + row * kp + c);
+        const float x0 = __fadd_rn(h.x, lo.x), x1 = __fadd_rn(h.y, lo.y);
+        const float z0 = (x0 - d[2 * half]) * inv_noise;
+        const float z1 = (x1 - d[2 * half + 1]) * inv_noise;
+        *reinterpret_cast<float2*>(z + (a0 + row) * kp + c) = make_float2(z0, z1);
+        acc[0] = df_add(acc[0], df_two_prod(x0, z0));
+        acc[1] = df_add(acc[1], df_two_prod(x1, z1));
       }
     }
     __syncthreads();  // stage st is free again
@@ -988,21 +1187,18 @@ __global__ void __launch_bounds__(kST, 1) kb_apply_z(const Table* __restrict__ T
   }
   // column sums: the 8 lanes of a column (same t) by a fixed butterfly, then the warps in order
 #pragma unroll
-  for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      double v = df_to_double(acc[nt][e]);
-      v += __shfl_xor_sync(0xffffffffu, v, 4);
-      v += __shfl_xor_sync(0xffffffffu, v, 8);
-      v += __shfl_xor_sync(0xffffffffu, v, 16);
-      const int c = 8 * nt + 2 * t + e;
-      if (g == 0 && c < kp) red[warp][c] = v;
-    }
+  for (int e = 0; e < 2; ++e) {
+    double v = df_to_double(acc[e]);
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    if (g == 0) red[warp][2 * t + e] = v;
+  }
   __syncthreads();
-  if ((int)threadIdx.x < kp) {
+  if (threadIdx.x < 8 && 8 * nt + (int)threadIdx.x < kp) {
     double v = 0.0;
     for (int w = 0; w < kWarps; ++w) v += red[w][threadIdx.x];
-    s.dpart2[local * kp + threadIdx.x] = v;
+    s.dpart2[vb * kp + 8 * nt + threadIdx.x] = v;
   }
   __syncthreads();
   SLOT_LOOP_END
@@ -1014,27 +1210,12 @@ size_t ring_smem_bytes(int kp) {
 }
 size_t apply_z_smem_bytes(int kp) { return ring_smem_bytes(kp) + 2 * (size_t)kMaxLd * kp * 4; }
 
-// kb_apply_z for the server's kp: NT = kp / 8 rounded up tiles of 8 columns.
 void launch_apply_z(int kp, const Table* T, cudaStream_t st) {
-  const size_t sm = apply_z_smem_bytes(kp);
-  switch ((kp + 7) / 8) {
-    case 1: launch_pdl_smem(kb_apply_z<1>, kRingGrid, kST, sm, st, T); break;
-    case 2: launch_pdl_smem(kb_apply_z<2>, kRingGrid, kST, sm, st, T); break;
-    case 3: launch_pdl_smem(kb_apply_z<3>, kRingGrid, kST, sm, st, T); break;
-    default: launch_pdl_smem(kb_apply_z<4>, kRingGrid, kST, sm, st, T); break;
-  }
+  launch_pdl_smem(kb_apply_z, kRingGrid, kST, apply_z_smem_bytes(kp), st, T);
 }
 cudaError_t apply_z_smem_attributes(int kp) {
-  const int sm = (int)apply_z_smem_bytes(kp);
-  cudaError_t e =
-      cudaFuncSetAttribute(kb_apply_z<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kb_apply_z<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kb_apply_z<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kb_apply_z<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  return e;
+  return cudaFuncSetAttribute(kb_apply_z, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)apply_z_smem_bytes(kp));
 }
 
 // kb_bt for the server's kp: KC = min(kp, 16) columns per pass.
@@ -1062,11 +1243,12 @@ cudaError_t bt_smem_attributes() {
 // ---- per-request set-up and read-out (single-request launches) ------------------------
 // Partials of <r, r> for the initial residual (the same virtual blocks as the iteration).
 __global__ void __launch_bounds__(kST) kb_norm(const Table* __restrict__ T) {
+  SLOT_AHEAD(U_VEC);
   pdl_enter();
   __shared__ double sh[kST * 4];
   const int kp = T->kp, G = kp / 4, groups = kST / G;
   const int g = threadIdx.x / G, col = (int)(threadIdx.x % G) * 4;
-  SLOT_LOOP(U_VEC)
+  SLOT_LOOP
   dfloat d[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
   if (g < groups) {
     for (int i = 0; i < kVecRows; ++i) {
@@ -1085,25 +1267,24 @@ __global__ void __launch_bounds__(kST) kb_norm(const Table* __restrict__ T) {
 
 __global__ void __launch_bounds__(kST) kb_init_scalars(const Table* __restrict__ T) {
   pdl_enter();
-  __shared__ double red[kST], trr[kMaxServeK], trz[kMaxServeK];
+  __shared__ double red[kST], red2[kST], trr[kMaxServeK], trz[kMaxServeK];
   const int q = blockIdx.x;
   if (q >= T->nslots) return;
   const SlotDev& s = T->s[q];
   const int kp = T->kp;
   const int64_t nvb = T->pre[U_VEC][q + 1] - T->pre[U_VEC][q];
-  const int64_t nvz = T->pre[U_Z][q + 1] - T->pre[U_Z][q];
-  slot_cols_total(s.dpart, nvb, kp, red, trr);
-  if (s.l) slot_cols_total(s.dpart2, nvz, kp, red, trz);
+  const int64_t nvz = (T->pre[U_Z][q + 1] - T->pre[U_Z][q]) / z_tiles(kp);
+  slot_cols_total(s.dpart, nvb, kp, red, trr, s.l ? s.dpart2 : nullptr, nvz, red2, trz);
   const int c = threadIdx.x;
   int on = 0;
   if (c < kp) {
     const double rr = trr[c];
     s.rho[c] = s.l ? trz[c] : rr;
     s.bnorm[c] = sqrt(rr);
-    s.alpha[c] = 0.0;
-    s.beta[c] = 0.0;
+    s.alpha[c] = {0.f, 0.f};
+    s.beta[c] = {0.f, 0.f};
     on = (rr > 0.0 && 1.0 > (double)s.tol && s.max_iter > 0) ? 1 : 0;
-    s.relres[c] = rr > 0.0 ? 1.0 : 0.0;
+    s.rr[c] = rr;
     s.active[c] = on;
   }
   const int any = __syncthreads_or(on);
@@ -1227,7 +1408,7 @@ struct Request {
   Lattice* L = nullptr;
   float *xh = nullptr, *xl = nullptr, *rh = nullptr, *rl = nullptr, *p = nullptr, *ap = nullptr;
   double* dpart = nullptr;
-  double* scal = nullptr;  // rho, bnorm, relres, alpha, beta: [5][kp]
+  double* scal = nullptr;  // rho, bnorm, rr, alpha, beta: [5][kp]
   int* ints = nullptr;     // active [kp], state [2], bulk-copy error [1]
   float* outd = nullptr;   // mean, var: [2][ns]
   Table* dtab1 = nullptr;  // one-request table for the set-up kernels
@@ -1241,7 +1422,7 @@ struct Request {
   double kappa = 0.0;
   float* Bh = nullptr;
   double* Minv = nullptr;
-  float *btpart = nullptr, *bt2 = nullptr, *u = nullptr;
+  float *btpart = nullptr, *u = nullptr;
   double *tvec = nullptr, *dpart2 = nullptr;
   std::vector<void*> ptrs;
   std::string setup_error;  // message of a failed set-up (set on the set-up thread)
@@ -1353,9 +1534,9 @@ void fill_slot(const sgp_server* S, const Request* R, SlotDev& s) {
   const int kp = S->kp;
   s.rho = R->scal;
   s.bnorm = R->scal + kp;
-  s.relres = R->scal + 2 * kp;
-  s.alpha = R->scal + 3 * kp;
-  s.beta = R->scal + 4 * kp;
+  s.rr = R->scal + 2 * kp;
+  s.alpha = reinterpret_cast<dfloat*>(R->scal + 3 * kp);
+  s.beta = reinterpret_cast<dfloat*>(R->scal + 4 * kp);
   s.active = R->ints;
   s.state = R->ints + kp;
   s.max_iter = S->o.max_iter;
@@ -1372,7 +1553,6 @@ void fill_slot(const sgp_server* S, const Request* R, SlotDev& s) {
   s.Bh = R->Bh;
   s.Minv = R->Minv;
   s.btpart = R->btpart;
-  s.bt2 = R->bt2;
   s.tvec = R->tvec;
   s.u = R->u;
   s.dpart2 = R->dpart2;
@@ -1382,17 +1562,14 @@ void unit_counts(const sgp_server* S, const Request* R, int64_t (&vb)[U_KINDS]) 
   const Lattice* L = R->L;
   const int groups = groups_of(S->kp);
   vb[U_SPLAT] = ceil_div(L->nseg, groups);
-  vb[U_MED] = ceil_div(L->nmed, groups);
-  vb[U_HUGE] = L->nhuge;
+  vb[U_FIX] = L->nhuge + ceil_div(L->nmed, groups);
   vb[U_BLUR] = ceil_div(L->sparse ? L->act_max : L->m, (int64_t)groups * kBlurU);
   vb[U_VEC] = ceil_div(L->n, (int64_t)groups * kVecRows);
   vb[U_VERT] = L->sparse ? ceil_div(L->m, (int64_t)groups * kBlurU) : 0;
-  const int64_t nch = ceil_div((int64_t)R->ld * S->kp, kST);  // output chunks of B^T r
   vb[U_BT] = R->l ? ceil_div(L->n, kBtVbRows) : 0;
-  vb[U_BTS] = R->l ? nch * ceil_div(vb[U_BT], kBtSeg) : 0;
-  vb[U_BTT] = R->l ? nch : 0;
-  vb[U_MINV] = R->l ? ceil_div((int64_t)R->ld * S->kp * 4, kST) : 0;
-  vb[U_Z] = R->l ? ceil_div(L->n, kZVbRows) : 0;
+  vb[U_BTT] = R->l ? ceil_div((int64_t)R->ld * S->kp, kBtOut) : 0;
+  vb[U_MINV] = R->l ? ceil_div((int64_t)R->ld * S->kp * 4, kMinvT) : 0;
+  vb[U_Z] = R->l ? ceil_div(L->n, kZVbRows) * z_tiles(S->kp) : 0;
 }
 
 // Lane of a built request: dimension class (D <= 4, 8, ..., 128), work class (blur,
@@ -1565,18 +1742,16 @@ sgp_status setup(sgp_server* S, Request* R, cudaStream_t st, Table& t1) {
       unit_counts(S, R, R->vb);
       SRV_CHECK(get((void**)&R->Bh, (size_t)n_all * ld * sizeof(float)), "alloc Nystrom B");
       SRV_CHECK(get((void**)&R->Minv, (size_t)l * l * sizeof(double)), "alloc Nystrom Minv");
-      const size_t nseg = (size_t)ceil_div(R->vb[U_BT], kBtSeg);
       SRV_CHECK(get((void**)&R->btpart, (size_t)R->vb[U_BT] * ld * kp * sizeof(float)),
                 "alloc B^T r partials");
-      SRV_CHECK(get((void**)&R->bt2, nseg * ld * kp * sizeof(float)), "alloc B^T r sums");
       SRV_CHECK(get((void**)&R->tvec, (size_t)ld * kp * sizeof(double)), "alloc B^T r");
       SRV_CHECK(get((void**)&R->u, (size_t)ld * kp * sizeof(float)), "alloc Minv B^T r");
-      SRV_CHECK(get((void**)&R->dpart2, (size_t)R->vb[U_Z] * kp * sizeof(double)),
+      SRV_CHECK(get((void**)&R->dpart2, (size_t)R->vb[U_Z] / z_tiles(kp) * kp * sizeof(double)),
                 "alloc <r, z> partials");
       pre_bytes = (size_t)n_all * ld * sizeof(float) + (size_t)l * l * sizeof(double) +
-                  ((size_t)R->vb[U_BT] + nseg) * ld * kp * sizeof(float) +
+                  (size_t)R->vb[U_BT] * ld * kp * sizeof(float) +
                   (size_t)ld * kp * (sizeof(double) + sizeof(float)) +
-                  (size_t)R->vb[U_Z] * kp * sizeof(double);
+                  (size_t)R->vb[U_Z] / z_tiles(kp) * kp * sizeof(double);
       void* scratch = nullptr;
       int* status_d = nullptr;
       SRV_CHECK(tmp.get(&scratch, nystrom_masked_scratch_bytes(l, n_all)),
@@ -1605,7 +1780,7 @@ sgp_status setup(sgp_server* S, Request* R, cudaStream_t st, Table& t1) {
   t1.err = R->ints + kp + 2;
   t1.wait_limit = kSpinLimit;
   fill_slot(S, R, t1.s[0]);
-  for (int u = 0; u < U_KINDS; ++u) t1.pre[u][1] = R->vb[u];
+  for (int u = 0; u < U_KINDS; ++u) std::fill(t1.pre[u] + 1, t1.pre[u] + kMaxSlots + 1, R->vb[u]);
   SRV_CHECK(cudaMemcpyAsync(R->dtab1, &t1, sizeof(Table), cudaMemcpyHostToDevice, st),
             "copy table");
   launch_pdl(kb_norm, kGrid, kST, st, R->dtab1);
@@ -1615,9 +1790,8 @@ sgp_status setup(sgp_server* S, Request* R, cudaStream_t st, Table& t1) {
     SRV_CHECK(cudaMemcpyAsync(R->ints + kp, &kOne, sizeof(int), cudaMemcpyHostToDevice, st),
               "mark the request active");
     launch_bt(kp, R->dtab1, st);
-    launch_pdl(kb_bt_seg, kGrid, kST, st, R->dtab1);
-    launch_pdl(kb_bt_total, kGrid, kST, st, R->dtab1);
-    launch_pdl(kb_minv, kGrid, kST, st, R->dtab1);
+    launch_pdl(kb_bt_sum, kGrid, kST, st, R->dtab1);
+    launch_pdl(kb_minv, kGrid, kMinvT, st, R->dtab1);
     launch_apply_z(kp, R->dtab1, st);
     note_launches(5);
   }
@@ -1658,9 +1832,9 @@ sgp_status finish(sgp_server* S, Request* R, cudaStream_t st) {
     SRV_CHECK(cudaMemcpyAsync(in.var, var_d, (size_t)in.ns * sizeof(float),
                               cudaMemcpyDeviceToHost, st),
               "copy var");
-  std::vector<double> relres(kp);
+  std::vector<double> norms(2 * kp);  // ||b||, then <r, r>
   std::vector<int> ints(kp + 3);
-  SRV_CHECK(cudaMemcpyAsync(relres.data(), R->scal + 2 * kp, kp * sizeof(double),
+  SRV_CHECK(cudaMemcpyAsync(norms.data(), R->scal + kp, 2 * kp * sizeof(double),
                             cudaMemcpyDeviceToHost, st),
             "copy residuals");
   SRV_CHECK(cudaMemcpyAsync(ints.data(), R->ints, (kp + 3) * sizeof(int), cudaMemcpyDeviceToHost,
@@ -1668,7 +1842,8 @@ sgp_status finish(sgp_server* S, Request* R, cudaStream_t st) {
             "copy state");
   SRV_CHECK(cudaStreamSynchronize(st), "finishing a request");
   double worst = 0.0;
-  for (int c = 0; c <= S->S; ++c) worst = std::max(worst, relres[c]);
+  for (int c = 0; c <= S->S; ++c)
+    if (norms[c] > 0.0) worst = std::max(worst, std::sqrt(norms[kp + c]) / norms[c]);
   R->st.iters = ints[kp + 1];
   R->st.rel_res = worst;
   R->st.bytes = R->held;
@@ -1726,8 +1901,7 @@ int enqueue_iteration_t(Lane* ln, int dmax, bool sparse, bool pre) {
   cudaStream_t st = ln->st;
   const Table* T = ln->dtab;
   launch_pdl(kb_splat<Sv>, kGrid, kST, st, T);
-  launch_pdl(kb_splat_med<Sv>, kGrid, kST, st, T);
-  launch_pdl(kb_splat_huge<Sv>, kGrid, kST, st, T);
+  launch_pdl(kb_splat_fix<Sv>, kGrid, kST, st, T);
   for (int t = 0; t < 2 * dmax; ++t) {
     launch_pdl(kb_blur<Rr, Sv>, kGrid, kST, st, T, t);
     if (sparse) launch_pdl(kb_sparse_store<Sv>, kGrid, kST, st, T, t);
@@ -1739,14 +1913,13 @@ int enqueue_iteration_t(Lane* ln, int dmax, bool sparse, bool pre) {
   if (pre) {
     const int kp = ln->htab->kp;
     launch_bt(kp, T, st);
-    launch_pdl(kb_bt_seg, kGrid, kST, st, T);
-    launch_pdl(kb_bt_total, kGrid, kST, st, T);
-    launch_pdl(kb_minv, kGrid, kST, st, T);
+    launch_pdl(kb_bt_sum, kGrid, kST, st, T);
+    launch_pdl(kb_minv, kGrid, kMinvT, st, T);
     launch_apply_z(kp, T, st);
   }
   launch_pdl(kb_check_beta, kMaxSlots, kST, st, T);
   launch_pdl(kb_update_p, kGrid, kST, st, T);
-  return 8 + 2 * dmax + (sparse ? 2 * dmax + 1 : 0) + (pre ? 5 : 0);
+  return 7 + 2 * dmax + (sparse ? 2 * dmax + 1 : 0) + (pre ? 4 : 0);
 }
 
 template <class Sv>
@@ -1994,6 +2167,8 @@ sgp_status launch(sgp_server* S, Lane* ln) {
         R->waited = true;
       }
     }
+    for (int u = 0; u < U_KINDS; ++u)
+      std::fill(t.pre[u] + ns + 1, t.pre[u] + kMaxSlots + 1, t.pre[u][ns]);
     SRV_CHECK(cudaMemcpyAsync(ln->dtab, &t, sizeof(Table), cudaMemcpyHostToDevice, ln->st),
               "copy table");
     ln->ntab = ns;

@@ -379,6 +379,20 @@ __device__ __forceinline__ void block_column_sums(const double (&acc)[VEC], int 
   }
 }
 
+// Whether ||r|| / ||b|| = sqrt(rr) / bnorm (fp64) is at most tol or not finite.  Decided in
+// fp32 unless the two are within 1e-4 of each other (or out of fp32's range): a square root
+// and a division in fp64 are some 60 dependent operations of a narrow pipe, 2 us.
+__device__ __forceinline__ bool cg_stops(double rr, double bnorm, float tol) {
+  const float r = (float)rr, b = (float)bnorm;
+  const float lim = tol * b * (tol * b);
+  if (r > 1e-30f && r < 1e30f && lim < 1e30f && lim > 1e-30f) {
+    if (r > lim * 1.0002f) return false;
+    if (r < lim * 0.9998f) return true;
+  }
+  const double rel = sqrt(rr) / bnorm;
+  return rel <= (double)tol || !isfinite(rel);
+}
+
 // ---- double-float arithmetic -------------------------------------------------------
 // FP64 throughput on this part is a small fraction of FP32, so quantities that need more
 // than fp32 precision per element (CG iterate and residual, dot-product accumulation) are
