@@ -161,7 +161,7 @@ __global__ void k_filter_finish(int64_t n, int d, float scale, const float* __re
 
 // dl_j = -sum_i dX_ij x_ij / l_j: per-block partials (thread t owns column t % d and
 // rows t / d, t / d + P, ... of the block's range, P = floor(256 / d)), combined in a
-// fixed order; then the blocks in order.
+// fixed order; then the blocks in a fixed order.
 __global__ void __launch_bounds__(256) k_dls_partial(int64_t n, int d, const float* __restrict__ X,
                                                      const float* __restrict__ dX,
                                                      double* __restrict__ partial) {
@@ -188,11 +188,15 @@ __global__ void __launch_bounds__(256) k_dls_partial(int64_t n, int d, const flo
 __global__ void k_dls_final(int nblk, int d, const double* __restrict__ partial,
                             const float* __restrict__ ls, float* __restrict__ dls) {
   pdl_enter();
-  const int j = threadIdx.x;
-  if (j >= d) return;
+  // eight lanes a dimension, every eighth block each (304 dependent fp64 additions: 27 us)
+  const int j = blockIdx.x * (blockDim.x / 8) + threadIdx.x / 8, lane = threadIdx.x % 8;
   double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += partial[(int64_t)b * d + j];
-  dls[j] = (float)(-s / (double)ls[j]);
+  if (j < d) {
+#pragma unroll 8
+    for (int b = lane; b < nblk; b += 8) s += partial[(int64_t)b * d + j];
+  }
+  for (int o = 4; o >= 1; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (j < d && lane == 0) dls[j] = (float)(-s / (double)ls[j]);
 }
 
 #define BW_CHECK(expr, what)                                  \
@@ -326,7 +330,7 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
     double* part = nullptr;
     BW_CHECK(w.get(&part, (size_t)kDlsBlocks * d * sizeof(double)), "alloc partials");
     launch_pdl(k_dls_partial, kDlsBlocks, 256, st, n, d, X, dXw, part);
-    launch_pdl(k_dls_final, 1, 128, st, kDlsBlocks, d, part, ls, dls);
+    launch_pdl(k_dls_final, (unsigned)ceil_div(d, 16), 128, st, kDlsBlocks, d, part, ls, dls);
     note_launches(2);
   }
   BW_CHECK(cudaGetLastError(), "launching the MVM backward");

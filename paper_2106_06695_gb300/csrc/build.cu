@@ -1219,7 +1219,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     launch_pdl(k_point_key, (unsigned)ceil_div(n, 256), 256, st, rem0, n, D, pk, ka, va);
     note_launches(1);
     // the packed cell occupies the top `used` bits; bits below are zero
-    const bool in_alt = used > 0 ? radix_sort_pairs(ka, va, kb, vb, n, 32, rt, st) : false;
+    const bool in_alt = radix_sort_pairs(ka, va, kb, vb, n, (32 - used) & ~7, 32, rt, st);
     SGP_CHECK(dalloc(&L->perm, n, st), "alloc perm");
     SGP_CHECK(cudaMemcpyAsync(L->perm, in_alt ? vb : va, n * sizeof(int32_t),
                               cudaMemcpyDeviceToDevice, st),
@@ -1314,7 +1314,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     launch_pdl(k_nbr_close, grid, 256, st, owner, L->idx, L->rank, m, d, r, L->nbr,
                lb);
     launch_pdl(k_hash_keys, grid, 256, st, vhash, m, 64 - bits, ka, va);
-    const bool in_alt = radix_sort_pairs(ka, va, kb, vb, m, bits, rt, st);
+    const bool in_alt = radix_sort_pairs(ka, va, kb, vb, m, 0, bits, rt, st);
     const uint32_t* ord = in_alt ? vb : va;
     launch_pdl(k_hash_index, grid, 256, st, in_alt ? kb : ka, ord, vhash, up, m, buckets,
                low, high, up_sorted, start);
@@ -1334,7 +1334,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     launch_pdl(k_iota, (unsigned)ceil_div(nD, 256), 256, st, va, nD);
     note_launches(1);
     const int bits = std::max(1, bits_for((uint64_t)(m > 0 ? m - 1 : 0)));
-    const bool in_alt = radix_sort_pairs(ka, va, kb, vb, nD, bits, rt, st);
+    const bool in_alt = radix_sort_pairs(ka, va, kb, vb, nD, 0, bits, rt, st);
     const uint32_t* sorted_ids = in_alt ? kb : ka;
     const uint32_t* sorted_entries = in_alt ? vb : va;
     SGP_CHECK(dalloc(&L->items, nD, st), "alloc items");
@@ -1351,19 +1351,17 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   // 7. splat segments (load balance)
   unsigned long long pairs = 0;  // (v, v + u_j) pairs: at least as many active vertices
   {
-    uint32_t *cnt, *slots, *med, *huge, *tot, *stmp;
+    uint32_t *cnt, *slots, *med, *huge, *tot;
     SGP_CHECK(tmp.get(&cnt, m), "alloc seg");
     SGP_CHECK(tmp.get(&slots, m), "alloc seg");
     SGP_CHECK(tmp.get(&med, m), "alloc seg");
     SGP_CHECK(tmp.get(&huge, m), "alloc seg");
     SGP_CHECK(tmp.get(&tot, 4), "alloc seg");
-    SGP_CHECK(tmp.get(&stmp, scan_temp_elems(m)), "alloc seg");
     launch_pdl(k_seg_count, (unsigned)ceil_div(m, 256), 256, st, L->row_ptr, m, cnt, slots, med, huge);
     note_launches(1);
-    exclusive_scan_u32(cnt, m, tot + 0, stmp, st);
-    exclusive_scan_u32(slots, m, tot + 1, stmp, st);
-    exclusive_scan_u32(med, m, tot + 2, stmp, st);
-    exclusive_scan_u32(huge, m, tot + 3, stmp, st);
+    uint32_t* const counted[4] = {cnt, slots, med, huge};
+    uint32_t* const sums[4] = {tot, tot + 1, tot + 2, tot + 3};
+    exclusive_scans_u32(counted, sums, 4, m, rt, st);  // rt holds nD / 8 and more
     uint32_t ht[4];
     SGP_CHECK(cudaMemcpyAsync(ht, tot, sizeof(ht), cudaMemcpyDeviceToHost, st), "read seg");
     SGP_CHECK(cudaMemcpyAsync(&pairs, counts + 2 * D, sizeof(pairs), cudaMemcpyDeviceToHost, st),

@@ -203,11 +203,15 @@ bool make_stencil(int kernel, int r, double spacing_override, double* s, double*
 size_t scan_temp_elems(int64_t n);
 void exclusive_scan_u32(uint32_t* data, int64_t n, uint32_t* total, uint32_t* tmp,
                         cudaStream_t st);
-// Stable LSD radix sort of (key, value) pairs by the low `bits` bits of the key.  Uses
-// the *_alt buffers as ping-pong storage; returns true when the result ended in *_alt.
+// `count` (at most 4) such scans by the same launches; `tmp` holds count times as much.
+void exclusive_scans_u32(uint32_t* const* data, uint32_t* const* totals, int count, int64_t n,
+                         uint32_t* tmp, cudaStream_t st);
+// Stable LSD radix sort of (key, value) pairs by bits begin .. end - 1 of the key (8 at a
+// time, so up to 7 more).  Uses the *_alt buffers as ping-pong storage; returns true when the
+// result ended in *_alt.
 size_t radix_temp_elems(int64_t n);
 bool radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
-                      int64_t n, int bits, uint32_t* tmp, cudaStream_t st);
+                      int64_t n, int begin, int end, uint32_t* tmp, cudaStream_t st);
 
 // ---- lattice construction (build.cu) ----
 sgp_status build_lattice(Lattice* L, const float* X, const float* ls);
