@@ -451,12 +451,18 @@ __global__ void k_point_key(const int16_t* __restrict__ rem0, int64_t n, int D, 
 // ---------------------------------------------------------------------------------
 // 3. Hash insert.
 // ---------------------------------------------------------------------------------
+// A slot only ever goes from empty to a vertex, whose owner only decreases: it is read before an
+// atomic is tried, and an entry above the owner seen there needs none (n = 628k, d = 3, where
+// 2.5M entries share a few thousand vertices: 450 us with an atomic per probe).  The linear hash
+// goes to hash_lo / hash_hi for the numbering.
 template <int MAXD>
 __global__ void __launch_bounds__(256) k_insert(const int32_t* __restrict__ perm,
                                                 const int16_t* __restrict__ rem0,
                                                 const uint8_t* __restrict__ rank, int64_t nD,
                                                 int d, unsigned long long* __restrict__ table,
                                                 uint64_t mask, int32_t* __restrict__ entry_slot,
+                                                uint32_t* __restrict__ hash_lo,
+                                                uint32_t* __restrict__ hash_hi,
                                                 unsigned* __restrict__ err) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -466,19 +472,23 @@ __global__ void __launch_bounds__(256) k_insert(const int32_t* __restrict__ perm
   const int k = (int)(e % D);
   int key[MAXD];
   for (int c = 0; c < D; ++c) key[c] = vertex_coord(rem0 + i * D, rank + i * D, d, k, c);
-  const uint64_t h = mix64(lin_hash(key, D));
+  const uint64_t lin = lin_hash(key, D);
+  hash_lo[e] = (uint32_t)lin;
+  hash_hi[e] = (uint32_t)(lin >> 32);
+  const uint64_t h = mix64(lin);
   const uint32_t tag = (uint32_t)(h >> 33);
   const unsigned long long mine = ((unsigned long long)tag << 32) | (uint32_t)e;
   uint64_t slot = h & mask;
   for (uint64_t probe = 0; probe <= mask; ++probe) {
-    const unsigned long long prev = atomicCAS(&table[slot], kEmpty, mine);
+    unsigned long long prev = __ldcg(&table[slot]);
+    if (prev == kEmpty) prev = atomicCAS(&table[slot], kEmpty, mine);
     if (prev == kEmpty) {
       entry_slot[e] = (int32_t)slot;
       return;
     }
     if ((uint32_t)(prev >> 32) == tag &&
         entry_has_key<MAXD>((uint32_t)prev, key, d, perm, rem0, rank)) {
-      atomicMin(&table[slot], mine);
+      if (mine < prev) atomicMin(&table[slot], mine);
       entry_slot[e] = (int32_t)slot;
       return;
     }
@@ -501,47 +511,43 @@ __global__ void k_owner_flags(const int32_t* __restrict__ entry_slot,
   flags[e] = (s >= 0 && (uint32_t)table[s] == (uint32_t)e) ? 1u : 0u;
 }
 
-__global__ void k_assign_ids(const uint32_t* __restrict__ scanned,
-                             const int32_t* __restrict__ entry_slot,
-                             const unsigned long long* __restrict__ table,
-                             const int32_t* __restrict__ perm, const int16_t* __restrict__ rem0,
-                             const uint8_t* __restrict__ rank, int64_t nD, int d,
-                             int32_t* __restrict__ slot_id, int16_t* __restrict__ keys,
-                             uint64_t* __restrict__ vhash, uint32_t* __restrict__ owner) {
+// Owners of a warp have consecutive ids, so their key rows are one piece of memory, which the
+// warp writes element by element (m = 10.5M, d = 20, 441 MB: 764 us with each thread writing its
+// own 42-byte row, hashing it and looking its slot up again).  An entry owns its vertex where the
+// scan steps.
+constexpr int kAssignThreads = 256;
+__global__ void __launch_bounds__(kAssignThreads)
+    k_assign_ids(const uint32_t* __restrict__ scanned, const uint32_t* __restrict__ total,
+                 const int32_t* __restrict__ entry_slot, const int32_t* __restrict__ perm,
+                 const int16_t* __restrict__ rem0, const uint8_t* __restrict__ rank,
+                 const uint32_t* __restrict__ hash_lo, const uint32_t* __restrict__ hash_hi,
+                 int64_t nD, int d, int32_t* __restrict__ slot_id, int16_t* __restrict__ keys,
+                 uint64_t* __restrict__ vhash, uint32_t* __restrict__ owner) {
   pdl_enter();
+  __shared__ int2 from[kAssignThreads / 32][32];  // (point, vertex) of the warp's owners in order
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nD) return;
-  const int32_t s = entry_slot[e];
-  if (s < 0 || (uint32_t)table[s] != (uint32_t)e) return;
   const int D = d + 1;
-  const uint32_t id = scanned[e];
-  slot_id[s] = (int32_t)id;
-  owner[id] = (uint32_t)e;
-  const int64_t i = perm[e / D];
-  const int k = (int)(e % D);
-  uint64_t h = 0;
-  int16_t* row = keys + (int64_t)id * D;
-  // the row's coordinates, stored two per 4-byte word where the row is 4-byte aligned
-  int c = 0;
-  if ((reinterpret_cast<uintptr_t>(row) & 3u) != 0) {
-    const int x = vertex_coord(rem0 + i * D, rank + i * D, d, k, 0);
-    row[0] = (int16_t)x;
-    h += coord_mult(0) * (uint64_t)(int64_t)x;
-    c = 1;
+  const uint32_t id = e < nD ? scanned[e] : 0u;
+  const uint32_t next = e + 1 < nD ? scanned[e + 1] : *total;
+  const bool own = e < nD && next != id;
+  const unsigned owners = __ballot_sync(0xffffffffu, own);
+  if (owners == 0) return;
+  if (own) {
+    from[warp][__popc(owners & ((1u << lane) - 1u))] = make_int2(perm[e / D], (int)(e % D));
+    slot_id[entry_slot[e]] = (int32_t)id;
+    owner[id] = (uint32_t)e;
+    vhash[id] = (uint64_t)hash_hi[e] << 32 | hash_lo[e];
   }
-  for (; c + 1 < D; c += 2) {
-    const int x0 = vertex_coord(rem0 + i * D, rank + i * D, d, k, c);
-    const int x1 = vertex_coord(rem0 + i * D, rank + i * D, d, k, c + 1);
-    *reinterpret_cast<uint32_t*>(row + c) =
-        (uint32_t)(uint16_t)(int16_t)x0 | ((uint32_t)(uint16_t)(int16_t)x1 << 16);
-    h += coord_mult(c) * (uint64_t)(int64_t)x0 + coord_mult(c + 1) * (uint64_t)(int64_t)x1;
+  __syncwarp();
+  int16_t* out = keys + (int64_t)__shfl_sync(0xffffffffu, id, __ffs(owners) - 1) * D;
+  const int many = __popc(owners) * D;
+  int row = lane / D, c = lane - row * D;
+  for (int q = lane; q < many; q += 32) {
+    const int2 p = from[warp][row];
+    out[q] = (int16_t)vertex_coord(rem0 + (int64_t)p.x * D, rank + (int64_t)p.x * D, d, p.y, c);
+    for (c += 32; c >= D; c -= D) ++row;
   }
-  if (c < D) {
-    const int x = vertex_coord(rem0 + i * D, rank + i * D, d, k, c);
-    row[c] = (int16_t)x;
-    h += coord_mult(c) * (uint64_t)(int64_t)x;
-  }
-  vhash[id] = h;
 }
 
 __global__ void k_entry_ids(const int32_t* __restrict__ entry_slot,
@@ -963,37 +969,63 @@ __global__ void k_splat_items(const uint32_t* __restrict__ sorted_entries,
   items[p] = make_int2((int)(e / D), __float_as_int(w[e]));
 }
 
-// Segment counts per vertex: total segments, partial slots, medium / huge flags.
-__global__ void k_seg_count(const int32_t* __restrict__ row_ptr, int64_t m,
-                            uint32_t* __restrict__ nseg, uint32_t* __restrict__ nslot,
-                            uint32_t* __restrict__ med, uint32_t* __restrict__ huge) {
-  pdl_enter();
-  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= m) return;
-  const int len = row_ptr[v + 1] - row_ptr[v];
-  const uint32_t c = (uint32_t)((len + kSplatSeg - 1) / kSplatSeg);
-  nseg[v] = c;
-  nslot[v] = c > 1 ? c : 0u;
-  med[v] = (c > 1 && c <= (uint32_t)kSplatMedSegs) ? 1u : 0u;
-  huge[v] = c > (uint32_t)kSplatMedSegs ? 1u : 0u;
+// What a vertex with the incidences [b, e) counts for: segments, partial slots, a medium and a
+// huge fix-up row (SEG_KINDS running counts).
+enum { SEG_ALL = 0, SEG_SLOT, SEG_MED, SEG_HUGE, SEG_KINDS };
+constexpr int kSegThreads = 512;  // vertices per block
+__device__ __forceinline__ void seg_counts(int b, int e, uint32_t (&c)[SEG_KINDS]) {
+  const uint32_t all = (uint32_t)((e - b + kSplatSeg - 1) / kSplatSeg);
+  c[SEG_ALL] = all;
+  c[SEG_SLOT] = all > 1 ? all : 0u;
+  c[SEG_MED] = (all > 1 && all <= (uint32_t)kSplatMedSegs) ? 1u : 0u;
+  c[SEG_HUGE] = all > (uint32_t)kSplatMedSegs ? 1u : 0u;
 }
 
-// After the exclusive scans: write every segment and the fix-up row lists.  A vertex of up to
+// Counts of each block of vertices, sums[kind][block], with a zero behind each row (its
+// exclusive scan is the row's total).  k_seg_fill counts again rather than reading offsets per
+// vertex: those are 32 bytes a vertex written and read for 4 read here (m = 10.5M: 390 us for
+// the counts, their scans and the fill, 90 with the block sums alone).
+__global__ void __launch_bounds__(kSegThreads) k_seg_sums(const int32_t* __restrict__ row_ptr,
+                                                          int64_t m, uint32_t* __restrict__ sums) {
+  pdl_enter();
+  const int64_t v = (int64_t)blockIdx.x * kSegThreads + threadIdx.x;
+  uint32_t c[SEG_KINDS] = {};
+  if (v < m) seg_counts(row_ptr[v], row_ptr[v + 1], c);
+  __shared__ uint32_t sum[SEG_KINDS][kSegThreads / 32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int q = 0; q < SEG_KINDS; ++q) {
+    const uint32_t t = __reduce_add_sync(0xffffffffu, c[q]);
+    if (lane == 0) sum[q][warp] = t;
+  }
+  __syncthreads();
+  if (warp < SEG_KINDS) {
+    const uint32_t t = __reduce_add_sync(0xffffffffu, lane < kSegThreads / 32 ? sum[warp][lane] : 0u);
+    uint32_t* row = sums + (int64_t)warp * (gridDim.x + 1);
+    if (lane == 0) row[blockIdx.x] = t;
+    if (lane == 0 && blockIdx.x == 0) row[gridDim.x] = 0;
+  }
+}
+
+// From the scanned sums: write every segment and the fix-up row lists.  A vertex of up to
 // 8 segments is written by its thread, a longer one by its warp (few dense vertices may hold
 // nearly all segments: n = 760k, d = 2, five vertices, 284 us with one thread each).
-__global__ void k_seg_fill(const int32_t* __restrict__ row_ptr, int64_t m,
-                           const uint32_t* __restrict__ seg_off,
-                           const uint32_t* __restrict__ slot_off,
-                           const uint32_t* __restrict__ med_off,
-                           const uint32_t* __restrict__ huge_off, int4* __restrict__ seg,
-                           int4* __restrict__ med_rows, int4* __restrict__ huge_rows) {
+__global__ void __launch_bounds__(kSegThreads)
+    k_seg_fill(const int32_t* __restrict__ row_ptr, int64_t m, const uint32_t* __restrict__ sums,
+               int4* __restrict__ seg, int4* __restrict__ med_rows, int4* __restrict__ huge_rows) {
   pdl_enter();
-  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t v = (int64_t)blockIdx.x * kSegThreads + threadIdx.x;
   const bool live = v < m;
   const int b = live ? row_ptr[v] : 0, e = live ? row_ptr[v + 1] : 0;
-  const int c = (e - b + kSplatSeg - 1) / kSplatSeg;
-  const int s0 = live ? (int)seg_off[v] : 0;
-  const int slot0 = c > 1 ? (int)slot_off[v] : -1;
+  uint32_t count[SEG_KINDS], at[SEG_KINDS] = {};
+  seg_counts(b, e, count);
+  const bool several = __syncthreads_or(count[SEG_ALL] > 1);
+#pragma unroll
+  for (int q = 0; q < SEG_KINDS; ++q)
+    if (q == SEG_ALL || several)
+      at[q] = sums[(int64_t)q * (gridDim.x + 1) + blockIdx.x] + block_exclusive_scan(count[q], nullptr);
+  const int c = (int)count[SEG_ALL], s0 = (int)at[SEG_ALL];
+  const int slot0 = c > 1 ? (int)at[SEG_SLOT] : -1;
   auto piece = [](int vertex, int first, int end, int slot, int j) {
     const int beg = first + j * kSplatSeg;
     return make_int4(vertex, beg, min(beg + kSplatSeg, end), slot >= 0 ? slot + j : -1);
@@ -1007,33 +1039,57 @@ __global__ void k_seg_fill(const int32_t* __restrict__ row_ptr, int64_t m,
     const int ss = __shfl_sync(0xffffffffu, s0, src), sl = __shfl_sync(0xffffffffu, slot0, src);
     for (int j = (int)(threadIdx.x & 31); j < cc; j += 32) seg[ss + j] = piece(vv, bb, ee, sl, j);
   }
-  if (c > 1 && c <= kSplatMedSegs) med_rows[med_off[v]] = make_int4((int)v, slot0, c, 0);
-  if (c > kSplatMedSegs) huge_rows[huge_off[v]] = make_int4((int)v, slot0, c, 0);
+  if (count[SEG_MED]) med_rows[at[SEG_MED]] = make_int4((int)v, slot0, c, 0);
+  if (count[SEG_HUGE]) huge_rows[at[SEG_HUGE]] = make_int4((int)v, slot0, c, 0);
 }
 
 // Within each window of kSegWindow consecutive segments, order the segments by length,
 // longest first (ties keep their order), so that the thread groups of a warp walk lists
 // of similar length and finish together.  Windows keep the vertex order of the lattice
 // at large, so the gathers of concurrently running warps stay local.  The splat's result
-// does not depend on the order in which segments are processed.
+// does not depend on the order in which segments are processed.  A counting sort: ranks by
+// comparison with the whole window are 128 steps a segment (10.5M segments: 238 us).
 constexpr int kSegWindow = 128;
 __global__ void __launch_bounds__(kSegWindow) k_seg_window_sort(const int4* __restrict__ in,
                                                                 int64_t nseg,
                                                                 int4* __restrict__ out) {
   pdl_enter();
-  __shared__ int len[kSegWindow];
+  constexpr int kWarps = kSegWindow / 32;
+  __shared__ int count[kWarps][kSplatSeg];  // [warp][kSplatSeg - length], then positions
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int b = threadIdx.x; b < kWarps * kSplatSeg; b += kSegWindow) (&count[0][0])[b] = 0;
   const int64_t s = (int64_t)blockIdx.x * kSegWindow + threadIdx.x;
-  const int4 sg = s < nseg ? in[s] : make_int4(0, 0, 0, 0);
-  const int mine = s < nseg ? sg.z - sg.y : -1;
-  len[threadIdx.x] = mine;
+  const bool live = s < nseg;
+  const int4 sg = live ? in[s] : make_int4(0, 0, 0, 0);
+  const int bin = live ? kSplatSeg - (sg.z - sg.y) : kSplatSeg;  // lengths are 1 .. kSplatSeg
   __syncthreads();
-  if (s >= nseg) return;
-  int rank = 0;
-  for (int j = 0; j < kSegWindow; ++j) {
-    const int o = len[j];
-    rank += (o > mine || (o == mine && j < (int)threadIdx.x)) ? 1 : 0;
+  const unsigned peers = __match_any_sync(0xffffffffu, bin);
+  const int before = __popc(peers & ((1u << lane) - 1u));
+  if (live && before == 0) count[warp][bin] = __popc(peers);
+  __syncthreads();
+  if (warp == 0) {
+    int run = 0;
+    for (int b0 = 0; b0 < kSplatSeg; b0 += 32) {
+      int c[kWarps], all = 0;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) all += c[w] = b0 + lane < kSplatSeg ? count[w][b0 + lane] : 0;
+      int inc = all;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      int at = run + inc - all;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) {
+        if (b0 + lane < kSplatSeg) count[w][b0 + lane] = at;
+        at += c[w];
+      }
+      run += __shfl_sync(0xffffffffu, inc, 31);
+    }
   }
-  out[(int64_t)blockIdx.x * kSegWindow + rank] = sg;
+  __syncthreads();
+  if (live) out[(int64_t)blockIdx.x * kSegWindow + count[warp][bin] + before] = sg;
 }
 
 __global__ void k_iota(uint32_t* __restrict__ out, int64_t count) {
@@ -1238,7 +1294,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   SGP_CHECK(tmp.get(&entry_slot, nD), "alloc entry slots");
   SGP_CHECK(cudaMemsetAsync(table, 0xff, cap * sizeof(unsigned long long), st), "memset table");
   SGP_DISPATCH_D(D, k_insert, (unsigned)ceil_div(nD, 256), 256, st, L->perm, rem0, rank, nD, d,
-                 table, mask, entry_slot, L->err);
+                 table, mask, entry_slot, ka, va, L->err);  // ka, va: free until the sorts below
   SGP_CHECK(cudaGetLastError(), "k_insert");
 
   // 4. numbering
@@ -1268,8 +1324,8 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   SGP_CHECK(tmp.get(&vhash, m), "alloc vertex hashes");
   uint32_t* owner = nullptr;  // [m] first entry of each vertex
   SGP_CHECK(tmp.get(&owner, m), "alloc owners");
-  launch_pdl(k_assign_ids, (unsigned)ceil_div(nD, 256), 256, st, flags, entry_slot, table, L->perm,
-             rem0, rank, nD, d, slot_id, L->keys, vhash, owner);
+  launch_pdl(k_assign_ids, (unsigned)ceil_div(nD, kAssignThreads), kAssignThreads, st, flags, total,
+             entry_slot, L->perm, rem0, rank, ka, va, nD, d, slot_id, L->keys, vhash, owner);
   note_launches(1);
   SGP_CHECK(dalloc(&L->idx, nD, st), "alloc idx");
   SGP_CHECK(dalloc(&L->w, nD, st), "alloc w");
@@ -1351,35 +1407,31 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
   // 7. splat segments (load balance)
   unsigned long long pairs = 0;  // (v, v + u_j) pairs: at least as many active vertices
   {
-    uint32_t *cnt, *slots, *med, *huge, *tot;
-    SGP_CHECK(tmp.get(&cnt, m), "alloc seg");
-    SGP_CHECK(tmp.get(&slots, m), "alloc seg");
-    SGP_CHECK(tmp.get(&med, m), "alloc seg");
-    SGP_CHECK(tmp.get(&huge, m), "alloc seg");
-    SGP_CHECK(tmp.get(&tot, 4), "alloc seg");
-    launch_pdl(k_seg_count, (unsigned)ceil_div(m, 256), 256, st, L->row_ptr, m, cnt, slots, med, huge);
+    const int64_t blocks = std::max<int64_t>(1, ceil_div(m, (int64_t)kSegThreads));
+    uint32_t* sums;
+    SGP_CHECK(tmp.get(&sums, SEG_KINDS * (blocks + 1)), "alloc seg");
+    launch_pdl(k_seg_sums, (unsigned)blocks, kSegThreads, st, L->row_ptr, m, sums);
     note_launches(1);
-    uint32_t* const counted[4] = {cnt, slots, med, huge};
-    uint32_t* const sums[4] = {tot, tot + 1, tot + 2, tot + 3};
-    exclusive_scans_u32(counted, sums, 4, m, rt, st);  // rt holds nD / 8 and more
-    uint32_t ht[4];
-    SGP_CHECK(cudaMemcpyAsync(ht, tot, sizeof(ht), cudaMemcpyDeviceToHost, st), "read seg");
+    exclusive_scan_rows_u32(sums, SEG_KINDS, blocks + 1, st);
+    uint32_t ht[SEG_KINDS];
+    SGP_CHECK(cudaMemcpy2DAsync(ht, sizeof(uint32_t), sums + blocks, (blocks + 1) * sizeof(uint32_t),
+                                sizeof(uint32_t), SEG_KINDS, cudaMemcpyDeviceToHost, st),
+              "read seg");
     SGP_CHECK(cudaMemcpyAsync(&pairs, counts + 2 * D, sizeof(pairs), cudaMemcpyDeviceToHost, st),
               "read pairs");
     SGP_CHECK(cudaStreamSynchronize(st), "sync seg");
-    L->nseg = ht[0];
-    L->nslots = ht[1];
-    L->nmed = ht[2];
-    L->nhuge = ht[3];
+    L->nseg = ht[SEG_ALL];
+    L->nslots = ht[SEG_SLOT];
+    L->nmed = ht[SEG_MED];
+    L->nhuge = ht[SEG_HUGE];
     SGP_CHECK(dalloc(&L->seg, L->nseg, st), "alloc seg");
     SGP_CHECK(dalloc(&L->med_rows, L->nmed, st), "alloc seg");
     SGP_CHECK(dalloc(&L->huge_rows, L->nhuge, st), "alloc seg");
     L->bytes += (L->nseg + L->nmed + L->nhuge) * sizeof(int4);
     int4* seg_unsorted = nullptr;
     SGP_CHECK(tmp.get(&seg_unsorted, std::max<int64_t>(L->nseg, 1)), "alloc seg");
-    launch_pdl(k_seg_fill, (unsigned)ceil_div(m, 256), 256, st, L->row_ptr, m, cnt, slots, med, huge,
-                                                          seg_unsorted, L->med_rows,
-                                                          L->huge_rows);
+    launch_pdl(k_seg_fill, (unsigned)blocks, kSegThreads, st, L->row_ptr, m, sums, seg_unsorted,
+               L->med_rows, L->huge_rows);
     if (L->nseg > 0)
       launch_pdl(k_seg_window_sort, (unsigned)ceil_div(L->nseg, kSegWindow), kSegWindow, st, 
           seg_unsorted, L->nseg, L->seg);

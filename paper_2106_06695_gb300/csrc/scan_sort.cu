@@ -8,7 +8,6 @@ namespace {
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanThreads * kScanItems;
-constexpr int kScanMany = 4;
 
 constexpr int kSortThreads = 512;
 constexpr int kSortWarps = kSortThreads / 32;
@@ -16,47 +15,9 @@ constexpr int kSortBatches = 8;                       // 32-item batches per war
 constexpr int kSortTile = kSortThreads * kSortBatches;  // 4096 items per block
 constexpr int kSortSelf = 128;  // up to this many blocks the scatter sums the histograms itself
 
-// Exclusive block scan of one value per thread; returns the block total in *total.
-__device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
-  __shared__ uint32_t warp_sums[32];
-  __shared__ uint32_t block_total;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t inc = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
-  }
-  if (lane == 31) warp_sums[warp] = inc;
-  __syncthreads();
-  const int nwarps = blockDim.x >> 5;
-  if (warp == 0) {
-    uint32_t s = lane < nwarps ? warp_sums[lane] : 0u;
-    uint32_t si = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, si, o);
-      if (lane >= o) si += t;
-    }
-    if (lane < nwarps) warp_sums[lane] = si - s;
-    if (lane == 31) block_total = si;  // nwarps <= 32
-  }
-  __syncthreads();
-  const uint32_t res = warp_sums[warp] + inc - v;
-  if (total) *total = block_total;
-  __syncthreads();
-  return res;
-}
-
-// Up to kScanMany arrays of one length scanned by the same launches (grid y: the array).
-struct ScanArrays {
-  uint32_t* data[kScanMany];
-  uint32_t* total[kScanMany];  // device, may be null
-};
-
-__global__ void k_scan_reduce(ScanArrays a, int64_t n, uint32_t* __restrict__ block_sums) {
+__global__ void k_scan_reduce(const uint32_t* __restrict__ data, int64_t n,
+                              uint32_t* __restrict__ block_sums) {
   pdl_enter();
-  const uint32_t* data = a.data[blockIdx.y];
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
   uint32_t s = 0;
 #pragma unroll
@@ -64,10 +25,10 @@ __global__ void k_scan_reduce(ScanArrays a, int64_t n, uint32_t* __restrict__ bl
     if (base + i < n) s += data[base + i];
   uint32_t total;
   block_exclusive_scan(s, &total);
-  if (threadIdx.x == 0) block_sums[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = total;
+  if (threadIdx.x == 0) block_sums[blockIdx.x] = total;
 }
 
-// Exclusive scan of the block sums in place (more blocks than k_scan_down adds up itself).
+// Exclusive scan in place of the rows of n sums, a block each.
 __global__ void k_scan_top(uint32_t* __restrict__ block_sums, int64_t nb) {
   pdl_enter();
   block_sums += blockIdx.y * nb;
@@ -95,10 +56,10 @@ __global__ void k_scan_top(uint32_t* __restrict__ block_sums, int64_t nb) {
 // SELF: the block adds up the sums of the blocks before it, one a thread (up to kScanThreads
 // blocks; a launch less than with k_scan_top, 2.5 us).
 template <bool SELF>
-__global__ void k_scan_down(ScanArrays a, int64_t n, const uint32_t* __restrict__ block_sums) {
+__global__ void k_scan_down(uint32_t* __restrict__ data, int64_t n,
+                            const uint32_t* __restrict__ block_sums,
+                            uint32_t* __restrict__ total) {
   pdl_enter();
-  uint32_t* data = a.data[blockIdx.y];
-  block_sums += (int64_t)blockIdx.y * gridDim.x;
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
   uint32_t v[kScanItems];
   uint32_t s = 0;
@@ -117,8 +78,7 @@ __global__ void k_scan_down(ScanArrays a, int64_t n, const uint32_t* __restrict_
     if (base + i < n) data[base + i] = run;
     run += v[i];
   }
-  if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1 && a.total[blockIdx.y])
-    *a.total[blockIdx.y] = before + mine;
+  if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1 && total) *total = before + mine;
 }
 
 // Digit counts of each block's items: [digit][block] for the scan, [block][digit] with SELF.
@@ -265,31 +225,27 @@ __global__ void __launch_bounds__(kSortThreads)
 
 size_t scan_temp_elems(int64_t n) { return (size_t)ceil_div(n > 0 ? n : 1, kScanTile); }
 
-void exclusive_scans_u32(uint32_t* const* data, uint32_t* const* totals, int count, int64_t n,
-                         uint32_t* tmp, cudaStream_t st) {
+void exclusive_scan_u32(uint32_t* data, int64_t n, uint32_t* total, uint32_t* tmp,
+                        cudaStream_t st) {
   if (n <= 0) {
-    for (int i = 0; i < count; ++i)
-      if (totals[i]) cudaMemsetAsync(totals[i], 0, sizeof(uint32_t), st);
+    if (total) cudaMemsetAsync(total, 0, sizeof(uint32_t), st);
     return;
   }
-  ScanArrays a{};
-  for (int i = 0; i < count; ++i) a.data[i] = data[i], a.total[i] = totals[i];
   const int64_t nb = ceil_div(n, kScanTile);
-  const dim3 grid((unsigned)nb, (unsigned)count);
-  launch_pdl(k_scan_reduce, grid, kScanThreads, st, a, n, tmp);
+  launch_pdl(k_scan_reduce, (unsigned)nb, kScanThreads, st, data, n, tmp);
   if (nb <= kScanThreads) {
-    launch_pdl(k_scan_down<true>, grid, kScanThreads, st, a, n, tmp);
+    launch_pdl(k_scan_down<true>, (unsigned)nb, kScanThreads, st, data, n, tmp, total);
     note_launches(2);
     return;
   }
-  launch_pdl(k_scan_top, dim3(1, (unsigned)count), kScanThreads, st, tmp, nb);
-  launch_pdl(k_scan_down<false>, grid, kScanThreads, st, a, n, tmp);
+  launch_pdl(k_scan_top, 1, kScanThreads, st, tmp, nb);
+  launch_pdl(k_scan_down<false>, (unsigned)nb, kScanThreads, st, data, n, tmp, total);
   note_launches(3);
 }
 
-void exclusive_scan_u32(uint32_t* data, int64_t n, uint32_t* total, uint32_t* tmp,
-                        cudaStream_t st) {
-  exclusive_scans_u32(&data, &total, 1, n, tmp, st);
+void exclusive_scan_rows_u32(uint32_t* data, int rows, int64_t n, cudaStream_t st) {
+  launch_pdl(k_scan_top, dim3(1, (unsigned)rows), kScanThreads, st, data, n);
+  note_launches(1);
 }
 
 size_t radix_temp_elems(int64_t n) {

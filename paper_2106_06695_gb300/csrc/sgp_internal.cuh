@@ -203,9 +203,8 @@ bool make_stencil(int kernel, int r, double spacing_override, double* s, double*
 size_t scan_temp_elems(int64_t n);
 void exclusive_scan_u32(uint32_t* data, int64_t n, uint32_t* total, uint32_t* tmp,
                         cudaStream_t st);
-// `count` (at most 4) such scans by the same launches; `tmp` holds count times as much.
-void exclusive_scans_u32(uint32_t* const* data, uint32_t* const* totals, int count, int64_t n,
-                         uint32_t* tmp, cudaStream_t st);
+// Exclusive scans in place of `rows` rows of n values, one block each (block sums).
+void exclusive_scan_rows_u32(uint32_t* data, int rows, int64_t n, cudaStream_t st);
 // Stable LSD radix sort of (key, value) pairs by bits begin .. end - 1 of the key (8 at a
 // time, so up to 7 more).  Uses the *_alt buffers as ping-pong storage; returns true when the
 // result ended in *_alt.
@@ -355,6 +354,38 @@ sgp_status run_logdet(Lattice* L, const float* Z, int s, float noise, int max_la
                       float tol, double* logdet, double* quad);
 
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// Exclusive block scan of one value per thread; returns the block total in *total.
+__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
+  __shared__ uint32_t warp_sums[32];
+  __shared__ uint32_t block_total;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) warp_sums[warp] = inc;
+  __syncthreads();
+  const int nwarps = blockDim.x >> 5;
+  if (warp == 0) {
+    uint32_t s = lane < nwarps ? warp_sums[lane] : 0u;
+    uint32_t si = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, si, o);
+      if (lane >= o) si += t;
+    }
+    if (lane < nwarps) warp_sums[lane] = si - s;
+    if (lane == 31) block_total = si;  // nwarps <= 32
+  }
+  __syncthreads();
+  const uint32_t res = warp_sums[warp] + inc - v;
+  if (total) *total = block_total;
+  __syncthreads();
+  return res;
+}
 
 // Per-column sums of per-thread fp64 partials inside one block, for kernels whose threads
 // own VEC consecutive columns of one row: thread t owns columns (t % G) VEC .. + VEC - 1
