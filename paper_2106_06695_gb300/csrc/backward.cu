@@ -29,6 +29,7 @@ namespace {
 constexpr int kBT = 128;
 constexpr int kDlsBlocks = 2 * 152;
 constexpr int kFilterChunk = 256;  // columns per filtering product
+constexpr size_t kPairBytes = 32u << 20;  // lattice values of two dense blurs done as one
 
 template <class S, int VEC>
 __device__ __forceinline__ float row_dot2(const float* g, const S* bu, const float* v,
@@ -59,9 +60,10 @@ __device__ __forceinline__ float row_dot2(const float* g, const S* bu, const flo
 }
 
 // Exact derivative through the weights: one thread per point (locality order p); dX in
-// the caller's order.  f[j] = scale / sqrt((j+1)(j+2)) are the elevation factors.
+// the caller's order.  Rows of all four arrays are ld apart.  f[j] = scale / sqrt((j+1)(j+2)) are
+// the elevation factors.
 template <int MAXD, int VEC, class S>
-__global__ void __launch_bounds__(kBT) k_weight_grad(int64_t n, int d, int k,
+__global__ void __launch_bounds__(kBT) k_weight_grad(int64_t n, int d, int k, int ld,
                                                      const int32_t* __restrict__ perm,
                                                      const int32_t* __restrict__ idx,
                                                      const uint8_t* __restrict__ rank,
@@ -79,7 +81,7 @@ __global__ void __launch_bounds__(kBT) k_weight_grad(int64_t n, int d, int k,
   float dw[MAXD];
   for (int kk = 0; kk < D; ++kk) {
     const int64_t v = idx[p * D + kk];
-    dw[kk] = alpha * row_dot2<S, VEC>(Gp + p * k, BU + v * k, Vp + p * k, BS + v * k, k);
+    dw[kk] = alpha * row_dot2<S, VEC>(Gp + p * ld, BU + v * ld, Vp + p * ld, BS + v * ld, k);
   }
   double dy[MAXD];
   for (int c = 0; c < D; ++c) {
@@ -220,13 +222,13 @@ struct Work {
 };
 
 template <class S, int VEC>
-void launch_weight_grad(const Lattice* L, int k, const void* BU, const void* BS, const float* Vp,
+void launch_weight_grad(const Lattice* L, int k, int ld, const void* BU, const void* BS, const float* Vp,
                         const float* Gp, float alpha, const double* f, const float* ls, float* dX,
                         cudaStream_t st) {
   const unsigned grid = (unsigned)ceil_div(L->n, kBT);
   const int D = L->D;
 #define SGP_WG(MAXD)                                                                        \
-  launch_pdl(k_weight_grad<MAXD, VEC, S>, grid, kBT, st, L->n, L->d, k, L->perm, L->idx, L->rank, \
+  launch_pdl(k_weight_grad<MAXD, VEC, S>, grid, kBT, st, L->n, L->d, k, ld, L->perm, L->idx, L->rank, \
                                                     (const S*)BU, (const S*)BS, Vp, Gp,      \
                                                     alpha, f, ls, dX)
   if (D <= 8) SGP_WG(8);
@@ -261,25 +263,47 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
     sgp_status s = ensure_product(L, k, st);
     if (s != SGP_OK) return s;
     const int kp = value_cols(L, k);
-    const size_t vb = lattice_value_bytes(L, kp);
+    // B^T W^T G and B W^T V, each over its factor (both blurs have as many passes and the same
+    // centre tap: one factor).  The symmetric blur is its own transpose, so the two can share
+    // their passes as the halves of rows of 2 kp columns: half the launches, and rows of 32
+    // bytes (k = 8) at random places cost DRAM 64 either way (n = 500k, d = 20, k = 8: 84 passes
+    // of 22.3 us apart, 42 of 33.5 together).  Done where it takes no more memory than apart (in-place
+    // blurs) or little of it.
+    const int kp2 = 2 * kp;
+    const size_t vb = lattice_value_bytes(L, kp), vb2 = 2 * vb;
+    const bool pair = want_x && blur == SGP_BLUR_SYMMETRIC && !L->tight_cols && kp2 <= 256 &&
+                      (blur_in_place(L) || (!L->sparse && vb2 <= kPairBytes));
+    const int ld = pair ? kp2 : kp;
+    const size_t one = sizeof(float);
     void *b0 = nullptr, *b1 = nullptr;
     float *Vp = nullptr, *Gp = nullptr;
-    BW_CHECK(w.get(&b0, vb), "alloc lattice values");
-    BW_CHECK(w.get(&b1, vb), "alloc lattice values");
-    BW_CHECK(w.get(&Vp, (size_t)n * kp * sizeof(float)), "alloc V");
-    BW_CHECK(w.get(&Gp, (size_t)n * kp * sizeof(float)), "alloc G");
-    enqueue_permute(L, G, k, kp, Gp, st);
-    // B^T W^T G into (b0, b1), B W^T V into the handle's buffers, each over its factor (both
-    // blurs have as many passes and the same centre tap: one factor)
+    const void *BS = nullptr, *BU = nullptr;
     double scale = 1.0;
-    const void* BS = enqueue_splat_blur(L, Gp, kp, k, transpose_blur(blur), b0, b1, L->partial,
-                                        st, &scale);
+    if (pair) {
+      float* part = nullptr;
+      BW_CHECK(w.get(&b0, vb2), "alloc lattice values");
+      if (!blur_in_place(L)) BW_CHECK(w.get(&b1, vb2), "alloc lattice values");
+      BW_CHECK(w.get(&part, (size_t)L->nslots * kp2 * one), "alloc splat partials");
+      BW_CHECK(w.get(&Gp, (size_t)n * kp2 * one), "alloc G, V");
+      Vp = Gp + kp;
+      enqueue_permute_pair(L, G, V, k, kp, Gp, st);
+      BS = enqueue_splat_blur(L, Gp, kp2, kp2, blur, b0, b1, part, st, &scale);
+      BU = static_cast<const char*>(BS) + vb / L->m;
+    } else {
+      BW_CHECK(w.get(&b0, vb), "alloc lattice values");
+      BW_CHECK(w.get(&b1, vb), "alloc lattice values");
+      BW_CHECK(w.get(&Vp, (size_t)n * kp * one), "alloc V");
+      BW_CHECK(w.get(&Gp, (size_t)n * kp * one), "alloc G");
+      enqueue_permute(L, G, k, kp, Gp, st);
+      BS = enqueue_splat_blur(L, Gp, kp, k, transpose_blur(blur), b0, b1, L->partial, st, &scale);
+    }
     alpha = (float)(alpha * scale);
-    if (dV) enqueue_slice_caller(L, BS, k, kp, alpha, dV, st);
+    if (dV) enqueue_slice_caller(L, BS, k, kp, ld, alpha, dV, st);
     if (want_x) {
-      enqueue_permute(L, V, k, kp, Vp, st);
-      const void* BU = enqueue_splat_blur(L, Vp, kp, k, blur, L->lat[0], L->lat[1],
-                                          L->partial, st, &scale);
+      if (!pair) {
+        enqueue_permute(L, V, k, kp, Vp, st);
+        BU = enqueue_splat_blur(L, Vp, kp, k, blur, L->lat[0], L->lat[1], L->partial, st, &scale);
+      }
       const double scale = std::sqrt((double)(d * (d + 1))) / L->s;
       std::vector<double> hf(d);
       for (int j = 0; j < d; ++j) hf[j] = scale / std::sqrt((double)((j + 1) * (j + 2)));
@@ -290,11 +314,11 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
                "copy f");
       const bool v4 = kp % 4 == 0;
       if (L->value_dtype == SGP_VALUES_BF16) {
-        if (v4) launch_weight_grad<bf16, 4>(L, kp, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
-        else launch_weight_grad<bf16, 1>(L, kp, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
+        if (v4) launch_weight_grad<bf16, 4>(L, kp, ld, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
+        else launch_weight_grad<bf16, 1>(L, kp, ld, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
       } else {
-        if (v4) launch_weight_grad<float, 4>(L, kp, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
-        else launch_weight_grad<float, 1>(L, kp, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
+        if (v4) launch_weight_grad<float, 4>(L, kp, ld, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
+        else launch_weight_grad<float, 1>(L, kp, ld, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
       }
     }
   } else {  // SGP_GRAD_FILTER

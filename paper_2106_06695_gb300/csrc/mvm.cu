@@ -582,9 +582,9 @@ __device__ __forceinline__ typename Vec<VEC>::T slice_row(int64_t p, int D, int 
   return acc;
 }
 
-// out = alpha W lat (+ beta V when beta != 0; V's row perm[p] of ko columns if vperm, the caller's, else rows of k in locality order).  PERM: out has the caller's
-// ko columns and row order (row perm[p]), written one value at a time unless WIDE (ko = k,
-// aligned rows); else out is [n][k] in locality order.
+// out = alpha W lat (+ beta Vp when beta != 0, rows of k in locality order) for the first G VEC of
+// lat's k columns.  PERM: out has the caller's ko columns and row order (row perm[p]), written one
+// value at a time unless WIDE (ko = G VEC, aligned rows); else out is [n][k] in locality order.
 template <int VEC, bool PERM, bool WIDE, class S>
 __global__ void __launch_bounds__(kThreads) k_slice(int64_t n, int G, int k, int ko, int D,
                                                     const int32_t* __restrict__ perm,
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(kThreads) k_slice(int64_t n, int G, int k, int
   typename Vt::T res = Vt::scale(alpha, acc);
   if (beta != 0.f) res = Vt::fma(beta, Vt::ld(Vp + p * k + col), res);
   if constexpr (!PERM || WIDE) {
-    Vt::st(out + i * k + col, res);
+    Vt::st(out + i * (PERM ? ko : k) + col, res);
   } else {
     const float* rr = reinterpret_cast<const float*>(&res);
 #pragma unroll
@@ -670,6 +670,34 @@ __global__ void __launch_bounds__(kThreads) k_permute_rows(int64_t n, int G, int
       if (col + j < ki) xx[j] = V[i * ki + col + j];
   }
   Vt::st(Vp + p * k + col, x);
+}
+
+// Out[p] = (A[perm[p]], B[perm[p]]): the caller's rows of two arrays (ki columns each, padded with
+// zero columns to kp) side by side.  VEC divides kp; WIDE: ki = kp and aligned rows.
+template <int VEC, bool WIDE>
+__global__ void __launch_bounds__(kThreads) k_permute_pair(int64_t n, int G, int kp, int ki,
+                                                           const int32_t* __restrict__ perm,
+                                                           const float* __restrict__ A,
+                                                           const float* __restrict__ B,
+                                                           float* __restrict__ out) {
+  pdl_enter();
+  using Vt = Vec<VEC>;
+  const int64_t p = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
+  if (p >= n) return;
+  const int at = (int)(threadIdx.x % G) * VEC;
+  const float* src = at < kp ? A : B;
+  const int col = at < kp ? at : at - kp;
+  const int64_t i = perm[p];
+  typename Vt::T x = Vt::zero();
+  if constexpr (WIDE) {
+    x = Vt::ld(src + i * ki + col);
+  } else {
+    float* xx = reinterpret_cast<float*>(&x);
+#pragma unroll
+    for (int j = 0; j < VEC; ++j)
+      if (col + j < ki) xx[j] = src[i * ki + col + j];
+  }
+  Vt::st(out + p * 2 * kp + at, x);
 }
 
 // Columns per thread and launch shape for rows of kp columns in library buffers (16-byte
@@ -760,19 +788,20 @@ void launch_blur_t(const Lattice* L, int j, const Taps& taps, const S* in, S* ou
 }
 
 // out = alpha W lat + beta Vp (Vp in locality order, rows of kp).  PERM: out is the caller's
-// [n][k]; else [n][kp] in locality order.
+// [n][k]; else [n][kp] in locality order.  lat_cols: columns of a row of lat (0: kp).
 template <bool PERM, class S>
 void launch_slice_t(const Lattice* L, const S* lat, const float* Vp, int k, int kp, float alpha,
-                    float beta, float* out, cudaStream_t st) {
+                    float beta, float* out, cudaStream_t st, int lat_cols = 0) {
+  if (lat_cols == 0) lat_cols = kp;
   const RowShape q = row_shape(L->n, kp);
   if (!Vp) beta = 0.f;
   by_vec(q.vec, [&](auto vec) {
     constexpr int VEC = decltype(vec)::value;
     if (!PERM || wide_ok(k, kp, out))
-      launch_pdl(k_slice<VEC, PERM, true, S>, q.blocks, q.threads, st, L->n, q.G, kp, k, L->D,
+      launch_pdl(k_slice<VEC, PERM, true, S>, q.blocks, q.threads, st, L->n, q.G, lat_cols, k, L->D,
                  L->perm, L->idx, L->w, lat, Vp, alpha, beta, out);
     else
-      launch_pdl(k_slice<VEC, PERM, false, S>, q.blocks, q.threads, st, L->n, q.G, kp, k, L->D,
+      launch_pdl(k_slice<VEC, PERM, false, S>, q.blocks, q.threads, st, L->n, q.G, lat_cols, k, L->D,
                  L->perm, L->idx, L->w, lat, Vp, alpha, beta, out);
   });
   note_launches(1);
@@ -1118,12 +1147,28 @@ void enqueue_permute(const Lattice* L, const float* V, int k, int kp, float* Vp,
   launch_permute(L, V, k, kp, Vp, st);
 }
 
-void enqueue_slice_caller(const Lattice* L, const void* lat, int k, int kp, float alpha, float* out,
-                          cudaStream_t st) {
+void enqueue_permute_pair(const Lattice* L, const float* A, const float* B, int k, int kp,
+                          float* out, cudaStream_t st) {
+  const int vec = kp % 4 == 0 ? 4 : 1;
+  const int G = 2 * kp / vec, rows = kThreads / G;
+  const unsigned blocks = (unsigned)ceil_div(L->n, rows);
+  auto go = [&](auto kernel) {
+    launch_pdl(kernel, blocks, rows * G, st, L->n, G, kp, k, L->perm, A, B, out);
+  };
+  if (vec == 4 && wide_ok(k, kp, A) && wide_ok(k, kp, B)) go(k_permute_pair<4, true>);
+  else if (vec == 4) go(k_permute_pair<4, false>);
+  else go(k_permute_pair<1, false>);
+  note_launches(1);
+}
+
+bool blur_in_place(const Lattice* L) { return L->sparse && chains_ok(L); }
+
+void enqueue_slice_caller(const Lattice* L, const void* lat, int k, int kp, int lat_cols,
+                          float alpha, float* out, cudaStream_t st) {
   if (L->value_dtype == SGP_VALUES_BF16)
-    launch_slice_t<true, bf16>(L, (const bf16*)lat, nullptr, k, kp, alpha, 0.f, out, st);
+    launch_slice_t<true, bf16>(L, (const bf16*)lat, nullptr, k, kp, alpha, 0.f, out, st, lat_cols);
   else
-    launch_slice_t<true, float>(L, (const float*)lat, nullptr, k, kp, alpha, 0.f, out, st);
+    launch_slice_t<true, float>(L, (const float*)lat, nullptr, k, kp, alpha, 0.f, out, st, lat_cols);
 }
 
 size_t lattice_value_bytes(const Lattice* L, int k) { return (size_t)L->m * k * value_size(L); }

@@ -255,13 +255,16 @@ void enqueue_mvm_into(const Lattice* L, const float* V, int k, int blur, float a
 // Pieces of the operator for the backward: splat a locality-ordered Vp (rows of kp) and blur
 // it (the result ends in the returned buffer, lat0 or lat1, of the handle's value type; kt
 // as enqueue_mvm's tree_k; the blurred values are *scale times what the buffer holds); gather
-// the caller's rows of k into locality-ordered rows of kp;
-// out (caller's order, rows of k) = alpha W lat.
+// the caller's rows of k into locality-ordered rows of kp (two arrays: side by side, 2 kp
+// columns); out (caller's order, rows of k) = alpha W lat, the first kp of lat's lat_cols columns.
 void* enqueue_splat_blur(const Lattice* L, const float* Vp, int kp, int kt, int blur, void* lat0,
                          void* lat1, float* partial, cudaStream_t st, double* scale);
 void enqueue_permute(const Lattice* L, const float* V, int k, int kp, float* Vp, cudaStream_t st);
-void enqueue_slice_caller(const Lattice* L, const void* lat, int k, int kp, float alpha, float* out,
-                          cudaStream_t st);
+void enqueue_permute_pair(const Lattice* L, const float* A, const float* B, int k, int kp,
+                          float* out, cudaStream_t st);
+bool blur_in_place(const Lattice* L);  // enqueue_splat_blur needs no second buffer (lat1)
+void enqueue_slice_caller(const Lattice* L, const void* lat, int k, int kp, int lat_cols,
+                          float alpha, float* out, cudaStream_t st);
 size_t lattice_value_bytes(const Lattice* L, int k);
 // Full operator on the handle's stream, allocating value buffers when needed.
 sgp_status run_mvm(Lattice* L, const float* V, int k, int blur, float alpha, float beta,
