@@ -14,9 +14,13 @@
 
 namespace sgp {
 
-int injected_fault() {
+int injected_fault(int* columns) {
   const char* f = getenv("SGP_FAULT");
   if (!f || !f[0]) return FAULT_NONE;
+  if (!strncmp(f, "cols_oom:", 9)) {
+    *columns = atoi(f + 9);
+    return FAULT_NONE;
+  }
   if (!strcmp(f, "oom")) return FAULT_OOM;
   if (!strcmp(f, "cuda_err")) return FAULT_CUDA;
   if (!strcmp(f, "hash_full")) return FAULT_HASH_FULL;
@@ -113,6 +117,11 @@ cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t st) {
   return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
+cudaError_t cols_malloc(const Lattice* L, int columns, void** p, size_t bytes, cudaStream_t st) {
+  if (L->fault_cols > 0 && columns > L->fault_cols) return cudaErrorMemoryAllocation;
+  return dev_malloc(p, bytes, st);
+}
+
 int64_t launches_so_far() { return g_launches.load(std::memory_order_relaxed); }
 
 sgp_status cuda_status(cudaError_t e, const char* what) {
@@ -188,7 +197,8 @@ sgp_status sgp_lattice_build(const float* X, const float* lengthscales, int64_t 
   }
   clear_pending_error();
   NvtxRange nvtx("sgp_build");
-  const int fault = injected_fault();
+  int fault_cols = 0;
+  const int fault = injected_fault(&fault_cols);
   if (fault == FAULT_OOM) {
     set_error("sgp_lattice_build: out of device memory (injected by SGP_FAULT=oom)");
     return SGP_ERR_OOM;
@@ -199,6 +209,7 @@ sgp_status sgp_lattice_build(const float* X, const float* lengthscales, int64_t 
   }
   Lattice* L = new Lattice();
   L->fault = fault;
+  L->fault_cols = fault_cols;
   L->n = n;
   L->d = d;
   L->D = d + 1;

@@ -22,7 +22,7 @@ enum : unsigned {
 
 // Faults injected on the host through SGP_FAULT (tests of the error paths).
 enum { FAULT_NONE = 0, FAULT_OOM, FAULT_CUDA, FAULT_HASH_FULL, FAULT_NAN_INPUT };
-int injected_fault();
+int injected_fault(int* columns);  // *columns: sgp_lattice::fault_cols
 
 // NVTX range for the lifetime of a scope (timeline profilers; no-op without one).
 struct NvtxRange {
@@ -66,6 +66,7 @@ struct sgp_lattice {
   int precond_power_iters = 1;
   uint64_t precond_seed = 0;
   int fault = 0;  // sgp::FAULT_* injected by SGP_FAULT into this lattice's construction
+  int fault_cols = 0;  // > 0: buffers of more columns than this fail to allocate (SGP_FAULT)
   int device = -1;  // CUDA device current at build time (the arrays live there)
   cudaStream_t stream = nullptr;
 
@@ -151,6 +152,8 @@ int64_t launches_so_far();
 // Stream-ordered device allocation from the library's pool on the current device (freed
 // with cudaFreeAsync; freed blocks stay mapped for reuse until sgp_trim_memory).
 cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t st);
+// The same for a buffer of `columns` columns that a call on L may fail to get.
+cudaError_t cols_malloc(const sgp_lattice* L, int columns, void** p, size_t bytes, cudaStream_t st);
 
 // ---- programmatic dependent launch ----
 // Back-to-back dependent kernels on one stream start about 4.1 us apart on GB300 when each
