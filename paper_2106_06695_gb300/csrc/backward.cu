@@ -214,8 +214,9 @@ struct Work {
     for (void* p : ptrs) (void)cudaFreeAsync(p, st);
   }
   template <class T>
-  cudaError_t get(T** p, size_t bytes) {
-    cudaError_t e = dev_malloc((void**)p, std::max<size_t>(bytes, 16), st);
+  cudaError_t get(T** p, size_t bytes, const Lattice* L = nullptr, int columns = 0) {
+    bytes = std::max<size_t>(bytes, 16);
+    cudaError_t e = L ? cols_malloc(L, columns, (void**)p, bytes, st) : dev_malloc((void**)p, bytes, st);
     if (e == cudaSuccess) ptrs.push_back((void*)*p);
     return e;
   }
@@ -246,11 +247,10 @@ int transpose_blur(int blur) {
                                       : SGP_BLUR_SYMMETRIC;
 }
 
-}  // namespace
-
-sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const float* V,
-                            const float* G, int k, int blur, float alpha, int grad, float* dV,
-                            float* dX, float* dls) {
+// may_pair: the symmetric blur's two products may share their passes; *paired: they did.
+sgp_status backward(Lattice* L, const float* X, const float* ls, const float* V, const float* G,
+                    int k, int blur, float alpha, int grad, float* dV, float* dX, float* dls,
+                    bool may_pair, bool* paired) {
   cudaStream_t st = L->stream;
   const int64_t n = L->n;
   const int d = L->d;
@@ -271,8 +271,10 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
     // blurs) or little of it.
     const int kp2 = 2 * kp;
     const size_t vb = lattice_value_bytes(L, kp), vb2 = 2 * vb;
-    const bool pair = want_x && blur == SGP_BLUR_SYMMETRIC && !L->tight_cols && kp2 <= 256 &&
+    const bool pair = may_pair && want_x && blur == SGP_BLUR_SYMMETRIC && !L->tight_cols &&
+                      kp2 <= 256 &&
                       (blur_in_place(L) || (!L->sparse && vb2 <= kPairBytes));
+    *paired = pair;
     const int ld = pair ? kp2 : kp;
     const size_t one = sizeof(float);
     void *b0 = nullptr, *b1 = nullptr;
@@ -281,19 +283,19 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
     double scale = 1.0;
     if (pair) {
       float* part = nullptr;
-      BW_CHECK(w.get(&b0, vb2), "alloc lattice values");
-      if (!blur_in_place(L)) BW_CHECK(w.get(&b1, vb2), "alloc lattice values");
-      BW_CHECK(w.get(&part, (size_t)L->nslots * kp2 * one), "alloc splat partials");
-      BW_CHECK(w.get(&Gp, (size_t)n * kp2 * one), "alloc G, V");
+      BW_CHECK(w.get(&b0, vb2, L, kp2), "alloc lattice values");
+      if (!blur_in_place(L)) BW_CHECK(w.get(&b1, vb2, L, kp2), "alloc lattice values");
+      BW_CHECK(w.get(&part, (size_t)L->nslots * kp2 * one, L, kp2), "alloc splat partials");
+      BW_CHECK(w.get(&Gp, (size_t)n * kp2 * one, L, kp2), "alloc G, V");
       Vp = Gp + kp;
       enqueue_permute_pair(L, G, V, k, kp, Gp, st);
       BS = enqueue_splat_blur(L, Gp, kp2, kp2, blur, b0, b1, part, st, &scale);
       BU = static_cast<const char*>(BS) + vb / L->m;
     } else {
-      BW_CHECK(w.get(&b0, vb), "alloc lattice values");
-      BW_CHECK(w.get(&b1, vb), "alloc lattice values");
-      BW_CHECK(w.get(&Vp, (size_t)n * kp * one), "alloc V");
-      BW_CHECK(w.get(&Gp, (size_t)n * kp * one), "alloc G");
+      BW_CHECK(w.get(&b0, vb, L, kp), "alloc lattice values");
+      BW_CHECK(w.get(&b1, vb, L, kp), "alloc lattice values");
+      BW_CHECK(w.get(&Vp, (size_t)n * kp * one, L, kp), "alloc V");
+      BW_CHECK(w.get(&Gp, (size_t)n * kp * one, L, kp), "alloc G");
       enqueue_permute(L, G, k, kp, Gp, st);
       BS = enqueue_splat_blur(L, Gp, kp, k, transpose_blur(blur), b0, b1, L->partial, st, &scale);
     }
@@ -359,6 +361,25 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
   }
   BW_CHECK(cudaGetLastError(), "launching the MVM backward");
   return SGP_OK;
+}
+
+}  // namespace
+
+// Where memory is short: without pairing, then without padded rows.  (A pass that ran out of memory
+// half way is done again from the start; it has written outputs only.)
+sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const float* V,
+                            const float* G, int k, int blur, float alpha, int grad, float* dV,
+                            float* dX, float* dls) {
+  bool paired = false;
+  auto run = [&](bool may_pair) {
+    return backward(L, X, ls, V, G, k, blur, alpha, grad, dV, dX, dls, may_pair, &paired);
+  };
+  sgp_status s = run(true);
+  if (s == SGP_ERR_OOM && paired) s = run(false);
+  if (s == SGP_ERR_OOM && (grad == SGP_GRAD_FILTER || padded_cols(k) != k) &&
+      give_up_padding(L, L->stream))
+    s = run(false);
+  return s;
 }
 
 }  // namespace sgp

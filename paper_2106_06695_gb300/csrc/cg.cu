@@ -384,7 +384,7 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
   // are rows of float4 and the MVM takes its vectorised kernels.  One or two Lanczos probes
   // (sgp_logdet) stay as they are; their huge vertices' sums keep the caller's k's shape.
   const int kb = k;
-  k = rec ? padded_cols(k) : (k + 3) / 4 * 4;
+  k = rec ? rec->cols : (k + 3) / 4 * 4;
   // CUDA graphs cannot be captured on the legacy default stream: use a private blocking
   // stream then (it is ordered with the legacy stream like any blocking stream).
   cudaStream_t st = L->stream;
@@ -413,7 +413,7 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
     }
   } cl{st, own, {}};
   auto get = [&](void** p, size_t bytes) {
-    cudaError_t e = dev_malloc(p, std::max<size_t>(bytes, 16), st);
+    cudaError_t e = cols_malloc(L, k, p, std::max<size_t>(bytes, 16), st);
     if (e == cudaSuccess) cl.ptrs.push_back(*p);
     return e;
   };

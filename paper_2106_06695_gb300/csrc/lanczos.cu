@@ -100,10 +100,9 @@ __global__ void __launch_bounds__(32) k_slq(const double* __restrict__ ha,
   if (lane == 0) part[c * kSlqWarps + w] = bnorm[c] * bnorm[c] * kSlqStep * sum;
 }
 
-}  // namespace
-
-sgp_status run_logdet(Lattice* L, const float* Z, int s, float noise, int max_lanczos, float tol,
-                      double* logdet, double* quad) {
+// sp: columns of the solver's rows (zero columns appended).
+sgp_status logdet_rows(Lattice* L, const float* Z, int s, int sp, float noise, int max_lanczos,
+                       float tol, double* logdet, double* quad) {
   cudaStream_t st = L->stream;
   const int cap = std::min(max_lanczos, kMaxLanczos);
   struct Bufs {
@@ -125,7 +124,7 @@ sgp_status run_logdet(Lattice* L, const float* Z, int s, float noise, int max_la
   } while (0)
   LanczosRecord rec{};
   rec.cap = cap;
-  const int sp = padded_cols(s);  // columns of the record (run_cg pads its vectors alike)
+  rec.cols = sp;
   float* X = nullptr;
   double* dq = nullptr;
   int* bad = nullptr;
@@ -163,6 +162,16 @@ sgp_status run_logdet(Lattice* L, const float* Z, int s, float noise, int max_la
     return SGP_ERR_NONFINITE;
   }
   return SGP_OK;
+}
+
+}  // namespace
+
+sgp_status run_logdet(Lattice* L, const float* Z, int s, float noise, int max_lanczos, float tol,
+                      double* logdet, double* quad) {
+  sgp_status st = logdet_rows(L, Z, s, value_cols(L, s), noise, max_lanczos, tol, logdet, quad);
+  if (st == SGP_ERR_OOM && padded_cols(s) != s && give_up_padding(L, L->stream))
+    st = logdet_rows(L, Z, s, s, noise, max_lanczos, tol, logdet, quad);
+  return st;
 }
 
 }  // namespace sgp

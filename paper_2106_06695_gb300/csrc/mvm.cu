@@ -1041,6 +1041,19 @@ size_t mvm_work_bytes(const Lattice* L, int k) {
          round256((size_t)L->nslots * k * sizeof(float)) + round256((size_t)L->n * k * sizeof(float));
 }
 
+void release_lattice_values(Lattice* L, cudaStream_t st) {
+  void** bufs[4] = {(void**)&L->lat[0], (void**)&L->lat[1], (void**)&L->partial,
+                    (void**)&L->vperm};
+  for (void** b : bufs) {
+    if (*b) cudaFreeAsync(*b, st);
+    *b = nullptr;
+  }
+  L->bytes -= L->lat_bytes;
+  L->lat_bytes = 0;
+  L->lat_elems = 0;
+  L->vperm_elems = 0;
+}
+
 sgp_status ensure_lattice_values(Lattice* L, int k, cudaStream_t st) {
   if (L->sparse && (!chains_ok(L) || L->table_blur) &&
       L->act_tmp_elems < (size_t)L->act_max * k) {
@@ -1054,16 +1067,9 @@ sgp_status ensure_lattice_values(Lattice* L, int k, cudaStream_t st) {
   }
   if (L->lat_elems >= (size_t)L->m * k && L->lat[0] && L->vperm_elems >= (size_t)L->n * k)
     return SGP_OK;
+  release_lattice_values(L, st);
   void** bufs[4] = {(void**)&L->lat[0], (void**)&L->lat[1], (void**)&L->partial,
                     (void**)&L->vperm};
-  for (void** b : bufs) {
-    if (*b) cudaFreeAsync(*b, st);
-    *b = nullptr;
-  }
-  L->bytes -= L->lat_bytes;
-  L->lat_bytes = 0;
-  L->lat_elems = 0;
-  L->vperm_elems = 0;
   const size_t vbytes = (size_t)L->m * k * value_size(L);
   const size_t sizes[4] = {vbytes, vbytes, (size_t)L->nslots * k * sizeof(float),
                            (size_t)L->n * k * sizeof(float)};
@@ -1178,12 +1184,17 @@ int padded_cols(int k) { return k <= 2 ? k : (k + 3) / 4 * 4; }
 
 int value_cols(const Lattice* L, int k) { return L->tight_cols ? k : padded_cols(k); }
 
+bool give_up_padding(Lattice* L, cudaStream_t st) {
+  if (L->tight_cols) return false;
+  L->tight_cols = true;
+  release_lattice_values(L, st);
+  return true;
+}
+
 sgp_status ensure_product(Lattice* L, int k, cudaStream_t st) {
   sgp_status s = ensure_lattice_values(L, value_cols(L, k), st);
-  if (s == SGP_ERR_OOM && !L->tight_cols && padded_cols(k) != k) {
-    L->tight_cols = true;  // no room for zero columns: products of this lattice go without
+  if (s == SGP_ERR_OOM && padded_cols(k) != k && give_up_padding(L, st))
     s = ensure_lattice_values(L, k, st);
-  }
   return s;
 }
 

@@ -226,6 +226,9 @@ sgp_status ensure_lattice_values(Lattice* L, int k, cudaStream_t st);
 // this lattice uses (k itself once the padded buffers did not fit).
 int padded_cols(int k);
 int value_cols(const Lattice* L, int k);
+// No room for zero columns: from now on this lattice's products go without, and the value
+// buffers are given back.  False when it was so before.
+bool give_up_padding(Lattice* L, cudaStream_t st);
 // ensure_lattice_values for a public k-column product (value_cols columns).
 sgp_status ensure_product(Lattice* L, int k, cudaStream_t st);
 // Enqueue out = alpha * W B W^T V + beta * V on `st` (buffers must be ready: ensure_product,
@@ -338,9 +341,11 @@ sgp_status run_mvm_backward(Lattice* L, const float* X, const float* ls, const f
 
 // ---- CG (cg.cu) ----
 // Device buffers that receive the CG coefficients of every column for the Lanczos
-// quadrature: alpha_j / beta_j of column c at [j][padded_cols(k)] for j < cap, ||b_c|| and the
-// iteration count per column.
+// quadrature: alpha_j / beta_j of column c at [j][cols] for j < cap, ||b_c|| and the
+// iteration count per column.  cols: what the solver rounds k up to (padded_cols(k), or k
+// itself where memory is short).
 struct LanczosRecord {
+  int cols;
   double* alpha;
   double* beta;
   int cap;
