@@ -42,12 +42,12 @@ constexpr int kThreads = 256;
 constexpr int kChunk = 8;
 
 // One thread-group of G = k / VEC threads per segment of at most kSplatSeg incidences;
-// blockDim.x is a multiple of G.
+// blockDim.x is a multiple of G.  scale: a power of two on the vertices' values (ChainRange).
 template <int VEC, class S>
 __global__ void __launch_bounds__(kThreads) k_splat(int64_t nseg, int G, int k,
                                                     const int4* __restrict__ seg,
                                                     const int2* __restrict__ items,
-                                                    const float* __restrict__ V,
+                                                    const float* __restrict__ V, float scale,
                                                     S* __restrict__ lat,
                                                     float* __restrict__ partial) {
   pdl_enter();
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kThreads) k_splat(int64_t nseg, int G, int k,
     for (int j = 0; j < kChunk; ++j)
       if (it[j].x >= 0) acc = Vt::fma(__int_as_float(it[j].y), row[j], acc);
   }
-  if (sg.w < 0) Vt::sts(lat + (int64_t)sg.x * k + col, acc);
+  if (sg.w < 0) Vt::sts(lat + (int64_t)sg.x * k + col, Vt::scale(scale, acc));
   else Vt::st(partial + (int64_t)sg.w * k + col, acc);
 }
 
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kThreads) k_splat_fix(int nhuge, int64_t nmed,
                                                         int k, const int4* __restrict__ huge_rows,
                                                         const int4* __restrict__ med_rows,
                                                         const float* __restrict__ partial,
-                                                        S* __restrict__ lat) {
+                                                        float scale, S* __restrict__ lat) {
   pdl_enter();
   using Vt = Vec<VEC>;
   __shared__ typename Vt::T red[kThreads];
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kThreads) k_splat_fix(int nhuge, int64_t nmed,
 #pragma unroll
     for (int j = 0; j < kSplatMedSegs; ++j)
       if (j < rw.z) acc = Vt::add(acc, x[j]);
-    Vt::sts(lat + (int64_t)rw.x * k + col, acc);
+    Vt::sts(lat + (int64_t)rw.x * k + col, Vt::scale(scale, acc));
     return;
   }
   const int4 rw = huge_rows[blockIdx.x];
@@ -125,7 +125,8 @@ __global__ void __launch_bounds__(kThreads) k_splat_fix(int nhuge, int64_t nmed,
       red[q] = Vt::add(red[q], red[q + half * G]);
     __syncthreads();
   }
-  for (int q = threadIdx.x; q < G; q += blockDim.x) Vt::sts(lat + (int64_t)rw.x * k + q * VEC, red[q]);
+  for (int q = threadIdx.x; q < G; q += blockDim.x)
+    Vt::sts(lat + (int64_t)rw.x * k + q * VEC, Vt::scale(scale, red[q]));
 }
 
 // ---- blur ----------------------------------------------------------------------------
@@ -395,7 +396,8 @@ __global__ void __launch_bounds__(1024) k_blur_cluster(ClusterBlur q, S* __restr
 // A vertex without a neighbour along a pass's direction is only scaled by the centre tap g0.
 // With fp32 values kept as y = x / g0^t after t passes such vertices do not change, a pass is
 // y[v] += (g1 / g0) (y[v - u_j] + y[v + u_j]) on the others, and the factor g0^passes is
-// applied once at the end (by the caller, through its alpha).
+// applied once at the end (by the caller, through its alpha).  ChainRange keeps y inside the
+// range that x has.
 //
 // One thread-group of G threads per chain v, v + u_j, v + 2 u_j, ...: it reads every row of the
 // chain once and writes it back in place, which no other group reads (chains are maximal).
@@ -726,16 +728,17 @@ void by_vec(int vec, F f) {
 }
 
 // ---- launchers -----------------------------------------------------------------------
+// scale: a power of two on the splatted values (1 but for fp32 chains).
 // kt: the column count that fixes the shape of the huge vertices' summation tree (the
 // caller's k, so that padding does not change a result).
 template <class S>
-void launch_splat_t(const Lattice* L, const float* V, int kp, int kt, S* lat, float* partial,
-                    cudaStream_t st) {
+void launch_splat_t(const Lattice* L, const float* V, int kp, int kt, float scale, S* lat,
+                    float* partial, cudaStream_t st) {
   by_vec(row_shape(1, kp).vec, [&](auto vec) {
     constexpr int VEC = decltype(vec)::value;
     const RowShape q = row_shape(L->nseg, kp);
-    launch_pdl(k_splat<VEC, S>, q.blocks, q.threads, st, L->nseg, q.G, kp, L->seg, L->items, V, lat,
-               partial);
+    launch_pdl(k_splat<VEC, S>, q.blocks, q.threads, st, L->nseg, q.G, kp, L->seg, L->items, V,
+               scale, lat, partial);
     note_launches(1);
     if (L->nmed > 0 || L->nhuge > 0) {
       const int gt = kt % 4 == 0 ? kt / 4 : kt;
@@ -743,7 +746,7 @@ void launch_splat_t(const Lattice* L, const float* V, int kp, int kt, S* lat, fl
       while (groups * 2 * gt <= kThreads) groups *= 2;
       const int64_t med_blocks = ceil_div(L->nmed, kThreads / q.G);
       launch_pdl(k_splat_fix<VEC, S>, (unsigned)(L->nhuge + med_blocks), kThreads, st, (int)L->nhuge,
-                 L->nmed, groups, q.G, kp, L->huge_rows, L->med_rows, partial, lat);
+                 L->nmed, groups, q.G, kp, L->huge_rows, L->med_rows, partial, scale, lat);
       note_launches(1);
     }
   });
@@ -888,6 +891,36 @@ bool blur_cluster_t(const Lattice* L, int blur, int passes, const Taps& tp, S* l
 // Sparse blurs run on chains (else on the direction lists).
 bool chains_ok(const Lattice* L) { return L->chain_max > 0 && L->chain_max <= kMaxChain; }
 
+// Centre and side tap of one pass.
+double tap0(const Lattice* L, int blur) { return (blur == SGP_BLUR_SYMMETRIC ? L->half : L->coef)[0]; }
+double tap1(const Lattice* L, int blur) { return (blur == SGP_BLUR_SYMMETRIC ? L->half : L->coef)[1]; }
+int pass_count(const Lattice* L, int blur) { return blur == SGP_BLUR_SYMMETRIC ? 2 * L->D : L->D; }
+
+// The values y = x / g0^t of fp32 chains grow past x by g0^-t (400 at d = 50 and the default
+// spacing, 3e22 at a spacing of 0.25): a product whose x has room in fp32 must not overflow in
+// y, nor its alpha g0^t underflow.  So the splat takes 2^-exponent off (exact, and no bit of a
+// product differs for it), with 2^exponent >= g0^-t, and the values are multiplied by g0^run
+// every `run` passes so that exponent <= 12 (never below 142 passes at the default spacing):
+// |y| <= |x|, and x down to 2^-114 keeps its 24 bits.
+struct ChainRange {
+  int run = 0;       // passes between rescalings (0: the values are x itself)
+  int exponent = 0;
+};
+template <class S>
+ChainRange chain_range(const Lattice* L, int blur, bool dense) {
+  const double g0 = tap0(L, blur);
+  if (!L->sparse || dense || !chains_ok(L) || std::is_same_v<S, bf16> || g0 >= 1.0) return {};
+  constexpr double kMaxExponent = 12.0;
+  const double bits = -std::log2(g0);  // growth of a pass
+  const int P = pass_count(L, blur);
+  const int most = std::max(1, (int)std::min<double>(P, kMaxExponent / bits));
+  const int runs = (P + most - 1) / most;
+  ChainRange c;
+  c.run = (P + runs - 1) / runs;
+  c.exponent = (int)std::ceil(c.run * bits);
+  return c;
+}
+
 // The blur passes of `blur` on the splatted values in lat0 (lat1: ping-pong buffer);
 // returns the buffer that holds the result divided by *scale.  Sparse lattices use their
 // chains or direction lists (lat1 unused) unless `dense` is set.
@@ -934,21 +967,18 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
     note_launches(1);
   };
   if (chains_ok(L)) {
-    const double g0 = blur == SGP_BLUR_SYMMETRIC ? L->half[0] : L->coef[0];
-    const double g1 = blur == SGP_BLUR_SYMMETRIC ? L->half[1] : L->coef[1];
-    // y / x = g0^-t grows with the passes: bring it back every kRescale passes (never for D
-    // <= 64) so that it stays far from the end of the exponent range
-    constexpr int kRescale = 64;
+    const double g0 = tap0(L, blur), g1 = tap1(L, blur);
+    const ChainRange range = chain_range<S>(L, blur, dense);
     int owed = 0;  // passes whose factor has not been applied
     by_vec(row_shape(1, k).vec, [&](auto vec) {
       constexpr int VEC = decltype(vec)::value;
       for (int t = 0; t < P; ++t) {
         const int j = dir(t);
         const int64_t count = L->chain_off[j + 1] - L->chain_off[j];
-        if (!lazy && g0 != 1.0 && P > 2 * kRescale && owed == kRescale) {
+        if (range.run > 0 && owed == range.run) {
           const RowShape q = row_shape(L->m, k);
           launch_pdl(k_rescale<VEC, S>, q.blocks, q.threads, st, L->m, q.G, k,
-                     (float)std::pow(g0, kRescale), lat0);
+                     (float)std::pow(g0, owed), lat0);
           note_launches(1);
           owed = 0;
         }
@@ -966,7 +996,7 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
       }
     });
     if (lazy) finish();
-    else *scale = std::pow(g0, owed);
+    else *scale = std::ldexp(std::pow(g0, owed), range.exponent);
     return lat0;
   }
   S* tmp = static_cast<S*>(L->act_tmp);
@@ -1004,7 +1034,8 @@ int enqueue_t(const Lattice* L, const float* V, int k, int kp, int kt, int blur,
     src = vperm;
   }
   if (ev) cudaEventRecordWithFlags(ev[2], st, cudaEventRecordExternal);
-  launch_splat_t<S>(L, src, kp, kt, lat0, partial, st);
+  const float take = std::ldexp(1.f, -chain_range<S>(L, blur, dense).exponent);
+  launch_splat_t<S>(L, src, kp, kt, take, lat0, partial, st);
   // External: inside a stream capture this becomes an event-record node of the graph
   if (ev) cudaEventRecordWithFlags(ev[0], st, cudaEventRecordExternal);
   int passes = 0;
@@ -1024,7 +1055,8 @@ int enqueue_t(const Lattice* L, const float* V, int k, int kp, int kt, int blur,
 template <class S>
 S* splat_blur_t(const Lattice* L, const float* Vp, int kp, int kt, int blur, S* lat0, S* lat1,
                 float* partial, cudaStream_t st, double* scale) {
-  launch_splat_t<S>(L, Vp, kp, kt, lat0, partial, st);
+  const float take = std::ldexp(1.f, -chain_range<S>(L, blur, false).exponent);
+  launch_splat_t<S>(L, Vp, kp, kt, take, lat0, partial, st);
   return blur_passes_t<S>(L, blur, lat0, lat1, kp, st, nullptr, false, scale);
 }
 
