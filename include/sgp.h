@@ -28,8 +28,9 @@
  *     a 1024-slot vertex table, so that the bounded probes of a larger lattice run out and
  *     the build returns SGP_ERR_HASH_FULL), "nan_input" (the elevation kernel treats the
  *     first point as NaN: SGP_ERR_NONFINITE), "cols_oom:<c>" (allocations of more than c
- *     columns fail in later calls on the lattice, as when memory is short).  None of them
- *     faults the device.
+ *     columns fail in later calls on the lattice, as when memory is short),
+ *     "no_cluster" (small lattices are blurred as on a device that holds no 16-block
+ *     cluster).  None of them faults the device.
  *   - Each stage pushes an NVTX range (sgp_build, sgp_mvm, sgp_cg, sgp_backward,
  *     sgp_logdet, sgp_serve_step) for timeline profilers.
  */

@@ -25,6 +25,7 @@ int injected_fault(int* columns) {
   if (!strcmp(f, "cuda_err")) return FAULT_CUDA;
   if (!strcmp(f, "hash_full")) return FAULT_HASH_FULL;
   if (!strcmp(f, "nan_input")) return FAULT_NAN_INPUT;
+  if (!strcmp(f, "no_cluster")) return FAULT_NO_CLUSTER;
   return FAULT_NONE;
 }
 

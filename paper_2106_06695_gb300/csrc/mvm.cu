@@ -845,12 +845,9 @@ void launch_permute(const Lattice* L, const float* V, int k, int kp, float* Vp, 
 // were never faster (m = 1k, d = 4: 38 us with one block, 31 with 16).
 constexpr int kClusterBlocks = 16, kClusterRows = 1024, kClusterGroups = 8;
 
-template <int VEC, int R, class S>
-cudaError_t launch_cluster(const ClusterBlur& q, int blocks, int groups, S* lat, cudaStream_t st) {
-  auto kernel = k_blur_cluster<VEC, R, S>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
-  cudaLaunchAttribute at[2]{};
+// Launch configuration of one cluster per column group; at: room for its two attributes.
+cudaLaunchConfig_t cluster_config(int blocks, int groups, int rows, cudaStream_t st,
+                                  cudaLaunchAttribute (&at)[2]) {
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   at[1].id = cudaLaunchAttributeClusterDimension;
@@ -858,34 +855,64 @@ cudaError_t launch_cluster(const ClusterBlur& q, int blocks, int groups, S* lat,
   at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)blocks, (unsigned)groups);
-  cfg.blockDim = (unsigned)(ceil_div(q.rows, 32) * 32);
+  cfg.blockDim = (unsigned)(ceil_div(rows, 32) * 32);
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kernel, q, lat);
+  return cfg;
 }
 
-// All passes on lat0 by k_blur_cluster; false when the lattice is not of its size.
+// Whether the current device can hold the largest cluster (on a partitioned one it may have
+// too few SMs together): asked before the first launch, because inside a stream capture a
+// launch is only recorded and would fail when the graph runs.
+template <int VEC, int R, class S>
+bool cluster_fits() {
+  static std::atomic<int> cache[64];  // 0: not asked yet, 1: fits, 2: does not
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  if (const int c = cache[dev].load()) return c == 1;
+  if (cudaPeekAtLastError() != cudaSuccess) return false;  // left for the caller's check
+  auto kernel = k_blur_cluster<VEC, R, S>;
+  cudaLaunchAttribute at[2]{};
+  const cudaLaunchConfig_t cfg = cluster_config(kClusterBlocks, 1, kClusterRows, nullptr, at);
+  int clusters = 0;
+  const bool fits =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+          cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0;
+  if (!fits) clear_pending_error();  // of these two calls
+  cache[dev].store(fits ? 1 : 2);
+  return fits;
+}
+
+// All passes on lat0 by k_blur_cluster; false when the lattice is not of its size, or the device
+// has no room for its clusters.
 template <class S>
 bool blur_cluster_t(const Lattice* L, int blur, int passes, const Taps& tp, S* lat0, int k,
                     cudaStream_t st) {
   const RowShape shape = row_shape(L->m, k);
-  if (L->m > kClusterBlocks * kClusterRows || shape.G > kClusterGroups || L->r > 2) return false;
+  if (L->m > kClusterBlocks * kClusterRows || shape.G > kClusterGroups || L->r > 2 ||
+      L->fault == FAULT_NO_CLUSTER)
+    return false;
   int blocks = 1;
   while (blocks < kClusterBlocks && L->m > 64 * blocks) blocks *= 2;
   const ClusterBlur q{(int)L->m, k, L->D, passes, blur, (int)ceil_div(L->m, blocks), tp, L->nbr};
-  cudaError_t e = cudaSuccess;
+  bool done = false;
   by_vec(shape.vec, [&](auto vec) {
     constexpr int VEC = decltype(vec)::value;
-    e = L->r == 1 ? launch_cluster<VEC, 1, S>(q, blocks, shape.G, lat0, st)
-                  : launch_cluster<VEC, 2, S>(q, blocks, shape.G, lat0, st);
+    auto go = [&](auto order) {
+      constexpr int R = decltype(order)::value;
+      if (!cluster_fits<VEC, R, S>()) return;
+      cudaLaunchAttribute at[2]{};
+      const cudaLaunchConfig_t cfg = cluster_config(blocks, shape.G, q.rows, st, at);
+      (void)cudaLaunchKernelEx(&cfg, k_blur_cluster<VEC, R, S>, q, lat0);  // as launch_pdl
+      done = true;
+    };
+    if (L->r == 1) go(std::integral_constant<int, 1>{});
+    else go(std::integral_constant<int, 2>{});
   });
-  if (e != cudaSuccess) {  // no room for such a cluster (e.g. a partitioned device)
-    clear_pending_error();
-    return false;
-  }
-  note_launches(1);
-  return true;
+  if (done) note_launches(1);
+  return done;
 }
 
 // Sparse blurs run on chains (else on the direction lists).

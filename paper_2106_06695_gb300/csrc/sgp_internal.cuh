@@ -21,7 +21,7 @@ enum : unsigned {
 };
 
 // Faults injected on the host through SGP_FAULT (tests of the error paths).
-enum { FAULT_NONE = 0, FAULT_OOM, FAULT_CUDA, FAULT_HASH_FULL, FAULT_NAN_INPUT };
+enum { FAULT_NONE = 0, FAULT_OOM, FAULT_CUDA, FAULT_HASH_FULL, FAULT_NAN_INPUT, FAULT_NO_CLUSTER };
 int injected_fault(int* columns);  // *columns: sgp_lattice::fault_cols
 
 // NVTX range for the lifetime of a scope (timeline profilers; no-op without one).
