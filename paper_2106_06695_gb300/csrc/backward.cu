@@ -67,12 +67,12 @@ __global__ void __launch_bounds__(kBT) k_weight_grad(int64_t n, int d, int k, in
                                                      const int32_t* __restrict__ perm,
                                                      const int32_t* __restrict__ idx,
                                                      const uint8_t* __restrict__ rank,
-                                                     const S* __restrict__ BU,
-                                                     const S* __restrict__ BS,
-                                                     const float* __restrict__ Vp,
-                                                     const float* __restrict__ Gp, float alpha,
-                                                     const double* __restrict__ f,
-                                                     const float* __restrict__ ls,
+                                                     const S* BU,
+                                                     const S* BS,
+                                                     const float* Vp,
+                                                     const float* Gp, float alpha,
+                                                     const double* f,
+                                                     const float* ls,
                                                      float* __restrict__ dX) {
   pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -101,8 +101,8 @@ __global__ void __launch_bounds__(kBT) k_weight_grad(int64_t n, int d, int k, in
 // Filter inputs, columns [col0, col0 + kc) of [z (.) g | g | z (.) v | v] ([n][kk],
 // kk = 2 k (d + 1); column c d + t of a z-block holds g_c z_t), caller's order.
 __global__ void k_filter_in(int64_t n, int d, int k, int col0, int kc,
-                            const float* __restrict__ X, const float* __restrict__ ls,
-                            const float* __restrict__ V, const float* __restrict__ G,
+                            const float* X, const float* ls,
+                            const float* V, const float* G,
                             float* __restrict__ out) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -127,9 +127,9 @@ __global__ void k_filter_in(int64_t n, int d, int k, int col0, int kc,
 // Accumulate the filtered columns [col0, col0 + kc) into dZ ([n][d], fp32, caller's order)
 // without the factor 2 alpha k'/k: one thread per point, columns in order.
 __global__ void k_filter_acc(int64_t n, int d, int k, int col0, int kc,
-                             const float* __restrict__ X, const float* __restrict__ ls,
-                             const float* __restrict__ V, const float* __restrict__ G,
-                             const float* __restrict__ F, float* __restrict__ dZ) {
+                             const float* X, const float* ls,
+                             const float* V, const float* G,
+                             const float* F, float* __restrict__ dZ) {
   pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -153,7 +153,7 @@ __global__ void k_filter_acc(int64_t n, int d, int k, int col0, int kc,
   }
 }
 
-__global__ void k_filter_finish(int64_t n, int d, float scale, const float* __restrict__ ls,
+__global__ void k_filter_finish(int64_t n, int d, float scale, const float* ls,
                                 float* __restrict__ dX) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -164,8 +164,8 @@ __global__ void k_filter_finish(int64_t n, int d, float scale, const float* __re
 // dl_j = -sum_i dX_ij x_ij / l_j: per-block partials (thread t owns column t % d and
 // rows t / d, t / d + P, ... of the block's range, P = floor(256 / d)), combined in a
 // fixed order; then the blocks in a fixed order.
-__global__ void __launch_bounds__(256) k_dls_partial(int64_t n, int d, const float* __restrict__ X,
-                                                     const float* __restrict__ dX,
+__global__ void __launch_bounds__(256) k_dls_partial(int64_t n, int d, const float* X,
+                                                     const float* dX,
                                                      double* __restrict__ partial) {
   pdl_enter();
   __shared__ double sh[256];
@@ -187,8 +187,8 @@ __global__ void __launch_bounds__(256) k_dls_partial(int64_t n, int d, const flo
   }
 }
 
-__global__ void k_dls_final(int nblk, int d, const double* __restrict__ partial,
-                            const float* __restrict__ ls, float* __restrict__ dls) {
+__global__ void k_dls_final(int nblk, int d, const double* partial,
+                            const float* ls, float* __restrict__ dls) {
   pdl_enter();
   // eight lanes a dimension, every eighth block each (304 dependent fp64 additions: 27 us)
   const int j = blockIdx.x * (blockDim.x / 8) + threadIdx.x / 8, lane = threadIdx.x % 8;

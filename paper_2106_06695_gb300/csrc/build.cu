@@ -177,7 +177,7 @@ __device__ __forceinline__ void note_range(int q, int c, int* qmin, int* qmax, u
 // n = 2M, d = 11: 0.91 ms, against 2.05 ms with per-thread local arrays and fp64 divisions.
 template <int MAXD>
 __global__ void __launch_bounds__(kElevT) k_elevate_small(
-    const float* __restrict__ X, const float* __restrict__ ls, const double* __restrict__ f,
+    const float* X, const float* ls, const double* f,
     int64_t n, int d, int16_t* __restrict__ rem0_out, uint8_t* __restrict__ rank_out,
     float* __restrict__ w_out, int* __restrict__ qmin, int* __restrict__ qmax,
     unsigned* __restrict__ err, int inject_nan) {
@@ -321,9 +321,9 @@ __global__ void __launch_bounds__(kElevT) k_elevate_small(
 // Any D <= MAXD: one thread per point, per-coordinate values in local memory (n = 500k, d =
 // 20: 0.46 ms, before 0.96; n = 60k, d = 50: 0.33 ms, before 0.48).
 template <int MAXD>
-__global__ void __launch_bounds__(kElevT) k_elevate(const float* __restrict__ X,
-                                                    const float* __restrict__ ls,
-                                                    const double* __restrict__ f, int64_t n,
+__global__ void __launch_bounds__(kElevT) k_elevate(const float* X,
+                                                    const float* ls,
+                                                    const double* f, int64_t n,
                                                     int d, int16_t* __restrict__ rem0_out,
                                                     uint8_t* __restrict__ rank_out,
                                                     float* __restrict__ w_out,
@@ -436,7 +436,7 @@ struct CellPack {
   int qmin[kMaxD];
 };
 
-__global__ void k_point_key(const int16_t* __restrict__ rem0, int64_t n, int D, CellPack pk,
+__global__ void k_point_key(const int16_t* rem0, int64_t n, int D, CellPack pk,
                             uint32_t* __restrict__ key, uint32_t* __restrict__ val) {
   pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -456,9 +456,9 @@ __global__ void k_point_key(const int16_t* __restrict__ rem0, int64_t n, int D, 
 // 2.5M entries share a few thousand vertices: 450 us with an atomic per probe).  The linear hash
 // goes to hash_lo / hash_hi for the numbering.
 template <int MAXD>
-__global__ void __launch_bounds__(256) k_insert(const int32_t* __restrict__ perm,
-                                                const int16_t* __restrict__ rem0,
-                                                const uint8_t* __restrict__ rank, int64_t nD,
+__global__ void __launch_bounds__(256) k_insert(const int32_t* perm,
+                                                const int16_t* rem0,
+                                                const uint8_t* rank, int64_t nD,
                                                 int d, unsigned long long* __restrict__ table,
                                                 uint64_t mask, int32_t* __restrict__ entry_slot,
                                                 uint32_t* __restrict__ hash_lo,
@@ -501,8 +501,8 @@ __global__ void __launch_bounds__(256) k_insert(const int32_t* __restrict__ perm
 // ---------------------------------------------------------------------------------
 // 4. Numbering: owner flags, then ids by scan, then slot -> id and vertex keys.
 // ---------------------------------------------------------------------------------
-__global__ void k_owner_flags(const int32_t* __restrict__ entry_slot,
-                              const unsigned long long* __restrict__ table, int64_t nD,
+__global__ void k_owner_flags(const int32_t* entry_slot,
+                              const unsigned long long* table, int64_t nD,
                               uint32_t* __restrict__ flags) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -517,10 +517,10 @@ __global__ void k_owner_flags(const int32_t* __restrict__ entry_slot,
 // scan steps.
 constexpr int kAssignThreads = 256;
 __global__ void __launch_bounds__(kAssignThreads)
-    k_assign_ids(const uint32_t* __restrict__ scanned, const uint32_t* __restrict__ total,
-                 const int32_t* __restrict__ entry_slot, const int32_t* __restrict__ perm,
-                 const int16_t* __restrict__ rem0, const uint8_t* __restrict__ rank,
-                 const uint32_t* __restrict__ hash_lo, const uint32_t* __restrict__ hash_hi,
+    k_assign_ids(const uint32_t* scanned, const uint32_t* total,
+                 const int32_t* entry_slot, const int32_t* perm,
+                 const int16_t* rem0, const uint8_t* rank,
+                 const uint32_t* hash_lo, const uint32_t* hash_hi,
                  int64_t nD, int d, int32_t* __restrict__ slot_id, int16_t* __restrict__ keys,
                  uint64_t* __restrict__ vhash, uint32_t* __restrict__ owner) {
   pdl_enter();
@@ -550,10 +550,10 @@ __global__ void __launch_bounds__(kAssignThreads)
   }
 }
 
-__global__ void k_entry_ids(const int32_t* __restrict__ entry_slot,
-                            const int32_t* __restrict__ slot_id,
-                            const int32_t* __restrict__ perm, const float* __restrict__ w_user,
-                            const uint8_t* __restrict__ rank_user, int64_t nD, int D,
+__global__ void k_entry_ids(const int32_t* entry_slot,
+                            const int32_t* slot_id,
+                            const int32_t* perm, const float* w_user,
+                            const uint8_t* rank_user, int64_t nD, int D,
                             int32_t* __restrict__ idx, float* __restrict__ w,
                             uint8_t* __restrict__ rank) {
   pdl_enter();
@@ -592,9 +592,9 @@ struct LinkBits {
 
 // nbr[j][t][side][v]: the links of v's owner simplex, -1 elsewhere; up[v]: the direction along
 // which v's link upwards lies.  owner[v]: its entry.
-__global__ void __launch_bounds__(256) k_nbr_init(const uint32_t* __restrict__ owner,
-                                                  const int32_t* __restrict__ idx,
-                                                  const uint8_t* __restrict__ rank, int64_t m, int d,
+__global__ void __launch_bounds__(256) k_nbr_init(const uint32_t* owner,
+                                                  const int32_t* idx,
+                                                  const uint8_t* rank, int64_t m, int d,
                                                   int r, int32_t* __restrict__ nbr,
                                                   uint8_t* __restrict__ up, LinkBits lb) {
   pdl_enter();
@@ -634,9 +634,9 @@ __global__ void __launch_bounds__(256) k_nbr_init(const uint32_t* __restrict__ o
 
 // The other ends of those links, where they belong to another simplex and so did not write
 // theirs.  (Several simplices may write one link; they write the same id.)
-__global__ void __launch_bounds__(256) k_nbr_close(const uint32_t* __restrict__ owner,
-                                                   const int32_t* __restrict__ idx,
-                                                   const uint8_t* __restrict__ rank, int64_t m,
+__global__ void __launch_bounds__(256) k_nbr_close(const uint32_t* owner,
+                                                   const int32_t* idx,
+                                                   const uint8_t* rank, int64_t m,
                                                    int d, int r, int32_t* __restrict__ nbr,
                                                    LinkBits lb) {
   pdl_enter();
@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(256) k_nbr_close(const uint32_t* __restrict__ 
 }
 
 // Sort keys: the top bits of the vertex hashes.
-__global__ void k_hash_keys(const uint64_t* __restrict__ vhash, int64_t m, int shift,
+__global__ void k_hash_keys(const uint64_t* vhash, int64_t m, int shift,
                             uint32_t* __restrict__ key, uint32_t* __restrict__ val) {
   pdl_enter();
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -672,8 +672,8 @@ __global__ void k_hash_keys(const uint64_t* __restrict__ vhash, int64_t m, int s
 
 // Of the i-th vertex in bucket order: its hash (low and high half) and its direction up;
 // start[b] = first i of bucket b (b <= buckets).
-__global__ void k_hash_index(const uint32_t* __restrict__ key, const uint32_t* __restrict__ ord,
-                             const uint64_t* __restrict__ vhash, const uint8_t* __restrict__ up,
+__global__ void k_hash_index(const uint32_t* key, const uint32_t* ord,
+                             const uint64_t* vhash, const uint8_t* up,
                              int64_t m, int64_t buckets, uint32_t* __restrict__ low,
                              uint32_t* __restrict__ high, uint8_t* __restrict__ up_sorted,
                              uint32_t* __restrict__ start) {
@@ -705,9 +705,9 @@ __device__ __forceinline__ bool steps_to(int16_t v, int16_t u, int c, int j, int
 constexpr int kNbrGroup = 4;
 template <bool WARP>
 __global__ void __launch_bounds__(256) k_neighbours(
-    const int16_t* __restrict__ keys, const uint32_t* __restrict__ low,
-    const uint32_t* __restrict__ high, const uint8_t* __restrict__ up,
-    const uint32_t* __restrict__ ord, const uint32_t* __restrict__ start, int shift, int64_t m,
+    const int16_t* keys, const uint32_t* low,
+    const uint32_t* high, const uint8_t* up,
+    const uint32_t* ord, const uint32_t* start, int shift, int64_t m,
     int d, int r, uint64_t sum_A, int32_t* __restrict__ nbr, unsigned long long* __restrict__ hits,
     LinkBits lb) {
   pdl_enter();
@@ -729,11 +729,11 @@ __global__ void __launch_bounds__(256) k_neighbours(
         const uint32_t* s = start + (x >> shift);
         const bool on = live && j0 + q < D && (t > 1 || j0 + q != given);
         want[q] = (uint32_t)x;
-        p[q] = on ? __ldg(s) : 0u;
-        end[q] = on ? __ldg(s + 1) : 0u;
+        p[q] = on ? *s : 0u;
+        end[q] = on ? s[1] : 0u;
       }
 #pragma unroll
-      for (int q = 0; q < kNbrGroup; ++q) at[q] = p[q] < end[q] ? __ldg(low + p[q]) : 0u;
+      for (int q = 0; q < kNbrGroup; ++q) at[q] = p[q] < end[q] ? low[p[q]] : 0u;
 #pragma unroll
       for (int q = 0; q < kNbrGroup; ++q) {
         const int j = j0 + q;
@@ -741,15 +741,15 @@ __global__ void __launch_bounds__(256) k_neighbours(
         bool more = true;
         while (more) {
           while (p[q] < end[q] && at[q] != want[q])
-            if (++p[q] < end[q]) at[q] = __ldg(low + p[q]);
+            if (++p[q] < end[q]) at[q] = low[p[q]];
           __syncwarp();
           const bool match = p[q] < end[q];
           unsigned todo = __ballot_sync(0xffffffffu, match);
           if (!todo) break;
           uint32_t u = 0, v = 0;
           if (match) {
-            u = __ldg(ord + p[q]);
-            v = __ldg(ord + i);
+            u = ord[p[q]];
+            v = ord[i];
           }
           bool ok = false;
           if (WARP) {
@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(256) k_neighbours(
 #pragma unroll
               for (int c0 = 0; c0 < kMaxD; c0 += 32)
                 if (c0 < D && c0 + lane < D)
-                  same = same & steps_to(__ldg(kv + c0 + lane), __ldg(ku + c0 + lane), c0 + lane, j, t, D);
+                  same = same & steps_to(kv[c0 + lane], ku[c0 + lane], c0 + lane, j, t, D);
               same = __all_sync(0xffffffffu, same);
               ok = ok || (same && lane == src);
             }
@@ -771,7 +771,7 @@ __global__ void __launch_bounds__(256) k_neighbours(
             ok = true;
 #pragma unroll
             for (int c = 0; c < 16; ++c)
-              if (c < D) ok = ok & steps_to(__ldg(kv + c), __ldg(ku + c), c, j, t, D);
+              if (c < D) ok = ok & steps_to(kv[c], ku[c], c, j, t, D);
           }
           if (ok) {
             plane[u] = (int32_t)v;
@@ -783,7 +783,7 @@ __global__ void __launch_bounds__(256) k_neighbours(
             found += t == 1 ? 1u : 0u;
             p[q] = end[q];
           } else if (match && ++p[q] < end[q]) {  // another vertex with these hash bits
-            at[q] = __ldg(low + p[q]);
+            at[q] = low[p[q]];
           }
           more = __any_sync(0xffffffffu, p[q] < end[q]);
         }
@@ -796,7 +796,7 @@ __global__ void __launch_bounds__(256) k_neighbours(
 
 // The link bits read off the table, where they were not recorded while it was made; for r > 1,
 // above = any neighbour along the direction and below = 0.
-__global__ void __launch_bounds__(256) k_link_bits(const int32_t* __restrict__ nbr, int64_t m,
+__global__ void __launch_bounds__(256) k_link_bits(const int32_t* nbr, int64_t m,
                                                    int D, int r, LinkBits lb) {
   pdl_enter();
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -849,7 +849,7 @@ __global__ void __launch_bounds__(256) k_link_counts(LinkBits lb, int64_t m, int
 // blur, which updates its vertices independently.
 constexpr int kFillThreads = 512;
 __global__ void __launch_bounds__(kFillThreads) k_active_fill(
-    const uint32_t* __restrict__ hasnb, int64_t m, int D, const int64_t* __restrict__ off,
+    const uint32_t* hasnb, int64_t m, int D, const int64_t* off,
     unsigned long long* __restrict__ fill, int32_t* __restrict__ act) {
   pdl_enter();
   constexpr int kWarps = kFillThreads / 32;
@@ -902,8 +902,8 @@ __global__ void __launch_bounds__(kFillThreads) k_active_fill(
 // chain slots per direction, and each head walks again to write its chain.  The order of
 // the chains is immaterial.  *longest: the longest chain.
 __global__ void __launch_bounds__(kFillThreads) k_chain_fill(
-    LinkBits lb, const int32_t* __restrict__ nbr, int64_t m, int D,
-    const int64_t* __restrict__ off, const int64_t* __restrict__ chain_off,
+    LinkBits lb, const int32_t* nbr, int64_t m, int D,
+    const int64_t* off, const int64_t* chain_off,
     unsigned long long* __restrict__ fill, unsigned long long* __restrict__ chain_fill,
     int32_t* __restrict__ act, uint2* __restrict__ chain, int* __restrict__ longest) {
   pdl_enter();
@@ -959,8 +959,8 @@ __global__ void __launch_bounds__(kFillThreads) k_chain_fill(
 // ---------------------------------------------------------------------------------
 // 6. Splat lists.
 // ---------------------------------------------------------------------------------
-__global__ void k_splat_items(const uint32_t* __restrict__ sorted_entries,
-                              const float* __restrict__ w,
+__global__ void k_splat_items(const uint32_t* sorted_entries,
+                              const float* w,
                               int64_t nD, int D, int2* __restrict__ items) {
   pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -985,7 +985,7 @@ __device__ __forceinline__ void seg_counts(int b, int e, uint32_t (&c)[SEG_KINDS
 // exclusive scan is the row's total).  k_seg_fill counts again rather than reading offsets per
 // vertex: those are 32 bytes a vertex written and read for 4 read here (m = 10.5M: 390 us for
 // the counts, their scans and the fill, 90 with the block sums alone).
-__global__ void __launch_bounds__(kSegThreads) k_seg_sums(const int32_t* __restrict__ row_ptr,
+__global__ void __launch_bounds__(kSegThreads) k_seg_sums(const int32_t* row_ptr,
                                                           int64_t m, uint32_t* __restrict__ sums) {
   pdl_enter();
   const int64_t v = (int64_t)blockIdx.x * kSegThreads + threadIdx.x;
@@ -1011,7 +1011,7 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_sums(const int32_t* __restr
 // 8 segments is written by its thread, a longer one by its warp (few dense vertices may hold
 // nearly all segments: n = 760k, d = 2, five vertices, 284 us with one thread each).
 __global__ void __launch_bounds__(kSegThreads)
-    k_seg_fill(const int32_t* __restrict__ row_ptr, int64_t m, const uint32_t* __restrict__ sums,
+    k_seg_fill(const int32_t* row_ptr, int64_t m, const uint32_t* sums,
                int4* __restrict__ seg, int4* __restrict__ med_rows, int4* __restrict__ huge_rows) {
   pdl_enter();
   const int64_t v = (int64_t)blockIdx.x * kSegThreads + threadIdx.x;
@@ -1050,7 +1050,7 @@ __global__ void __launch_bounds__(kSegThreads)
 // does not depend on the order in which segments are processed.  A counting sort: ranks by
 // comparison with the whole window are 128 steps a segment (10.5M segments: 238 us).
 constexpr int kSegWindow = 128;
-__global__ void __launch_bounds__(kSegWindow) k_seg_window_sort(const int4* __restrict__ in,
+__global__ void __launch_bounds__(kSegWindow) k_seg_window_sort(const int4* in,
                                                                 int64_t nseg,
                                                                 int4* __restrict__ out) {
   pdl_enter();
@@ -1098,7 +1098,7 @@ __global__ void k_iota(uint32_t* __restrict__ out, int64_t count) {
   if (p < count) out[p] = (uint32_t)p;
 }
 
-__global__ void k_row_ptr(const uint32_t* __restrict__ sorted_ids, int64_t nD, int64_t m,
+__global__ void k_row_ptr(const uint32_t* sorted_ids, int64_t nD, int64_t m,
                           int32_t* __restrict__ row_ptr) {
   pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

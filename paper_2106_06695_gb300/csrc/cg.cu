@@ -191,7 +191,7 @@ __device__ __forceinline__ void stf(float* p, const float (&v)[VEC]) {
 // The caller's B has kb <= k columns; columns kb .. k - 1 of the solver's vectors are zero
 // right-hand sides (inactive from the start).
 template <int VEC>
-__global__ void k_cg_init(const float* __restrict__ B, int kb, const int32_t* __restrict__ perm,
+__global__ void k_cg_init(const float* B, int kb, const int32_t* __restrict__ perm,
                           float* __restrict__ xh, float* __restrict__ xl,
                           float* __restrict__ rh, float* __restrict__ rl, float* __restrict__ p,
                           int64_t n, int k, CgState S) {
@@ -230,7 +230,7 @@ __global__ void k_cg_init(const float* __restrict__ B, int kb, const int32_t* __
 template <int VEC>
 __global__ void k_cg_update_xr(float* __restrict__ xh, float* __restrict__ xl,
                                float* __restrict__ rh, float* __restrict__ rl,
-                               const float* __restrict__ p, const float* __restrict__ Ap,
+                               const float* p, const float* Ap,
                                int64_t n, int k, CgState S) {
   pdl_enter();
   dfloat acc[VEC], a[VEC], na[VEC];
@@ -294,7 +294,7 @@ __global__ void k_cg_update_xr(float* __restrict__ xh, float* __restrict__ xl,
 
 // Preconditioned CG: p = z + beta p on active columns (first == true: p = z).
 template <int VEC, bool FIRST>
-__global__ void k_cg_update_p_z(float* __restrict__ p, const float* __restrict__ z, int64_t n,
+__global__ void k_cg_update_p_z(float* __restrict__ p, const float* z, int64_t n,
                                 int k, CgState S) {
   pdl_enter();
   dfloat b[VEC];
@@ -327,8 +327,8 @@ __global__ void k_cg_update_p_z(float* __restrict__ p, const float* __restrict__
 
 // p = r + beta p on active columns (double-float sum, rounded to fp32).
 template <int VEC>
-__global__ void k_cg_update_p(float* __restrict__ p, const float* __restrict__ rh,
-                              const float* __restrict__ rl, int64_t n, int k, CgState S) {
+__global__ void k_cg_update_p(float* __restrict__ p, const float* rh,
+                              const float* rl, int64_t n, int k, CgState S) {
   pdl_enter();
   dfloat b[VEC];
   bool on[VEC];
@@ -358,7 +358,7 @@ __global__ void k_cg_update_p(float* __restrict__ p, const float* __restrict__ r
 }
 
 template <int VEC>
-__global__ void k_cg_store_x(const float* __restrict__ xh, const float* __restrict__ xl,
+__global__ void k_cg_store_x(const float* xh, const float* xl,
                              const int32_t* __restrict__ perm, float* __restrict__ X, int kb,
                              int64_t n, int k) {
   pdl_enter();

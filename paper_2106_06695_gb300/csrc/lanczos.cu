@@ -39,10 +39,10 @@ constexpr double kSlqStep = 0.45;  // trapezoid step in log t
 // QL iteration with one thread per probe (a serial chain of about 15,000 rotations, 21.8 ms
 // for 10 probes of 100 steps); the whole log determinant at n = 46k, d = 9 went from 39.4 to
 // 17.5 ms.  Against 50-digit arithmetic its values are off by 0 to 2e-16, QL's by up to 1e-12.
-__global__ void __launch_bounds__(32) k_slq(const double* __restrict__ ha,
-                                            const double* __restrict__ hb, int k, int cap,
-                                            const int* __restrict__ iters,
-                                            const double* __restrict__ bnorm,
+__global__ void __launch_bounds__(32) k_slq(const double* ha,
+                                            const double* hb, int k, int cap,
+                                            const int* iters,
+                                            const double* bnorm,
                                             double* __restrict__ part, int* __restrict__ bad) {
   pdl_enter();
   __shared__ double al[kMaxLanczos], be[kMaxLanczos];

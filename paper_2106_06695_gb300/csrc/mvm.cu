@@ -47,7 +47,7 @@ template <int VEC, class S>
 __global__ void __launch_bounds__(kThreads) k_splat(int64_t nseg, int G, int k,
                                                     const int4* __restrict__ seg,
                                                     const int2* __restrict__ items,
-                                                    const float* __restrict__ V, float scale,
+                                                    const float* V, float scale,
                                                     S* __restrict__ lat,
                                                     float* __restrict__ partial) {
   pdl_enter();
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kThreads) k_splat(int64_t nseg, int G, int k,
     typename Vt::T row[kChunk];
 #pragma unroll
     for (int j = 0; j < kChunk; ++j)
-      row[j] = it[j].x >= 0 ? Vt::ldg(V + (int64_t)it[j].x * k + col) : Vt::zero();
+      row[j] = it[j].x >= 0 ? Vt::ld(V + (int64_t)it[j].x * k + col) : Vt::zero();
 #pragma unroll
     for (int j = 0; j < kChunk; ++j)
       if (it[j].x >= 0) acc = Vt::fma(__int_as_float(it[j].y), row[j], acc);
@@ -83,7 +83,7 @@ template <int VEC, class S>
 __global__ void __launch_bounds__(kThreads) k_splat_fix(int nhuge, int64_t nmed, int groups, int G,
                                                         int k, const int4* __restrict__ huge_rows,
                                                         const int4* __restrict__ med_rows,
-                                                        const float* __restrict__ partial,
+                                                        const float* partial,
                                                         float scale, S* __restrict__ lat) {
   pdl_enter();
   using Vt = Vec<VEC>;
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kThreads) k_splat_fix(int nhuge, int64_t nmed,
     const float* base = partial + (int64_t)rw.y * k + col;
     typename Vt::T x[kSplatMedSegs], acc = Vt::zero();
 #pragma unroll
-    for (int j = 0; j < kSplatMedSegs; ++j) x[j] = j < rw.z ? Vt::ldg(base + (int64_t)j * k) : Vt::zero();
+    for (int j = 0; j < kSplatMedSegs; ++j) x[j] = j < rw.z ? Vt::ld(base + (int64_t)j * k) : Vt::zero();
 #pragma unroll
     for (int j = 0; j < kSplatMedSegs; ++j)
       if (j < rw.z) acc = Vt::add(acc, x[j]);
@@ -112,11 +112,11 @@ __global__ void __launch_bounds__(kThreads) k_splat_fix(int nhuge, int64_t nmed,
     for (; j + 15 * groups < rw.z; j += 16 * groups) {  // 16 loads in flight, summed in order
       typename Vt::T x[16];
 #pragma unroll
-      for (int e = 0; e < 16; ++e) x[e] = Vt::ldg(base + (int64_t)(j + e * groups) * k);
+      for (int e = 0; e < 16; ++e) x[e] = Vt::ld(base + (int64_t)(j + e * groups) * k);
 #pragma unroll
       for (int e = 0; e < 16; ++e) acc = Vt::add(acc, x[e]);
     }
-    for (; j < rw.z; j += groups) acc = Vt::add(acc, Vt::ldg(base + (int64_t)j * k));
+    for (; j < rw.z; j += groups) acc = Vt::add(acc, Vt::ld(base + (int64_t)j * k));
     red[q] = acc;
   }
   __syncthreads();
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kThreads) k_splat_fix(int nhuge, int64_t nmed,
 template <class S>
 __global__ void __launch_bounds__(kThreads) k_blur(int64_t m, int k, int r, Taps tp,
                                                    const int32_t* __restrict__ nbr,
-                                                   const S* __restrict__ in, S* __restrict__ out) {
+                                                   const S* in, S* __restrict__ out) {
   pdl_enter();
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t v = gid / k;
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kThreads) k_blur(int64_t m, int k, int r, Taps
 template <int VEC, int CH, int U, int R, class S>
 __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k, Taps tp,
                                                         const int32_t* __restrict__ nbr,
-                                                        const S* __restrict__ in,
+                                                        const S* in,
                                                         S* __restrict__ out) {
   static_assert(CH == 1 || (CH == 2 && VEC == 4), "one group of columns per thread, or 2 x 4");
   using Vt = Vec<VEC>;
@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k,
   }
   pdl_enter();  // the ids do not change: loaded before the wait
   auto load = [&](int64_t row, T* x) {
-    if constexpr (CH == 2) Store<S>::ldg8(in + row * k + col, x[0], x[1]);
-    else x[0] = Vt::ldgs(in + row * k + col);
+    if constexpr (CH == 2) Store<S>::ld8(in + row * k + col, x[0], x[1]);
+    else x[0] = Vt::lds(in + row * k + col);
   };
   T own[U][CH], sa[U][R][CH], sc[U][R][CH];
 #pragma unroll
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k,
 template <class S>
 __global__ void __launch_bounds__(kThreads) k_blur_pipe(int64_t m, int G, int k, Taps tp,
                                                         const int32_t* __restrict__ nbr,
-                                                        const S* __restrict__ in,
+                                                        const S* in,
                                                         S* __restrict__ out) {
   pdl_enter();
   const int rows_per_block = blockDim.x / G;
@@ -239,9 +239,9 @@ __global__ void __launch_bounds__(kThreads) k_blur_pipe(int64_t m, int G, int k,
   };
   auto load = [&](int64_t v, int a, int c, float4 (&x)[3][2]) {  // own, minus, plus rows
     x[0][0] = x[0][1] = x[1][0] = x[1][1] = x[2][0] = x[2][1] = zero;
-    if (v < m) Store<S>::ldg8(in + v * k + col, x[0][0], x[0][1]);
-    if (a >= 0) Store<S>::ldg8(in + (int64_t)a * k + col, x[1][0], x[1][1]);
-    if (c >= 0) Store<S>::ldg8(in + (int64_t)c * k + col, x[2][0], x[2][1]);
+    if (v < m) Store<S>::ld8(in + v * k + col, x[0][0], x[0][1]);
+    if (a >= 0) Store<S>::ld8(in + (int64_t)a * k + col, x[1][0], x[1][1]);
+    if (c >= 0) Store<S>::ld8(in + (int64_t)c * k + col, x[2][0], x[2][1]);
   };
   int a0, c0, a1, c1;
   ids(row, a0, c0);
@@ -496,9 +496,9 @@ __global__ void __launch_bounds__(kThreads) k_sparse_blur(int64_t count, int G, 
                                                           const int32_t* __restrict__ act,
                                                           const int32_t* __restrict__ nbr_j,
                                                           int64_t m,
-                                                          const int32_t* __restrict__ epoch,
+                                                          const int32_t* epoch,
                                                           const float* __restrict__ pw,
-                                                          const S* __restrict__ stored,
+                                                          const S* stored,
                                                           S* __restrict__ tmp) {
   pdl_enter();
   using Vt = Vec<VEC>;
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(kThreads) k_sparse_blur(int64_t count, int G, 
 template <int VEC, class S>
 __global__ void __launch_bounds__(kThreads) k_sparse_store(int64_t count, int G, int k, int t,
                                                            const int32_t* __restrict__ act,
-                                                           const S* __restrict__ tmp,
+                                                           const S* tmp,
                                                            S* __restrict__ stored,
                                                            int32_t* __restrict__ epoch) {
   pdl_enter();
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(kThreads) k_sparse_store(int64_t count, int G,
 
 template <int VEC, class S>
 __global__ void __launch_bounds__(kThreads) k_sparse_finish(int64_t m, int G, int k, int P,
-                                                            const int32_t* __restrict__ epoch,
+                                                            const int32_t* epoch,
                                                             const float* __restrict__ pw,
                                                             S* __restrict__ stored) {
   pdl_enter();
@@ -560,7 +560,7 @@ template <int VEC, class S>
 __device__ __forceinline__ typename Vec<VEC>::T slice_row(int64_t p, int D, int k, int col,
                                                           const int32_t* __restrict__ idx,
                                                           const float* __restrict__ w,
-                                                          const S* __restrict__ lat) {
+                                                          const S* lat) {
   using Vt = Vec<VEC>;
   typename Vt::T acc = Vt::zero();
   const int64_t e0 = p * D;
@@ -576,7 +576,7 @@ __device__ __forceinline__ typename Vec<VEC>::T slice_row(int64_t p, int D, int 
     typename Vt::T row[kChunk];
 #pragma unroll
     for (int j = 0; j < kChunk; ++j)
-      row[j] = id[j] >= 0 ? Vt::ldgs(lat + (int64_t)id[j] * k + col) : Vt::zero();
+      row[j] = id[j] >= 0 ? Vt::lds(lat + (int64_t)id[j] * k + col) : Vt::zero();
 #pragma unroll
     for (int j = 0; j < kChunk; ++j)
       if (id[j] >= 0) acc = Vt::fma(wt[j], row[j], acc);
@@ -592,8 +592,8 @@ __global__ void __launch_bounds__(kThreads) k_slice(int64_t n, int G, int k, int
                                                     const int32_t* __restrict__ perm,
                                                     const int32_t* __restrict__ idx,
                                                     const float* __restrict__ w,
-                                                    const S* __restrict__ lat,
-                                                    const float* __restrict__ Vp, float alpha,
+                                                    const S* lat,
+                                                    const float* Vp, float alpha,
                                                     float beta, float* __restrict__ out) {
   pdl_enter();
   using Vt = Vec<VEC>;
@@ -621,8 +621,8 @@ template <int VEC, class S>
 __global__ void __launch_bounds__(kThreads) k_slice_dot(int64_t n, int G, int k, int D,
                                                         const int32_t* __restrict__ idx,
                                                         const float* __restrict__ w,
-                                                        const S* __restrict__ lat,
-                                                        const float* __restrict__ V, float alpha,
+                                                        const S* lat,
+                                                        const float* V, float alpha,
                                                         float beta, float* __restrict__ out,
                                                         double* __restrict__ dot_partial) {
   pdl_enter();
@@ -654,7 +654,7 @@ __global__ void __launch_bounds__(kThreads) k_slice_dot(int64_t n, int G, int k,
 template <int VEC, bool WIDE>
 __global__ void __launch_bounds__(kThreads) k_permute_rows(int64_t n, int G, int k, int ki,
                                                            const int32_t* __restrict__ perm,
-                                                           const float* __restrict__ V,
+                                                           const float* V,
                                                            float* __restrict__ Vp) {
   pdl_enter();
   using Vt = Vec<VEC>;
@@ -679,8 +679,8 @@ __global__ void __launch_bounds__(kThreads) k_permute_rows(int64_t n, int G, int
 template <int VEC, bool WIDE>
 __global__ void __launch_bounds__(kThreads) k_permute_pair(int64_t n, int G, int kp, int ki,
                                                            const int32_t* __restrict__ perm,
-                                                           const float* __restrict__ A,
-                                                           const float* __restrict__ B,
+                                                           const float* A,
+                                                           const float* B,
                                                            float* __restrict__ out) {
   pdl_enter();
   using Vt = Vec<VEC>;

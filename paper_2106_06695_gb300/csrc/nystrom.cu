@@ -49,7 +49,7 @@ __device__ __forceinline__ float to_f(float x) { return x; }
 // else L = X.  X: [n][ld] (first l columns used).  out: partial[block][l][l] (fp64 of
 // fp32 block sums).
 template <bool OMEGA, class TX>
-__global__ void k_gram(const TX* __restrict__ X, int ld, const int32_t* __restrict__ perm,
+__global__ void k_gram(const TX* X, int ld, const int32_t* __restrict__ perm,
                        int64_t n, int l, uint64_t seed, double* __restrict__ partial) {
   pdl_enter();
   extern __shared__ float sh[];
@@ -92,7 +92,7 @@ __global__ void k_gram(const TX* __restrict__ X, int ld, const int32_t* __restri
 }
 
 // out[e] = sum over blocks of partial[b][e], in block order.
-__global__ void k_sum_blocks(const double* __restrict__ partial, int nblk, int count,
+__global__ void k_sum_blocks(const double* partial, int nblk, int count,
                              double* __restrict__ out) {
   pdl_enter();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -152,7 +152,7 @@ __global__ void k_cholesky(double* __restrict__ A, int l, double shift, double r
 
 // T = (R^-1)^T for lower-triangular R (fp64), written as fp32 [l][l] (upper triangular):
 // thread c solves R x = e_c by forward substitution.
-__global__ void k_tri_inv_t(const double* __restrict__ R, int l, double* __restrict__ work,
+__global__ void k_tri_inv_t(const double* R, int l, double* __restrict__ work,
                             float* __restrict__ T) {
   pdl_enter();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -168,7 +168,7 @@ __global__ void k_tri_inv_t(const double* __restrict__ R, int l, double* __restr
 
 // Minv = (Q Q^T)^-1 for lower-triangular Q (fp64): W = Q^-1 by forward substitution per
 // column (thread c), then Minv = W^T W.  `work` holds W ([l][l]).
-__global__ void k_inv_from_cholesky(const double* __restrict__ Q, int l, double* __restrict__ W,
+__global__ void k_inv_from_cholesky(const double* Q, int l, double* __restrict__ W,
                                     double* __restrict__ Minv) {
   pdl_enter();
   for (int c = threadIdx.x; c < l; c += blockDim.x) {
@@ -204,7 +204,7 @@ __global__ void k_fill_sketch_chunk(const int32_t* __restrict__ perm, int64_t n,
 // the last chunk also zeroes the padding columns l..ld-1.
 __global__ void k_gather_chunk(const int32_t* __restrict__ perm, int64_t n, int64_t n_train,
                                int l, int ld, int c0, int kp, uint64_t seed, float nu,
-                               const float* __restrict__ KV, float* __restrict__ Y) {
+                               const float* KV, float* __restrict__ Y) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n * kp) return;
@@ -220,7 +220,7 @@ __global__ void k_gather_chunk(const int32_t* __restrict__ perm, int64_t n, int6
 
 // In place, row by row: Y[row][0..l) = Y[row][0..l) T (T in shared memory).  Each block
 // stages its rows before it writes any of them, and no other block touches those rows.
-__global__ void k_rows_times_inplace(float* Y, const float* __restrict__ T, int64_t n, int l,
+__global__ void k_rows_times_inplace(float* Y, const float* T, int64_t n, int l,
                                      int ld) {
   pdl_enter();
   extern __shared__ float sh[];

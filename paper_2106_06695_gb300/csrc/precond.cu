@@ -65,7 +65,7 @@ __device__ __forceinline__ float sketch_sign(uint64_t seed, int64_t i, int j, in
 
 // G[i][j] = sum over splits of partial[s][i][j] (fp64, in split order) for the tiles on
 // and below the diagonal, mirrored above it.
-__global__ void k_sum_splits(const float* __restrict__ partial, int splits, int ldp,
+__global__ void k_sum_splits(const float* partial, int splits, int ldp,
                              double* __restrict__ G) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -109,7 +109,7 @@ constexpr int kTcThreads = 160;               // warp 0: issue; warps 1-4: epilo
 // the split right-hand side as rows of 64 bf16 (columns 48..63 stay zero), MN-major for
 // the B^T r MMAs.  One row per thread, 16-byte stores.  (The CG's x, r update writes the
 // first 16 columns' split itself; this kernel serves the CG start and further chunks.)
-__global__ void k_split_r(const float* __restrict__ rh, const float* __restrict__ rl, int k,
+__global__ void k_split_r(const float* rh, const float* rl, int k,
                           int c_off, int kc, int64_t n, __nv_bfloat16* __restrict__ r3) {
   pdl_enter();
   const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -144,7 +144,7 @@ __global__ void k_split_r(const float* __restrict__ rh, const float* __restrict_
 // one warp; the loads of the next eight splits are in flight while eight are added.  131
 // splits of 256 x 16 outputs: 14.7 us (a chain of 131 fp64 additions), 23.5 with 256 outputs
 // and their conversions on each of 16 SMs.
-__global__ void __launch_bounds__(32) k_sum_t(const float* __restrict__ tpart, int splits, int ld,
+__global__ void __launch_bounds__(32) k_sum_t(const float* tpart, int splits, int ld,
                                               float* __restrict__ t) {
   pdl_enter();
   const int e = blockIdx.x * 32 + threadIdx.x;  // ld * 16 is a multiple of 32
@@ -172,8 +172,8 @@ __global__ void __launch_bounds__(32) k_sum_t(const float* __restrict__ tpart, i
 // takes j = 32 q' + q (coalesced reads of the row), then a fixed butterfly over the lanes.
 // Stored split in three bf16 parts, transposed: u3[part][c][i] (the K-major [48][ld]
 // operand).
-__global__ void __launch_bounds__(256) k_minv_u(const float* __restrict__ Minv, int ld,
-                                                const float* __restrict__ t,
+__global__ void __launch_bounds__(256) k_minv_u(const float* Minv, int ld,
+                                                const float* t,
                                                 __nv_bfloat16* __restrict__ u3) {
   pdl_enter();
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // update ends in a FastTwoSum, so fl(hi + lo) = hi), and the low words are not read.
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_z_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapU,
-           const float* __restrict__ rh, int k, int c_off, int kc, int64_t n, int ld,
+           const float* rh, int k, int c_off, int kc, int64_t n, int ld,
            float inv_tau, float* __restrict__ z, double* __restrict__ dot,
            int* __restrict__ err) {
   pdl_enter();
@@ -672,7 +672,7 @@ __global__ void k_cols3(__nv_bfloat16* __restrict__ P3, int ld, int c0, float* _
 
 // T3 = the three planes of (float)A for the l x l block of A (fp64, leading dimension lda),
 // zero elsewhere in [ld][ld].
-__global__ void k_split3_pad(const double* __restrict__ A, int lda, int l, int ld,
+__global__ void k_split3_pad(const double* A, int lda, int l, int ld,
                              __nv_bfloat16* __restrict__ T3) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -958,7 +958,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // the diagonal, strict upper triangle zero (l x l, leading dimension lda), and zero in the
 // rest of the lda x lda array; out of place, any grid (each block reads the diagonal for
 // the maximum).
-__global__ void __launch_bounds__(256) k_prepare_spd(const double* __restrict__ src,
+__global__ void __launch_bounds__(256) k_prepare_spd(const double* src,
                                                      double* __restrict__ dst, int l, int lda,
                                                      double shift, double rel) {
   pdl_enter();
@@ -1091,7 +1091,7 @@ __global__ void __launch_bounds__(256) k_syrk_trailing(double* __restrict__ A, i
 
 // Inverse of each 32 x 32 lower diagonal block of L into X (forward substitution per
 // column in shared memory); the strict upper part of the block is zero.
-__global__ void k_trtri_diag(const double* __restrict__ L, double* __restrict__ X, int lda,
+__global__ void k_trtri_diag(const double* L, double* __restrict__ X, int lda,
                              int l) {
   pdl_enter();
   __shared__ double a[kNB][kNB + 1], x[kNB][kNB + 1];
@@ -1134,7 +1134,7 @@ __global__ void k_trtri_diag(const double* __restrict__ L, double* __restrict__ 
 // (blockIdx.x = pair, row tile, column tile), 4 outputs per thread.  Reads beyond l are
 // zero.
 template <int MODE>
-__global__ void __launch_bounds__(256) k_trtri_level(const double* __restrict__ L,
+__global__ void __launch_bounds__(256) k_trtri_level(const double* L,
                                                       double* __restrict__ X,
                                                       double* __restrict__ S, int lda, int l,
                                                       int b) {
@@ -1185,7 +1185,7 @@ __global__ void __launch_bounds__(256) k_trtri_level(const double* __restrict__ 
 
 // M = X^T X for lower-triangular X (l x l), both triangles written; one 32 x 32 tile of the
 // lower triangle per block (mirrored).  Rows of X below the tiles' columns only.
-__global__ void __launch_bounds__(256) k_xtx(const double* __restrict__ X, int lda, int l,
+__global__ void __launch_bounds__(256) k_xtx(const double* X, int lda, int l,
                                              double* __restrict__ M) {
   pdl_enter();
   __shared__ double xa[kNB][kNB + 1], xb[kNB][kNB + 1];
@@ -1227,7 +1227,7 @@ __global__ void __launch_bounds__(256) k_xtx(const double* __restrict__ X, int l
 }
 
 // y = M v (M symmetric l x l, fp64): one warp per row.
-__global__ void k_symv(const double* __restrict__ M, int lda, int l, const double* __restrict__ v,
+__global__ void k_symv(const double* M, int lda, int l, const double* v,
                        double* __restrict__ y) {
   pdl_enter();
   const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
@@ -1241,7 +1241,7 @@ __global__ void k_symv(const double* __restrict__ M, int lda, int l, const doubl
 
 // Power-iteration step for the largest eigenvalue of M (v unit): rq = v^T y, v <- y / |y|.
 // One block of 1024 threads; v0 != 0 on entry.
-__global__ void k_power_step(double* __restrict__ v, const double* __restrict__ y, int l,
+__global__ void k_power_step(double* __restrict__ v, const double* y, int l,
                              double* __restrict__ rq) {
   pdl_enter();
   __shared__ double s1[1024], s2[1024];
@@ -1272,7 +1272,7 @@ __global__ void k_init_unit(double* __restrict__ v, int l) {
 }
 
 // out[i][j] = (float)A[i][j] for i, j < l, 0 elsewhere in [ld][ld].
-__global__ void k_to_f32_pad(const double* __restrict__ A, int lda, int l, int ld,
+__global__ void k_to_f32_pad(const double* A, int lda, int l, int ld,
                              float* __restrict__ out) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1282,7 +1282,7 @@ __global__ void k_to_f32_pad(const double* __restrict__ A, int lda, int l, int l
 }
 
 // A[i][j] = src[i][j] + d (i == j) on the l x l block.
-__global__ void k_copy_shift(const double* __restrict__ src, double* __restrict__ A, int lda,
+__global__ void k_copy_shift(const double* src, double* __restrict__ A, int lda,
                              int l, double d) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -15,7 +15,7 @@ constexpr int kSortBatches = 8;                       // 32-item batches per war
 constexpr int kSortTile = kSortThreads * kSortBatches;  // 4096 items per block
 constexpr int kSortSelf = 128;  // up to this many blocks the scatter sums the histograms itself
 
-__global__ void k_scan_reduce(const uint32_t* __restrict__ data, int64_t n,
+__global__ void k_scan_reduce(const uint32_t* data, int64_t n,
                               uint32_t* __restrict__ block_sums) {
   pdl_enter();
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
@@ -57,7 +57,7 @@ __global__ void k_scan_top(uint32_t* __restrict__ block_sums, int64_t nb) {
 // blocks; a launch less than with k_scan_top, 2.5 us).
 template <bool SELF>
 __global__ void k_scan_down(uint32_t* __restrict__ data, int64_t n,
-                            const uint32_t* __restrict__ block_sums,
+                            const uint32_t* block_sums,
                             uint32_t* __restrict__ total) {
   pdl_enter();
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
@@ -83,7 +83,7 @@ __global__ void k_scan_down(uint32_t* __restrict__ data, int64_t n,
 
 // Digit counts of each block's items: [digit][block] for the scan, [block][digit] with SELF.
 template <bool SELF>
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t* __restrict__ keys,
+__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t* keys,
                                                              int64_t n, int shift,
                                                              uint32_t* __restrict__ hist,
                                                              int64_t nblk) {
@@ -118,9 +118,9 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t* __r
 // them, 1.5 us in place of the three launches of a scan.
 template <bool SELF>
 __global__ void __launch_bounds__(kSortThreads)
-    k_radix_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
+    k_radix_scatter(const uint32_t* kin, const uint32_t* vin,
                     uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, int64_t n, int shift,
-                    const uint32_t* __restrict__ offs, int64_t nblk) {
+                    const uint32_t* offs, int64_t nblk) {
   pdl_enter();
   __shared__ uint32_t cnt[kSortWarps][256];
   __shared__ uint32_t item[kSortTile];

@@ -156,6 +156,14 @@ struct SlotWalk {
 // kernel before (SLOT_AHEAD, then pdl_enter()).  A kernel that reads more ahead (ids,
 // weights, the state word) calls pdl_enter() inside the loop, where a second call costs
 // nothing; every block calls it at least once, also one without work.
+// Fields that change in an iteration and are read ahead of the wait; each writer has to stay two
+// launches or more ahead of each such reader, the kernels between them waiting before they end:
+//   state[0], state[1]  written by kb_check_beta (kb_update_p and kb_splat, which wait first,
+//                       follow it); read ahead by kb_splat_fix, kb_blur, kb_slice_dot, kb_alpha,
+//                       kb_update_xr and the next kb_check_beta
+//   rho                 written by kb_check_beta; read ahead by kb_alpha and kb_check_beta
+//   active              written by kb_check_beta (read ahead by kb_alpha) and by kb_alpha (read
+//                       ahead by kb_check_beta, with kb_update_xr between them)
 #define SLOT_AHEAD(KIND) const SlotWalk walk_(T->pre[KIND])
 #define SLOT_AHEAD_IN_LOOP(KIND)          \
   SLOT_AHEAD(KIND);                       \
@@ -388,7 +396,7 @@ __global__ void __launch_bounds__(kST) kb_blur(const Table* __restrict__ T, int 
       const int64_t e = (local * kBlurU + u) * groups + g;
       if (e >= count) break;
       const int64_t v = s.act[base + e];
-      const float4 own = Store<S>::ldg4(lat + v * kp + col);
+      const float4 own = Store<S>::ld4(lat + v * kp + col);
       const float fo = s.g0pow[t - s.epoch[v]];
       float4 acc = make_float4(s.taps[0] * fo * own.x, s.taps[0] * fo * own.y,
                                s.taps[0] * fo * own.z, s.taps[0] * fo * own.w);
@@ -399,12 +407,12 @@ __global__ void __launch_bounds__(kST) kb_blur(const Table* __restrict__ T, int 
         const int ic = nbr[(int64_t)(2 * tt + 1) * s.m + v];
         if (ia >= 0) {
           const float f = s.g0pow[t - s.epoch[ia]];
-          const float4 x = Store<S>::ldg4(lat + (int64_t)ia * kp + col);
+          const float4 x = Store<S>::ld4(lat + (int64_t)ia * kp + col);
           sum = make_float4(f * x.x, f * x.y, f * x.z, f * x.w);
         }
         if (ic >= 0) {
           const float f = s.g0pow[t - s.epoch[ic]];
-          const float4 x = Store<S>::ldg4(lat + (int64_t)ic * kp + col);
+          const float4 x = Store<S>::ld4(lat + (int64_t)ic * kp + col);
           sum = make_float4(sum.x + f * x.x, sum.y + f * x.y, sum.z + f * x.z, sum.w + f * x.w);
         }
         const float wt = s.taps[tt + 1];
@@ -435,11 +443,11 @@ __global__ void __launch_bounds__(kST) kb_blur(const Table* __restrict__ T, int 
   float4 own[kBlurU], sa[kBlurU][R], sc[kBlurU][R];
 #pragma unroll
   for (int u = 0; u < kBlurU; ++u) {
-    own[u] = v[u] < m ? Store<S>::ldg4(in + v[u] * kp + col) : zero;
+    own[u] = v[u] < m ? Store<S>::ld4(in + v[u] * kp + col) : zero;
 #pragma unroll
     for (int tt = 0; tt < R; ++tt) {
-      sa[u][tt] = ia[u][tt] >= 0 ? Store<S>::ldg4(in + (int64_t)ia[u][tt] * kp + col) : zero;
-      sc[u][tt] = ic[u][tt] >= 0 ? Store<S>::ldg4(in + (int64_t)ic[u][tt] * kp + col) : zero;
+      sa[u][tt] = ia[u][tt] >= 0 ? Store<S>::ld4(in + (int64_t)ia[u][tt] * kp + col) : zero;
+      sc[u][tt] = ic[u][tt] >= 0 ? Store<S>::ld4(in + (int64_t)ic[u][tt] * kp + col) : zero;
     }
   }
   if (SLOT_LAST) pdl_leave();
@@ -1314,7 +1322,7 @@ __global__ void k_probe_fill(float* __restrict__ V, int64_t n_all, int64_t n_tra
 
 // Largest training-row sum max_i KZ[i][kp - 1] (i < n_train) of outputscale K~_XX; the
 // entries are non-negative, so the float bits order like the values (*out preset to 0).
-__global__ void k_rowsum_max(const float* __restrict__ KZ, int64_t n_train, int kp,
+__global__ void k_rowsum_max(const float* KZ, int64_t n_train, int kp,
                              int* __restrict__ out) {
   pdl_enter();
   __shared__ float red[256];
@@ -1333,8 +1341,8 @@ __global__ void k_rowsum_max(const float* __restrict__ KZ, int64_t n_train, int 
 
 // b (locality order): training rows [y, (KX* z)_1..S, 0 ...], test rows 0; r = p = b,
 // x = 0.  KZ is the probe product in the caller's order.
-__global__ void k_rhs(const int32_t* __restrict__ perm, const float* __restrict__ y,
-                      const float* __restrict__ KZ, int64_t n_all, int64_t n_train, int kp,
+__global__ void k_rhs(const int32_t* __restrict__ perm, const float* y,
+                      const float* KZ, int64_t n_all, int64_t n_train, int kp,
                       int S, float* __restrict__ xh, float* __restrict__ xl,
                       float* __restrict__ rh, float* __restrict__ rl, float* __restrict__ p) {
   pdl_enter();
@@ -1352,7 +1360,7 @@ __global__ void k_rhs(const int32_t* __restrict__ perm, const float* __restrict_
   p[e] = b;
 }
 
-__global__ void k_x_sum(const float* __restrict__ xh, const float* __restrict__ xl,
+__global__ void k_x_sum(const float* xh, const float* xl,
                         float* __restrict__ out, int64_t count) {
   pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1360,7 +1368,7 @@ __global__ void k_x_sum(const float* __restrict__ xh, const float* __restrict__ 
 }
 
 // mean[t] = (K*X W)[t][0]; var[t] = outputscale - (1/S) sum_s z_s[t] (K*X W)[t][1 + s].
-__global__ void k_predict(const int32_t* __restrict__ perm, const float* __restrict__ KW,
+__global__ void k_predict(const int32_t* __restrict__ perm, const float* KW,
                           int64_t n_all, int64_t n_train, int kp, int S, uint64_t seed,
                           float outputscale, float* __restrict__ mean, float* __restrict__ var) {
   pdl_enter();

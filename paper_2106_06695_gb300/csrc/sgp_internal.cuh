@@ -160,10 +160,19 @@ cudaError_t cols_malloc(const sgp_lattice* L, int columns, void** p, size_t byte
 // launch waits for the previous grid to drain, and 1.4-1.6 us apart when it is set up
 // beforehand and only waits for the data (measured: 200 dependent kernels of 152 blocks,
 // legacy and created streams; inside a graph 1.15 and 0.94 us).  launch_pdl marks a launch as
-// such a dependent; every kernel launched with it starts with pdl_enter(), which waits until
-// all work before this grid has completed and is visible.  Nothing is read or written
-// before that wait but arrays that do not change after the build (neighbour ids), so ordering is
-// as with ordinary launches.  Dependents are not let in early (griddepcontrol.launch_dependents
+// such a dependent; every block of a kernel launched with it calls pdl_enter(), which waits until
+// all work before this grid has completed and is visible.  What keeps the order that ordinary
+// launches have:
+//  - Nothing is written before the wait.
+//  - Read before it are only arrays that do not change after the build (neighbour ids), and data
+//    whose last writer is a grid that the grid right before this one has itself waited for, so
+//    at least two launches back (the server's table kernels: the list stands at SLOT_AHEAD).
+//  - What grids of the same stream write is read by ordinary loads: neither __ldg nor pointers
+//    that are const and __restrict__.  Those stand for data that do not change while the kernel
+//    runs, and a dependent runs already while the writer does; the compiler might also move
+//    such a load ahead of the wait.  Only the arrays that are fixed after the build (and the
+//    server's table) are declared so.
+// Dependents are not let in early (griddepcontrol.launch_dependents
 // at the top of each kernel): their waiting blocks take slots from the running grid (a
 // product at n = 50k, d = 8, k = 9: 63 us without, 78 us with it; eight CG iterations at n =
 // 86k, d = 8: 998 and 1154 us).  After the last loads are issued it does no harm (pdl_leave).

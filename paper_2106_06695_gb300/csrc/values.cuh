@@ -18,15 +18,12 @@ struct Store<float> {
   static __device__ __forceinline__ float4 ld4(const float* p) {
     return *reinterpret_cast<const float4*>(p);
   }
-  static __device__ __forceinline__ float4 ldg4(const float* p) {
-    return __ldg(reinterpret_cast<const float4*>(p));
-  }
   static __device__ __forceinline__ void st4(float* p, float4 v) {
     *reinterpret_cast<float4*>(p) = v;
   }
-  static __device__ __forceinline__ void ldg8(const float* p, float4& a, float4& b) {
-    a = __ldg(reinterpret_cast<const float4*>(p));
-    b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  static __device__ __forceinline__ void ld8(const float* p, float4& a, float4& b) {
+    a = reinterpret_cast<const float4*>(p)[0];
+    b = reinterpret_cast<const float4*>(p)[1];
   }
   static __device__ __forceinline__ void st8(float* p, float4 a, float4 b) {
     reinterpret_cast<float4*>(p)[0] = a;
@@ -34,9 +31,6 @@ struct Store<float> {
   }
   static __device__ __forceinline__ float2 ld2(const float* p) {
     return *reinterpret_cast<const float2*>(p);
-  }
-  static __device__ __forceinline__ float2 ldg2(const float* p) {
-    return __ldg(reinterpret_cast<const float2*>(p));
   }
   static __device__ __forceinline__ void st2(float* p, float2 v) {
     *reinterpret_cast<float2*>(p) = v;
@@ -66,14 +60,11 @@ struct Store<bf16> {
   static __device__ __forceinline__ float4 ld4(const bf16* p) {
     return cvt(*reinterpret_cast<const uint2*>(p));
   }
-  static __device__ __forceinline__ float4 ldg4(const bf16* p) {
-    return cvt(__ldg(reinterpret_cast<const uint2*>(p)));
-  }
   static __device__ __forceinline__ void st4(bf16* p, float4 v) {
     *reinterpret_cast<uint2*>(p) = make_uint2(pack2(v.x, v.y), pack2(v.z, v.w));
   }
-  static __device__ __forceinline__ void ldg8(const bf16* p, float4& a, float4& b) {
-    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+  static __device__ __forceinline__ void ld8(const bf16* p, float4& a, float4& b) {
+    const uint4 u = *reinterpret_cast<const uint4*>(p);
     a = cvt(make_uint2(u.x, u.y));
     b = cvt(make_uint2(u.z, u.w));
   }
@@ -83,9 +74,6 @@ struct Store<bf16> {
   }
   static __device__ __forceinline__ float2 ld2(const bf16* p) {
     return unpack2(*reinterpret_cast<const uint32_t*>(p));
-  }
-  static __device__ __forceinline__ float2 ldg2(const bf16* p) {
-    return unpack2(__ldg(reinterpret_cast<const uint32_t*>(p)));
   }
   static __device__ __forceinline__ void st2(bf16* p, float2 v) {
     *reinterpret_cast<uint32_t*>(p) = pack2(v.x, v.y);
@@ -113,13 +101,8 @@ struct Vec<4> {
   static __device__ __forceinline__ T zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
   static __device__ __forceinline__ T ld(const float* p) { return *reinterpret_cast<const float4*>(p); }
   static __device__ __forceinline__ void st(float* p, T v) { *reinterpret_cast<float4*>(p) = v; }
-  static __device__ __forceinline__ T ldg(const float* p) {
-    return __ldg(reinterpret_cast<const float4*>(p));
-  }
   template <class S>
   static __device__ __forceinline__ T lds(const S* p) { return Store<S>::ld4(p); }
-  template <class S>
-  static __device__ __forceinline__ T ldgs(const S* p) { return Store<S>::ldg4(p); }
   template <class S>
   static __device__ __forceinline__ void sts(S* p, T v) { Store<S>::st4(p, v); }
   static __device__ __forceinline__ T fma(float a, T x, T y) {
@@ -138,13 +121,8 @@ struct Vec<2> {
   static __device__ __forceinline__ T zero() { return make_float2(0.f, 0.f); }
   static __device__ __forceinline__ T ld(const float* p) { return *reinterpret_cast<const float2*>(p); }
   static __device__ __forceinline__ void st(float* p, T v) { *reinterpret_cast<float2*>(p) = v; }
-  static __device__ __forceinline__ T ldg(const float* p) {
-    return __ldg(reinterpret_cast<const float2*>(p));
-  }
   template <class S>
   static __device__ __forceinline__ T lds(const S* p) { return Store<S>::ld2(p); }
-  template <class S>
-  static __device__ __forceinline__ T ldgs(const S* p) { return Store<S>::ldg2(p); }
   template <class S>
   static __device__ __forceinline__ void sts(S* p, T v) { Store<S>::st2(p, v); }
   static __device__ __forceinline__ T fma(float a, T x, T y) {
@@ -159,11 +137,8 @@ struct Vec<1> {
   static __device__ __forceinline__ T zero() { return 0.f; }
   static __device__ __forceinline__ T ld(const float* p) { return *p; }
   static __device__ __forceinline__ void st(float* p, T v) { *p = v; }
-  static __device__ __forceinline__ T ldg(const float* p) { return __ldg(p); }
   template <class S>
   static __device__ __forceinline__ T lds(const S* p) { return Store<S>::ld1(p); }
-  template <class S>
-  static __device__ __forceinline__ T ldgs(const S* p) { return Store<S>::ld1(p); }
   template <class S>
   static __device__ __forceinline__ void sts(S* p, T v) { Store<S>::st1(p, v); }
   static __device__ __forceinline__ T fma(float a, T x, T y) { return fmaf(a, x, y); }
