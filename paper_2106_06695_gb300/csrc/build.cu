@@ -560,10 +560,13 @@ __global__ void k_entry_ids(const int32_t* entry_slot,
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nD) return;
   const int32_t s = entry_slot[e];
-  idx[e] = s >= 0 ? slot_id[s] : 0;
   const int64_t u = (int64_t)perm[e / D] * D + (e % D);
-  w[e] = w_user[u];
-  rank[e] = rank_user[u];
+  const int32_t id = s >= 0 ? slot_id[s] : 0;  // all loads ahead of the stores
+  const float wt = w_user[u];
+  const uint8_t rk = rank_user[u];
+  idx[e] = id;
+  w[e] = wt;
+  rank[e] = rk;
 }
 
 // ---------------------------------------------------------------------------------
@@ -680,12 +683,14 @@ __global__ void k_hash_index(const uint32_t* key, const uint32_t* ord,
   pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
-  const uint64_t h = vhash[ord[i]];
+  const uint32_t v = ord[i];
+  const int64_t own = key[i], first = i == 0 ? 0 : (int64_t)key[i - 1] + 1;
+  const uint64_t h = vhash[v];  // all loads ahead of the stores
+  const uint8_t dir = up[v];
   low[i] = (uint32_t)h;
   high[i] = (uint32_t)(h >> 32);
-  up_sorted[i] = up[ord[i]];
-  const int64_t own = key[i];
-  for (int64_t b = i == 0 ? 0 : (int64_t)key[i - 1] + 1; b <= own; ++b) start[b] = (uint32_t)i;
+  up_sorted[i] = dir;
+  for (int64_t b = first; b <= own; ++b) start[b] = (uint32_t)i;
   if (i == m - 1)
     for (int64_t b = own + 1; b <= buckets; ++b) start[b] = (uint32_t)m;
 }
@@ -702,9 +707,10 @@ __device__ __forceinline__ bool steps_to(int16_t v, int16_t u, int c, int j, int
 // the keys by the thread itself for D <= 16 (every row load in flight at once), by the whole
 // warp, one after another, above (a lane alone would walk a row of D loads while 31 wait).
 // *hits receives the number of pairs (v, v + u_j).
+// Five blocks an SM (48 registers): n = 500k, d = 20 0.93 ms, 1.08 with the 54 registers it would take.
 constexpr int kNbrGroup = 4;
 template <bool WARP>
-__global__ void __launch_bounds__(256) k_neighbours(
+__global__ void __launch_bounds__(256, 5) k_neighbours(
     const int16_t* keys, const uint32_t* low,
     const uint32_t* high, const uint8_t* up,
     const uint32_t* ord, const uint32_t* start, int shift, int64_t m,
@@ -746,11 +752,7 @@ __global__ void __launch_bounds__(256) k_neighbours(
           const bool match = p[q] < end[q];
           unsigned todo = __ballot_sync(0xffffffffu, match);
           if (!todo) break;
-          uint32_t u = 0, v = 0;
-          if (match) {
-            u = ord[p[q]];
-            v = ord[i];
-          }
+          const uint32_t u = match ? ord[p[q]] : 0u, v = match ? ord[i] : 0u;
           bool ok = false;
           if (WARP) {
             while (todo) {
