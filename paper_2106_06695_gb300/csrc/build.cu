@@ -851,7 +851,7 @@ __global__ void __launch_bounds__(256) k_link_counts(LinkBits lb, int64_t m, int
 // blur, which updates its vertices independently.
 constexpr int kFillThreads = 512;
 __global__ void __launch_bounds__(kFillThreads) k_active_fill(
-    const uint32_t* hasnb, int64_t m, int D, const int64_t* off,
+    LinkBits lb, int64_t m, int D, const int64_t* off,
     unsigned long long* __restrict__ fill, int32_t* __restrict__ act) {
   pdl_enter();
   constexpr int kWarps = kFillThreads / 32;
@@ -862,7 +862,7 @@ __global__ void __launch_bounds__(kFillThreads) k_active_fill(
   for (int e = threadIdx.x; e < kWarps * kMaxD; e += blockDim.x) (&wpos[0][0])[e] = 0;
   __syncthreads();
   for (int w = 0; w * 32 < D; ++w) {
-    const uint32_t bits = live ? hasnb[(int64_t)w * m + v] : 0u;
+    const uint32_t bits = live ? lb.above[(int64_t)w * m + v] | lb.below[(int64_t)w * m + v] : 0u;
     uint32_t seen = __reduce_or_sync(0xffffffffu, bits);
     while (seen) {
       const int b = __ffs(seen) - 1;
@@ -885,7 +885,7 @@ __global__ void __launch_bounds__(kFillThreads) k_active_fill(
   }
   __syncthreads();
   for (int w = 0; w * 32 < D; ++w) {
-    const uint32_t bits = live ? hasnb[(int64_t)w * m + v] : 0u;
+    const uint32_t bits = live ? lb.above[(int64_t)w * m + v] | lb.below[(int64_t)w * m + v] : 0u;
     uint32_t seen = __reduce_or_sync(0xffffffffu, bits);
     while (seen) {
       const int b = __ffs(seen) - 1;
@@ -902,7 +902,8 @@ __global__ void __launch_bounds__(kFillThreads) k_active_fill(
 // which it heads a chain.  Every head walks its chain for the length (all lanes at once: the
 // walks are chains of dependent loads), the block takes one range of list slots and one of
 // chain slots per direction, and each head walks again to write its chain.  The order of
-// the chains is immaterial.  *longest: the longest chain.
+// the chains is immaterial.  *longest: the longest chain; beyond kMaxChain the walks stop, the
+// lists are incomplete and the host has k_active_fill write them.
 __global__ void __launch_bounds__(kFillThreads) k_chain_fill(
     LinkBits lb, const int32_t* nbr, int64_t m, int D,
     const int64_t* off, const int64_t* chain_off,
@@ -917,11 +918,13 @@ __global__ void __launch_bounds__(kFillThreads) k_chain_fill(
   auto heads = [&](int w) {
     return live ? lb.above[(int64_t)w * m + v] & ~lb.below[(int64_t)w * m + v] : 0u;
   };
-  // length of the chain v heads along j (at most m steps: a line visits no vertex twice)
+  // length of the chain v heads along j, as far as it matters: a chain may run over 64000 / D
+  // vertices, each a dependent load (n = 3400, d = 20 with a chain of 3000: 1930 us a build,
+  // 460 with the limit)
   auto length = [&](int j) {
     const int32_t* above = nbr + ((int64_t)j * 2 + 1) * m;
     unsigned len = 1;
-    for (int32_t x = above[v]; x >= 0 && len < (unsigned)m; x = above[x]) ++len;
+    for (int32_t x = above[v]; x >= 0 && len <= (unsigned)kMaxChain; x = above[x]) ++len;
     return len;
   };
   int most = 0;
@@ -1491,8 +1494,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
         SGP_CHECK(cudaMemcpyAsync(&L->chain_max, longest, sizeof(int), cudaMemcpyDeviceToHost, st),
                   "read chains");
       } else {
-        launch_pdl(k_active_fill, grid, kFillThreads, st, lb.above, m, D, L->act_off_dev, counts + D,
-                   L->act);
+        launch_pdl(k_active_fill, grid, kFillThreads, st, lb, m, D, L->act_off_dev, counts + D, L->act);
       }
       note_launches(1);
       // powers of the symmetric blur's centre tap g_0 (stored rows are rescaled lazily)
@@ -1506,6 +1508,17 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
     }
   }
   SGP_CHECK(cudaStreamSynchronize(st), "sync build");
+  if (L->chain_max > kMaxChain) {  // blurred through the direction lists, without chains
+    SGP_CHECK(cudaFreeAsync(L->chain, st), "free chains");
+    L->chain = nullptr;
+    L->bytes -= (size_t)L->chain_off.back() * sizeof(uint2);
+    SGP_CHECK(cudaMemsetAsync(counts + D, 0, D * sizeof(unsigned long long), st), "clear list fill");
+    launch_pdl(k_active_fill, (unsigned)ceil_div(m, kFillThreads), kFillThreads, st, lb, m, D,
+               L->act_off_dev, counts + D, L->act);
+    note_launches(1);
+    SGP_CHECK(cudaGetLastError(), "direction lists");
+    SGP_CHECK(cudaStreamSynchronize(st), "sync direction lists");
+  }
   return SGP_OK;
 }
 
