@@ -1466,8 +1466,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
       total += (int64_t)hc[j];
       largest = std::max<int64_t>(largest, (int64_t)hc[j]);
     }
-    if (m > 0 && (double)total <= kSparseFrac * (double)D * (double)m &&
-        total <= (int64_t)0xffffffff) {  // chains hold 32-bit positions
+    if (m > 0 && (double)total <= kSparseFrac * (double)D * (double)m) {
       L->sparse = true;
       L->act_max = largest;
       L->act_off.assign(D + 1, 0);
@@ -1483,7 +1482,7 @@ sgp_status build_lattice(Lattice* L, const float* X, const float* ls) {
                                 cudaMemcpyHostToDevice, st),
                 "copy list offsets");
       const unsigned grid = (unsigned)ceil_div(m, kFillThreads);
-      if (r == 1) {
+      if (r == 1 && total <= (int64_t)0xffffffff) {  // chains hold 32-bit positions in the lists
         L->chain_off.assign(offsets.begin() + D + 1, offsets.end());
         const int64_t chains = L->chain_off.back();
         SGP_CHECK(dalloc(&L->chain, std::max<int64_t>(chains, 1), st), "alloc chains");

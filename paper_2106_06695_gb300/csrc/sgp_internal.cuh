@@ -104,7 +104,7 @@ struct sgp_lattice {
   // chain[chain_off[j] .. chain_off[j+1]) holds (begin, end) of direction j's chains in act.
   uint2* chain = nullptr;
   std::vector<int64_t> chain_off;  // [D + 1], host
-  int chain_max = 0;             // longest chain; 0: no chains (order > 1)
+  int chain_max = 0;  // longest chain, kMaxChain + 1 for any longer one; 0: no chains (order > 1)
   bool table_blur = false;       // blurred by the server's table kernels too (needs act_tmp)
   int32_t* epoch = nullptr;      // [m] pass after which a vertex's stored row was written
   void* act_tmp = nullptr;       // [act_max][k] new values of one pass
