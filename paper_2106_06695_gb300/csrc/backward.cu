@@ -289,7 +289,7 @@ sgp_status backward(Lattice* L, const float* X, const float* ls, const float* V,
       BW_CHECK(w.get(&Gp, (size_t)n * kp2 * one, L, kp2), "alloc G, V");
       Vp = Gp + kp;
       enqueue_permute_pair(L, G, V, k, kp, Gp, st);
-      BS = enqueue_splat_blur(L, Gp, kp2, kp2, blur, b0, b1, part, st, &scale);
+      BS = enqueue_splat_blur(L, Gp, kp2, k, blur, b0, b1, part, st, &scale);
       BU = static_cast<const char*>(BS) + vb / L->m;
     } else {
       BW_CHECK(w.get(&b0, vb, L, kp), "alloc lattice values");

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kThreads) k_splat(int64_t nseg, int G, int k,
 
 // Fix-up of the vertices with several segments, in one launch.  Blocks below `nhuge`: one
 // vertex of more than kSplatMedSegs segments each, in `groups` (a power of two, groups G <=
-// kThreads) strided partial sums and a fixed-shape shared-memory tree over them (the result
+// kThreads, or twice that where two products share the rows) strided partial sums and a fixed-shape shared-memory tree over them (the result
 // depends on `groups` only, not on how the threads share the work).  The blocks after them:
 // one thread-group per vertex of 2..kSplatMedSegs segments, summed in order.
 template <int VEC, class S>
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kThreads) k_splat_fix(int nhuge, int64_t nmed,
                                                         float scale, S* __restrict__ lat) {
   pdl_enter();
   using Vt = Vec<VEC>;
-  __shared__ typename Vt::T red[kThreads];
+  __shared__ typename Vt::T red[2 * kThreads];
   if ((int)blockIdx.x >= nhuge) {
     const int rows = kThreads / G;
     const int64_t q = (int64_t)((int)blockIdx.x - nhuge) * rows + threadIdx.x / G;
@@ -730,7 +730,8 @@ void by_vec(int vec, F f) {
 // ---- launchers -----------------------------------------------------------------------
 // scale: a power of two on the splatted values (1 but for fp32 chains).
 // kt: the column count that fixes the shape of the huge vertices' summation tree (the
-// caller's k, so that padding does not change a result).
+// caller's k, so that neither padding nor a second product beside it changes a result); kp is
+// at most twice kt rounded up.
 template <class S>
 void launch_splat_t(const Lattice* L, const float* V, int kp, int kt, float scale, S* lat,
                     float* partial, cudaStream_t st) {
