@@ -31,8 +31,9 @@ constexpr double kSlqStep = 0.45;  // trapezoid step in log t
 
 // Block (w, c): warp w of probe c.  Warps 0 .. kSlqWarps - 1 sum the integrand at the nodes
 // 32 w + lane (+ 256, ...), in a fixed order, into part[c][w] (scaled: the probe's value is
-// the plain sum of its parts); warp kSlqWarps sets *bad when T is not numerically positive
-// definite (a pivot of its LDL^T at or below zero, or an entry that is not finite).
+// the plain sum of its parts; a probe without iterations has none); warp kSlqWarps sets bad[c] when
+// T is not numerically positive definite (a pivot of its LDL^T at or below zero, or an entry that
+// is not finite).
 //
 // Bound by the latency of one fp64 division per step of the fraction.  The nodes are spread
 // over one-warp blocks, so that a probe uses nine SMs' fp64 pipes.  It replaced an implicit
@@ -65,7 +66,7 @@ __global__ void __launch_bounds__(32) k_slq(const double* ha,
       prev = piv;
       ok = piv > 0.0 && isfinite(piv) && isfinite(off2);
     }
-    if (!ok) atomicOr(bad, 1);
+    bad[c] = ok ? 0 : 1;
     return;
   }
   double sum = 0.0;
@@ -97,7 +98,7 @@ __global__ void __launch_bounds__(32) k_slq(const double* ha,
     }
   }
   for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if (lane == 0) part[c * kSlqWarps + w] = bnorm[c] * bnorm[c] * kSlqStep * sum;
+  if (lane == 0) part[c * kSlqWarps + w] = m > 0 ? bnorm[c] * bnorm[c] * kSlqStep * sum : 0.0;
 }
 
 // sp: columns of the solver's rows (zero columns appended).
@@ -134,8 +135,7 @@ sgp_status logdet_rows(Lattice* L, const float* Z, int s, int sp, float noise, i
   LZ_CHECK(get((void**)&rec.iters, (size_t)sp * sizeof(int)), "alloc Lanczos record");
   LZ_CHECK(get((void**)&X, (size_t)L->n * s * sizeof(float)), "alloc CG solution");
   LZ_CHECK(get((void**)&dq, (size_t)s * kSlqWarps * sizeof(double)), "alloc quadratures");
-  LZ_CHECK(get((void**)&bad, sizeof(int)), "alloc flag");
-  LZ_CHECK(cudaMemsetAsync(bad, 0, sizeof(int), st), "clear flag");
+  LZ_CHECK(get((void**)&bad, (size_t)s * sizeof(int)), "alloc flags");
   sgp_status status = run_cg(L, Z, s, SGP_BLUR_SYMMETRIC, noise, tol, cap, X, nullptr, nullptr,
                              0, 0, &rec);
   if (status != SGP_OK) return status;
@@ -144,21 +144,23 @@ sgp_status logdet_rows(Lattice* L, const float* Z, int s, int sp, float noise, i
   note_launches(1);
   LZ_CHECK(cudaGetLastError(), "Lanczos quadrature");
   std::vector<double> hq(s, 0.0), hp((size_t)s * kSlqWarps);
-  int hbad = 0;
+  std::vector<int> hbad(s, 0);
   LZ_CHECK(cudaMemcpyAsync(hp.data(), dq, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, st),
            "read quadratures");
-  LZ_CHECK(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, st), "read flag");
+  LZ_CHECK(cudaMemcpyAsync(hbad.data(), bad, s * sizeof(int), cudaMemcpyDeviceToHost, st),
+           "read flags");
   LZ_CHECK(cudaStreamSynchronize(st), "sync Lanczos");
 #undef LZ_CHECK
-  for (int c = 0; c < s; ++c)
+  for (int c = 0; c < s; ++c) {
     for (int w = 0; w < kSlqWarps; ++w) hq[c] += hp[(size_t)c * kSlqWarps + w];
+    if (hbad[c]) hq[c] = std::nan("");
+  }
   if (quad) std::copy(hq.begin(), hq.end(), quad);
   double sum = 0.0;
   for (double v : hq) sum += v;
   if (logdet) *logdet = sum / s;
-  if (hbad) {
-    set_error("sgp_logdet: a Lanczos tridiagonal was not positive definite or its eigenvalues "
-              "did not converge");
+  if (std::find(hbad.begin(), hbad.end(), 1) != hbad.end()) {
+    set_error("sgp_logdet: a Lanczos tridiagonal was not numerically positive definite");
     return SGP_ERR_NONFINITE;
   }
   return SGP_OK;
