@@ -29,11 +29,60 @@ constexpr int kMaxLanczos = 256;
 constexpr int kSlqWarps = 8;     // node warps per probe (256 nodes: one round as a rule)
 constexpr double kSlqStep = 0.45;  // trapezoid step in log t
 
+constexpr double kQlFree = 1e-12;
+constexpr int kQlSweeps = 64;  // QL iterations allowed per eigenvalue
+
+// Whether the implicit QL iteration with Wilkinson shifts (Bowdler, Martin, Reinsch & Wilkinson
+// 1968) finds all eigenvalues of the symmetric tridiagonal (diagonal d, e[i] coupling i and i + 1)
+// above zero.  Overwrites d and e.
+__device__ __noinline__ bool ql_positive(double* d, double* e, int m) {
+  for (int l = 0; l < m; ++l) {
+    for (int sweep = 0;; ++sweep) {
+      int mm = l;
+      for (; mm < m - 1; ++mm)
+        if (fabs(e[mm]) <= 1e-15 * (fabs(d[mm]) + fabs(d[mm + 1]))) break;
+      if (mm == l) break;
+      if (sweep == kQlSweeps) return false;
+      double g = (d[l + 1] - d[l]) / (2.0 * e[l]);  // shift from the leading 2 x 2 block
+      double r = hypot(g, 1.0);
+      g = d[mm] - d[l] + e[l] / (g + copysign(r, g));
+      double s = 1.0, c = 1.0, p = 0.0;
+      int i = mm - 1;
+      for (; i >= l; --i) {
+        const double f = s * e[i], b = c * e[i];
+        r = hypot(f, g);
+        e[i + 1] = r;
+        if (r == 0.0) {  // split: deflate and restart this eigenvalue
+          d[i + 1] -= p;
+          e[mm] = 0.0;
+          break;
+        }
+        s = f / r;
+        c = g / r;
+        g = d[i + 1] - p;
+        r = (d[i] - g) * s + 2.0 * c * b;
+        p = s * r;
+        d[i + 1] = g + p;
+        g = c * r - b;
+      }
+      if (r == 0.0 && i >= l) continue;
+      d[l] -= p;
+      e[l] = g;
+      e[mm] = 0.0;
+    }
+    if (!(d[l] > 0.0)) return false;  // not touched again
+  }
+  return true;
+}
+
 // Block (w, c): warp w of probe c.  Warps 0 .. kSlqWarps - 1 sum the integrand at the nodes
 // 32 w + lane (+ 256, ...), in a fixed order, into part[c][w] (scaled: the probe's value is
 // the plain sum of its parts; a probe without iterations has none); warp kSlqWarps sets bad[c] when
-// T is not numerically positive definite (a pivot of its LDL^T at or below zero, or an entry that
-// is not finite).
+// T is not numerically positive definite: an entry that is not finite, or an eigenvalue that the QL
+// iteration rounds to zero or below.  (Every pivot of T's LDL^T is 1 / alpha_j > 0, whatever the
+// operator: a singular one shows only in what rounding does to T's smallest eigenvalues.)  QL's
+// eigenvalues are off by some 1e-13 ||T|| at most, so it need not run when all are above kQlFree
+// ||T||, which the LDL^T of the shifted T tells: m divisions in place of some 150 m rotations.
 //
 // Bound by the latency of one fp64 division per step of the fraction.  The nodes are spread
 // over one-warp blocks, so that a probe uses nine SMs' fp64 pipes.  It replaced an implicit
@@ -55,18 +104,28 @@ __global__ void __launch_bounds__(32) k_slq(const double* ha,
   }
   __syncwarp();
   if (w == kSlqWarps) {
-    if (lane != 0) return;
-    double prev = 1.0, off2 = 0.0;  // previous pivot, squared coupling to it
+    __shared__ double d[kMaxLanczos], e[kMaxLanczos];
+    double norm = 0.0;
     bool ok = true;
-    for (int j = 0; j < m && ok; ++j) {
-      const double d = 1.0 / al[j] + (j > 0 ? be[j - 1] / al[j - 1] : 0.0);
-      const double piv = d - off2 / prev;
-      const double o = sqrt(be[j]) / al[j];
-      off2 = o * o;
-      prev = piv;
-      ok = piv > 0.0 && isfinite(piv) && isfinite(off2);
+    for (int j = lane; j < m; j += 32) {
+      d[j] = 1.0 / al[j] + (j > 0 ? be[j - 1] / al[j - 1] : 0.0);
+      e[j] = sqrt(be[j]) / al[j];  // 0 for the last
+      norm = fmax(norm, d[j] + 2.0 * e[j]);
+      ok = ok && isfinite(d[j]) && isfinite(e[j]);
     }
-    bad[c] = ok ? 0 : 1;
+    // twice the largest of the rows' d + 2 e bounds what Gershgorin's circles reach
+    for (int o = 16; o >= 1; o >>= 1) norm = fmax(norm, __shfl_xor_sync(0xffffffffu, norm, o));
+    norm *= 2.0;
+    ok = __all_sync(0xffffffffu, ok);
+    __syncwarp();
+    if (lane != 0) return;
+    bool clear = true;  // T - kQlFree norm I is positive definite
+    double piv = 1.0;
+    for (int j = 0; j < m && ok && clear; ++j) {
+      piv = d[j] - kQlFree * norm - (j > 0 ? e[j - 1] * e[j - 1] / piv : 0.0);
+      clear = piv > 0.0;
+    }
+    bad[c] = ok && (clear || ql_positive(d, e, m)) ? 0 : 1;
     return;
   }
   double sum = 0.0;
