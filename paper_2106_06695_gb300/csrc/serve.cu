@@ -29,9 +29,9 @@
 // An iteration of a small request is a chain of latencies, not of bytes: the kernels read the
 // table (and ids and weights where they can) ahead of the wait for the kernel before, and
 // issue the loads of several rows or items together.  40,000 points, d = 8, 12 columns, rank
-// 100: 142 us an iteration of 30 kernels (blur 18 x 4.4, z 16, B^T r 13, slice 12.5, x/r 11.6,
+// 100: 142 us an iteration of 29 kernels (blur 18 x 4.4, z 16, B^T r 13, slice 12.5, x/r 11.6,
 // splat 9.9, the others 4.4 to 5.8 each when run apart); 196 with table searches, single loads
-// in flight and 32 kernels.
+// in flight and 31 kernels.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -1801,7 +1801,7 @@ sgp_status setup(sgp_server* S, Request* R, cudaStream_t st, Table& t1) {
     launch_pdl(kb_bt_sum, kGrid, kST, st, R->dtab1);
     launch_pdl(kb_minv, kGrid, kMinvT, st, R->dtab1);
     launch_apply_z(kp, R->dtab1, st);
-    note_launches(5);
+    note_launches(4);
   }
   launch_pdl(kb_init_scalars, 1, kST, st, R->dtab1);
   note_launches(1);
