@@ -426,10 +426,11 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
   float *xh, *xl, *rh, *rl, *p, *Ap;
   CgState S{};
   const int vec = k % 4 == 0 ? 4 : 1;
-  const int T = column_block_threads(k, vec);
+  const int kt = rec ? kb : k;  // shapes the sums
+  const int T = column_block_threads(k, vec, kt);
   const int64_t rows_per_block = T / (k / vec);
   const unsigned vblocks = (unsigned)std::min<int64_t>(kVecBlocks, std::max<int64_t>(1, ceil_div(n, rows_per_block)));
-  const int64_t sblocks = slice_dot_blocks(L, k);
+  const int64_t sblocks = slice_dot_blocks(L, k, kt);
   const bool want_pre = precond_rank > 0 && noise > 0.f && !rec;
   // bounds ShiftedNystrom::dot_blocks (its z blocks: at most one per 128-row tile)
   const int64_t pblocks = want_pre ? ceil_div(n, 128) : 0;
@@ -511,7 +512,7 @@ sgp_status run_cg(Lattice* L, const float* B, int k, int blur, float noise, floa
   auto iteration = [&]() {
     // Ap = outputscale K~ p + noise p, with the slice also summing <p, Ap>: alpha
     passes = enqueue_mvm(L, p, k, blur, L->outputscale, noise, Ap, st, ev, /*internal=*/true,
-                         S.partial, rec ? kb : k);
+                         S.partial, kt);
     end(CG_ALPHA, sblocks);
     if (vec == 4)
       launch_pdl(k_cg_update_xr<4>, vblocks, T, st, xh, xl, rh, rl, p, Ap, n, k, S);

@@ -812,11 +812,11 @@ void launch_slice_t(const Lattice* L, const S* lat, const float* Vp, int k, int 
 }
 
 template <class S>
-void launch_slice_dot(const Lattice* L, const S* lat, const float* V, int k, float alpha,
+void launch_slice_dot(const Lattice* L, const S* lat, const float* V, int k, int kt, float alpha,
                       float beta, float* out, double* dot_partial, cudaStream_t st) {
   const int vec = k % 4 == 0 ? 4 : 1;
-  const int T = column_block_threads(k, vec);
-  const unsigned grid = (unsigned)slice_dot_blocks(L, k);
+  const int T = column_block_threads(k, vec, kt);
+  const unsigned grid = (unsigned)slice_dot_blocks(L, k, kt);
   if (vec == 4)
     launch_pdl(k_slice_dot<4, S>, grid, T, st, L->n, k / 4, k, L->D, L->idx, L->w, lat, V, alpha, beta,
                                           out, dot_partial);
@@ -1071,7 +1071,7 @@ int enqueue_t(const Lattice* L, const float* V, int k, int kp, int kt, int blur,
   S* a = blur_passes_t<S>(L, blur, lat0, lat1, kp, st, &passes, dense, &scale);
   alpha = (float)(alpha * scale);
   if (ev) cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal);
-  if (internal && dot_partial) launch_slice_dot<S>(L, a, V, kp, alpha, beta, out, dot_partial, st);
+  if (internal && dot_partial) launch_slice_dot<S>(L, a, V, kp, kt, alpha, beta, out, dot_partial, st);
   else if (internal) launch_slice_t<false, S>(L, a, V, kp, kp, alpha, beta, out, st);
   else launch_slice_t<true, S>(L, a, src, k, kp, alpha, beta, out, st);
   if (ev) cudaEventRecordWithFlags(ev[3], st, cudaEventRecordExternal);
@@ -1162,10 +1162,10 @@ void enqueue_mvm_bf16_values(const Lattice* L, const float* V, int k, int blur, 
                   L->partial, L->vperm, st, nullptr, /*internal=*/true);
 }
 
-int64_t slice_dot_blocks(const Lattice* L, int k) {
+int64_t slice_dot_blocks(const Lattice* L, int k, int tree_k) {
   const int vec = k % 4 == 0 ? 4 : 1;
   const int G = k / vec;
-  const int T = column_block_threads(k, vec);
+  const int T = column_block_threads(k, vec, tree_k);
   // one wave: as many blocks as the device keeps resident (a grid-stride kernel whose
   // grid exceeds that runs a second, mostly idle wave)
   int per_sm = 0, sms = 0, dev = 0;
