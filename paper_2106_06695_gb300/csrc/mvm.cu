@@ -716,6 +716,22 @@ RowShape row_shape(int64_t rows, int kp) {
   q.blocks = (unsigned)ceil_div(rows, q.threads / q.G);
   return q;
 }
+// The direction lists' kernels read 2 r + 1 rows a vertex one after another, so rows of one thread
+// leave a short list with too few warps: rows of two columns, and short lists of four, go a
+// column a thread.  Log determinants of 15 steps (d = 33, order 3, 10,000 vertices a list):
+// two probes 3.39 ms, 4.06 with two columns a thread; three (rows of four) 3.29, 3.54 with
+// four.  Lists of 54,000 (d = 20, order 2): 2.95 and 3.08 ms, of 80,000 (d = 33, order 3): 7.79 and
+// 6.53.
+RowShape list_shape(int64_t rows, int kp) {
+  RowShape q = row_shape(rows, kp);
+  if (kp == 2 || (kp == 4 && rows <= 1 << 16)) {
+    q.vec = 1;
+    q.G = kp;
+    q.threads = kThreads;
+    q.blocks = (unsigned)ceil_div(rows, kThreads / kp);
+  }
+  return q;
+}
 bool wide_ok(int k, int kp, const void* user) {
   return k == kp && (uintptr_t)user % (kp % 4 == 0 ? 16 : kp == 2 ? 8 : 4) == 0;
 }
@@ -1028,22 +1044,22 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
     return lat0;
   }
   S* tmp = static_cast<S*>(L->act_tmp);
-  by_vec(row_shape(1, k).vec, [&](auto vec) {
-    constexpr int VEC = decltype(vec)::value;
-    for (int t = 0; t < P; ++t) {
-      const int j = dir(t);
-      const int64_t count = L->act_off[j + 1] - L->act_off[j];
-      if (count == 0) continue;
-      const int32_t* act = L->act + L->act_off[j];
-      const int32_t* nbr_j = L->nbr + (size_t)j * L->r * 2 * L->m;
-      const RowShape q = row_shape(count, k);
+  for (int t = 0; t < P; ++t) {
+    const int j = dir(t);
+    const int64_t count = L->act_off[j + 1] - L->act_off[j];
+    if (count == 0) continue;
+    const int32_t* act = L->act + L->act_off[j];
+    const int32_t* nbr_j = L->nbr + (size_t)j * L->r * 2 * L->m;
+    const RowShape q = list_shape(count, k);
+    by_vec(q.vec, [&](auto vec) {
+      constexpr int VEC = decltype(vec)::value;
       launch_pdl(k_sparse_blur<VEC, S>, q.blocks, q.threads, st, count, q.G, k, L->r, tp, t, act,
                  nbr_j, L->m, L->epoch, pw, lat0, tmp);
       launch_pdl(k_sparse_store<VEC, S>, q.blocks, q.threads, st, count, q.G, k, t, act, tmp, lat0,
                  L->epoch);
       note_launches(2);
-    }
-  });
+    });
+  }
   if (pw) finish();
   return lat0;
 }
