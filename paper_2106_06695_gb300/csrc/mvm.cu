@@ -218,7 +218,15 @@ __global__ void __launch_bounds__(kThreads) k_blur_rows(int64_t m, int G, int k,
 // stride (own and both neighbours) and the neighbour ids of v + 2 stride are in flight, so
 // the memory system sees a steady stream instead of one burst per block.  Same arithmetic
 // as k_blur_rows (bitwise equal results).
-template <class S>
+//
+// RO: the rows through the read-only path, not launched as a dependent (the rule at launch_pdl).
+// fp32 values of kReadOnlyBytes or more blur faster so, although a launch costs 2.5 us more:
+// symmetric products, read-only / ordinary loads: m = 2.24M, k = 64 (547 MiB) 6.34 / 7.14 ms, k =
+// 48 (410) 5.01 / 5.11, k = 40 (342) 4.27 / 4.29, k = 32 (273) 3.25 / 3.20, k = 16 (137) 1.79 / 1.72;
+// m = 440k, k = 256 (429) 5.49 / 5.93, k = 192 (322) 4.08 / 4.10.  BF16 ones do not (m = 2.24M, k =
+// 192, 820 MiB: 13.12 / 13.11), nor do rows of k_blur_rows.
+constexpr size_t kReadOnlyBytes = (size_t)350 << 20;
+template <bool RO, class S>
 __global__ void __launch_bounds__(kThreads) k_blur_pipe(int64_t m, int G, int k, Taps tp,
                                                         const int32_t* __restrict__ nbr,
                                                         const S* in,
@@ -239,9 +247,13 @@ __global__ void __launch_bounds__(kThreads) k_blur_pipe(int64_t m, int G, int k,
   };
   auto load = [&](int64_t v, int a, int c, float4 (&x)[3][2]) {  // own, minus, plus rows
     x[0][0] = x[0][1] = x[1][0] = x[1][1] = x[2][0] = x[2][1] = zero;
-    if (v < m) Store<S>::ld8(in + v * k + col, x[0][0], x[0][1]);
-    if (a >= 0) Store<S>::ld8(in + (int64_t)a * k + col, x[1][0], x[1][1]);
-    if (c >= 0) Store<S>::ld8(in + (int64_t)c * k + col, x[2][0], x[2][1]);
+    auto row = [&](int64_t u, float4 (&y)[2]) {
+      if constexpr (RO) Store<S>::ro8(in + u * k + col, y[0], y[1]);
+      else Store<S>::ld8(in + u * k + col, y[0], y[1]);
+    };
+    if (v < m) row(v, x[0]);
+    if (a >= 0) row(a, x[1]);
+    if (c >= 0) row(c, x[2]);
   };
   int a0, c0, a1, c1;
   ids(row, a0, c0);
@@ -276,8 +288,8 @@ __global__ void __launch_bounds__(kThreads) k_blur_pipe(int64_t m, int G, int k,
   }
 }
 
-// Blocks of k_blur_pipe<S> the device keeps resident (one wave), cached per device.
-template <class S>
+// Blocks of k_blur_pipe<RO, S> the device keeps resident (one wave), cached per device.
+template <bool RO, class S>
 int blur_pipe_blocks() {
   static std::atomic<int> cache[64];
   int dev = 0;
@@ -285,7 +297,7 @@ int blur_pipe_blocks() {
   int b = cache[dev].load();
   if (b > 0) return b;
   int per_sm = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_blur_pipe<S>, kThreads, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_blur_pipe<RO, S>, kThreads, 0) !=
           cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     clear_pending_error();
@@ -555,7 +567,10 @@ __global__ void __launch_bounds__(kThreads) k_sparse_finish(int64_t m, int G, in
 
 // ---- slice ---------------------------------------------------------------------------
 // sum_c w[p][c] lat[idx[p][c]] for the VEC columns at col, in vertex order c = 0..D-1,
-// loading the ids and weights of kChunk vertices before their rows.
+// loading the ids and weights of kChunk vertices before their rows.  Where a row's bytes count,
+// the last D % kChunk vertices go in rounds of 4, 2 and 1 without conditions (k_slice, n = 2M, d =
+// 11, k = 64: 420 us, 623 with every load under a condition); with one or two columns the
+// rounds' latency counts (n = 46k, d = 9, k = 1: 33.5 us a product, 34.8 with more rounds).
 template <int VEC, class S>
 __device__ __forceinline__ typename Vec<VEC>::T slice_row(int64_t p, int D, int k, int col,
                                                           const int32_t* __restrict__ idx,
@@ -564,22 +579,51 @@ __device__ __forceinline__ typename Vec<VEC>::T slice_row(int64_t p, int D, int 
   using Vt = Vec<VEC>;
   typename Vt::T acc = Vt::zero();
   const int64_t e0 = p * D;
-  for (int c0 = 0; c0 < D; c0 += kChunk) {
-    int id[kChunk];
-    float wt[kChunk];
+  if constexpr (VEC == 4) {
+    auto run = [&](int c0, auto count) {
+      constexpr int N = decltype(count)::value;
+      int id[N];
+      float wt[N];
 #pragma unroll
-    for (int j = 0; j < kChunk; ++j) {
-      const bool in = c0 + j < D;
-      id[j] = in ? __ldg(idx + e0 + c0 + j) : -1;
-      wt[j] = in ? __ldg(w + e0 + c0 + j) : 0.f;
+      for (int j = 0; j < N; ++j) {
+        id[j] = __ldg(idx + e0 + c0 + j);
+        wt[j] = __ldg(w + e0 + c0 + j);
+      }
+      typename Vt::T row[N];
+#pragma unroll
+      for (int j = 0; j < N; ++j) row[j] = Vt::lds(lat + (int64_t)id[j] * k + col);
+#pragma unroll
+      for (int j = 0; j < N; ++j) acc = Vt::fma(wt[j], row[j], acc);
+    };
+    int c0 = 0;
+    for (; c0 + kChunk <= D; c0 += kChunk) run(c0, std::integral_constant<int, kChunk>{});
+    if (c0 + 4 <= D) {
+      run(c0, std::integral_constant<int, 4>{});
+      c0 += 4;
     }
-    typename Vt::T row[kChunk];
+    if (c0 + 2 <= D) {
+      run(c0, std::integral_constant<int, 2>{});
+      c0 += 2;
+    }
+    if (c0 < D) run(c0, std::integral_constant<int, 1>{});
+  } else {
+    for (int c0 = 0; c0 < D; c0 += kChunk) {
+      int id[kChunk];
+      float wt[kChunk];
 #pragma unroll
-    for (int j = 0; j < kChunk; ++j)
-      row[j] = id[j] >= 0 ? Vt::lds(lat + (int64_t)id[j] * k + col) : Vt::zero();
+      for (int j = 0; j < kChunk; ++j) {
+        const bool in = c0 + j < D;
+        id[j] = in ? __ldg(idx + e0 + c0 + j) : -1;
+        wt[j] = in ? __ldg(w + e0 + c0 + j) : 0.f;
+      }
+      typename Vt::T row[kChunk];
 #pragma unroll
-    for (int j = 0; j < kChunk; ++j)
-      if (id[j] >= 0) acc = Vt::fma(wt[j], row[j], acc);
+      for (int j = 0; j < kChunk; ++j)
+        row[j] = id[j] >= 0 ? Vt::lds(lat + (int64_t)id[j] * k + col) : Vt::zero();
+#pragma unroll
+      for (int j = 0; j < kChunk; ++j)
+        if (id[j] >= 0) acc = Vt::fma(wt[j], row[j], acc);
+    }
   }
   return acc;
 }
@@ -790,8 +834,19 @@ void launch_blur_t(const Lattice* L, int j, const Taps& taps, const S* in, S* ou
   const int32_t* nbr = L->nbr + (size_t)j * L->r * 2 * L->m;
   if (k % 8 == 0 && k / 8 <= kThreads && L->r == 1) {  // eight columns, pipelined rows
     const int G = k / 8, threads = G * (kThreads / G);
-    const int64_t blocks = std::min<int64_t>(blur_pipe_blocks<S>(), ceil_div(L->m, threads / G));
-    launch_pdl(k_blur_pipe<S>, (unsigned)blocks, threads, st, L->m, G, k, taps, nbr, in, out);
+    const int64_t most = ceil_div(L->m, threads / G);
+    bool done = false;
+    if constexpr (std::is_same_v<S, float>) {
+      if ((size_t)L->m * k * sizeof(float) >= kReadOnlyBytes) {  // not as a dependent
+        const unsigned blocks = (unsigned)std::min<int64_t>(blur_pipe_blocks<true, S>(), most);
+        k_blur_pipe<true, S><<<blocks, threads, 0, st>>>(L->m, G, k, taps, nbr, in, out);
+        done = true;
+      }
+    }
+    if (!done) {
+      const unsigned blocks = (unsigned)std::min<int64_t>(blur_pipe_blocks<false, S>(), most);
+      launch_pdl(k_blur_pipe<false, S>, blocks, threads, st, L->m, G, k, taps, nbr, in, out);
+    }
   } else if (k % 8 == 0 && k / 8 <= kThreads) {  // eight columns of two rows per thread
     launch_blur_rows<4, 2, 2, S>(L, nbr, taps, in, out, k, st);
   } else if (k % 4 == 0 && k / 4 <= kThreads) {

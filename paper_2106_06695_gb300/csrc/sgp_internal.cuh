@@ -171,7 +171,8 @@ cudaError_t cols_malloc(const sgp_lattice* L, int columns, void** p, size_t byte
 //    that are const and __restrict__.  Those stand for data that do not change while the kernel
 //    runs, and a dependent runs already while the writer does; the compiler might also move
 //    such a load ahead of the wait.  Only the arrays that are fixed after the build (and the
-//    server's table) are declared so.
+//    server's table) are declared so, and only a kernel that is launched the ordinary way may
+//    load others so (k_blur_pipe<RO = true>).
 // Dependents are not let in early (griddepcontrol.launch_dependents
 // at the top of each kernel): their waiting blocks take slots from the running grid (a
 // product at n = 50k, d = 8, k = 9: 63 us without, 78 us with it; eight CG iterations at n =

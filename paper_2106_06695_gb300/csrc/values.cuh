@@ -25,6 +25,11 @@ struct Store<float> {
     a = reinterpret_cast<const float4*>(p)[0];
     b = reinterpret_cast<const float4*>(p)[1];
   }
+  // Read-only path: for data that no running grid writes.
+  static __device__ __forceinline__ void ro8(const float* p, float4& a, float4& b) {
+    a = __ldg(reinterpret_cast<const float4*>(p));
+    b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  }
   static __device__ __forceinline__ void st8(float* p, float4 a, float4 b) {
     reinterpret_cast<float4*>(p)[0] = a;
     reinterpret_cast<float4*>(p)[1] = b;
@@ -65,6 +70,11 @@ struct Store<bf16> {
   }
   static __device__ __forceinline__ void ld8(const bf16* p, float4& a, float4& b) {
     const uint4 u = *reinterpret_cast<const uint4*>(p);
+    a = cvt(make_uint2(u.x, u.y));
+    b = cvt(make_uint2(u.z, u.w));
+  }
+  static __device__ __forceinline__ void ro8(const bf16* p, float4& a, float4& b) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
     a = cvt(make_uint2(u.x, u.y));
     b = cvt(make_uint2(u.z, u.w));
   }

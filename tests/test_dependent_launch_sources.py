@@ -42,9 +42,23 @@ def test_every_kernel_waits(name):
         assert "pdl_enter()" in body or "SLOT_AHEAD_IN_LOOP" in body, kernel
 
 
+def test_read_only_rows_are_for_ordinary_launches():
+    """The read-only loads of lattice rows (ro8) stand under RO alone, in one kernel, and that
+    instance is never launched as a dependent."""
+    for name, text in SOURCES.items():
+        if name != "values.cuh":
+            for line in text.splitlines():
+                assert "ro8(" not in line or "if constexpr (RO)" in line, line
+    mvm = SOURCES["mvm.cu"]
+    assert mvm.count("k_blur_pipe<true, S><<<") == 1
+    assert not re.search(r"launch_pdl\w*\([^;]*<true, S>", mvm)
+
+
 @pytest.mark.parametrize("name", sorted(SOURCES))
 def test_read_only_path_is_for_fixed_arrays(name):
     fixed = set() if name == "build.cu" else FIXED  # the build itself writes all of them
+    if name == "values.cuh":
+        fixed = fixed | {"p"}  # ro8
     for pointer in re.findall(r"const [\w ]+\* ?__restrict__ (\w+)", SOURCES[name]):
         assert pointer in fixed, pointer
     for pointer in re.findall(r"__ldg\(\(?(?:reinterpret_cast<[^>]*>\()?(\w+)", SOURCES[name]):
