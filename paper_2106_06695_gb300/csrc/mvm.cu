@@ -570,8 +570,10 @@ __global__ void __launch_bounds__(kThreads) k_sparse_finish(int64_t m, int G, in
 // loading the ids and weights of kChunk vertices before their rows.  Where a row's bytes count,
 // the last D % kChunk vertices go in rounds of 4, 2 and 1 without conditions (k_slice, n = 2M, d =
 // 11, k = 64: 420 us, 623 with every load under a condition); with one or two columns the
-// rounds' latency counts (n = 46k, d = 9, k = 1: 33.5 us a product, 34.8 with more rounds).
-template <int VEC, class S>
+// rounds' latency counts (n = 46k, d = 9, k = 1: 33.5 us a product, 34.8 with more rounds), and
+// the CG's slice of BF16 values keeps more loads in flight with conditions (n = 200k, d = 33: 62 us,
+// 97 without).
+template <int VEC, bool EXACT, class S>
 __device__ __forceinline__ typename Vec<VEC>::T slice_row(int64_t p, int D, int k, int col,
                                                           const int32_t* __restrict__ idx,
                                                           const float* __restrict__ w,
@@ -579,7 +581,7 @@ __device__ __forceinline__ typename Vec<VEC>::T slice_row(int64_t p, int D, int 
   using Vt = Vec<VEC>;
   typename Vt::T acc = Vt::zero();
   const int64_t e0 = p * D;
-  if constexpr (VEC == 4) {
+  if constexpr (EXACT) {
     auto run = [&](int c0, auto count) {
       constexpr int N = decltype(count)::value;
       int id[N];
@@ -644,7 +646,7 @@ __global__ void __launch_bounds__(kThreads) k_slice(int64_t n, int G, int k, int
   const int64_t p = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
   if (p >= n) return;
   const int col = (int)(threadIdx.x % G) * VEC;
-  const typename Vt::T acc = slice_row<VEC, S>(p, D, k, col, idx, w, lat);
+  const typename Vt::T acc = slice_row<VEC, VEC == 4, S>(p, D, k, col, idx, w, lat);
   const int64_t i = PERM ? (int64_t)perm[p] : p;
   typename Vt::T res = Vt::scale(alpha, acc);
   if (beta != 0.f) res = Vt::fma(beta, Vt::ld(Vp + p * k + col), res);
@@ -678,7 +680,8 @@ __global__ void __launch_bounds__(kThreads) k_slice_dot(int64_t n, int G, int k,
   for (int j = 0; j < VEC; ++j) d[j] = {0.f, 0.f};
   for (int64_t p = (int64_t)blockIdx.x * rows + threadIdx.x / G; p < n;
        p += (int64_t)gridDim.x * rows) {
-    const typename Vt::T acc = slice_row<VEC, S>(p, D, k, col, idx, w, lat);
+    const typename Vt::T acc =
+        slice_row<VEC, VEC == 4 && std::is_same_v<S, float>, S>(p, D, k, col, idx, w, lat);
     const typename Vt::T v = Vt::ld(V + p * k + col);
     const typename Vt::T res = Vt::fma(beta, v, Vt::scale(alpha, acc));
     Vt::st(out + p * k + col, res);
