@@ -1057,7 +1057,7 @@ __global__ void __launch_bounds__(kMinvT) kb_minv(const Table* __restrict__ T) {
   if (o < cnt && j < l) {
     const double* row = s.Minv + (int64_t)j * l;
     const double* tv = s.tvec + c;
-    for (int i0 = part; i0 < l; i0 += 4 * 13) {  // 13 terms loaded ahead (l = 100: two rounds)
+    for (int i0 = part; i0 < l; i0 += 4 * 13) {  // 13 ahead: the default rank 100 in two rounds, 128 in three
       double m[13], t[13];
 #pragma unroll
       for (int u = 0; u < 13; ++u) {
