@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kBT) k_weight_grad(int64_t n, int d, int k, in
                                                      const S* BU,
                                                      const S* BS,
                                                      const float* Vp,
-                                                     const float* Gp, float alpha,
+                                                     const float* Gp, dfloat alpha,
                                                      const double* f,
                                                      const float* ls,
                                                      float* __restrict__ dX) {
@@ -83,7 +83,8 @@ __global__ void __launch_bounds__(kBT) k_weight_grad(int64_t n, int d, int k, in
   float dw[MAXD];
   for (int kk = 0; kk < D; ++kk) {
     const int64_t v = idx[p * D + kk];
-    dw[kk] = alpha * row_dot2<S, VEC>(Gp + p * ld, BU + v * ld, Vp + p * ld, BS + v * ld, k);
+    const float dot = row_dot2<S, VEC>(Gp + p * ld, BU + v * ld, Vp + p * ld, BS + v * ld, k);
+    dw[kk] = alpha.lo != 0.f ? fmaf(alpha.hi, dot, alpha.lo * dot) : alpha.hi * dot;
   }
   double dy[MAXD];
   for (int c = 0; c < D; ++c) {
@@ -226,7 +227,7 @@ struct Work {
 
 template <class S, int VEC>
 void launch_weight_grad(const Lattice* L, int k, int ld, const void* BU, const void* BS, const float* Vp,
-                        const float* Gp, float alpha, const double* f, const float* ls, float* dX,
+                        const float* Gp, dfloat alpha, const double* f, const float* ls, float* dX,
                         cudaStream_t st) {
   const unsigned grid = (unsigned)ceil_div(L->n, kBT);
   const int D = L->D;
@@ -301,8 +302,8 @@ sgp_status backward(Lattice* L, const float* X, const float* ls, const float* V,
       enqueue_permute(L, G, k, kp, Gp, st);
       BS = enqueue_splat_blur(L, Gp, kp, k, transpose_blur(blur), b0, b1, L->partial, st, &scale);
     }
-    alpha = (float)(alpha * scale);
-    if (dV) enqueue_slice_caller(L, BS, k, kp, ld, alpha, dV, st);
+    const dfloat factor = split_factor(alpha * scale);
+    if (dV) enqueue_slice_caller(L, BS, k, kp, ld, factor, dV, st);
     if (want_x) {
       if (!pair) {
         enqueue_permute(L, V, k, kp, Vp, st);
@@ -318,11 +319,11 @@ sgp_status backward(Lattice* L, const float* X, const float* ls, const float* V,
                "copy f");
       const bool v4 = kp % 4 == 0;
       if (L->value_dtype == SGP_VALUES_BF16) {
-        if (v4) launch_weight_grad<bf16, 4>(L, kp, ld, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
-        else launch_weight_grad<bf16, 1>(L, kp, ld, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
+        if (v4) launch_weight_grad<bf16, 4>(L, kp, ld, BU, BS, Vp, Gp, factor, f, ls, dXw, st);
+        else launch_weight_grad<bf16, 1>(L, kp, ld, BU, BS, Vp, Gp, factor, f, ls, dXw, st);
       } else {
-        if (v4) launch_weight_grad<float, 4>(L, kp, ld, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
-        else launch_weight_grad<float, 1>(L, kp, ld, BU, BS, Vp, Gp, alpha, f, ls, dXw, st);
+        if (v4) launch_weight_grad<float, 4>(L, kp, ld, BU, BS, Vp, Gp, factor, f, ls, dXw, st);
+        else launch_weight_grad<float, 1>(L, kp, ld, BU, BS, Vp, Gp, factor, f, ls, dXw, st);
       }
     }
   } else {  // SGP_GRAD_FILTER

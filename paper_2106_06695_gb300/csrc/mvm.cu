@@ -486,15 +486,24 @@ __global__ void __launch_bounds__(kThreads) k_chain_blur(int64_t chains, int G, 
   }
 }
 
+// (a.hi + a.lo) x with one rounding of the result: an fp32 factor alone would put its own rounding
+// error, up to 6e-8, on every value alike.  a.lo = 0 but where the blur leaves a power of the
+// centre tap to the factor.
+template <int VEC>
+__device__ __forceinline__ typename Vec<VEC>::T times(dfloat a, typename Vec<VEC>::T x) {
+  using Vt = Vec<VEC>;
+  return a.lo != 0.f ? Vt::fma(a.hi, x, Vt::scale(a.lo, x)) : Vt::scale(a.hi, x);
+}
+
 template <int VEC, class S>
-__global__ void __launch_bounds__(kThreads) k_rescale(int64_t m, int G, int k, float f,
+__global__ void __launch_bounds__(kThreads) k_rescale(int64_t m, int G, int k, dfloat f,
                                                       S* __restrict__ vals) {
   pdl_enter();
   using Vt = Vec<VEC>;
   const int64_t v = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
   if (v >= m) return;
   S* p = vals + v * k + (int)(threadIdx.x % G) * VEC;
-  Vt::sts(p, Vt::scale(f, Vt::lds(p)));
+  Vt::sts(p, times<VEC>(f, Vt::lds(p)));
 }
 
 // The general form (stencil orders above 1, chains longer than kMaxChain): stored rows carry
@@ -639,7 +648,7 @@ __global__ void __launch_bounds__(kThreads) k_slice(int64_t n, int G, int k, int
                                                     const int32_t* __restrict__ idx,
                                                     const float* __restrict__ w,
                                                     const S* lat,
-                                                    const float* Vp, float alpha,
+                                                    const float* Vp, dfloat alpha,
                                                     float beta, float* __restrict__ out) {
   pdl_enter();
   using Vt = Vec<VEC>;
@@ -648,7 +657,7 @@ __global__ void __launch_bounds__(kThreads) k_slice(int64_t n, int G, int k, int
   const int col = (int)(threadIdx.x % G) * VEC;
   const typename Vt::T acc = slice_row<VEC, VEC == 4, S>(p, D, k, col, idx, w, lat);
   const int64_t i = PERM ? (int64_t)perm[p] : p;
-  typename Vt::T res = Vt::scale(alpha, acc);
+  typename Vt::T res = times<VEC>(alpha, acc);
   if (beta != 0.f) res = Vt::fma(beta, Vt::ld(Vp + p * k + col), res);
   if constexpr (!PERM || WIDE) {
     Vt::st(out + i * (PERM ? ko : k) + col, res);
@@ -668,7 +677,7 @@ __global__ void __launch_bounds__(kThreads) k_slice_dot(int64_t n, int G, int k,
                                                         const int32_t* __restrict__ idx,
                                                         const float* __restrict__ w,
                                                         const S* lat,
-                                                        const float* V, float alpha,
+                                                        const float* V, dfloat alpha,
                                                         float beta, float* __restrict__ out,
                                                         double* __restrict__ dot_partial) {
   pdl_enter();
@@ -683,7 +692,7 @@ __global__ void __launch_bounds__(kThreads) k_slice_dot(int64_t n, int G, int k,
     const typename Vt::T acc =
         slice_row<VEC, VEC == 4 && std::is_same_v<S, float>, S>(p, D, k, col, idx, w, lat);
     const typename Vt::T v = Vt::ld(V + p * k + col);
-    const typename Vt::T res = Vt::fma(beta, v, Vt::scale(alpha, acc));
+    const typename Vt::T res = Vt::fma(beta, v, times<VEC>(alpha, acc));
     Vt::st(out + p * k + col, res);
     const float* vv = reinterpret_cast<const float*>(&v);
     const float* rr = reinterpret_cast<const float*>(&res);
@@ -868,7 +877,7 @@ void launch_blur_t(const Lattice* L, int j, const Taps& taps, const S* in, S* ou
 // out = alpha W lat + beta Vp (Vp in locality order, rows of kp).  PERM: out is the caller's
 // [n][k]; else [n][kp] in locality order.  lat_cols: columns of a row of lat (0: kp).
 template <bool PERM, class S>
-void launch_slice_t(const Lattice* L, const S* lat, const float* Vp, int k, int kp, float alpha,
+void launch_slice_t(const Lattice* L, const S* lat, const float* Vp, int k, int kp, dfloat alpha,
                     float beta, float* out, cudaStream_t st, int lat_cols = 0) {
   if (lat_cols == 0) lat_cols = kp;
   const RowShape q = row_shape(L->n, kp);
@@ -886,7 +895,7 @@ void launch_slice_t(const Lattice* L, const S* lat, const float* Vp, int k, int 
 }
 
 template <class S>
-void launch_slice_dot(const Lattice* L, const S* lat, const float* V, int k, int kt, float alpha,
+void launch_slice_dot(const Lattice* L, const S* lat, const float* V, int k, int kt, dfloat alpha,
                       float beta, float* out, double* dot_partial, cudaStream_t st) {
   const int vec = k % 4 == 0 ? 4 : 1;
   const int T = column_block_threads(k, vec, kt);
@@ -1080,7 +1089,7 @@ S* blur_passes_t(const Lattice* L, int blur, S* lat0, S* lat1, int k, cudaStream
         if (range.run > 0 && owed == range.run) {
           const RowShape q = row_shape(L->m, k);
           launch_pdl(k_rescale<VEC, S>, q.blocks, q.threads, st, L->m, q.G, k,
-                     (float)std::pow(g0, owed), lat0);
+                     split_factor(std::pow(g0, owed)), lat0);
           note_launches(1);
           owed = 0;
         }
@@ -1143,11 +1152,11 @@ int enqueue_t(const Lattice* L, const float* V, int k, int kp, int kt, int blur,
   int passes = 0;
   double scale = 1.0;
   S* a = blur_passes_t<S>(L, blur, lat0, lat1, kp, st, &passes, dense, &scale);
-  alpha = (float)(alpha * scale);
+  const dfloat factor = split_factor(alpha * scale);
   if (ev) cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal);
-  if (internal && dot_partial) launch_slice_dot<S>(L, a, V, kp, kt, alpha, beta, out, dot_partial, st);
-  else if (internal) launch_slice_t<false, S>(L, a, V, kp, kp, alpha, beta, out, st);
-  else launch_slice_t<true, S>(L, a, src, k, kp, alpha, beta, out, st);
+  if (internal && dot_partial) launch_slice_dot<S>(L, a, V, kp, kt, factor, beta, out, dot_partial, st);
+  else if (internal) launch_slice_t<false, S>(L, a, V, kp, kp, factor, beta, out, st);
+  else launch_slice_t<true, S>(L, a, src, k, kp, factor, beta, out, st);
   if (ev) cudaEventRecordWithFlags(ev[3], st, cudaEventRecordExternal);
   return passes;
 }
@@ -1305,7 +1314,7 @@ void enqueue_permute_pair(const Lattice* L, const float* A, const float* B, int 
 bool blur_in_place(const Lattice* L) { return L->sparse && chains_ok(L); }
 
 void enqueue_slice_caller(const Lattice* L, const void* lat, int k, int kp, int lat_cols,
-                          float alpha, float* out, cudaStream_t st) {
+                          dfloat alpha, float* out, cudaStream_t st) {
   if (L->value_dtype == SGP_VALUES_BF16)
     launch_slice_t<true, bf16>(L, (const bf16*)lat, nullptr, k, kp, alpha, 0.f, out, st, lat_cols);
   else

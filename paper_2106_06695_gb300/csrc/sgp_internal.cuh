@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
 #include <string>
 #include <utility>
 #include <vector>
@@ -138,6 +139,17 @@ struct sgp_lattice {
 namespace sgp {
 
 using Lattice = ::sgp_lattice;
+
+// An unevaluated sum of two fp32 numbers (the arithmetic stands below).
+struct dfloat {
+  float hi, lo;
+};
+// A factor to 48 bits; lo = 0 for an fp32 number.
+inline dfloat split_factor(double x) {
+  const float hi = (float)x;
+  const float lo = (float)(x - (double)hi);
+  return {hi, std::isfinite(lo) ? lo : 0.f};
+}
 
 // ---- error reporting and launch accounting (api.cu) ----
 void set_error(const std::string& msg);
@@ -281,7 +293,7 @@ void enqueue_permute_pair(const Lattice* L, const float* A, const float* B, int 
                           float* out, cudaStream_t st);
 bool blur_in_place(const Lattice* L);  // enqueue_splat_blur needs no second buffer (lat1)
 void enqueue_slice_caller(const Lattice* L, const void* lat, int k, int kp, int lat_cols,
-                          float alpha, float* out, cudaStream_t st);
+                          dfloat alpha, float* out, cudaStream_t st);
 size_t lattice_value_bytes(const Lattice* L, int k);
 // Full operator on the handle's stream, allocating value buffers when needed.
 sgp_status run_mvm(Lattice* L, const float* V, int k, int blur, float alpha, float beta,
@@ -457,9 +469,6 @@ __device__ __forceinline__ bool cg_stops(double rr, double bnorm, float tol) {
 // transformations: TwoSum (Knuth), FastTwoSum (Dekker, |a| >= |b|) and TwoProd through a
 // fused multiply-add.  The _rn intrinsics keep the compiler from contracting or
 // reordering the steps.  About 48 significant bits.
-struct dfloat {
-  float hi, lo;
-};
 
 __device__ __forceinline__ dfloat df_two_sum(float a, float b) {
   const float s = __fadd_rn(a, b);
