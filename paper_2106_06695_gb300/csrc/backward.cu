@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kBT) k_weight_grad(int64_t n, int d, int k, in
   for (int kk = 0; kk < D; ++kk) {
     const int64_t v = idx[p * D + kk];
     const float dot = row_dot2<S, VEC>(Gp + p * ld, BU + v * ld, Vp + p * ld, BS + v * ld, k);
-    dw[kk] = alpha.lo != 0.f ? fmaf(alpha.hi, dot, alpha.lo * dot) : alpha.hi * dot;
+    dw[kk] = df_times(alpha, dot);
   }
   double dy[MAXD];
   for (int c = 0; c < D; ++c) {

@@ -486,13 +486,13 @@ __global__ void __launch_bounds__(kThreads) k_chain_blur(int64_t chains, int G, 
   }
 }
 
-// (a.hi + a.lo) x with one rounding of the result: an fp32 factor alone would put its own rounding
-// error, up to 6e-8, on every value alike.  a.lo = 0 but where the blur leaves a power of the
-// centre tap to the factor.
+// df_times on VEC columns.
 template <int VEC>
 __device__ __forceinline__ typename Vec<VEC>::T times(dfloat a, typename Vec<VEC>::T x) {
-  using Vt = Vec<VEC>;
-  return a.lo != 0.f ? Vt::fma(a.hi, x, Vt::scale(a.lo, x)) : Vt::scale(a.hi, x);
+  float* v = reinterpret_cast<float*>(&x);
+#pragma unroll
+  for (int j = 0; j < VEC; ++j) v[j] = df_times(a, v[j]);
+  return x;
 }
 
 template <int VEC, class S>

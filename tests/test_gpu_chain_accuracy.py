@@ -38,3 +38,27 @@ def test_common_factor(d):
     f = factor(out, want), factor(dV, ref.mvm(G.astype(np.float64), mode=2))
     print("d=%d: product 1 %+.1e, dV 1 %+.1e" % (d, f[0] - 1, f[1] - 1))
     assert max(abs(x - 1) for x in f) <= 1e-8
+
+
+@pytest.mark.parametrize("d", [14, 20, 90])
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+def test_infinities_stay(d, value):
+    """An entry that is not finite reaches the points that share vertices with it, as it is (all
+    taps and weights are positive); the others keep their bits."""
+    n = 300
+    X = synth.gmm_points(n, d, 7)
+    ref = OracleLattice(X, np.ones(d, np.float32))
+    lat = Lattice(gpu(X), 1.0, spacing=ref.s)
+    assert lat.sparse_blur
+    one = np.zeros((n, 1))
+    one[n // 2] = 1.0
+    V = synth.gaussian_values(n, 1, 3)
+    W = V.copy()
+    W[n // 2] = value
+    for blur, mode in (("symmetric", 2), ("sequential", 0)):
+        got = lat.mvm(gpu(W), blur=blur).cpu().numpy()
+        other = lat.mvm(gpu(V), blur=blur).cpu().numpy()
+        hit = ref.mvm(one, mode=mode) != 0.0
+        assert np.array_equal(got[~hit], other[~hit])
+        assert hit[n // 2] and np.array_equal(got[hit], np.full(hit.sum(), value, np.float32),
+                                              equal_nan=True)
